@@ -117,6 +117,12 @@ struct CompressPlan {
 };
 CompressPlan make_compress_plan(int64_t n, int64_t k, dropit_dtype dtype);
 
+// Tensors of up to this many elements are compressed by one thread-block cluster (compress_small.cu).  Returns false if
+// the tensor is larger or the device has no room for such a cluster; 0 < k <= n.
+constexpr int64_t kSmallMaxElems = 1 << 19;
+bool small_compress(const void* x, int64_t n, int64_t k, dropit_dtype dtype, bool index32, void* values, void* meta,
+                    uint32_t* offsets, cudaStream_t stream, dropit_status* status);
+
 inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s); }
 
 // Kernel launches enqueued by this library since it was loaded (diagnostic counter).

@@ -569,6 +569,8 @@ extern "C" dropit_status dropit_compress(const void* x, int64_t n, double gamma,
                                    workspace_bytes, dev_status, stream);
     const CompressPlan plan = make_compress_plan(n, k, dtype);
     if (workspace_bytes < plan.total_bytes) return DROPIT_ERR_WORKSPACE;
+    dropit_status s;   // three digit passes and a tiled compaction are for tensors that outgrow one cluster
+    if (small_compress(x, n, k, dtype, format == DROPIT_FMT_INDEX32, values, meta, offsets, stream, &s)) return s;
 
     unsigned char* ws = reinterpret_cast<unsigned char*>(workspace);
     SelectState* st = reinterpret_cast<SelectState*>(ws);
@@ -576,7 +578,7 @@ extern "C" dropit_status dropit_compress(const void* x, int64_t n, double gamma,
     unsigned long long* desc = reinterpret_cast<unsigned long long*>(ws + plan.desc_offset);
     if (cudaMemsetAsync(ws, 0, plan.total_bytes, stream) != cudaSuccess) return DROPIT_ERR_CUDA;
 
-    dropit_status s = launch_hist<F32Traits, 11, 20, 0, true, false>(x, n, k, st, hist, stream);
+    s = launch_hist<F32Traits, 11, 20, 0, true, false>(x, n, k, st, hist, stream);
     if (s != DROPIT_OK) return s;
     s = launch_hist<F32Traits, 10, 10, 1, false, false>(x, n, k, st, hist + 2048, stream);
     if (s != DROPIT_OK) return s;

@@ -40,7 +40,7 @@ constexpr int kWarpBins = 64;                                  // per-warp band 
 constexpr int kRowWords = kWarpBins + 2;                       // per-CTA row: bins, #key>hi, pad
 constexpr int kMaxGrid = 512;                                  // < 4096: departures are counted in 12 bits of the barrier word
 constexpr int kSampleVecs = 2048;                              // 16384 sampled elements
-constexpr int64_t kSampleMinElems = 1 << 19;                   // below this the band is the full key range
+constexpr int64_t kSampleMinElems = kSmallMaxElems;            // below this the band is the full key range (the call normally goes to compress_small.cu)
 constexpr int kBarrierSpinLimit = 1 << 22;
 constexpr uint32_t kHiBits = 0x80008000u;
 // The streaming passes work on super-blocks of two blocks (1024 elements): a lane owns 32 CONSECUTIVE
@@ -1010,6 +1010,9 @@ dropit_status fused_compress_bf16_prepared(const void* x, int64_t n, int64_t k, 
                                            int32_t* dev_status, cudaStream_t stream, const unsigned char* prep) {
     const FusedPlan plan = make_fused_plan(n);
     if (workspace_bytes < plan.total_bytes) return DROPIT_ERR_WORKSPACE;
+    dropit_status small_status;   // a tensor too small to be sampled
+    if (n <= kSmallMaxElems && small_compress(x, n, k, DROPIT_BF16, index32, values, meta, offsets, stream, &small_status))
+        return small_status;
     unsigned char* ws = reinterpret_cast<unsigned char*>(workspace);
     static_assert(kRingBytes >= (size_t)kKeySpace * 4, "the sample's and the general path's histogram live in the ring's memory");
     const size_t smem_mask = kRingBytes + kStageBytes + sizeof(FusedShared);

@@ -1,0 +1,33 @@
+"""One-cluster selection (tensors of up to 2^19 elements): bit-exact against the oracle where its work partition changes."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2202_13808_b200 as dropit
+from _parity import assert_cache_matches_oracle, oracle_cache
+
+pytestmark = pytest.mark.gpu
+
+# one CTA / two CTAs / the full cluster, its last element and the first size that another kernel takes; ragged in between
+SIZES = [8 * 1024, 8 * 1024 + 1, 16 * 8 * 1024, 16 * 8 * 1024 + 1023, 300_007, (1 << 19) - 1, 1 << 19, (1 << 19) + 1]
+
+
+def _draw(n, law, dtype):
+    g = torch.Generator().manual_seed(n)
+    if law == "normal":
+        return torch.randn(n, generator=g).to(dtype)
+    if law == "relu":        # half zeros: the threshold falls inside the ties at gamma = 0.3
+        return torch.relu(torch.randn(n, generator=g)).to(dtype)
+    return torch.randint(0, 3, (n,), generator=g).to(dtype)     # three levels: every digit round ends in one bin
+
+
+@pytest.mark.parametrize("fmt", ["bitmask", "index32"])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32], ids=["bf16", "f32"])
+@pytest.mark.parametrize("n", SIZES)
+def test_small_tensors_match_the_oracle(cuda_device, n, dtype, fmt):
+    for law, gamma in (("normal", 0.9), ("relu", 0.3), ("levels", 0.5)):
+        x = _draw(n, law, dtype)
+        bits, dt, keep, k = oracle_cache(x, gamma)
+        cache = dropit.dropit_compress(x.to(cuda_device), gamma, fmt)
+        dropit.check_device_status(cuda_device)
+        assert_cache_matches_oracle(cache, bits, dt, keep, k, fmt)
