@@ -292,9 +292,10 @@ dropit_status dropit_conv_weight_grad_workspace(int B, int Ca, int H, int W, int
  *   dy [device, B x Cz x Ho x Wo, dtype] with Ho = (H + 2 pad - R)/stride + 1,
  *   Wo likewise; values/meta/offsets [device] = cache of a [B x Ca x H x W];
  *   dw [device, Cz x Ca x R x S, float], overwritten or accumulated into.
- * bf16 with S <= 7 (and Wo <= W when stride is 1) runs on the tensor cores (one implicit GEMM per
- * filter tap over (n, y, x), fp32 accumulation, fixed summation order); other shapes and
- * fp32 inputs use an fp32 FMA kernel.  A bounded device wait that expires is reported
+ * bf16 bitmask caches with filters of up to 3 x 3 and stride 1 or 2 are multiplied on the tensor cores
+ * straight from the cache; other bf16 shapes with S <= 7 (and Wo <= W when stride is 1) on the tensor
+ * cores from dense copies (one implicit GEMM per filter tap over (n, y, x)); fp32 accumulation and a
+ * fixed summation order either way.  The rest and fp32 inputs use an fp32 FMA kernel.  A bounded device wait that expires is reported
  * through dev_status as DROPIT_ERR_TIMEOUT.
  */
 dropit_status dropit_conv_weight_grad(const void* dy, const void* values, const void* meta, const uint32_t* offsets,

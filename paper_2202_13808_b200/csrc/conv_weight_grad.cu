@@ -18,6 +18,19 @@ dropit_status conv_tc_run(const void* dy, const void* values, const void* meta, 
                           float* dw, int accumulate, void* workspace, size_t workspace_bytes, int32_t* dev_status,
                           cudaStream_t stream);
 
+// Straight from a bitmask cache (bf16, filters of up to 3 x 3), defined in conv_weight_grad_fused.cu.  It takes every shape
+// it can but one: a 1 x 1 filter of stride 1 on planes of whole 16-byte groups is a plain GEMM on the decompressed tensor
+// without any further copy, and the dense path's TMA tiles then beat the producer warps (64 x 256 x 56 x 56 -> 64: 55 against
+// 68 us, 64 -> 256: 38 against 72).
+size_t conv_fused_workspace_bytes(int B, int Ca, int H, int W, int Cz, int R, int S, int stride, int pad);
+dropit_status conv_fused_run(const void* dy, const void* values, const void* mask, const uint32_t* offsets, int B, int Ca, int H,
+                             int W, int Cz, int R, int S, int stride, int pad, int64_t k, float* dw, int accumulate,
+                             void* workspace, size_t workspace_bytes, int32_t* dev_status, cudaStream_t stream);
+static bool conv_fused_takes(int H, int W, int R, int S, int stride, int pad, dropit_dtype dtype, dropit_format format) {
+    if (dtype != DROPIT_BF16 || format != DROPIT_FMT_BITMASK) return false;
+    return !(R == 1 && S == 1 && stride == 1 && pad == 0 && (int64_t)H * W % 8 == 0);
+}
+
 constexpr int kConvTJ = 32;     // output channels per block
 constexpr int kConvTC = 8;      // input channels per block
 constexpr int kConvMaxUV = 9;   // filter taps accumulated per sweep
@@ -156,6 +169,12 @@ extern "C" dropit_status dropit_conv_weight_grad_workspace(int B, int Ca, int H,
     if ((dtype != DROPIT_BF16 && dtype != DROPIT_F32) || (format != DROPIT_FMT_BITMASK && format != DROPIT_FMT_INDEX32))
         return DROPIT_ERR_INVALID_ARG;
     if (workspace_bytes) {
+        const size_t fused = (B > 0 && conv_fused_takes(H, W, R, S, stride, pad, dtype, format))
+                                 ? conv_fused_workspace_bytes(B, Ca, H, W, Cz, R, S, stride, pad) : 0;
+        if (fused) {
+            *workspace_bytes = fused;
+            return DROPIT_OK;
+        }
         const size_t tc = (B > 0) ? conv_tc_workspace_bytes(B, Ca, H, W, Cz, R, S, stride, pad, dtype) : 0;
         const ConvPlan p = make_conv_plan(B, Ca, H, W, Cz, R, S, stride, pad, dtype);
         *workspace_bytes = tc ? tc : (p.total_bytes ? p.total_bytes : 256);
@@ -186,6 +205,11 @@ extern "C" dropit_status dropit_conv_weight_grad(const void* dy, const void* val
         return DROPIT_ERR_INVALID_ARG;
     if (format == DROPIT_FMT_BITMASK && (!offsets || !is_aligned16(offsets))) return DROPIT_ERR_INVALID_ARG;
     if (!workspace || !is_aligned16(workspace)) return DROPIT_ERR_INVALID_ARG;
+    if (conv_fused_takes(H, W, R, S, stride, pad, dtype, format)) {
+        s = conv_fused_run(dy, values, meta, offsets, B, Ca, H, W, Cz, R, S, stride, pad, k, dw, accumulate, workspace,
+                           workspace_bytes, dev_status, stream);
+        if (s != DROPIT_ERR_UNSUPPORTED) return s;
+    }
     if (conv_tc_workspace_bytes(B, Ca, H, W, Cz, R, S, stride, pad, dtype) != 0)
         return conv_tc_run(dy, values, meta, offsets, B, Ca, H, W, Cz, R, S, stride, pad, k, format, dw, accumulate,
                            workspace, workspace_bytes, dev_status, stream);

@@ -1,0 +1,616 @@
+// Conv2d weight gradient straight from the compressed cache (Eq. 4-5, retained term), bf16, filters of up to 3 x 3:
+//   dW[j,c,u,v] = sum_{n,y,x} dY[n,j,y,x] * R(a-hat)[n,c, y*stride+u-pad, x*stride+v-pad]
+//
+// No dense copy of the input exists in global memory.  A CTA owns 128 output channels j and a block of input channels, walks
+// over bands of image rows (or whole small images), and for every band its producer warps
+//   * inflate the band's piece of R(a-hat) into shared memory: a lane owns a pixel and builds the 16 bytes of its eight
+//     channels from eight mask words (each the same for the whole warp), reading the retained values with predicated loads
+//     that are contiguous over the warp, so that one 16-byte store per lane writes zeros and values alike,
+//   * transpose the band of dY into shared memory (8 channels x 8 pixels per lane, in registers),
+// while one thread feeds the previous band to tcgen05.mma.  Both operands lie pixel-major: 8 channels (16 bytes) of
+// consecutive pixels of one image row follow one another,
+//   address = row * row_pitch + (channel / 8) * group_pitch + pixel * 16 + (channel % 8) * 2,
+// which is the canonical MN-major layout without swizzle.  In it
+//   * the horizontal tap offset v is a start address 16 * v bytes further on (no shifted copies: with the 128-byte swizzle
+//     or with pixels innermost an offset of one pixel could not be expressed),
+//   * the filter rows u are extra columns of the product: row_pitch = (channels / 8) * group_pitch, so the column groups
+//     behind the block's last one are the next image row, and N = R * channels in one instruction,
+//   * rows need no common multiple: the two 8-pixel halves of a K = 16 step may lie in different rows (the descriptor's
+//     K stride says how far apart they are).
+// Stride 2 keeps the even and the odd padded columns in separate planes.  The reduction is split over the CTAs; every split
+// stores its accumulator as it comes out of tensor memory and a second kernel adds the splits in order.
+//
+// Bound by the producers: a band is two dependent trips to memory (mask and table entry, then values) and some 130 warp
+// instructions per 32 pixels x 8 channels; the MMAs take a third to a half of the time.  20 producer warps: 16 are slower
+// where rows are long (3 x 3 on 56 x 56: 56 against 50 us), 24 spill.  Against the dense copies of conv_weight_grad_tc.cu
+// (decompression, shifted or gathered copies, GEMM on 64-pixel rows; per call at batch 64, gamma 0.8, graph replay): 3 x 3
+// 64 -> 64 on 56 x 56 59 -> 50 us, 128 -> 128 on 28 x 28 130 -> 46, 256 -> 256 on 14 x 14 126 -> 51, 512 -> 512 on 7 x 7
+// 332 -> 93, stride 2 128 -> 128 on 56 x 56 212 -> 70; 1 x 1 1024 -> 256 on 14 x 14 113 -> 54.
+#include "weight_grad_common.cuh"
+
+namespace dropit {
+
+namespace {
+
+constexpr int kProdWarps = 20;
+constexpr int kThreads = 32 * (kProdWarps + 1);      // producer warps, then the MMA warp
+constexpr int kMaxStages = 4;
+constexpr int kMaxPairs = 64;                        // K = 16 steps of a band
+constexpr size_t kSmemBudget = 222 * 1024;
+
+struct FusedConvParams {
+    int B, Ca, H, W, Cz, Ho, Wo;                     // flat (1x1, stride 1): H = Ho = 1, W = Wo = pixels of the plane
+    int R, S, stride, pad;
+    int cb, mt;                                      // channels per block (multiple of 16), rows of dY kept per band (64 or 128)
+    int flat;
+    int yb, ni;                                      // output rows per band; images per band (> 1 only for whole images)
+    int xb;                                          // flat: pixels per band
+    int cores;                                       // 8-pixel groups per output row
+    int gp, gpy;                                     // pixels per channel group and row: X (one plane), dY
+    int planes;                                      // column parities kept (1 or 2)
+    int row_step, x_rows;                            // X rows per output row; X rows of one image in a band
+    int in_step;                                     // input rows per X row
+    // the X side of a band: segments of consecutive input pixels (a whole image's rows, or one row where every other row is
+    // skipped), cut into slots of 32 pixels, in the order [channel group][image][segment][slot]
+    int segs, seg_pixels, seg_slots, slots;          // segments of an image, pixels and slots of a segment, slots of the band
+    uint32_t seg_magic, segs_magic, ni_magic;        // slot / seg_slots = (slot * seg_magic) >> 20 and so on
+    uint32_t w_magic;                                // pixel / W
+    uint32_t cores_magic, yb_magic, step_magic;      // core / cores, row / yb, dY task / dY steps
+    int x_bytes, dy_bytes, stages;                   // per pipeline stage
+    int bands, bands_total, bands_per_split, splits; // bands per image (or per group of images); over the batch; per CTA
+    int tiles_c, tiles_j;
+    int ncols, chunks;                               // accumulator columns R * S * cb; 32-column chunks
+    uint32_t tmem_cols;
+    uint32_t k;
+    uint2 pairs[kMaxPairs];                          // low descriptor words of a band's K = 16 steps, relative to the stage: dY, X
+};
+
+struct FusedConvCtl {
+    uint64_t full[kMaxStages], empty[kMaxStages], accum;
+    uint32_t tmem_base;
+    int abort_flag;
+    alignas(16) uint2 home[kProdWarps][4];   // per producer warp: where the slots of its task go
+    uint2 meta[kProdWarps][32];  // per producer warp: [slot of a task][channel] (mask bits, position of their first value)
+};
+
+// x / d for x * d < 2^20, with magic = 2^20 / d + 1
+__host__ __device__ __forceinline__ uint32_t magic_of(uint32_t d) { return (1u << 20) / d + 1u; }
+__host__ __device__ __forceinline__ uint32_t quotient(uint32_t x, uint32_t magic) { return (x * magic) >> 20; }
+
+// Shared-memory matrix descriptor without swizzle, MN-major.  Low word: start address and the distance between the two 8-row
+// groups of a K = 16 step; high word: the distance between groups of eight columns, and the descriptor version.
+__host__ __device__ __forceinline__ uint32_t desc_low(uint32_t addr, uint32_t k_stride) { return (addr >> 4) | ((k_stride >> 4) << 16); }
+__device__ __forceinline__ uint64_t desc_of(uint32_t low, uint32_t high) { return (uint64_t)low | ((uint64_t)high << 32); }
+__device__ __forceinline__ uint32_t desc_high(uint32_t mn_stride) { return (mn_stride >> 4) | (1u << 14); }
+
+__device__ __forceinline__ void sts_zero16(uint32_t addr) {
+    asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(addr), "r"(0u) : "memory");
+}
+
+// *p if `bit` is not zero, else 0; a predicated load, not a branch.
+__device__ __forceinline__ uint32_t ldg_u16_if(const uint16_t* p, uint32_t bit) {
+    uint32_t v;
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\tmov.u32 %0, 0;\n\t@p ld.global.nc.u16 %0, [%1];\n\t}"
+        : "=r"(v) : "l"(p), "r"(bit));
+    return v;
+}
+
+struct Place {
+    uint32_t group, img, seg, pixel;     // pixel: of the slot's first element inside the segment
+};
+__device__ __forceinline__ Place place_of(const FusedConvParams& p, uint32_t index, int groups) {
+    Place r;
+    const uint32_t a = quotient(index, p.seg_magic), b = quotient(a, p.segs_magic);
+    r.pixel = (index - a * p.seg_slots) * 32;
+    r.seg = a - b * p.segs;
+    r.group = quotient(b, p.ni_magic);
+    r.img = b - r.group * p.ni;
+    return r;
+}
+
+// VEC: pixels per load of dY (8: rows are whole aligned 16-byte groups; 2; 1)
+template <int VEC>
+__global__ void __launch_bounds__(kThreads, 1)
+conv_wg_fused_kernel(const uint16_t* __restrict__ dy, const uint16_t* __restrict__ values, const uint32_t* __restrict__ mask,
+                     const uint32_t* __restrict__ offsets, const __grid_constant__ FusedConvParams p, float* __restrict__ partial,
+                     int32_t* dev_status, uint32_t wait_limit) {
+    extern __shared__ __align__(128) uint8_t csm[];
+    const int warp = __shfl_sync(kFullMask, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: uniform
+    const int stage_bytes = p.x_bytes + p.dy_bytes;
+    const uint32_t smem0 = ptx::smem_u32(csm);
+    FusedConvCtl* ctl = reinterpret_cast<FusedConvCtl*>(csm + (size_t)p.stages * stage_bytes);
+    const int tile = blockIdx.x, split = blockIdx.y;
+    const int c0 = (tile % p.tiles_c) * p.cb, j0 = (tile / p.tiles_c) * kBM;
+    const int band0 = split * p.bands_per_split;
+    const int nb = min(p.bands_total, band0 + p.bands_per_split) - band0;     // >= 1
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < p.stages; ++s) {
+            ptx::mbar_init(&ctl->full[s], kProdWarps);
+            ptx::mbar_init(&ctl->empty[s], 1);
+        }
+        ptx::mbar_init(&ctl->accum, 1);
+        ctl->abort_flag = 0;
+        ptx::fence_mbar_init();
+    }
+    if (warp == kProdWarps) {
+        ptx::tmem_alloc(&ctl->tmem_base, p.tmem_cols);
+        ptx::tmem_relinquish();
+    }
+    const uint32_t row_pitch = (uint32_t)(p.cb / 8) * p.gp * 16, dy_pitch = (uint32_t)(p.mt / 8) * p.gpy * 16;
+    // padding columns, and the rows of dY behind a band's last one, are read but never written: zero
+    for (int i = threadIdx.x; i < p.stages * stage_bytes / 16; i += kThreads) sts_zero16(smem0 + i * 16);
+    const int total_cores = p.ni * p.yb * p.cores, pairs = (total_cores + 1) / 2;
+    ptx::fence_proxy_async_smem();
+    ptx::tc_fence_before();
+    __syncthreads();
+    ptx::tc_fence_after();
+    const uint32_t tmem_base = ctl->tmem_base;
+    volatile int* abort_flag = &ctl->abort_flag;
+    ptx::grid_dependency_wait();
+
+    if (warp < kProdWarps) {
+        // ---------------- producers ----------------
+        const uint32_t nwords = (uint32_t)(((int64_t)p.B * p.Ca * p.H * p.W + 31) / 32);
+        const uint32_t plane_elems = (uint32_t)p.H * p.W, plane_pitch = (uint32_t)p.x_bytes / p.planes;
+        const int groups = p.cb / 8, x_tasks = (p.slots + 3) / 4;
+        const int dy_steps = (total_cores + 3) / 4, dy_tasks = dy_steps * (p.mt / 64);
+        const size_t dy_plane = (size_t)p.Ho * p.Wo;
+        const int slot = lane >> 3, sub = lane & 7;
+        uint2* meta = ctl->meta[warp];
+        uint2* home = ctl->home[warp];
+        const uint32_t lane_bit = 1u << lane, lane_below = lane_bit - 1u;
+        int n0 = (band0 / p.bands) * p.ni, piece = band0 % p.bands;      // image and piece of the image
+        for (int i = 0; i < nb; ++i) {
+            const int s = i % p.stages;
+            const int y0 = p.flat ? 0 : piece * p.yb, k0 = p.flat ? piece * p.xb : 0;
+            const uint32_t xbuf = smem0 + s * stage_bytes, ybuf = xbuf + p.x_bytes;
+            // ---- X: a task is four slots, a slot 32 consecutive pixels of 8 channels.  First the mask bits of every slot and
+            // channel and the position of their first value: lane = (channel sub, slot)
+            const int yi0 = y0 * p.stride - p.pad;
+            const int run_end = p.flat ? min(p.W, k0 + p.xb) : (int)plane_elems;   // no pixel of the plane from here on
+            struct Bits { uint4 chunk; uint32_t next, first, at, lead, len; };
+            auto request = [&](uint32_t index) {
+                Bits r;
+                r.chunk = make_uint4(0, 0, 0, 0);
+                r.next = r.first = r.at = r.lead = r.len = 0;
+                if (index >= (uint32_t)p.slots) return r;
+                const Place at = place_of(p, index, groups);
+                const int row = yi0 + (int)at.seg * p.in_step;                     // first input row of the segment
+                const int px = (p.flat ? k0 : row * p.W) + (int)at.pixel;
+                const int c = c0 + (int)at.group * 8 + sub;
+                int lo = max(px, 0), hi = min(min(px + 32, run_end), px + p.seg_pixels - (int)at.pixel);
+                if (n0 + (int)at.img < p.B && c < p.Ca && lo < hi) {
+                    r.at = ((uint32_t)(n0 + at.img) * p.Ca + c) * plane_elems + lo;   // flat index of the slot's first element
+                    r.lead = lo - px;
+                    r.len = hi - lo;
+                    const uint32_t ch = r.at >> 7, w1 = (r.at >> 5) + 1;
+                    r.first = __ldg(offsets + ch);
+                    if (w1 < nwords) r.next = __ldg(mask + w1);
+                    if (ch * 4 + 3 < nwords) {
+                        r.chunk = __ldg(reinterpret_cast<const uint4*>(mask) + ch);
+                    } else {                             // the tensor's last chunk may be short
+                        r.chunk.x = __ldg(mask + ch * 4);
+                        if (ch * 4 + 1 < nwords) r.chunk.y = __ldg(mask + ch * 4 + 1);
+                        if (ch * 4 + 2 < nwords) r.chunk.z = __ldg(mask + ch * 4 + 2);
+                    }
+                }
+                return r;
+            };
+            auto record = [&](const Bits& r) {
+                const uint32_t in = (r.at >> 5) & 3u, sh = r.at & 31u;
+                uint32_t m = r.chunk.x, pos = r.first;
+                if (in > 0) { pos += __popc(m); m = r.chunk.y; }
+                if (in > 1) { pos += __popc(m); m = r.chunk.z; }
+                if (in > 2) { pos += __popc(m); m = r.chunk.w; }
+                pos += __popc(m & ((1u << sh) - 1u));
+                uint32_t bits = __funnelshift_r(m, r.next, sh);
+                if (r.len < 32) bits &= (1u << r.len) - 1u;
+                if (pos + __popc(bits) > p.k) bits = 0;   // a table that does not match the mask must not read past the values
+                return make_uint2(bits << r.lead, pos);
+            };
+            Bits ahead = request(warp * 4 + slot);
+            if (i >= p.stages) {
+                const bool ok = ptx::mbar_wait_warp(&ctl->empty[s], ((i / p.stages) - 1) & 1, wait_limit);
+                if (!ok) *abort_flag = 1;
+            }
+            if (__any_sync(kFullMask, *abort_flag != 0)) break;
+            for (int t = warp; t < x_tasks; t += kProdWarps) {
+                meta[lane] = record(ahead);
+                if (lane < 4) {
+                    const uint32_t index = t * 4 + lane;
+                    const Place at = place_of(p, index, groups);
+                    home[lane] = make_uint2(xbuf + (at.img * p.x_rows + at.seg) * row_pitch + at.group * p.gp * 16,
+                                            index < (uint32_t)p.slots ? at.pixel : (uint32_t)p.seg_pixels);
+                }
+                ahead = request((t + kProdWarps) * 4 + slot);
+                __syncwarp();
+                // a slot at a time: the lane builds the 16 bytes of its pixel's 8 channels
+#pragma unroll 2
+                for (int q = 0; q < 4; ++q) {
+                    uint32_t v[8];
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const uint4 m = reinterpret_cast<const uint4*>(meta)[q * 4 + h];
+                        v[2 * h] = ldg_u16_if(values + (m.y + __popc(m.x & lane_below)), m.x & lane_bit);
+                        v[2 * h + 1] = ldg_u16_if(values + (m.w + __popc(m.z & lane_below)), m.z & lane_bit);
+                    }
+                    const uint2 at = home[q];            // where the slot's first pixel is: segment's address, pixel of the segment
+                    const uint32_t rel = at.y + lane;
+                    bool keep = rel < (uint32_t)p.seg_pixels;
+                    uint32_t x = rel, to = at.x;
+                    if (!p.flat) {
+                        const uint32_t row = quotient(rel, p.w_magic);
+                        x = rel - row * p.W + p.pad;
+                        to += row * row_pitch;
+                        if (p.stride == 2) {             // even and odd columns in separate planes
+                            if (x & 1u) {
+                                keep = keep && p.planes == 2;
+                                to += plane_pitch;
+                            }
+                            x >>= 1;
+                        }
+                    }
+                    if (keep)
+                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(to + x * 16), "r"(v[0] | (v[1] << 16)),
+                                     "r"(v[2] | (v[3] << 16)), "r"(v[4] | (v[5] << 16)), "r"(v[6] | (v[7] << 16)) : "memory");
+                }
+                __syncwarp();                            // the records may be overwritten
+            }
+
+            // ---- dY: 8 channels x 8 pixels per lane, transposed in registers.  The eight lanes of a quarter-warp take eight
+            // channel groups (their pitch is 16 bytes modulo 128, so that the stores of a quarter-warp do not collide)
+            for (int t = (warp + kProdWarps - x_tasks % kProdWarps) % kProdWarps; t < dy_tasks; t += kProdWarps) {   // goes on where the X tasks ended
+                const int jset = (int)quotient(t, p.step_magic);
+                const int core = (t - jset * dy_steps) * 4 + slot, jg = jset * 8 + sub;
+                if (core >= total_cores) continue;
+                const int row = (int)quotient(core, p.cores_magic), xc = core - row * p.cores;
+                const int img = (int)quotient(row, p.yb_magic), y = y0 + row - img * p.yb;
+                const int x = k0 + xc * 8, nv = min(8, p.Wo - x);          // pixels that exist
+                const bool in = n0 + img < p.B && y < p.Ho && nv > 0;
+                const int j = j0 + jg * 8;
+                const uint16_t* src = dy + ((size_t)(n0 + img) * p.Cz + j) * dy_plane + (size_t)y * p.Wo + x;
+                uint32_t w[8][4];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    w[e][0] = w[e][1] = w[e][2] = w[e][3] = 0;
+                    if (in && j + e < p.Cz) {
+                        if constexpr (VEC == 8) {
+                            const uint4 v = ld_stream(reinterpret_cast<const uint4*>(src));
+                            w[e][0] = v.x; w[e][1] = v.y; w[e][2] = v.z; w[e][3] = v.w;
+                        } else if constexpr (VEC == 2) {
+#pragma unroll
+                            for (int h = 0; h < 4; ++h)
+                                if (2 * h < nv) w[e][h] = __ldg(reinterpret_cast<const uint32_t*>(src) + h);
+                        } else {
+#pragma unroll
+                            for (int h = 0; h < 8; ++h)
+                                if (h < nv) w[e][h >> 1] |= (uint32_t)__ldg(src + h) << ((h & 1) * 16);
+                        }
+                    }
+                    src += dy_plane;
+                }
+                const uint32_t dst = ybuf + row * dy_pitch + (jg * p.gpy + xc * 8) * 16;
+#pragma unroll
+                for (int px = 0; px < 8; ++px) {
+                    uint32_t o[4];
+#pragma unroll
+                    for (int h = 0; h < 4; ++h)
+                        o[h] = __byte_perm(w[2 * h][px >> 1], w[2 * h + 1][px >> 1], (px & 1) ? 0x7632 : 0x5410);
+                    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + px * 16), "r"(o[0]), "r"(o[1]), "r"(o[2]),
+                                 "r"(o[3]) : "memory");
+                }
+            }
+
+            ptx::fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(&ctl->full[s]);
+            if (i + 1 < nb) {
+                // the next band's dY is brought into L2 meanwhile (a lane's eight rows, one 16-byte piece of each 128-byte line)
+                const bool turn = piece + 1 == p.bands;
+                const int n1 = turn ? n0 + p.ni : n0, piece1 = turn ? 0 : piece + 1;
+                const int rows1 = p.flat ? 1 : min(p.yb, p.Ho - piece1 * p.yb);
+                const size_t first = p.flat ? (size_t)piece1 * p.xb : (size_t)piece1 * p.yb * p.Wo;
+                const int lines = (rows1 * (p.flat ? min(p.xb, p.Wo - piece1 * p.xb) : p.Wo) * 2 + 127) / 128;
+                const int per_img = min(p.mt, p.Cz - j0) * lines;
+                for (int q = threadIdx.x; q < per_img * min(p.ni, p.B - n1); q += 32 * kProdWarps) {
+                    const int img = q / per_img, rest = q - img * per_img, j = rest / lines, l = rest - j * lines;
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(dy + ((size_t)(n1 + img) * p.Cz + j0 + j) * dy_plane + first + l * 64));
+                }
+            }
+            if (++piece == p.bands) {
+                piece = 0;
+                n0 += p.ni;
+            }
+        }
+        ptx::launch_dependents();
+        // ---------------- epilogue: the accumulator leaves in the order it has in tensor memory ----------------
+        bool ok = ptx::mbar_wait_warp(&ctl->accum, 0, wait_limit);
+        if (!ok || *abort_flag) {
+            *abort_flag = 1;
+        } else {
+            ptx::tc_fence_after();
+            const int quarter = warp & 3;
+            if (j0 + 32 * quarter < p.Cz) {
+                float4* plane = reinterpret_cast<float4*>(partial) + ((size_t)split * gridDim.x + tile) * p.chunks * 8 * kBM;
+                for (int ch = warp >> 2; ch < p.chunks; ch += kProdWarps / 4) {
+                    uint32_t r[32];
+                    ptx::tmem_ld_32x32(tmem_base + ((uint32_t)(32 * quarter) << 16) + ch * 32, r);
+                    ptx::tmem_ld_wait();
+#pragma unroll
+                    for (int e4 = 0; e4 < 8; ++e4)
+                        __stcg(plane + (size_t)(ch * 8 + e4) * kBM + 32 * quarter + lane,
+                               make_float4(__uint_as_float(r[4 * e4]), __uint_as_float(r[4 * e4 + 1]), __uint_as_float(r[4 * e4 + 2]),
+                                           __uint_as_float(r[4 * e4 + 3])));
+                }
+            }
+        }
+    } else {
+        // ---------------- MMA issuer (the whole warp runs the loop, one thread issues) ----------------
+        const uint32_t leader = ptx::elect_one();
+        const uint32_t n_inst = (uint32_t)(p.R * p.cb);
+        const uint32_t idesc = ptx::make_idesc_bf16(kBM, (int)n_inst, true, true);
+        const uint32_t high_a = desc_high(p.gpy * 16), high_b = desc_high(p.gp * 16);
+        const uint32_t plane_pitch = (uint32_t)p.x_bytes / p.planes;
+        // where a horizontal tap's columns start, in descriptor units
+        const uint32_t shift1 = (p.stride == 2 ? plane_pitch : 16u) >> 4, shift2 = (p.stride == 2 ? 16u : 32u) >> 4;
+        for (int i = 0; i < nb; ++i) {
+            const int s = i % p.stages;
+            if (!__all_sync(kFullMask, !*abort_flag && ptx::mbar_wait_spin(&ctl->full[s], (i / p.stages) & 1, wait_limit))) {
+                *abort_flag = 1;
+                break;
+            }
+            ptx::tc_fence_after();
+            const uint32_t stage = (smem0 + s * stage_bytes) >> 4;
+#pragma unroll 2
+            for (int q = 0; q < pairs; ++q) {
+                const uint64_t ad = desc_of(p.pairs[q].x + stage, high_a);
+                const uint32_t b_low = p.pairs[q].y + stage, acc = (i > 0 || q > 0) ? 1u : 0u;
+                ptx::umma_bf16_elected(tmem_base, ad, desc_of(b_low, high_b), idesc, acc, leader);
+                if (p.S > 1) ptx::umma_bf16_elected(tmem_base + n_inst, ad, desc_of(b_low + shift1, high_b), idesc, acc, leader);
+                if (p.S > 2) ptx::umma_bf16_elected(tmem_base + 2 * n_inst, ad, desc_of(b_low + shift2, high_b), idesc, acc, leader);
+            }
+            if (leader) ptx::umma_commit(&ctl->empty[s]);
+            __syncwarp();
+        }
+        if (leader) ptx::umma_commit(&ctl->accum);      // also after an abort: it then tells when the MMAs in flight are done
+        __syncwarp();
+        ptx::mbar_wait_warp(&ctl->accum, 0, kWaitLimit);   // no MMA may be in flight when tensor memory is freed
+    }
+    ptx::tc_fence_before();
+    __syncthreads();
+    if (warp == kProdWarps) {
+        ptx::tc_fence_after();
+        ptx::tmem_dealloc(tmem_base, p.tmem_cols);
+    }
+    if (*abort_flag && threadIdx.x == 0 && dev_status) atomicExch(dev_status, (int)DROPIT_ERR_TIMEOUT);
+}
+
+// dw[j,c,u,v] (=|+=) sum over splits, in split order within a warp's share and then over the warps.  A block takes 32 rows of
+// one 4-column group; its eight warps share out the splits.
+constexpr int kRedWarps = 8;
+__global__ void __launch_bounds__(32 * kRedWarps)
+conv_fused_reduce_kernel(const float4* __restrict__ partial, const FusedConvParams p, float* __restrict__ dw, int accumulate) {
+    __shared__ float4 sums[kRedWarps][32];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int quarters = (min(kBM, p.Cz) + 31) / 32;
+    int b = blockIdx.x;
+    const int quarter = b % quarters; b /= quarters;
+    const int e4 = b % (p.chunks * 8), tile = b / (p.chunks * 8);
+    const int tiles = p.tiles_c * p.tiles_j;
+    const int c0 = (tile % p.tiles_c) * p.cb, j = (tile / p.tiles_c) * kBM + 32 * quarter + lane;
+    const int col = e4 * 4;
+    ptx::grid_dependency_wait();                        // the partial tiles come from the kernel before this one
+    if (col >= p.ncols || j - lane >= p.Cz) return;
+    const size_t plane = (size_t)tiles * p.chunks * 8 * kBM;
+    const float4* src = partial + ((size_t)tile * p.chunks * 8 + e4) * kBM + 32 * quarter + lane;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    int s = g;
+    for (; s + 3 * kRedWarps < p.splits; s += 4 * kRedWarps) {
+        float4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = __ldcg(src + (size_t)(s + u * kRedWarps) * plane);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { acc.x += v[u].x; acc.y += v[u].y; acc.z += v[u].z; acc.w += v[u].w; }
+    }
+    for (; s < p.splits; s += kRedWarps) {
+        const float4 v = __ldcg(src + (size_t)s * plane);
+        acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+    }
+    sums[g][lane] = acc;
+    __syncthreads();
+    if (g == 0 && j < p.Cz) {
+#pragma unroll
+        for (int w = 1; w < kRedWarps; ++w) {
+            const float4 v = sums[w][lane];
+            acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+        }
+        const int n_inst = p.R * p.cb;
+        const int v = col / n_inst, u = (col % n_inst) / p.cb, c = c0 + col % p.cb;   // cb is a multiple of 16: one tap
+        const float a[4] = {acc.x, acc.y, acc.z, acc.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (c + e < p.Ca) {
+                float* d = dw + (((size_t)j * p.Ca + c + e) * p.R + u) * p.S + v;
+                *d = accumulate ? *d + a[e] : a[e];
+            }
+        }
+    }
+}
+
+size_t stage_bytes_of(FusedConvParams& p) {
+    const size_t row_pitch = (size_t)(p.cb / 8) * p.gp * 16, dy_pitch = (size_t)(p.mt / 8) * p.gpy * 16;
+    // With an odd number of 8-pixel groups the last K = 16 step reads one more K row than the band has: zeros in dY,
+    // anything finite in X.  With 64 rows of dY per band the instruction's rows 64..127 are the next image row (their
+    // results are not used).
+    const int odd = (p.ni * p.yb * p.cores) & 1;
+    const size_t x = (size_t)(p.ni * p.x_rows + odd * p.row_step) * row_pitch * p.planes;
+    const size_t y = (size_t)(p.ni * p.yb + odd + (p.mt == 64 ? 1 : 0)) * dy_pitch;
+    p.x_bytes = (int)align_up(x, 128 * p.planes);
+    p.dy_bytes = (int)align_up(y, 128);
+    return (size_t)p.x_bytes + p.dy_bytes;
+}
+
+bool make_fused_conv_plan(FusedConvParams& p, int B, int Ca, int H, int W, int Cz, int R, int S, int stride, int pad, int64_t k) {
+    p = FusedConvParams{};
+    if (R > 3 || S > 3 || stride > 2 || pad > 2 || B < 1) return false;
+    p.B = B; p.Ca = Ca; p.Cz = Cz; p.R = R; p.S = S; p.stride = stride; p.pad = pad; p.k = (uint32_t)k;
+    p.H = H; p.W = W;
+    p.Ho = (H + 2 * pad - R) / stride + 1;
+    p.Wo = (W + 2 * pad - S) / stride + 1;
+    p.flat = R == 1 && S == 1 && stride == 1 && pad == 0;
+    if (p.flat) { p.W = p.Wo = H * W; p.H = p.Ho = 1; }
+    const int cb_max = (256 / R < 512 / (R * S) ? 256 / R : 512 / (R * S)) / 16 * 16;   // N <= 256 columns, 512 of tensor memory
+    const int blocks = (Ca + cb_max - 1) / cb_max;
+    p.cb = (int)align_up((size_t)(Ca + blocks - 1) / blocks, 16);
+    p.mt = Cz > 64 ? 128 : 64;
+    p.planes = stride == 2 && S > 1 ? 2 : 1;
+    p.row_step = R == 1 ? 1 : stride;
+    p.in_step = R == 1 ? stride : 1;
+    p.tiles_c = (Ca + p.cb - 1) / p.cb;
+    p.tiles_j = (Cz + kBM - 1) / kBM;
+    p.stages = 2;
+    const int64_t tiles = (int64_t)p.tiles_c * p.tiles_j;
+    if (tiles > 65535) return false;
+    if (!p.flat) {
+        p.cores = (p.Wo + 7) / 8;
+        p.gpy = p.cores * 8 + 1;
+        // columns an 8-pixel group of any tap can reach, at the plane's resolution
+        const int reach = p.cores * 8 + (S - 1) / stride + 1, padded = ((W + 7) / 8 * 8 + pad + stride - 1) / stride + 1;
+        p.gp = reach > padded ? reach : padded;
+    }
+    // An image in `pieces` equal bands (pieces == 1: `ni` images in one band); returns what the slowest CTA takes, in units
+    // of a producer task, or -1 if such a band does not fit.  A band costs half a task on top of its rounds of tasks
+    // (handing the stage over, waiting for the product of the band before last).
+    auto set_band = [&](int pieces, int ni) -> float {
+        p.ni = ni;
+        if (p.flat) {
+            p.xb = (int)align_up((size_t)(p.W + pieces - 1) / pieces, pieces > 1 ? 32 : 16);
+            p.cores = p.xb / 8;
+            p.gp = p.gpy = p.xb + 1;
+            p.yb = 1;
+            p.bands = (p.W + p.xb - 1) / p.xb;
+        } else {
+            p.yb = (p.Ho + pieces - 1) / pieces;
+            p.bands = (p.Ho + p.yb - 1) / p.yb;
+        }
+        p.x_rows = (p.yb - 1) * p.row_step + R;
+        if (p.ni * p.yb * p.cores > 2 * kMaxPairs || stage_bytes_of(p) * p.stages + sizeof(FusedConvCtl) + 128 > kSmemBudget) return -1.f;
+        p.bands_total = (B + ni - 1) / ni * p.bands;
+        p.segs = p.in_step > 1 ? p.x_rows : 1;
+        p.seg_pixels = p.flat ? p.xb : (p.in_step > 1 ? W : p.x_rows * W);
+        p.seg_slots = (p.seg_pixels + 31) / 32;
+        p.slots = p.seg_slots * p.segs * p.ni * (p.cb / 8);
+        int splits = (int)(sm_count() / tiles);
+        if (splits < 1) splits = 1;
+        if (splits > p.bands_total) splits = p.bands_total;
+        p.bands_per_split = (p.bands_total + splits - 1) / splits;
+        p.splits = (p.bands_total + p.bands_per_split - 1) / p.bands_per_split;
+        const int tasks = (p.slots + 3) / 4 + (p.ni * p.yb * p.cores + 3) / 4 * (p.mt / 64);
+        return p.bands_per_split * (0.5f + (float)((tasks + kProdWarps - 1) / kProdWarps));
+    };
+    int best_pieces = 0, best_ni = 0;
+    float best = 0.f;
+    const int most_pieces = p.flat ? (p.W + 31) / 32 : p.Ho;
+    for (int pieces = 1; pieces <= most_pieces && pieces <= 64; ++pieces) {
+        if (!p.flat && pieces > 1 && (p.Ho + pieces - 1) / pieces == (p.Ho + pieces - 2) / (pieces - 1)) continue;
+        for (int ni = 1; ni <= (pieces == 1 ? B : 1); ++ni) {
+            const float cost = set_band(pieces, ni);
+            if (cost < 0.f) break;
+            if (best_ni == 0 || cost < best) { best = cost; best_pieces = pieces; best_ni = ni; }
+        }
+    }
+    if (best_ni == 0) return false;
+    set_band(best_pieces, best_ni);
+    const int cores_total = p.ni * p.yb * p.cores;
+    p.seg_magic = magic_of((uint32_t)p.seg_slots);
+    p.segs_magic = magic_of((uint32_t)p.segs);
+    p.ni_magic = magic_of((uint32_t)p.ni);
+    p.w_magic = magic_of((uint32_t)W);
+    p.cores_magic = magic_of((uint32_t)p.cores);
+    p.yb_magic = magic_of((uint32_t)p.yb);
+    p.step_magic = magic_of((uint32_t)((cores_total + 3) / 4));
+    // what the division by multiplication and the table of K steps can take
+    const int64_t most = p.slots + 4 * kProdWarps + 4;
+    if (cores_total > 2 * kMaxPairs || most * p.seg_slots >= (1 << 20) || most * p.segs >= (1 << 20) || most * p.ni >= (1 << 20) ||
+        (int64_t)cores_total * p.cores >= (1 << 20) || (!p.flat && (int64_t)(p.seg_pixels + 32) * W >= (1 << 20)))
+        return false;
+    p.ncols = R * S * p.cb;
+    p.chunks = (p.ncols + 31) / 32;
+    p.tmem_cols = 32;
+    while ((int)p.tmem_cols < p.chunks * 32) p.tmem_cols *= 2;
+    if (p.tmem_cols > 512) return false;
+    {
+        const uint32_t row_pitch = (uint32_t)(p.cb / 8) * p.gp * 16, dy_pitch = (uint32_t)(p.mt / 8) * p.gpy * 16;
+        for (int i = 0; i < (cores_total + 1) / 2; ++i) {
+            uint32_t a[2], b[2];
+            for (int h = 0; h < 2; ++h) {
+                const int core = 2 * i + h, row = core / p.cores, xc = core % p.cores;
+                // the group behind the last row counts as a row of the last image
+                const int img = row / p.yb < p.ni ? row / p.yb : p.ni - 1, y = row - img * p.yb;
+                a[h] = p.x_bytes + row * dy_pitch + xc * 128;
+                b[h] = (img * p.x_rows + y * p.row_step) * row_pitch + xc * 128;
+            }
+            p.pairs[i] = make_uint2(desc_low(a[0], a[1] - a[0]), desc_low(b[0], b[1] - b[0]));
+        }
+    }
+    return true;
+}
+
+}  // namespace
+
+// 0 when this kernel does not take the shape.
+size_t conv_fused_workspace_bytes(int B, int Ca, int H, int W, int Cz, int R, int S, int stride, int pad) {
+    FusedConvParams p;
+    if (!make_fused_conv_plan(p, B, Ca, H, W, Cz, R, S, stride, pad, 0)) return 0;
+    return (size_t)p.splits * p.tiles_c * p.tiles_j * p.chunks * 32 * kBM * 4;
+}
+
+// Caller has validated pointers, sizes and alignment, and B >= 1, k >= 1; bitmask caches only.
+dropit_status conv_fused_run(const void* dy, const void* values, const void* mask, const uint32_t* offsets, int B, int Ca, int H,
+                             int W, int Cz, int R, int S, int stride, int pad, int64_t k, float* dw, int accumulate,
+                             void* workspace, size_t workspace_bytes, int32_t* dev_status, cudaStream_t stream) {
+    FusedConvParams p;
+    if (!make_fused_conv_plan(p, B, Ca, H, W, Cz, R, S, stride, pad, k)) return DROPIT_ERR_UNSUPPORTED;
+    const int tiles = p.tiles_c * p.tiles_j;
+    if (workspace_bytes < (size_t)p.splits * tiles * p.chunks * 32 * kBM * 4) return DROPIT_ERR_WORKSPACE;
+    const int vec = p.Wo % 8 == 0 ? 8 : (p.Wo % 2 == 0 ? 2 : 1);
+    auto kern = vec == 8 ? conv_wg_fused_kernel<8> : (vec == 2 ? conv_wg_fused_kernel<2> : conv_wg_fused_kernel<1>);
+    static PerDeviceOnce attr[3];
+    PerDeviceOnce& once = attr[vec == 8 ? 0 : (vec == 2 ? 1 : 2)];
+    if (once.needed()) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess)
+            return DROPIT_ERR_CUDA;
+        once.mark();
+    }
+    float* partial = reinterpret_cast<float*>(workspace);
+    cudaLaunchAttribute pdl[1];
+    pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)tiles, (unsigned)p.splits);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = (size_t)p.stages * (p.x_bytes + p.dy_bytes) + sizeof(FusedConvCtl);
+    cfg.stream = stream;
+    cfg.attrs = pdl;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, kern, reinterpret_cast<const uint16_t*>(dy), reinterpret_cast<const uint16_t*>(values),
+                           reinterpret_cast<const uint32_t*>(mask), offsets, p, partial, dev_status,
+                           spin_limit(kWaitLimit)) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return DROPIT_ERR_CUDA;
+    }
+    dropit_status st = check_launch();
+    if (st != DROPIT_OK) return st;
+    const int quarters = ((Cz < kBM ? Cz : kBM) + 31) / 32;
+    cfg.gridDim = dim3((unsigned)(tiles * p.chunks * 8 * quarters));
+    cfg.blockDim = dim3(32 * kRedWarps);
+    cfg.dynamicSmemBytes = 0;
+    if (cudaLaunchKernelEx(&cfg, conv_fused_reduce_kernel, reinterpret_cast<const float4*>(partial), p, dw, accumulate) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return DROPIT_ERR_CUDA;
+    }
+    return check_launch();
+}
+
+}  // namespace dropit

@@ -1,4 +1,5 @@
-// Conv2d weight gradient on the tensor cores (Eq. 4-5, retained term), bf16, stride 1:
+// Conv2d weight gradient on the tensor cores from dense copies of R(a-hat) (Eq. 4-5, retained term), bf16: 1 x 1 filters on
+// planes of whole 16-byte groups, filters wider than 3, index32 caches (conv_weight_grad_fused.cu takes the rest).  Stride 1:
 //   dW[j,c,u,v] = sum_{n,y,x} dY[n,j,y,x] * R(a-hat)[n,c, y+u-pad, x+v-pad]
 // One implicit GEMM per filter tap (u,v): M = output channels j, N = input channels c, and the
 // reduction runs over (n, y, x) with x innermost, which is the contiguous axis of both NCHW operands,
