@@ -15,8 +15,14 @@
 //           histograms.  No second counting pass.
 //   phase 3 second read (L2 hits for tensors that fit L2): element i is retained iff key_i > T, or
 //           key_i == T and fewer than q equal keys precede it; #retained before i =
-//           gt_before + min(eq_before, q).  A lane owns 32 consecutive elements of a super-block; retained values are
-//           staged per warp and leave in aligned 16-byte pieces.
+//           gt_before + min(eq_before, q).  The quota ends inside one warp's run; in all others one threshold decides.
+//           A lane owns 32 consecutive elements of a super-block; retained values are staged per warp and leave in
+//           aligned 16-byte pieces.
+// Bound by issue in both streaming phases (some 250 warp instructions per super-block each) on top of 11 us of fixed steps
+// (sample 5.5, barrier 2, phase 2 2.5).  What the one threshold, the flags gathered by a prmt with msb replication, the
+// walk of dense words from registers and the rarer flushes gave, per call over rotating inputs (graph replay, gamma 0.9):
+// 12608 x 768 20.7 -> 19.3 us, 12608 x 3072 42.3 -> 39.1; 32768 x 768 at 0.5 48.3 -> 40.9; 32768 x 3072 at 0.8 96 -> 89,
+// at 0.5 134 -> 112 us (3.7 TB/s of the two reads and the outputs).
 // When the band is wider than the per-warp histogram (small tensors, which are not sampled; key
 // distributions that are flat around T; a sample that missed) a general path is taken instead:
 // full CTA histogram in shared memory, global histogram by atomics, then one extra counting read.
@@ -51,8 +57,11 @@ constexpr int kSbBytes = kSbVecs * 16;                         // 2 KB
 constexpr int kSbChunks = kSbElems / DROPIT_CHUNK;             // 8 seek-table entries
 constexpr int kRingSlots = 2;
 constexpr size_t kRingBytes = (size_t)kFusedWarps * kRingSlots * kSbBytes;   // 128 KB
-constexpr int kStageVals = kSbElems + 8;                       // per-warp staging: a super-block's retained values behind < 8 carried ones
-constexpr size_t kStageBytes = (size_t)kFusedWarps * kStageVals * 2;   // 64.5 KB
+// per-warp staging of retained values: whole 16-byte pieces leave once more than kStageKeep are waiting (every third
+// super-block or so at gamma 0.9), so that a super-block's values always find room behind them
+constexpr int kStageKeep = 264;
+constexpr int kStageVals = kSbElems + kStageKeep + 8;
+constexpr size_t kStageBytes = (size_t)kFusedWarps * kStageVals * 2;   // 81 KB
 static_assert(kStageBytes >= (size_t)kKeySpace * 2, "the sample's 16-bit histogram lives in the staging area");
 
 struct FusedState {
@@ -154,6 +163,46 @@ __device__ __forceinline__ uint32_t flags8(uint32_t x0, uint32_t x1, uint32_t x2
     const uint32_t r0 = __byte_perm(x0, x1, 0x7531), r1 = __byte_perm(x2, x3, 0x7531);
     const uint32_t u = ((r0 >> 7) & 0x01010101u) | ((r1 >> 3) & 0x10101010u);
     return (u * 0x01020408u) >> 24;
+}
+
+// Which of the lane's 32 elements have a key >= bound (c = ge_const(bound)); m: the keys, w & 0x7FFF7FFF, of the lane's 16
+// words as sb_read delivers them (register 4 * j + i holds word 4 * (j ^ rot) + i).  Words u and u + 8 share one prmt, which
+// turns their four flags into four bytes of ones (msb replication): word u's low and high half, word u + 8's low and high
+// half.  A bit of each byte is kept, bit u mod 8, so that the element of word u, half h ends at bit 16 (u / 8) + 8 h + u % 8.
+struct GatherLane {
+    uint32_t sel;              // prmt selector: registers j and j ^ 2 come in word order or the other way round
+    uint32_t place[2];         // 1 << 4 * ((j ^ rot) & 1)
+};
+__device__ __forceinline__ GatherLane gather_lane(uint32_t rot) {
+    GatherLane g;
+    g.sel = (rot & 2u) ? 0xB9FDu : 0xFDB9u;
+    g.place[0] = (rot & 1u) ? 16u : 1u;
+    g.place[1] = (rot & 1u) ? 1u : 16u;
+    return g;
+}
+__device__ __forceinline__ uint32_t ge_bits(const uint32_t (&m)[16], uint32_t c, const GatherLane& g) {
+    uint32_t all = 0;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        uint32_t four = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            uint32_t bytes;
+            asm("prmt.b32 %0, %1, %2, %3;" : "=r"(bytes) : "r"(m[4 * j + i] + c), "r"(m[4 * (j + 2) + i] + c), "r"(g.sel));
+            four |= bytes & (0x01010101u << i);
+        }
+        all += four * g.place[j];
+    }
+    return all;
+}
+// Such bits in element order: element 2 u + h.
+__device__ __forceinline__ uint32_t element_order(uint32_t x) {
+    uint32_t t = (x ^ (x >> 4)) & 0x00F000F0u;
+    x ^= t ^ (t << 4);
+    t = (x ^ (x >> 2)) & 0x0C0C0C0Cu;
+    x ^= t ^ (t << 2);
+    t = (x ^ (x >> 1)) & 0x22222222u;
+    return x ^ t ^ (t << 1);
 }
 
 // Exclusive prefix over the block's threads of `v`; also returns the block total.
@@ -448,7 +497,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                       uint16_t* __restrict__ values, uint32_t* __restrict__ mask, int32_t* __restrict__ indices,
                       uint32_t* __restrict__ offsets, int32_t* dev_status, int spin_max, const unsigned char* prep) {
     // shared memory: [input ring, 128 KB | general path: full key histogram]
-    //                [phase 3: per-warp value staging, 64 KB | sample step: 16-bit key histogram]
+    //                [phase 3: per-warp value staging, 81 KB | sample step: 16-bit key histogram]
     //                [control block of phases 1-2]
     extern __shared__ __align__(16) unsigned char fsm[];
     uint32_t* bins = reinterpret_cast<uint32_t*>(fsm);
@@ -464,6 +513,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
     const uint32_t ring_copy = ring_warp + lane * 16;   // where the lane's copies of a slot start
     const uint32_t ring_own = ring_warp + lane * 64;    // the lane's 32 elements of a slot
     const uint32_t rot = (uint32_t)(lane >> 1) & 3u;     // see sb_read
+    const GatherLane gl = gather_lane(rot);
     const int64_t nvec_full = n / 8;
     const int64_t blocks_total = (n + kBlkElems - 1) / kBlkElems;
     const int64_t blk0 = ((int64_t)blockIdx.x * kFusedWarps + warp) * blocks_per_warp;   // even
@@ -504,7 +554,8 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
         rows = const_cast<uint32_t*>(prep_rows(prep));
         __syncthreads();
     } else {
-        sample_band(x, n, k, sample_bins, sh.warp, sh.band, st, [&] { issue_sb(sb0, 0); }, [](const uint4& v) { return v; });
+        sample_band(x, n, k, sample_bins, sh.warp, sh.band, st,
+                    [&] { if (sb0 < sb1) issue_sb(sb1 - 1, 0); }, [](const uint4& v) { return v; });
     }
     bool prefetched = !prepared;
     uint32_t lo = sh.band[0], hi = sh.band[1];
@@ -565,12 +616,37 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                 }
             };
             if (narrow) {
-                // stream the run through the ring, one super-block ahead
-                if (!prefetched) issue_sb(sb0, 0);
+                // stream the run through the ring, one super-block ahead, LAST super-block first: phase 3 walks forward and
+                // so begins with what this pass has just read (of a tensor larger than L2, half is still there)
+                if (!prefetched && sb0 < sb1) issue_sb(sb1 - 1, 0);
+                auto issue_before = [&](int64_t sb, int to) {
+                    if (sb > sb0) issue_sb(sb - 1, to);
+                    else asm volatile("cp.async.commit_group;" ::: "memory");
+                };
                 int slot = 0;
-                auto count_sb = [&](int64_t sb, auto full_tag) {
-                    constexpr bool FULL = decltype(full_tag)::value;
-                    issue_sb(sb + 1, slot ^ 1);
+                uint32_t at = 0;    // the current slot's offset in the ring
+                auto count_fast = [&]() {
+                    sb_wait();
+                    __syncwarp();   // the lane reads vectors that other lanes copied
+                    const uint32_t own = ring_own + at;
+                    uint32_t w[16];
+                    sb_read(own, rot, w);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) w[i] &= 0x7FFF7FFFu;
+                    const uint32_t g = ge_bits(w, c_hi, gl);
+                    uint32_t pending = element_order(ge_bits(w, c_lo, gl) & ~g);
+                    cnt_hi += __popc(g);
+                    while (pending) {   // a few percent of the elements: the band histogram (their order is irrelevant)
+                        const uint32_t e = top_bit(pending);
+                        pending ^= 1u << e;
+                        const uint32_t d = (lds_u16(own + 2u * e) & 0x7FFFu) - lo;
+                        if (d == 0) ++cnt_lo; else atomicAdd(&hist[d], 1u);
+                    }
+                    __syncwarp();   // every lane is done with the slot before it is refilled
+                    at ^= kSbBytes;
+                };
+                auto count_sb = [&](int64_t sb) {   // the tensor's ragged last super-block
+                    issue_before(sb, slot ^ 1);
                     sb_wait();
                     __syncwarp();   // the lane reads vectors that other lanes copied
                     const uint32_t own = ring_own + slot * kSbBytes;
@@ -592,7 +668,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                         pending |= flags8(b[0], b[1], b[2], b[3]) << ((g ^ rot) << 3);
                     }
                     cnt_hi += __popc(hi_flags);
-                    if constexpr (!FULL) pending &= valid_mask32(sb * kSbElems + lane * 32, n);   // zero padding is no data
+                    pending &= valid_mask32(sb * kSbElems + lane * 32, n);   // zero padding is no data
                     while (pending) {   // a few percent of the elements: the band histogram (their order is irrelevant)
                         const uint32_t e = top_bit(pending);
                         pending ^= 1u << e;
@@ -602,9 +678,20 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                     __syncwarp();   // every lane is done with the slot before it is refilled
                     slot ^= 1;
                 };
-                int64_t sb = sb0;
-                for (; sb < sb_full_end; ++sb) count_sb(sb, std::true_type{});
-                for (; sb < sb1; ++sb) count_sb(sb, std::false_type{});
+                int64_t sb = sb1 - 1;
+                for (; sb >= sb0 && sb >= sb_full_end; --sb) count_sb(sb);
+                if (sb >= sb0) {
+                    at = slot * kSbBytes;
+                    const uint4* src = x + sb * kSbVecs + lane;
+                    for (; sb > sb0; --sb) {
+                        src -= kSbVecs;
+                        sb_issue_full(ring_copy + (at ^ kSbBytes), src);
+                        count_fast();
+                    }
+                    asm volatile("cp.async.commit_group;" ::: "memory");
+                    count_fast();
+                    --sb;
+                }
                 asm volatile("cp.async.wait_all;" ::: "memory");
             } else {
                 int64_t blk = blk0;
@@ -684,7 +771,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                 // thread (g, c) adds column c of rows g, g + kGroups, ...: consecutive threads read consecutive
                 // words of a row, and a thread's loads are independent of one another
                 constexpr int kGroups = kFusedThreads / kRowWords;
-                constexpr int kInFlight = 8;
+                constexpr int kInFlight = 10;
                 const uint32_t g = threadIdx.x / kRowWords, c = threadIdx.x - g * kRowWords;
                 if (g < (uint32_t)kGroups && (c <= width || c == (uint32_t)kWarpBins)) {
                     uint32_t t_sum = 0, p_sum = 0;
@@ -875,10 +962,129 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
     uint32_t gpos = run_gt + min(run_eq, q);   // retained elements before this warp's next super-block
     uint32_t head = gpos & ~7u;                // first position not yet written to `values` (16-byte aligned)
     uint32_t foreign = gpos & 7u;              // leading slots of the first piece that belong to the previous warp
+    // The quota of ties runs out inside one warp's run at most.  In every other run either all ties are retained or none, so
+    // that one threshold decides: key >= T or key >= T + 1.
+    bool one_threshold = false;
+    uint32_t c_keep = 0;
+    {
+        const uint32_t run_ties = sh.wpre_eq[warp];
+        const bool all = run_eq + run_ties <= q, none = run_eq >= q;
+        if (all || none) {
+            one_threshold = true;
+            c_keep = all ? c_ge : c_gt;
+            run_gt = gpos;                     // from here on positions count from gpos, with a quota that never or always binds
+            run_eq = 0;
+            q = all ? 0x40000000u : 0u;
+        }
+    }
+    // write the whole 16-byte pieces that are staged, carry the rest to the front
+    auto flush = [&]() {
+        const uint32_t staged = gpos - head;
+        const uint32_t pieces = staged / 8;
+        for (uint32_t c = lane; c < pieces; c += 32) {
+            if (c == 0 && foreign) {
+                for (uint32_t e = foreign; e < 8; ++e) values[head + e] = s_vals[e];
+            } else {
+                *reinterpret_cast<uint4*>(values + head + c * 8) = *reinterpret_cast<const uint4*>(s_vals + c * 8);
+            }
+        }
+        if (pieces) {
+            foreign = 0;
+            const uint32_t rem = staged - pieces * 8;
+            uint16_t carry = 0;
+            if (lane < (int)rem) carry = s_vals[pieces * 8 + lane];
+            __syncwarp();
+            if (lane < (int)rem) s_vals[lane] = carry;
+            head += pieces * 8;
+            __syncwarp();
+        }
+    };
     issue_sb(sb0, 0);
     int slot = 0;
-    auto compact_sb = [&](int64_t sb, auto full_tag) {
-        constexpr bool FULL = decltype(full_tag)::value;
+    // a super-block under the one threshold; `at` = offset of its slot in the ring, `out` = where its mask words and table
+    // entries go, `first_idx` = the lane's first element
+    uint32_t at = 0;
+    uint32_t* mask_out = INDEX32 ? nullptr : mask + sb0 * (kSbElems / 32) + lane;
+    uint32_t* offs_out = offsets + sb0 * kSbChunks + (lane >> 2);
+    [[maybe_unused]] int32_t first_idx = (int32_t)(sb0 * kSbElems) + lane * 32;
+    auto compact_fast = [&](auto dense_tag) {
+        constexpr bool DENSE = decltype(dense_tag)::value;
+        sb_wait();
+        __syncwarp();   // the lane reads vectors that other lanes copied
+        const uint32_t own = ring_own + at;
+        uint32_t w[16];
+        sb_read(own, rot, w);
+        uint32_t m[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) m[i] = w[i] & 0x7FFF7FFFu;
+        const uint32_t keep = element_order(ge_bits(m, c_keep, gl));
+        const uint32_t cnt = __popc(keep);
+        uint32_t inc = cnt;                    // prefix over the lanes = over the super-block's elements
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFullMask, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const uint32_t pos = gpos + inc - cnt;
+        if ((lane & 3) == 0) *offs_out = pos;
+        offs_out += kSbChunks;
+        if constexpr (!INDEX32) {
+            *mask_out = keep;
+            mask_out += kSbElems / 32;
+        }
+        const uint32_t stage0 = s_vals_addr - 2u * head;      // position p is staged at stage0 + 2 p
+        if constexpr (DENSE) {
+            // straight from the registers, element by element
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t v8 = ((uint32_t)j ^ rot) * 8;       // the lane's elements in registers 4 * j ..
+                const uint32_t bits = keep >> v8;
+                [[maybe_unused]] uint32_t p_abs = pos + __popc(keep & ((1u << v8) - 1u));
+                uint32_t to = stage0 + 2u * p_abs;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const uint32_t v = (e & 1) ? w[4 * j + e / 2] >> 16 : w[4 * j + e / 2];
+                    if (bits & (1u << e)) {
+                        asm volatile("st.shared.u16 [%0], %1;" ::"r"(to), "h"((uint16_t)v) : "memory");
+                        to += 2;
+                        if constexpr (INDEX32) indices[p_abs++] = first_idx + (int32_t)(v8 + e);
+                    }
+                }
+            }
+        } else {
+            // highest first: read from the ring, staged at their final position
+            uint32_t left = keep;
+            [[maybe_unused]] uint32_t p_abs = gpos + inc;
+            uint32_t to = stage0 + 2u * (gpos + inc);
+            while (left) {
+                const uint32_t e = top_bit(left);
+                left ^= 1u << e;
+                to -= 2;
+                const uint32_t v = lds_u16(own + 2u * e);
+                asm volatile("st.shared.u16 [%0], %1;" ::"r"(to), "h"((uint16_t)v) : "memory");
+                if constexpr (INDEX32) indices[--p_abs] = first_idx + (int32_t)e;
+            }
+        }
+        if constexpr (INDEX32) first_idx += kSbElems;
+        gpos += __shfl_sync(kFullMask, inc, 31);
+        __syncwarp();   // staged values visible to the warp; every lane is done with the ring slot
+        at ^= kSbBytes;
+        if (gpos - head > (uint32_t)kStageKeep) flush();
+    };
+    auto compact_run = [&](auto dense_tag) {
+        const uint4* src = x + sb0 * kSbVecs + lane;
+        for (int more = (int)(sb_full_end - sb0) - 1; more > 0; --more) {
+            src += kSbVecs;
+            sb_issue_full(ring_copy + (at ^ kSbBytes), src);
+            compact_fast(dense_tag);
+        }
+        slot = at / kSbBytes;
+        issue_sb(sb_full_end, slot ^ 1);
+        compact_fast(dense_tag);
+        slot ^= 1;
+    };
+    // any super-block: the run in which the quota ends, and the tensor's ragged last super-block
+    auto compact_sb = [&](int64_t sb) {
         issue_sb(sb + 1, slot ^ 1);
         sb_wait();
         __syncwarp();   // the lane reads vectors that other lanes copied
@@ -901,7 +1107,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
             }
         }
         uint32_t e32 = ge32 & ~g32;   // key == T
-        if constexpr (!FULL) e32 &= valid_mask32(sb * kSbElems + lane * 32, n);   // zero padding must not tie with T = 0
+        e32 &= valid_mask32(sb * kSbElems + lane * 32, n);   // zero padding must not tie with T = 0
         const uint32_t cnt = __popc(g32) | (__popc(e32) << 16);
         // packed (gt | eq << 16) prefix over the lanes = over the super-block's elements
         uint32_t inc = cnt;
@@ -929,19 +1135,11 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
         }
         const uint32_t pos = run_gt + (excl & 0xFFFFu) + min(eq_before, q);   // retained elements before this lane's first
         if ((lane & 3) == 0) {   // the lane opens a 128-element chunk
-            if constexpr (FULL) {
-                offsets[sb * kSbChunks + (lane >> 2)] = pos;
-            } else {
-                if (sb * kSbElems + lane * 32 < n) offsets[sb * kSbChunks + (lane >> 2)] = pos;
-            }
+            if (sb * kSbElems + lane * 32 < n) offsets[sb * kSbChunks + (lane >> 2)] = pos;
         }
         if constexpr (!INDEX32) {
             const int64_t wi = sb * (kSbElems / 32) + lane;
-            if constexpr (FULL) {
-                mask[wi] = keep;
-            } else {
-                if (wi < nwords) mask[wi] = keep;
-            }
+            if (wi < nwords) mask[wi] = keep;
         }
         {
             // the lane's retained elements, highest first: read from the ring, staged at their final position
@@ -962,32 +1160,23 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
         gpos = run_gt + min(run_eq, q);
         __syncwarp();   // staged values visible to the warp; every lane is done with the ring slot
         slot ^= 1;
-        // write the whole 16-byte pieces, carry the rest to the front
-        const uint32_t staged = gpos - head;
-        const uint32_t pieces = staged / 8;
-        if (pieces) {
-            for (uint32_t c = lane; c < pieces; c += 32) {
-                if (c == 0 && foreign) {
-                    for (uint32_t e = foreign; e < 8; ++e) values[head + e] = s_vals[e];
-                } else {
-                    *reinterpret_cast<uint4*>(values + head + c * 8) = *reinterpret_cast<const uint4*>(s_vals + c * 8);
-                }
-            }
-            foreign = 0;
-            const uint32_t rem = staged - pieces * 8;
-            uint16_t carry = 0;
-            if (lane < (int)rem) carry = s_vals[pieces * 8 + lane];
-            __syncwarp();
-            if (lane < (int)rem) s_vals[lane] = carry;
-            head += pieces * 8;
-            __syncwarp();
-        }
+        if (gpos - head > (uint32_t)kStageKeep) flush();
     };
     {
         int64_t sb = sb0;
-        for (; sb < sb_full_end; ++sb) compact_sb(sb, std::true_type{});
-        for (; sb < sb1; ++sb) compact_sb(sb, std::false_type{});
+        if (one_threshold && sb0 < sb_full_end) {
+            // Words with many retained elements go element by element from the registers (a fixed 32 predicated stores), words
+            // with few through a loop over the set bits (the warp makes as many trips as its fullest lane): with a tenth
+            // retained 40.9 against 39.8 us on 12608 x 3072, with a fifth 35.0 against 35.8 us and with half 41.3 against
+            // 47.8 us on 32768 x 768, so the line lies in between.
+            if (k * 20 > (unsigned long long)n * 3) compact_run(std::true_type{});
+            else compact_run(std::false_type{});
+            run_gt = gpos;
+            sb = sb_full_end;
+        }
+        for (; sb < sb1; ++sb) compact_sb(sb);
     }
+    flush();
     // the elements of the last, partial piece (the warp behind this one writes the rest of that piece)
     if (lane >= (int)foreign && head + lane < gpos) values[head + lane] = s_vals[lane];
     // Leave the barrier word stale.  A launch replayed from a captured graph carries the same epoch again; if the
