@@ -7,6 +7,7 @@ import threading
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libdropit.so")
+NATIVE_PATH = os.path.join(_PKG, "_native.so")
 
 _lock = threading.Lock()
 _lib = None
@@ -43,6 +44,17 @@ SIGNATURES = {
     "dropit_conv_weight_grad": (c_int, [c_vp, c_vp, c_vp, c_vp] + [c_int] * 10 + [c_i64, c_int, c_int, c_vp, c_int,
                                         c_vp, c_sz, c_vp, c_vp]),
 }
+
+
+def load_native():
+    """The native binding of the calls that a training step makes; raises if it is absent."""
+    load()      # fails with a message of its own if the CUDA library is missing
+    if not os.path.exists(NATIVE_PATH):
+        raise RuntimeError(
+            "_native.so is not built (%s). Run `python -m paper_2202_13808_b200.build`; "
+            "there is no fallback path." % NATIVE_PATH)
+    from . import _native
+    return _native
 
 
 def load():

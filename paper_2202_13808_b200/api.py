@@ -1,7 +1,8 @@
 """Torch-facing binding of the C ABI in include/dropit.h.
 
 Argument marshalling only: every step (selection, packing, recovery, weight gradients) runs in
-the CUDA library.  torch supplies device memory and the current stream.
+the CUDA library.  torch supplies device memory and the current stream.  The calls of a training
+step go through the native module (csrc/native.cpp), the others through ctypes.
 """
 from __future__ import annotations
 
@@ -89,14 +90,21 @@ class DropITCache:
         return sum(t.numel() * t.element_size() for t in parts if t is not None)
 
 
-_status_words = {}
+_native_module = None
+
+
+def _native():
+    """The native binding; raises if it has not been built."""
+    global _native_module
+    if _native_module is None:
+        mod = _lib.load_native()
+        mod.set_error_class(DropITError)
+        _native_module = mod
+    return _native_module
 
 
 def _status_word(device: torch.device) -> torch.Tensor:
-    key = (device.type, device.index)
-    if key not in _status_words:
-        _status_words[key] = torch.zeros(4, dtype=torch.int32, device=device)
-    return _status_words[key]
+    return _native().status_word(_device_index(device))
 
 
 def check_device_status(device=None) -> None:
@@ -135,24 +143,9 @@ def _require_cuda(t: torch.Tensor, name: str):
 
 def dropit_compress(x: torch.Tensor, gamma: float, fmt="bitmask", workspace: Optional[torch.Tensor] = None) -> DropITCache:
     """D(a), min-k (Sec. 3.3): retain the k largest-|x| elements of the whole tensor."""
-    _require_cuda(x, "x")
-    lib = _lib.load()
-    fmt = _FMT_CODE[fmt]
-    dt = _DTYPE_CODE[x.dtype]
-    n = x.numel()
-    vb, mb, ob, wb = dropit_cache_sizes(n, gamma, dt, fmt)
-    k = dropit_keep_count(n, gamma)
-    dev = x.device
-    values = torch.empty(vb // x.element_size(), dtype=x.dtype, device=dev)
-    meta = torch.empty(mb // 4, dtype=torch.int32, device=dev)
-    offsets = torch.empty(ob // 4, dtype=torch.int32, device=dev)
-    if workspace is None or workspace.numel() < wb:
-        workspace = torch.empty(max(wb, 16), dtype=torch.uint8, device=dev)
-    with _on_device(dev):
-        code = lib.dropit_compress(_ptr(x), n, float(gamma), dt, fmt, _ptr(values), _ptr(meta), _ptr(offsets),
-                                   _ptr(workspace), workspace.numel(), _ptr(_status_word(dev)), _stream_ptr(dev))
-    _check(code, "dropit_compress")
-    return DropITCache(values, meta, offsets, n, k, tuple(x.shape), x.dtype, fmt, float(gamma))
+    fmt, gamma = _FMT_CODE[fmt], float(gamma)
+    values, meta, offsets, k = _native().compress(x, gamma, fmt, workspace)
+    return DropITCache(values, meta, offsets, x.numel(), k, tuple(x.shape), x.dtype, fmt, gamma)
 
 
 def dropit_quantize_cache(cache: DropITCache) -> DropITCache:
@@ -230,39 +223,15 @@ def dropit_produce(x: torch.Tensor, gamma: float, act: str = "identity", table: 
         code_act = ACT_TABLE
     else:
         code_act = {"identity": ACT_IDENTITY, "relu": ACT_RELU}[act]
-    n = x.numel()
-    y = torch.empty_like(x) if (want_y or code_act != ACT_IDENTITY) else None
-    prep = torch.empty(max(dropit_produce_workspace(n), 16), dtype=torch.uint8, device=dev)
-    with _on_device(dev):
-        code = _lib.load().dropit_produce(_ptr(x), n, float(gamma), code_act, _ptr(table), _ptr(y), _ptr(prep),
-                                          prep.numel(), _stream_ptr(dev))
-    _check(code, "dropit_produce")
-    return y, prep
+    return _native().produce(x, float(gamma), code_act, table, want_y or code_act != ACT_IDENTITY)
 
 
 def dropit_compress_prepared(y: torch.Tensor, gamma: float, prep: torch.Tensor, fmt="bitmask",
                              workspace: Optional[torch.Tensor] = None) -> DropITCache:
     """dropit_compress of a tensor whose selection statistics dropit_produce has already taken: one read of y."""
-    _require_cuda(y, "y")
-    if y.dtype != torch.bfloat16:
-        raise TypeError("dropit_compress_prepared takes bf16 tensors")
-    lib = _lib.load()
-    fmt = _FMT_CODE[fmt]
-    n = y.numel()
-    vb, mb, ob, wb = dropit_cache_sizes(n, gamma, BF16, fmt)
-    k = dropit_keep_count(n, gamma)
-    dev = y.device
-    values = torch.empty(vb // 2, dtype=torch.bfloat16, device=dev)
-    meta = torch.empty(mb // 4, dtype=torch.int32, device=dev)
-    offsets = torch.empty(ob // 4, dtype=torch.int32, device=dev)
-    if workspace is None or workspace.numel() < wb:
-        workspace = torch.empty(max(wb, 16), dtype=torch.uint8, device=dev)
-    with _on_device(dev):
-        code = lib.dropit_compress_prepared(_ptr(y), n, float(gamma), fmt, _ptr(values), _ptr(meta), _ptr(offsets),
-                                            _ptr(prep), prep.numel(), _ptr(workspace), workspace.numel(),
-                                            _ptr(_status_word(dev)), _stream_ptr(dev))
-    _check(code, "dropit_compress_prepared")
-    return DropITCache(values, meta, offsets, n, k, tuple(y.shape), y.dtype, fmt, float(gamma))
+    fmt, gamma = _FMT_CODE[fmt], float(gamma)
+    values, meta, offsets, k = _native().compress_prepared(y, gamma, prep, fmt, workspace)
+    return DropITCache(values, meta, offsets, y.numel(), k, tuple(y.shape), y.dtype, fmt, gamma)
 
 
 @functools.lru_cache(maxsize=4096)
@@ -343,32 +312,10 @@ def dropit_weight_grad(dy: torch.Tensor, cache: DropITCache, out: Optional[torch
     """Eq. 6: dW[j, c] = sum over retained (n, c) of dY[n, j] a[n, c]; returns fp32 [Cz, Ca].
 
     fused=True calls dropit_weight_grad_fused (cache expanded inside the GEMM, no dense scratch)."""
-    cache = dropit_dequantize_cache(cache)
-    _require_cuda(dy, "dy")
-    if dy.dtype != cache.dtype:
-        raise TypeError("dy dtype %s != cache dtype %s" % (dy.dtype, cache.dtype))
-    Ca = cache.shape[-1]
-    M = cache.n // Ca if Ca else 0
-    Cz = dy.shape[-1]
-    if dy.numel() != M * Cz:
-        raise ValueError("dy has %d elements, expected %d x %d" % (dy.numel(), M, Cz))
-    lib = _lib.load()
-    dev = dy.device
-    dt = _DTYPE_CODE[cache.dtype]
-    if out is None:
-        if accumulate:
-            raise ValueError("accumulate=True needs out")
-        out = torch.empty((Cz, Ca), dtype=torch.float32, device=dev)
-    wb = dropit_weight_grad_workspace(M, Ca, Cz, dt, cache.fmt, dev)
-    if workspace is None or workspace.numel() < wb:
-        workspace = torch.empty(max(wb, 16), dtype=torch.uint8, device=dev)
-    with _on_device(dev):
-        fn = lib.dropit_weight_grad_fused if fused else lib.dropit_weight_grad
-        code = fn(_ptr(dy), _ptr(cache.values), _ptr(cache.meta), _ptr(cache.offsets), M, Ca, Cz,
-                                      cache.k, dt, cache.fmt, _ptr(out), int(bool(accumulate)), _ptr(workspace),
-                                      workspace.numel(), _ptr(_status_word(dev)), _stream_ptr(dev))
-    _check(code, "dropit_weight_grad_fused" if fused else "dropit_weight_grad")
-    return out
+    if cache.values is None:
+        cache = dropit_dequantize_cache(cache)
+    return _native().weight_grad(dy, cache.values, cache.meta, cache.offsets, cache.n, cache.shape[-1], cache.k, cache.fmt, out,
+                                 accumulate, workspace, fused)
 
 
 @functools.lru_cache(maxsize=4096)
@@ -390,27 +337,9 @@ def dropit_conv_weight_grad(dy: torch.Tensor, cache: DropITCache, kernel_size: T
                             pad: int = 0, dilation: int = 1, out: Optional[torch.Tensor] = None,
                             accumulate: bool = False, workspace: Optional[torch.Tensor] = None) -> torch.Tensor:
     """Eq. 4-5 retained term: dW[j,c,u,v] from dY [B,Cz,Ho,Wo] and the cache of a [B,Ca,H,W]; fp32."""
-    cache = dropit_dequantize_cache(cache)
-    _require_cuda(dy, "dy")
-    if dy.dtype != cache.dtype:
-        raise TypeError("dy dtype %s != cache dtype %s" % (dy.dtype, cache.dtype))
+    if cache.values is None:
+        cache = dropit_dequantize_cache(cache)
     B, Ca, H, W = cache.shape
     R, S = kernel_size
-    Cz = dy.shape[1]
-    lib = _lib.load()
-    dev = dy.device
-    dt = _DTYPE_CODE[cache.dtype]
-    if out is None:
-        if accumulate:
-            raise ValueError("accumulate=True needs out")
-        out = torch.empty((Cz, Ca, R, S), dtype=torch.float32, device=dev)
-    wb = dropit_conv_weight_grad_workspace(B, Ca, H, W, Cz, R, S, stride, pad, dt, cache.fmt, dev)
-    if workspace is None or workspace.numel() < wb:
-        workspace = torch.empty(max(wb, 16), dtype=torch.uint8, device=dev)
-    with _on_device(dev):
-        code = lib.dropit_conv_weight_grad(_ptr(dy), _ptr(cache.values), _ptr(cache.meta), _ptr(cache.offsets), B, Ca,
-                                           H, W, Cz, R, S, stride, pad, dilation, cache.k, dt, cache.fmt, _ptr(out),
-                                           int(bool(accumulate)), _ptr(workspace), workspace.numel(),
-                                           _ptr(_status_word(dev)), _stream_ptr(dev))
-    _check(code, "dropit_conv_weight_grad")
-    return out
+    return _native().conv_weight_grad(dy, cache.values, cache.meta, cache.offsets, B, Ca, H, W, R, S, stride, pad, dilation, cache.k,
+                                      cache.fmt, out, accumulate, workspace)

@@ -26,6 +26,8 @@
 // (decompression, shifted or gathered copies, GEMM on 64-pixel rows; per call at batch 64, gamma 0.8, graph replay): 3 x 3
 // 64 -> 64 on 56 x 56 59 -> 50 us, 128 -> 128 on 28 x 28 130 -> 46, 256 -> 256 on 14 x 14 126 -> 51, 512 -> 512 on 7 x 7
 // 332 -> 93, stride 2 128 -> 128 on 56 x 56 212 -> 70; 1 x 1 1024 -> 256 on 14 x 14 113 -> 54.
+#include <cstring>
+
 #include "weight_grad_common.cuh"
 
 namespace dropit {
@@ -557,12 +559,32 @@ bool make_fused_conv_plan(FusedConvParams& p, int B, int Ca, int H, int W, int C
     return true;
 }
 
+// The plan of the last shape that this thread asked for: the search over bands costs some ten microseconds, and a layer is
+// planned twice per call (workspace query and launch).
+bool cached_fused_conv_plan(FusedConvParams& p, int B, int Ca, int H, int W, int Cz, int R, int S, int stride, int pad, int64_t k) {
+    struct Last {
+        int key[10];
+        bool ok;
+        FusedConvParams p;
+    };
+    static thread_local Last last = {};
+    const int key[10] = {B, Ca, H, W, Cz, R, S, stride, pad, sm_count()};
+    if (std::memcmp(key, last.key, sizeof(key)) != 0) {
+        last.ok = make_fused_conv_plan(last.p, B, Ca, H, W, Cz, R, S, stride, pad, 0);
+        std::memcpy(last.key, key, sizeof(key));
+    }
+    if (!last.ok) return false;
+    p = last.p;
+    p.k = (uint32_t)k;
+    return true;
+}
+
 }  // namespace
 
 // 0 when this kernel does not take the shape.
 size_t conv_fused_workspace_bytes(int B, int Ca, int H, int W, int Cz, int R, int S, int stride, int pad) {
     FusedConvParams p;
-    if (!make_fused_conv_plan(p, B, Ca, H, W, Cz, R, S, stride, pad, 0)) return 0;
+    if (!cached_fused_conv_plan(p, B, Ca, H, W, Cz, R, S, stride, pad, 0)) return 0;
     return (size_t)p.splits * p.tiles_c * p.tiles_j * p.chunks * 32 * kBM * 4;
 }
 
@@ -571,7 +593,7 @@ dropit_status conv_fused_run(const void* dy, const void* values, const void* mas
                              int W, int Cz, int R, int S, int stride, int pad, int64_t k, float* dw, int accumulate,
                              void* workspace, size_t workspace_bytes, int32_t* dev_status, cudaStream_t stream) {
     FusedConvParams p;
-    if (!make_fused_conv_plan(p, B, Ca, H, W, Cz, R, S, stride, pad, k)) return DROPIT_ERR_UNSUPPORTED;
+    if (!cached_fused_conv_plan(p, B, Ca, H, W, Cz, R, S, stride, pad, k)) return DROPIT_ERR_UNSUPPORTED;
     const int tiles = p.tiles_c * p.tiles_j;
     if (workspace_bytes < (size_t)p.splits * tiles * p.chunks * 32 * kBM * 4) return DROPIT_ERR_WORKSPACE;
     const int vec = p.Wo % 8 == 0 ? 8 : (p.Wo % 2 == 0 ? 2 : 1);

@@ -137,41 +137,16 @@ class DropITConv2dFn(torch.autograd.Function):
         return dx, dw, db, None, None, None, None, None
 
 
-class DropITGeluLinearFn(torch.autograd.Function):
+class DropITGeluLinearFn:
     """z = GELU(x) W^T + b for bf16 tensors, with the GELU written by the library's producer kernel so that the
     selection statistics of GELU(x), the tensor the Linear caches, are taken while it is written (Sec. 3.5: the
-    activation keeps its own cache x; only the Linear's cache is replaced by D(GELU(x)))."""
+    activation keeps its own cache x; only the Linear's cache is replaced by D(GELU(x))).  The autograd node is native
+    (csrc/native.cpp): forward and backward make a dozen calls, whose host side in Python took twice their GPU time."""
 
     @staticmethod
-    def forward(ctx, x, weight, bias, gamma: float, fmt: str):
+    def apply(x, weight, bias, gamma: float, fmt: str):
         _check_input(x)
-        x2 = x.reshape(-1, x.shape[-1])
-        x2 = x2 if x2.is_contiguous() else x2.contiguous()
-        y, prep = api.dropit_produce(x2, gamma, "gelu")
-        z = F.linear(y, weight, bias).reshape(*x.shape[:-1], weight.shape[0])
-        ctx.has_bias = bias is not None
-        ctx.x_shape = tuple(x.shape)
-        cache = api.dropit_compress_prepared(y, gamma, prep, fmt)
-        ctx.cache_meta = (cache.n, cache.k, cache.shape, cache.dtype, cache.fmt, cache.gamma)
-        ctx.save_for_backward(x2, weight, cache.values, cache.meta, cache.offsets)
-        return z
-
-    @staticmethod
-    def backward(ctx, dz):
-        x2, weight, values, meta, offsets = ctx.saved_tensors
-        dx = dw = db = None
-        dz2 = dz.reshape(-1, dz.shape[-1])
-        if ctx.needs_input_grad[0]:
-            dy = dz2 @ weight                                             # Eq. 3: exact, needs theta only
-            dx = torch.ops.aten.gelu_backward(dy, x2).reshape(ctx.x_shape)   # the activation's own cache is x
-        if ctx.needs_input_grad[1]:
-            n, k, shape, dtype, fmt, gamma = ctx.cache_meta
-            cache = api.DropITCache(values, meta, offsets, n, k, shape, dtype, fmt, gamma)
-            dzc = dz2 if dz2.is_contiguous() else dz2.contiguous()
-            dw = api.dropit_weight_grad(dzc.to(dtype), cache).to(weight.dtype)   # Eq. 6
-        if ctx.has_bias and ctx.needs_input_grad[2]:
-            db = dz2.sum(0)
-        return dx, dw, db, None, None
+        return api._native().gelu_linear(x, weight, bias, gamma, api._FMT_CODE[fmt], api.dropit_activation_table("gelu", x.device))
 
 
 class _Strategy:
