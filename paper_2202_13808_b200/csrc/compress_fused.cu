@@ -1001,12 +1001,14 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
     };
     issue_sb(sb0, 0);
     int slot = 0;
-    // a super-block under the one threshold; `at` = offset of its slot in the ring, `out` = where its mask words and table
-    // entries go, `first_idx` = the lane's first element
+    // a super-block under the one threshold; `at` = offset of its slot in the ring, *_out = where its mask words and table
+    // entries go, sb_first = its first element.  Many indices leave coalesced, through the slot (scattered straight from the
+    // lanes they took the call from 41 to 112 us on 32768 x 768 at gamma 0.5, through the slot 53 us); few go straight
+    // (12608 x 768 at gamma 0.9: 20 against 22 us).
     uint32_t at = 0;
     uint32_t* mask_out = INDEX32 ? nullptr : mask + sb0 * (kSbElems / 32) + lane;
     uint32_t* offs_out = offsets + sb0 * kSbChunks + (lane >> 2);
-    [[maybe_unused]] int32_t first_idx = (int32_t)(sb0 * kSbElems) + lane * 32;
+    [[maybe_unused]] int32_t sb_first = (int32_t)(sb0 * kSbElems);
     auto compact_fast = [&](auto dense_tag) {
         constexpr bool DENSE = decltype(dense_tag)::value;
         sb_wait();
@@ -1034,6 +1036,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
         }
         const uint32_t stage0 = s_vals_addr - 2u * head;      // position p is staged at stage0 + 2 p
         if constexpr (DENSE) {
+            if constexpr (INDEX32) __syncwarp();   // the slot has been read by all lanes: it takes the element numbers
             // straight from the registers, element by element
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -1047,9 +1050,18 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                     if (bits & (1u << e)) {
                         asm volatile("st.shared.u16 [%0], %1;" ::"r"(to), "h"((uint16_t)v) : "memory");
                         to += 2;
-                        if constexpr (INDEX32) indices[p_abs++] = first_idx + (int32_t)(v8 + e);
+                        if constexpr (INDEX32) {
+                            asm volatile("st.shared.u16 [%0], %1;" ::"r"(ring_warp + at + 2u * (p_abs - gpos)), "h"((uint16_t)(lane * 32 + v8 + e)) : "memory");
+                            ++p_abs;
+                        }
                     }
                 }
+            }
+            if constexpr (INDEX32) {
+                __syncwarp();
+                const uint32_t kept = __shfl_sync(kFullMask, inc, 31);
+                for (uint32_t i = lane; i < kept; i += 32)
+                    indices[gpos + i] = sb_first + (int32_t)lds_u16(ring_warp + at + 2u * i);
             }
         } else {
             // highest first: read from the ring, staged at their final position
@@ -1062,10 +1074,10 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                 to -= 2;
                 const uint32_t v = lds_u16(own + 2u * e);
                 asm volatile("st.shared.u16 [%0], %1;" ::"r"(to), "h"((uint16_t)v) : "memory");
-                if constexpr (INDEX32) indices[--p_abs] = first_idx + (int32_t)e;
+                if constexpr (INDEX32) indices[--p_abs] = sb_first + lane * 32 + (int32_t)e;
             }
         }
-        if constexpr (INDEX32) first_idx += kSbElems;
+        if constexpr (INDEX32) sb_first += kSbElems;
         gpos += __shfl_sync(kFullMask, inc, 31);
         __syncwarp();   // staged values visible to the warp; every lane is done with the ring slot
         at ^= kSbBytes;

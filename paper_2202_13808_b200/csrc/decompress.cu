@@ -210,6 +210,64 @@ decompress_bitmask_kernel(const typename Tr::elem_t* __restrict__ values, const 
     }
 }
 
+// Coordinate format: a warp inflates 1024 elements per step in a zeroed image in shared memory; the seek table tells which
+// retained values fall into the step.  One launch and full-line stores, where a memset and a scatter kernel wrote the tensor
+// twice (2-byte stores all over it): 591 x 768 bf16 3.8 us and a launch gap -> 2.6, 18706 x 472 at gamma 0.64 12.6 -> 7 us.
+constexpr int kIdxWarps = 8;
+template <typename Tr>
+__global__ void __launch_bounds__(32 * kIdxWarps)
+decompress_index32_kernel(const typename Tr::elem_t* __restrict__ values, const uint32_t* __restrict__ idx,
+                          const uint32_t* __restrict__ offsets, int64_t n, int64_t k, typename Tr::elem_t* __restrict__ out) {
+    using elem_t = typename Tr::elem_t;
+    constexpr int G = Tr::kVecElems;
+    __shared__ __align__(16) elem_t image[kIdxWarps][1024];
+    ptx::grid_dependency_wait();
+    ptx::launch_dependents();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint4* img = reinterpret_cast<uint4*>(image[warp]);
+    const uint32_t steps = (uint32_t)((n + 1023) / 1024), stride = gridDim.x * kIdxWarps;
+    const uint32_t nchunks = (uint32_t)((n + DROPIT_CHUNK - 1) / DROPIT_CHUNK), k32 = (uint32_t)k;
+    auto entry = [&](uint32_t t) -> uint32_t { return t * 8 < nchunks ? min(__ldg(offsets + t * 8), k32) : k32; };
+    uint32_t t = blockIdx.x * kIdxWarps + warp;
+    uint32_t next0 = t < steps ? entry(t) : 0u, next1 = t < steps ? entry(t + 1) : 0u;
+    for (; t < steps; t += stride) {
+        const uint32_t r0 = next0, r1 = next1;
+        if (t + stride < steps) {
+            next0 = entry(t + stride);
+            next1 = entry(t + stride + 1);
+        }
+#pragma unroll
+        for (int i = 0; i < 1024 / G / 32; ++i) img[i * 32 + lane] = make_uint4(0, 0, 0, 0);
+        __syncwarp();
+        for (uint32_t r = r0 + lane; r < r1; r += 128) {          // four pairs in flight per lane
+            uint32_t at[4];
+            elem_t val[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                at[u] = 1024;
+                val[u] = 0;
+                if (r + 32 * u < r1) {
+                    at[u] = __ldg(idx + r + 32 * u) - t * 1024;
+                    val[u] = __ldg(values + r + 32 * u);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (at[u] < 1024) image[warp][at[u]] = val[u];     // (an index outside the step is dropped)
+        }
+        __syncwarp();
+        const int64_t e0 = (int64_t)t * 1024;
+        if (e0 + 1024 <= n) {
+#pragma unroll
+            for (int i = 0; i < 1024 / G / 32; ++i) reinterpret_cast<uint4*>(out + e0)[i * 32 + lane] = img[i * 32 + lane];
+        } else {
+            for (int e = lane; e0 + e < n; e += 32) out[e0 + e] = image[warp][e];
+        }
+        __syncwarp();
+    }
+}
+
+// ... without a seek table
 template <typename Tr>
 __global__ void __launch_bounds__(256)
 scatter_index32_kernel(const typename Tr::elem_t* __restrict__ values, const int32_t* __restrict__ idx, int64_t k,
@@ -246,6 +304,27 @@ static dropit_status run_decompress(const void* values, const void* meta, const 
         if (cudaLaunchKernelEx(&cfg, decompress_bitmask_kernel<Tr>, reinterpret_cast<const elem_t*>(values),
                                reinterpret_cast<const uint32_t*>(meta), offsets, n, k, reinterpret_cast<elem_t*>(out)) !=
             cudaSuccess) {
+            (void)cudaGetLastError();
+            return DROPIT_ERR_CUDA;
+        }
+        return check_launch();
+    }
+    if (offsets != nullptr) {
+        const int64_t steps = (n + 1023) / 1024;
+        int64_t blocks = (steps + kIdxWarps - 1) / kIdxWarps;
+        const int64_t resident = (int64_t)sm_count() * (Tr::kElemBytes == 2 ? 8 : 6);
+        if (blocks > resident) blocks = resident;
+        cudaLaunchAttribute pdl[1];
+        pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        pdl[0].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)blocks);
+        cfg.blockDim = dim3(32 * kIdxWarps);
+        cfg.stream = stream;
+        cfg.attrs = pdl;
+        cfg.numAttrs = 1;
+        if (cudaLaunchKernelEx(&cfg, decompress_index32_kernel<Tr>, reinterpret_cast<const elem_t*>(values),
+                               reinterpret_cast<const uint32_t*>(meta), offsets, n, k, reinterpret_cast<elem_t*>(out)) != cudaSuccess) {
             (void)cudaGetLastError();
             return DROPIT_ERR_CUDA;
         }

@@ -791,56 +791,165 @@ wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
 }
 
 // ---------------------------------------------------------------------------------------------
-// FFMA kernel: fp32 inputs, or bf16 shapes that the TMA path cannot take.  64x64 output tile,
-// 16 tokens per step, 4x4 outputs per thread.
+// FFMA kernel: fp32 inputs, or bf16 shapes that the TMA path cannot take.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ float to_float(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }
 __device__ __forceinline__ float to_float(float f) { return f; }
 
-template <typename T>
+// dY tile (kFmaK tokens x TILE outputs) and R(a-hat) tile (x TILE channels) in shared memory, the next ones on their way in
+// registers.  A thread holds MICRO x MICRO sums, packed in pairs for the two-wide FMA; the threads form groups that each
+// cover the tile and share out the tokens of a stage, and the groups' sums are added in group order.  64-wide tiles: 8 x 8
+// sums, 4 groups of 64 threads.  32-wide tiles, for outputs too small to fill the chip with 64-wide ones: 4 x 4 sums, 4 groups.
+// Bound by the FMA rate (256 x 768 x 768: 2.2 us at the two-wide rate) and the latency of its eight stages.
+constexpr int kFmaK = 32;
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(unsigned long long v, float& lo, float& hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+template <typename T, int TILE>
 __global__ void __launch_bounds__(256)
 wg_ffma_kernel(const T* __restrict__ dy, const T* __restrict__ xd, int M, int Ca, int Cz, float* __restrict__ dw,
                int accumulate) {
-    __shared__ float sA[16][64 + 4];
-    __shared__ float sB[16][64 + 4];
-    const int j0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    const int lr = threadIdx.x >> 4, lc = (threadIdx.x & 15) * 4;
-    float acc[4][4] = {};
-    for (int k0 = 0; k0 < M; k0 += 16) {
-        const int n = k0 + lr;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int j = j0 + lc + e, c = c0 + lc + e;
-            sA[lr][lc + e] = (n < M && j < Cz) ? to_float(dy[(size_t)n * Cz + j]) : 0.f;
-            sB[lr][lc + e] = (n < M && c < Ca) ? to_float(xd[(size_t)n * Ca + c]) : 0.f;
+    constexpr int kMicro = TILE / 8;                           // 8 or 4
+    constexpr int kGroups = 4, kSide = 8;                      // 4 groups of 8 x 8 threads
+    constexpr int kCols4 = TILE / 4;
+    constexpr int kUnits = kFmaK * kCols4 / 256;               // 4-element pieces per thread and operand
+    constexpr int kPitch = TILE + 4;
+    __shared__ __align__(16) float smem[2][2][kFmaK][kPitch];  // [operand][buffer]
+    auto& sA = smem[0];
+    auto& sB = smem[1];
+    const int j0 = blockIdx.y * TILE, c0 = blockIdx.x * TILE;
+    const int group = threadIdx.x / (kSide * kSide), tg = threadIdx.x % (kSide * kSide);
+    const int tx = tg % kSide, ty = tg / kSide;                // a thread's sums: 4-wide pieces 32 columns (rows) apart
+    const bool vec_a = (Cz & 3) == 0, vec_b = (Ca & 3) == 0;   // rows start on a 4-element boundary
+    float4 ra[kUnits], rb[kUnits];
+    auto load4 = [&](const T* p, int n, int col, int cols, bool vec) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (n >= M) return v;
+        const T* q = p + (size_t)n * cols + col;
+        if (vec && col + 4 <= cols) {
+            if constexpr (sizeof(T) == 4) {
+                v = __ldg(reinterpret_cast<const float4*>(q));
+            } else {
+                const uint2 u = __ldg(reinterpret_cast<const uint2*>(q));
+                v = make_float4(to_float((T)(u.x & 0xFFFFu)), to_float((T)(u.x >> 16)), to_float((T)(u.y & 0xFFFFu)), to_float((T)(u.y >> 16)));
+            }
+        } else {
+            if (col < cols) v.x = to_float(q[0]);
+            if (col + 1 < cols) v.y = to_float(q[1]);
+            if (col + 2 < cols) v.z = to_float(q[2]);
+            if (col + 3 < cols) v.w = to_float(q[3]);
         }
-        __syncthreads();
+        return v;
+    };
+    auto load_stage = [&](int k0) {
 #pragma unroll
-        for (int k = 0; k < 16; ++k) {
-            float a[4], b[4];
+        for (int u = 0; u < kUnits; ++u) {
+            const int unit = u * 256 + threadIdx.x, row = unit / kCols4, col = (unit % kCols4) * 4;
+            ra[u] = load4(dy, k0 + row, j0 + col, Cz, vec_a);
+            rb[u] = load4(xd, k0 + row, c0 + col, Ca, vec_b);
+        }
+    };
+    auto store_stage = [&](int buf) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                a[i] = sA[k][ty * 4 + i];
-                b[i] = sB[k][tx * 4 + i];
+        for (int u = 0; u < kUnits; ++u) {
+            const int unit = u * 256 + threadIdx.x, row = unit / kCols4, col = (unit % kCols4) * 4;
+            *reinterpret_cast<float4*>(&sA[buf][row][col]) = ra[u];
+            *reinterpret_cast<float4*>(&sB[buf][row][col]) = rb[u];
+        }
+    };
+    unsigned long long acc[kMicro][kMicro / 2];                // pairs of neighbouring channels
+#pragma unroll
+    for (int i = 0; i < kMicro; ++i)
+#pragma unroll
+        for (int l = 0; l < kMicro / 2; ++l) acc[i][l] = 0ull;
+    ptx::grid_dependency_wait();                               // the dense scratch comes from the kernel before this one
+    load_stage(0);
+    store_stage(0);
+    __syncthreads();
+    int buf = 0;
+    for (int k0 = 0; k0 < M; k0 += kFmaK, buf ^= 1) {
+        const bool more = k0 + kFmaK < M;
+        if (more) load_stage(k0 + kFmaK);
+#pragma unroll
+        for (int kk = 0; kk < kFmaK / kGroups; ++kk) {
+            const int row = group * (kFmaK / kGroups) + kk;
+            float a[kMicro];
+            unsigned long long b[kMicro / 2];
+#pragma unroll
+            for (int h = 0; h < kMicro / 4; ++h) {
+                const float4 a4 = *reinterpret_cast<const float4*>(&sA[buf][row][h * 32 + ty * 4]);
+                const float4 b4 = *reinterpret_cast<const float4*>(&sB[buf][row][h * 32 + tx * 4]);
+                a[4 * h] = a4.x; a[4 * h + 1] = a4.y; a[4 * h + 2] = a4.z; a[4 * h + 3] = a4.w;
+                b[2 * h] = pack2(b4.x, b4.y);
+                b[2 * h + 1] = pack2(b4.z, b4.w);
             }
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < kMicro; ++i) {
+                const unsigned long long aa = pack2(a[i], a[i]);
 #pragma unroll
-                for (int l = 0; l < 4; ++l) acc[i][l] = fmaf(a[i], b[l], acc[i][l]);
+                for (int l = 0; l < kMicro / 2; ++l) fma2(acc[i][l], aa, b[l]);
+            }
         }
+        if (more) store_stage(buf ^ 1);                        // last read before the previous barrier
         __syncthreads();
     }
+    float out[kMicro][kMicro];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < kMicro; ++i)
 #pragma unroll
-        for (int l = 0; l < 4; ++l) {
-            const int j = j0 + ty * 4 + i, c = c0 + tx * 4 + l;
-            if (j < Cz && c < Ca) {
-                float* d = dw + (size_t)j * Ca + c;
-                *d = accumulate ? (*d + acc[i][l]) : acc[i][l];
+        for (int l = 0; l < kMicro / 2; ++l) unpack2(acc[i][l], out[i][2 * l], out[i][2 * l + 1]);
+    // the groups' sums, in group order, one group after the other through the (finished) buffers
+    float4* share = reinterpret_cast<float4*>(&smem[0][0][0][0]);
+    constexpr int kPieces = kMicro * kMicro / 4;
+    static_assert(sizeof(smem) >= (size_t)kSide * kSide * kPieces * sizeof(float4), "room for one group's sums");
+    for (int g = 1; g < kGroups; ++g) {
+        if (group == g)
+#pragma unroll
+            for (int q = 0; q < kPieces; ++q) {
+                const int i = q / (kMicro / 4), h = (q % (kMicro / 4)) * 4;
+                share[q * (kSide * kSide) + tg] = make_float4(out[i][h], out[i][h + 1], out[i][h + 2], out[i][h + 3]);
+            }
+        __syncthreads();
+        if (group == 0)
+#pragma unroll
+            for (int q = 0; q < kPieces; ++q) {
+                const int i = q / (kMicro / 4), h = (q % (kMicro / 4)) * 4;
+                const float4 v = share[q * (kSide * kSide) + tg];
+                out[i][h] += v.x; out[i][h + 1] += v.y; out[i][h + 2] += v.z; out[i][h + 3] += v.w;
+            }
+        __syncthreads();
+    }
+    if (group != 0) return;
+#pragma unroll
+    for (int i = 0; i < kMicro; ++i) {
+        const int j = j0 + (i / 4) * 32 + ty * 4 + i % 4;
+        if (j >= Cz) continue;
+#pragma unroll
+        for (int h = 0; h < kMicro / 4; ++h) {
+            const int c = c0 + h * 32 + tx * 4;
+            float* d = dw + (size_t)j * Ca + c;
+            if (vec_b && c + 4 <= Ca) {
+                float4 v = make_float4(out[i][4 * h], out[i][4 * h + 1], out[i][4 * h + 2], out[i][4 * h + 3]);
+                if (accumulate) {
+                    const float4 o = *reinterpret_cast<const float4*>(d);
+                    v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+                }
+                *reinterpret_cast<float4*>(d) = v;
+            } else {
+#pragma unroll
+                for (int l = 0; l < 4; ++l)
+                    if (c + l < Ca) d[l] = accumulate ? d[l] + out[i][4 * h + l] : out[i][4 * h + l];
             }
         }
+    }
 }
 
 __global__ void zero_or_keep_kernel(float* dw, int64_t count, int accumulate) {
@@ -894,15 +1003,31 @@ static dropit_status weight_grad_impl(const void* dy, const void* values, const 
     if (s != DROPIT_OK) return s;
 
     if (!plan.tensor_core) {
-        dim3 grid(plan.tiles_n, plan.tiles_m);
+        // 32-wide tiles where 64-wide ones would leave more than half of the chip idle
+        const bool narrow = 2 * (int64_t)plan.tiles_n * plan.tiles_m <= sm_count();
+        const int tile = narrow ? 32 : 64;
+        cudaLaunchAttribute pdl[1];
+        pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        pdl[0].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)((Ca + tile - 1) / tile), (unsigned)((Cz + tile - 1) / tile));
+        cfg.blockDim = dim3(256);
+        cfg.stream = stream;
+        cfg.attrs = pdl;
+        cfg.numAttrs = 1;
+        cudaError_t err;
         if (dtype == DROPIT_BF16)
-            wg_ffma_kernel<uint16_t><<<grid, 256, 0, stream>>>(reinterpret_cast<const uint16_t*>(dy),
-                                                             reinterpret_cast<const uint16_t*>(dense), (int)M, (int)Ca,
-                                                             (int)Cz, dw, accumulate);
+            err = cudaLaunchKernelEx(&cfg, narrow ? wg_ffma_kernel<uint16_t, 32> : wg_ffma_kernel<uint16_t, 64>,
+                                     reinterpret_cast<const uint16_t*>(dy), reinterpret_cast<const uint16_t*>(dense), (int)M, (int)Ca,
+                                     (int)Cz, dw, accumulate);
         else
-            wg_ffma_kernel<float><<<grid, 256, 0, stream>>>(reinterpret_cast<const float*>(dy),
-                                                          reinterpret_cast<const float*>(dense), (int)M, (int)Ca,
-                                                          (int)Cz, dw, accumulate);
+            err = cudaLaunchKernelEx(&cfg, narrow ? wg_ffma_kernel<float, 32> : wg_ffma_kernel<float, 64>,
+                                     reinterpret_cast<const float*>(dy), reinterpret_cast<const float*>(dense), (int)M, (int)Ca,
+                                     (int)Cz, dw, accumulate);
+        if (err != cudaSuccess) {
+            (void)cudaGetLastError();
+            return DROPIT_ERR_CUDA;
+        }
         return check_launch();
     }
 
