@@ -15,7 +15,7 @@
 //  * wg_tc_kernel (this file; Cz <= 128, or DROPIT_WG_PATH=single): the same with one CTA per 128 x 256 tile.
 //  * weight_grad_tmem.cu (dropit_weight_grad_fused): no scratch; the cache is expanded into tensor memory in
 //    front of the MMAs.  One launch, no workspace, slower.
-// Small output matrices are split along n ("split-K").  The splits of a tile add up through global memory:
+// Small output matrices are split along n ("split-K"; which way, make_wg_plan decides by cost).  The splits of a tile add up through global memory:
 // the tile is cut into as many parts as there are splits, every CTA stores the parts it does not finish into its
 // plane of the workspace and finishes the others, tickets deciding who finishes what (wg_tc_kernel with 2 or 4
 // splits: the splits form a thread-block cluster and exchange through distributed shared memory instead).
@@ -46,6 +46,8 @@ struct WgPlan {
     bool fused;               // weight_grad_tmem.cu: the cache is expanded into tensor memory inside the GEMM (no dense scratch)
     bool cluster;             // the splits of a tile form a thread-block cluster and add up through shared memory
     bool pair;                // CTA pairs compute 256 x 256 tiles (wg_pair_kernel); the splits add up through global memory
+    int stream_pairs;         // > 0: that many pairs share out all tiles' token blocks evenly (see StreamSplit), a second kernel adds up
+    int stream_slots;         // most pairs that share a tile
     int tiles_m, tiles_n, splits, kb_total, kb_per_split;
     size_t counters_off, counters_bytes;
     size_t dense_off, dense_bytes;
@@ -64,6 +66,32 @@ static bool wg_path_is(const char* name) {
     const char* e = std::getenv("DROPIT_WG_PATH");
     return e && std::strcmp(e, name) == 0;
 }
+
+// Even split: pair p of `pairs` takes the token blocks [p * units / pairs, (p + 1) * units / pairs) of the sequence
+// "all blocks of tile 0, all blocks of tile 1, ..." (units = tiles * kb_total).  With at least as many pairs as tiles it touches
+// two tiles at most.
+__host__ __device__ __forceinline__ int stream_begin(int p, int units, int pairs) { return (int)((int64_t)p * units / pairs); }
+// The first pair that touches the tile whose blocks start at `unit`.
+__host__ __device__ __forceinline__ int stream_first_pair(int unit, int units, int pairs) {
+    int p = (int)((int64_t)unit * pairs / units);
+    while (p > 0 && stream_begin(p, units, pairs) > unit) --p;
+    while (stream_begin(p + 1, units, pairs) <= unit) ++p;
+    return p;
+}
+
+// Splits used to be as many as the SMs hold, whatever adding them up costs.  Measured per call, decompression included, before
+// and after choosing by cost: 591 x 768 -> 768 16.9 -> 12.5 us (no split), 1000 x 1024 -> 1024 21.8 -> 14.2, 8000 x 768 -> 768
+// 34.2 -> 26.3, 20000 x 256 -> 768 37.2 -> 27.2 and 25000 x 200 -> 800 40.9 -> 33.1 (even split).
+// Microseconds, fitted on B200 (768 .. 3072 wide outputs, 591 .. 32768 tokens): a 144-token block of a pair's main loop,
+// and what adding up costs: tickets by the number of splits, or partial tiles written and read again by a second kernel.
+constexpr float kBlockUs = 0.66f;
+constexpr int64_t kStreamMaxBytes = (int64_t)80 << 20;
+static float ticket_us(int splits) {
+    return splits == 1 ? 0.f : (splits == 2 ? 3.8f : (splits == 3 ? 6.f : (splits == 4 ? 8.4f : (splits < 8 ? 10.f : 20.f))));
+}
+// Pairs of CTAs that the device holds at once (not every SM finds a neighbour), defined behind the kernel.
+static int resident_pairs();
+static float stream_us(int pairs, int tiles) { return 6.f + 0.07f * (float)(pairs + tiles); }
 
 static WgPlan make_wg_plan(int64_t M, int64_t Ca, int64_t Cz, dropit_dtype dtype, dropit_format format, bool fused) {
     WgPlan p{};
@@ -95,6 +123,33 @@ static WgPlan make_wg_plan(int64_t M, int64_t Ca, int64_t Cz, dropit_dtype dtype
         if (splits < 1) splits = 1;
         if (splits > 255) splits = 255;                                  // the tile counters hold eight bits
         if (splits > p.kb_total) splits = p.kb_total;
+        if (p.pair) {
+            // the cheaper of: whole ranges of the token axis per pair, with tickets; all blocks shared out evenly
+            const int most = splits, pair_tiles = tiles / 2, units = pair_tiles * p.kb_total;
+            float best = 0.f;
+            for (int s = 1; s <= most; ++s) {
+                const float us = kBlockUs * ((p.kb_total + s - 1) / s) + ticket_us(s);
+                if (s == 1 || us < best) { best = us; splits = s; }
+            }
+            const int all_pairs = resident_pairs() < units ? resident_pairs() : units;
+            // Under the even split the pairs are at different tokens at any time, so that a row of dY or of the scratch that
+            // several tiles share is read from HBM for each of them unless L2 holds both operands (32768 x 768 -> 2304, 201 MB:
+            // 122 us against 92 with aligned ranges).
+            const bool in_l2 = (M * Ca + M * Cz) * 2 <= kStreamMaxBytes;
+            for (int s = 2; s <= most + 1 && pair_tiles <= all_pairs && in_l2; ++s) {
+                const int pairs = s * pair_tiles < all_pairs ? s * pair_tiles : all_pairs;
+                const float us = kBlockUs * ((units + pairs - 1) / pairs) + stream_us(pairs, pair_tiles);
+                if (us < best) { best = us; p.stream_pairs = pairs; }
+            }
+            if (p.stream_pairs) {
+                splits = 1;
+                for (int t = 0; t < pair_tiles; ++t) {
+                    const int first = stream_first_pair(t * p.kb_total, units, p.stream_pairs);
+                    const int last = stream_first_pair((t + 1) * p.kb_total - 1, units, p.stream_pairs);
+                    if (last - first + 1 > p.stream_slots) p.stream_slots = last - first + 1;
+                }
+            }
+        }
         p.kb_per_split = (p.kb_total + splits - 1) / splits;
         p.splits = (p.kb_total + p.kb_per_split - 1) / p.kb_per_split;   // every split owns >= 1 block
         p.cluster = !p.pair && (p.splits == 2 || p.splits == 4);
@@ -108,7 +163,8 @@ static WgPlan make_wg_plan(int64_t M, int64_t Ca, int64_t Cz, dropit_dtype dtype
     p.dense_off = p.counters_off + p.counters_bytes;
     p.dense_bytes = align_up((size_t)M * Ca * es, 256);
     p.partial_off = p.dense_off + p.dense_bytes;
-    p.partial_bytes = (p.splits > 1 && !p.cluster) ? (size_t)p.splits * p.tiles_m * p.tiles_n * kBM * kBN * 4 : 0;   // whole tiles
+    const int planes = p.stream_pairs ? p.stream_slots : (p.splits > 1 && !p.cluster ? p.splits : 0);
+    p.partial_bytes = (size_t)planes * p.tiles_m * p.tiles_n * kBM * kBN * 4;   // whole tiles
     p.total_bytes = p.partial_off + p.partial_bytes;
     if (p.total_bytes == 0) p.total_bytes = 256;
     return p;
@@ -584,7 +640,7 @@ constexpr uint32_t kPairStageTx = kPairAStageBytes + kPairBStageBytes;
 struct PairSmem {
     uint64_t full[kPairStages];
     uint64_t empty[kPairStages];
-    uint64_t accum;
+    uint64_t accum[2];               // per segment (see PairSegments)
     uint32_t tmem_base;
     int abort_flag;
     int finisher;
@@ -597,11 +653,21 @@ constexpr size_t kPairSmemBytes = 1024 + (size_t)kPairStages * (kPairAStageBytes
 static_assert(kPairStages * (kPairAStageBytes + kPairBStageBytes) >= (int)(kEpiWarps * kEpiWarpFloats * sizeof(float)),
               "the epilogue stages its chunks in the pipeline buffers");
 
+// What a pair works on: `first` token blocks of one tile from kb_begin on and, under the even split, the blocks up to nkb from
+// the beginning of the next tile.
+struct PairSegments {
+    int nkb, first, kb_begin;
+    int j0, cb;                      // first row of dY's columns / first of the tile's channels that this CTA loads
+    int next_j0, next_cb;
+};
+
 // One producer thread: token blocks i = p, p + 3, p + 6, ... of this CTA's range (block i lives in slot i % stages,
 // so the thread only ever touches the slots s with s % 3 == p).
+template <bool STREAM>
 __device__ __forceinline__ void pair_producer(PairSmem* ctl, uint8_t* sA, uint8_t* sB, const CUtensorMap* map_dy,
-                                              const CUtensorMap* map_x, int p, int member, uint32_t leader_rank, int nkb,
-                                              int kb_begin, int j0, int cb, int grouped_maps, uint32_t wait_limit) {
+                                              const CUtensorMap* map_x, int p, int member, uint32_t leader_rank,
+                                              const PairSegments& seg, int grouped_maps, uint32_t wait_limit) {
+    const int nkb = seg.nkb;
     volatile int* abort_flag = &ctl->abort_flag;
     const uint32_t full0 = ptx::map_shared_to_cta(ptx::smem_u32(&ctl->full[0]), leader_rank);
     int rounds[kPairStages / kPairProducers];
@@ -622,7 +688,9 @@ __device__ __forceinline__ void pair_producer(PairSmem* ctl, uint8_t* sA, uint8_
             }
             const uint32_t bar = full0 + 8u * (uint32_t)s;
             if (!member) ptx::mbar_arrive_expect_tx(&ctl->full[s], 2u * kPairStageTx);
-            const int k0 = (kb_begin + i) * kPairBK;
+            const bool next = STREAM && i >= seg.first;
+            const int k0 = (next ? i - seg.first : seg.kb_begin + i) * kPairBK;
+            const int j0 = next ? seg.next_j0 : seg.j0, cb = next ? seg.next_cb : seg.cb;
             uint8_t* a = sA + s * kPairAStageBytes;
             uint8_t* b = sB + s * kPairBStageBytes;
             if (grouped_maps) {   // one copy per operand
@@ -645,11 +713,12 @@ __device__ __forceinline__ void pair_producer(PairSmem* ctl, uint8_t* sA, uint8_
     }
 }
 
+template <bool STREAM>
 __global__ void __launch_bounds__(kTcThreads, 1)
 wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CUtensorMap map_x, int Ca, int Cz,
                int tiles_n, int splits, int kb_per_split, int kb_total, float* __restrict__ dw, int accumulate,
                float* __restrict__ partial, uint32_t* counters, int32_t* dev_status, int grouped_maps,
-               uint32_t wait_limit, uint32_t epoch) {
+               uint32_t wait_limit, uint32_t epoch, int stream_pairs) {
     extern __shared__ uint8_t smem_raw[];
     // same offsets in both CTAs: the MMA addresses the operands of both with one descriptor
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -662,15 +731,29 @@ wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
     const uint32_t rank = ptx::cluster_ctarank();
     const int member = (int)(rank & 1u);           // 0: leader
     const uint32_t leader_rank = rank & ~1u;
-    const int tile = blockIdx.x;                   // the pair's CTAs are neighbours along x
     const int split = blockIdx.y;
-    const int pair = tile >> 1;
+    int pair = blockIdx.x >> 1;                    // pair of tiles; the pair's CTAs are neighbours along x
+    PairSegments seg;
+    if constexpr (STREAM) {
+        const int units = (int)(((Cz + 2 * kBM - 1) / (2 * kBM)) * tiles_n * kb_total);
+        const int u0 = stream_begin(pair, units, stream_pairs);
+        seg.nkb = stream_begin(pair + 1, units, stream_pairs) - u0;
+        pair = u0 / kb_total;
+        seg.kb_begin = u0 - pair * kb_total;
+        seg.first = min(seg.nkb, kb_total - seg.kb_begin);
+    } else {
+        seg.kb_begin = split * kb_per_split;
+        seg.first = seg.nkb = min(kb_total, seg.kb_begin + kb_per_split) - seg.kb_begin;
+    }
+    const int segments = STREAM && seg.first < seg.nkb ? 2 : 1;
+    const int tile = 2 * pair + member;
     const int j0 = ((pair / tiles_n) * 2 + member) * kBM;
     const int c0 = (pair % tiles_n) * kBN;
-    const int cb = c0 + member * (kBN / 2);        // the half of the tile's columns whose x this CTA loads
-    const int kb_begin = split * kb_per_split;
-    const int kb_end = min(kb_total, kb_begin + kb_per_split);
-    const int nkb = kb_end - kb_begin;
+    seg.j0 = j0;
+    seg.cb = c0 + member * (kBN / 2);              // the half of the tile's columns whose x this CTA loads
+    seg.next_j0 = (((pair + 1) / tiles_n) * 2 + member) * kBM;
+    seg.next_cb = ((pair + 1) % tiles_n) * kBN + member * (kBN / 2);
+    constexpr uint32_t tmem_cols = STREAM ? 2 * kBN : kBN;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kPairStages; ++s) {
@@ -679,7 +762,8 @@ wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
             ctl->issued[s] = 0;
             ctl->peer_issued[s] = 0;
         }
-        ptx::mbar_init(&ctl->accum, 1);
+        ptx::mbar_init(&ctl->accum[0], 1);
+        ptx::mbar_init(&ctl->accum[1], 1);
         ctl->abort_flag = 0;
         ctl->finisher = 1;
         ctl->consumed = 0;
@@ -689,7 +773,7 @@ wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
         ptx::prefetch_tensormap(&map_x);
     }
     if (warp == 1) {
-        ptx::tmem_alloc_pair(&ctl->tmem_base, kBN);
+        ptx::tmem_alloc_pair(&ctl->tmem_base, tmem_cols);
         ptx::tmem_relinquish_pair();
     }
     ptx::tc_fence_before();
@@ -702,7 +786,7 @@ wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
         // ---------------- TMA producer 0 (both CTAs) ----------------
         if (lane == 0) {
             ptx::grid_dependency_wait();   // the dense scratch is written by the kernel before this one
-            pair_producer(ctl, sA, sB, &map_dy, &map_x, 0, member, leader_rank, nkb, kb_begin, j0, cb, grouped_maps, wait_limit);
+            pair_producer<STREAM>(ctl, sA, sB, &map_dy, &map_x, 0, member, leader_rank, seg, grouped_maps, wait_limit);
         }
     } else if (warp == 1) {
         // ---------------- MMA issuer (leader only) ----------------
@@ -712,7 +796,14 @@ wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
             const uint16_t both = (uint16_t)(3u << leader_rank);
             int consumed = 0, s = 0;
             uint32_t round_parity = 0;
-            for (int i = 0; i < nkb; ++i) {
+            uint32_t tmem_d = tmem_base;
+            bool fresh = true;                           // the segment's first MMA overwrites its accumulator
+            for (int i = 0; i < seg.nkb; ++i) {
+                if (STREAM && i == seg.first) {          // on to the next tile, in the other half of tensor memory
+                    ptx::umma_commit_pair(&ctl->accum[0], both);
+                    tmem_d = tmem_base + kBN;
+                    fresh = true;
+                }
                 if (*abort_flag || !ptx::mbar_wait_poll(&ctl->full[s], round_parity, wait_limit)) {
                     *abort_flag = 1;
                     break;
@@ -725,13 +816,14 @@ wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
                 for (int kk = 0; kk < kPairBK / 16; ++kk) {
                     const uint64_t ad = ptx::make_smem_desc_sw128(a_addr + kk * 2048, kGroupBytes, 1024);
                     const uint64_t bd = ptx::make_smem_desc_sw128(b_addr + kk * 2048, kGroupBytes, 1024);
-                    ptx::umma_bf16_pair(tmem_base, ad, bd, idesc, (i > 0 || kk > 0) ? 1u : 0u);
+                    ptx::umma_bf16_pair(tmem_d, ad, bd, idesc, (fresh && kk == 0) ? 0u : 1u);
                 }
+                fresh = false;
                 ptx::umma_commit_pair(&ctl->empty[s], both);
                 if (++s == kPairStages) { s = 0; round_parity ^= 1u; }
             }
             ctl->consumed = consumed;
-            ptx::umma_commit_pair(&ctl->accum, both);   // also after an abort: tells both CTAs when the MMAs in flight are done
+            ptx::umma_commit_pair(&ctl->accum[segments - 1], both);   // also after an abort: tells both CTAs when the MMAs in flight are done
         }
     } else {
         // ---------------- epilogue: TMEM -> global (both CTAs, each its own 128 rows) ----------------
@@ -744,17 +836,46 @@ wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
         if (warp - 2 >= 1 && warp - 2 < kPairProducers) {   // producers 1 and 2 first
             if (lane == 0) {
                 ptx::grid_dependency_wait();
-                pair_producer(ctl, sA, sB, &map_dy, &map_x, warp - 2, member, leader_rank, nkb, kb_begin, j0, cb, grouped_maps, wait_limit);
+                pair_producer<STREAM>(ctl, sA, sB, &map_dy, &map_x, warp - 2, member, leader_rank, seg, grouped_maps, wait_limit);
             }
             __syncwarp();
         }
-        bool ok = ptx::mbar_wait_warp(&ctl->accum, 0, wait_limit);
-        ok = __all_sync(kFullMask, ok) && !*abort_flag;
-        if (!ok) *abort_flag = 1;
-        // every MMA has read its operands in both CTAs: the pipeline buffers serve as the staging area
-        ticket_epilogue(tmem_base, reinterpret_cast<float*>(smem), warp, lane, j0, c0, Ca, Cz, split, splits, dw, accumulate,
-                        partial, counters + (size_t)tile * 2 * kMaxParts, counters + (size_t)tile * 2 * kMaxParts + kMaxParts, epoch,
-                        first_ticket, &ctl->finisher, abort_flag);
+        if constexpr (STREAM) {
+            // Every segment's accumulator leaves for the pair's plane of the tile as it is.  The first of two does so under the
+            // main loop of the second, by the four warps that do not produce.
+            const int units = (int)(((Cz + 2 * kBM - 1) / (2 * kBM)) * tiles_n * kb_total);
+            const size_t stride = (size_t)2 * ((Cz + 2 * kBM - 1) / (2 * kBM)) * tiles_n * kPlaneTileFloats;
+            for (int sg = 0; sg < segments; ++sg) {
+                const bool shared_out = sg == segments - 1;         // all eight warps
+                if (!shared_out && warp < 6) continue;
+                bool ok = ptx::mbar_wait_warp(&ctl->accum[sg], 0, wait_limit);
+                ok = __all_sync(kFullMask, ok) && !*abort_flag;
+                if (!ok) { *abort_flag = 1; break; }
+                ptx::tc_fence_after();
+                const int slot = (int)(blockIdx.x >> 1) - stream_first_pair((pair + sg) * kb_total, units, stream_pairs);
+                float* plane = partial + (size_t)slot * stride + (size_t)(tile + 2 * sg) * kPlaneTileFloats;
+                const int g = warp & 3;
+                for (int ch = shared_out ? (warp - 2) >> 2 : 0; ch < kBN / 32; ch += shared_out ? kEpiSubs : 1) {
+                    uint32_t r[32];
+                    ptx::tmem_ld_32x32(tmem_base + sg * kBN + ((uint32_t)(32 * g) << 16) + ch * 32, r);
+                    ptx::tmem_ld_wait();
+                    float* dst = plane + plane_offset(ch, g, 0, lane);
+#pragma unroll
+                    for (int e4 = 0; e4 < 8; ++e4)
+                        __stcg(reinterpret_cast<float4*>(dst + e4 * 128),
+                               make_float4(__uint_as_float(r[4 * e4]), __uint_as_float(r[4 * e4 + 1]), __uint_as_float(r[4 * e4 + 2]),
+                                           __uint_as_float(r[4 * e4 + 3])));
+                }
+            }
+        } else {
+            bool ok = ptx::mbar_wait_warp(&ctl->accum[0], 0, wait_limit);
+            ok = __all_sync(kFullMask, ok) && !*abort_flag;
+            if (!ok) *abort_flag = 1;
+            // every MMA has read its operands in both CTAs: the pipeline buffers serve as the staging area
+            ticket_epilogue(tmem_base, reinterpret_cast<float*>(smem), warp, lane, j0, c0, Ca, Cz, split, splits, dw, accumulate,
+                            partial, counters + (size_t)tile * 2 * kMaxParts, counters + (size_t)tile * 2 * kMaxParts + kMaxParts, epoch,
+                            first_ticket, &ctl->finisher, abort_flag);
+        }
     }
 
     // Neither CTA leaves while the other may still signal its barriers or read its shared memory.  After a wait
@@ -783,11 +904,90 @@ wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
     ptx::cluster_sync_all();
     if (warp == 1) {
         // tensor memory is given back by both CTAs, and only once no MMA can still write to it
-        ptx::mbar_wait_warp(&ctl->accum, 0, kWaitLimit);
+        ptx::mbar_wait_warp(&ctl->accum[segments - 1], 0, kWaitLimit);
         ptx::tc_fence_after();
-        ptx::tmem_dealloc_pair(tmem_base, kBN);
+        ptx::tmem_dealloc_pair(tmem_base, tmem_cols);
     }
     if (*abort_flag && threadIdx.x == 0 && dev_status) atomicExch(dev_status, (int)DROPIT_ERR_TIMEOUT);
+}
+
+static int resident_pairs() {
+    static std::atomic<int> cached[64];                        // 0 = not looked up yet
+    const int dev = current_device();
+    if (dev < 0 || dev >= 64) return sm_count() / 2;
+    int v = cached[dev].load(std::memory_order_acquire);
+    if (v == 0) {
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 2;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(2);
+        cfg.blockDim = dim3(kTcThreads);
+        cfg.dynamicSmemBytes = kPairSmemBytes;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaFuncSetAttribute(wg_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmemBytes) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&v, wg_pair_kernel<true>, &cfg) != cudaSuccess || v <= 0)
+            v = sm_count() / 2;
+        (void)cudaGetLastError();
+        cached[dev].store(v, std::memory_order_release);
+    }
+    return v;
+}
+
+// dw (=|+=) the planes of every tile, in pair order, after wg_pair_kernel under the even split.  A warp takes 32 rows x 32
+// columns: its lanes read their row's columns of each plane (512 contiguous bytes per load), turn the sum through shared
+// memory and write 128-byte row segments.
+__global__ void __launch_bounds__(128)
+wg_stream_reduce_kernel(const float* __restrict__ partial, int Ca, int Cz, int tiles_n, int kb_total, int stream_pairs,
+                        float* __restrict__ dw, int accumulate) {
+    __shared__ __align__(16) float stage_all[4 * kEpiWarpFloats];
+    const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* stage = stage_all + g * kEpiWarpFloats;
+    const int tile = blockIdx.x / (kBN / 32), ch = blockIdx.x % (kBN / 32);
+    const int pair_tiles = ((Cz + 2 * kBM - 1) / (2 * kBM)) * tiles_n, units = pair_tiles * kb_total;
+    const int pair = tile >> 1, member = tile & 1;
+    const int j0 = ((pair / tiles_n) * 2 + member) * kBM, c0 = (pair % tiles_n) * kBN;
+    ptx::grid_dependency_wait();
+    if (j0 + 32 * g >= Cz || c0 + ch * 32 >= Ca) return;       // uniform over the warp
+    const int first = stream_first_pair(pair * kb_total, units, stream_pairs);
+    const int count = stream_first_pair((pair + 1) * kb_total - 1, units, stream_pairs) - first + 1;
+    const size_t stride = (size_t)2 * pair_tiles * kPlaneTileFloats;
+    const float* src = partial + (size_t)tile * kPlaneTileFloats + plane_offset(ch, g, 0, lane);
+    float4 acc[8], next[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) next[e] = __ldcg(reinterpret_cast<const float4*>(src + e * 128));
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s = 0; s < count; ++s) {
+        float4 cur[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) cur[e] = next[e];
+        if (s + 1 < count) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) next[e] = __ldcg(reinterpret_cast<const float4*>(src + (size_t)(s + 1) * stride + e * 128));
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) { acc[e].x += cur[e].x; acc[e].y += cur[e].y; acc[e].z += cur[e].z; acc[e].w += cur[e].w; }
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) *reinterpret_cast<float4*>(stage + lane * kEpiRowFloats + 4 * e) = acc[e];
+    __syncwarp();
+    const int rr0 = lane >> 3, q = lane & 7, col = c0 + ch * 32 + 4 * q;
+#pragma unroll
+    for (int it = 0; it < 8; ++it) {
+        const int row = j0 + 32 * g + it * 4 + rr0;
+        if (col < Ca && row < Cz) {                             // Ca is a multiple of 8
+            float4 v = *reinterpret_cast<const float4*>(stage + (it * 4 + rr0) * kEpiRowFloats + 4 * q);
+            float* dst = dw + (size_t)row * Ca + col;
+            if (accumulate) {
+                const float4 o = *reinterpret_cast<const float4*>(dst);
+                v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+            }
+            *reinterpret_cast<float4*>(dst) = v;
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1048,11 +1248,12 @@ static dropit_status weight_grad_impl(const void* dy, const void* values, const 
     static PerDeviceOnce smem_attr;
     if (smem_attr.needed()) {
         if (cudaFuncSetAttribute(wg_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemBytes) != cudaSuccess ||
-            cudaFuncSetAttribute(wg_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmemBytes) != cudaSuccess)
+            cudaFuncSetAttribute(wg_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmemBytes) != cudaSuccess ||
+            cudaFuncSetAttribute(wg_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmemBytes) != cudaSuccess)
             return DROPIT_ERR_CUDA;
         smem_attr.mark();
     }
-    dim3 grid(plan.tiles_m * plan.tiles_n, plan.splits);
+    dim3 grid(plan.stream_pairs ? 2 * plan.stream_pairs : plan.tiles_m * plan.tiles_n, plan.splits);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(kTcThreads);
@@ -1073,13 +1274,26 @@ static dropit_status weight_grad_impl(const void* dy, const void* values, const 
     attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
     ++cfg.numAttrs;
     const cudaError_t err =
-        plan.pair ? cudaLaunchKernelEx(&cfg, wg_pair_kernel, map_dy, map_x, (int)Ca, (int)Cz, plan.tiles_n, plan.splits,
+        plan.pair ? cudaLaunchKernelEx(&cfg, plan.stream_pairs ? wg_pair_kernel<true> : wg_pair_kernel<false>, map_dy, map_x, (int)Ca, (int)Cz, plan.tiles_n, plan.splits,
                                        plan.kb_per_split, plan.kb_total, dw, accumulate, partial, counters, dev_status,
-                                       grouped ? 1 : 0, spin_limit(kWaitLimit), epoch)
+                                       grouped ? 1 : 0, spin_limit(kWaitLimit), epoch, plan.stream_pairs)
                   : cudaLaunchKernelEx(&cfg, wg_tc_kernel, map_dy, map_x, (int)Ca, (int)Cz, plan.tiles_n, plan.splits,
                                        plan.kb_per_split, plan.kb_total, dw, accumulate, partial, counters, dev_status,
                                        plan.cluster ? 1 : 0, grouped ? 1 : 0, spin_limit(kWaitLimit), epoch);
     if (err != cudaSuccess) {
+        (void)cudaGetLastError();
+        return DROPIT_ERR_CUDA;
+    }
+    if (plan.stream_pairs == 0) return check_launch();
+    s = check_launch();
+    if (s != DROPIT_OK) return s;
+    cfg.gridDim = dim3((unsigned)(plan.tiles_m * plan.tiles_n * (kBN / 32)));
+    cfg.blockDim = dim3(128);
+    cfg.dynamicSmemBytes = 0;
+    attr[0] = attr[cfg.numAttrs - 1];            // programmatic launch only
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, wg_stream_reduce_kernel, (const float*)partial, (int)Ca, (int)Cz, plan.tiles_n, plan.kb_total,
+                           plan.stream_pairs, dw, accumulate) != cudaSuccess) {
         (void)cudaGetLastError();
         return DROPIT_ERR_CUDA;
     }
