@@ -3,9 +3,9 @@
 //
 // No dense copy of the input exists in global memory.  A CTA owns 128 output channels j and a block of input channels, walks
 // over bands of image rows (or whole small images), and for every band its producer warps
-//   * inflate the band's piece of R(a-hat) into shared memory: a lane owns a pixel and builds the 16 bytes of its eight
-//     channels from eight mask words (each the same for the whole warp), reading the retained values with predicated loads
-//     that are contiguous over the warp, so that one 16-byte store per lane writes zeros and values alike,
+//   * inflate the band's piece of R(a-hat) into shared memory: a lane owns two pixels and builds the 16 bytes of their eight
+//     channels from eight mask words (the same for a half-warp), reading the retained values with predicated loads that are
+//     contiguous over the warp, so that 16-byte stores write zeros and values alike,
 //   * transpose the band of dY into shared memory (8 channels x 8 pixels per lane, in registers),
 // while one thread feeds the previous band to tcgen05.mma.  Both operands lie pixel-major: 8 channels (16 bytes) of
 // consecutive pixels of one image row follow one another,
@@ -20,13 +20,16 @@
 // Stride 2 keeps the even and the odd padded columns in separate planes.  The reduction is split over the CTAs; every split
 // stores its accumulator as it comes out of tensor memory and a second kernel adds the splits in order.
 //
-// Bound by the producers: a band is two dependent trips to memory (mask and table entry, then values) and some 130 warp
-// instructions per 32 pixels x 8 channels; the MMAs take a third to a half of the time.  20 producer warps: 16 are slower
-// where rows are long (3 x 3 on 56 x 56: 56 against 50 us), 24 spill.  Against the dense copies of conv_weight_grad_tc.cu
-// (decompression, shifted or gathered copies, GEMM on 64-pixel rows; per call at batch 64, gamma 0.8, graph replay): 3 x 3
-// 64 -> 64 on 56 x 56 59 -> 50 us, 128 -> 128 on 28 x 28 130 -> 46, 256 -> 256 on 14 x 14 126 -> 51, 512 -> 512 on 7 x 7
-// 332 -> 93, stride 2 128 -> 128 on 56 x 56 212 -> 70; 1 x 1 1024 -> 256 on 14 x 14 113 -> 54.
+// Bound by the producers (some 150 warp instructions per 64 pixels x 8 channels of X) beside MMAs that take most of the shared
+// memory's bandwidth; both lanes' pixels of a pair share one mask lookup, the mask words are requested a task ahead and
+// the loads of a warp's first tasks are under way before it waits for the stage, so that one trip to memory per band is
+// exposed.  The taps of a K step share the dY operand in the collector.  16 producer warps: 20 (80 registers) are up to 8 %
+// slower.  Measured per call at batch 64, gamma 0.8 (graph replay), dense copies of conv_weight_grad_tc.cu (decompression,
+// shifted or gathered copies, GEMM on 64-pixel rows) -> first version of this kernel -> now: 3 x 3 64 -> 64 on 56 x 56
+// 59 -> 50 -> 50 us, 128 -> 128 on 28 x 28 131 -> 46 -> 39, 256 -> 256 on 14 x 14 125 -> 51 -> 45, 512 -> 512 on 7 x 7
+// 334 -> 93 -> 86, stride 2 128 -> 128 on 56 x 56 213 -> 70 -> 59; 1 x 1 of stride 2 256 -> 512 on 56 x 56 292 -> 170 -> 129.
 #include <cstring>
+#include <type_traits>
 
 #include "weight_grad_common.cuh"
 
@@ -34,7 +37,7 @@ namespace dropit {
 
 namespace {
 
-constexpr int kProdWarps = 20;
+constexpr int kProdWarps = 16;                       // four per lane quarter of the accumulator in the epilogue
 constexpr int kThreads = 32 * (kProdWarps + 1);      // producer warps, then the MMA warp
 constexpr int kMaxStages = 4;
 constexpr int kMaxPairs = 64;                        // K = 16 steps of a band
@@ -53,7 +56,7 @@ struct FusedConvParams {
     int row_step, x_rows;                            // X rows per output row; X rows of one image in a band
     int in_step;                                     // input rows per X row
     // the X side of a band: segments of consecutive input pixels (a whole image's rows, or one row where every other row is
-    // skipped), cut into slots of 32 pixels, in the order [channel group][image][segment][slot]
+    // skipped), cut into slots of 64 pixels, in the order [channel group][image][segment][slot]
     int segs, seg_pixels, seg_slots, slots;          // segments of an image, pixels and slots of a segment, slots of the band
     uint32_t seg_magic, segs_magic, ni_magic;        // slot / seg_slots = (slot * seg_magic) >> 20 and so on
     uint32_t w_magic;                                // pixel / W
@@ -71,8 +74,8 @@ struct FusedConvCtl {
     uint64_t full[kMaxStages], empty[kMaxStages], accum;
     uint32_t tmem_base;
     int abort_flag;
-    alignas(16) uint2 home[kProdWarps][4];   // per producer warp: where the slots of its task go
-    uint2 meta[kProdWarps][32];  // per producer warp: [slot of a task][channel] (mask bits, position of their first value)
+    alignas(16) uint2 home[kProdWarps][2];   // per producer warp: where the slots of its task go
+    uint2 meta[kProdWarps][32];  // ... [word of a task][channel] (mask bits, position of their first value)
 };
 
 // x / d for x * d < 2^20, with magic = 2^20 / d + 1
@@ -97,20 +100,30 @@ __device__ __forceinline__ uint32_t ldg_u16_if(const uint16_t* p, uint32_t bit) 
     return v;
 }
 
+// The values of two neighbouring elements of a 32-element word of the mask, bits bit0 and bit0 + 1; pos = position of the
+// word's first value.
+__device__ __forceinline__ void load_two(const uint16_t* __restrict__ values, uint32_t word, uint32_t pos, uint32_t bit0, uint32_t& v0,
+                                         uint32_t& v1) {
+    const uint32_t b = word >> bit0;
+    const uint16_t* src = values + (pos + __popc(word & ((1u << bit0) - 1u)));
+    v0 = ldg_u16_if(src, b & 1u);
+    v1 = ldg_u16_if(src + (b & 1u), b & 2u);
+}
+
 struct Place {
     uint32_t group, img, seg, pixel;     // pixel: of the slot's first element inside the segment
 };
 __device__ __forceinline__ Place place_of(const FusedConvParams& p, uint32_t index, int groups) {
     Place r;
     const uint32_t a = quotient(index, p.seg_magic), b = quotient(a, p.segs_magic);
-    r.pixel = (index - a * p.seg_slots) * 32;
+    r.pixel = (index - a * p.seg_slots) * 64;
     r.seg = a - b * p.segs;
     r.group = quotient(b, p.ni_magic);
     r.img = b - r.group * p.ni;
     return r;
 }
 
-// VEC: pixels per load of dY (8: rows are whole aligned 16-byte groups; 2; 1)
+// VEC: pixels per load of dY that the row length allows (8: rows are whole aligned 16-byte groups; 4; 2; 1: rows that start anywhere)
 template <int VEC>
 __global__ void __launch_bounds__(kThreads, 1)
 conv_wg_fused_kernel(const uint16_t* __restrict__ dy, const uint16_t* __restrict__ values, const uint32_t* __restrict__ mask,
@@ -155,90 +168,181 @@ conv_wg_fused_kernel(const uint16_t* __restrict__ dy, const uint16_t* __restrict
         // ---------------- producers ----------------
         const uint32_t nwords = (uint32_t)(((int64_t)p.B * p.Ca * p.H * p.W + 31) / 32);
         const uint32_t plane_elems = (uint32_t)p.H * p.W, plane_pitch = (uint32_t)p.x_bytes / p.planes;
-        const int groups = p.cb / 8, x_tasks = (p.slots + 3) / 4;
+        const int groups = p.cb / 8, x_tasks = (p.slots + 1) / 2;
         const int dy_steps = (total_cores + 3) / 4, dy_tasks = dy_steps * (p.mt / 64);
         const size_t dy_plane = (size_t)p.Ho * p.Wo;
+        [[maybe_unused]] const size_t dy_total = dy_plane * p.Cz * p.B;
+        const int dy_first = (warp + kProdWarps - x_tasks % kProdWarps) % kProdWarps;   // goes on where the X tasks end
         const int slot = lane >> 3, sub = lane & 7;
         uint2* meta = ctl->meta[warp];
         uint2* home = ctl->home[warp];
-        const uint32_t lane_bit = 1u << lane, lane_below = lane_bit - 1u;
+        const uint32_t bit0 = (2u * lane) & 31u;       // the lane's first pixel in its 32-pixel word
         int n0 = (band0 / p.bands) * p.ni, piece = band0 % p.bands;      // image and piece of the image
+        // ---- X: a task is two slots, a slot 64 consecutive pixels of 8 channels.  The mask bits of its four 32-pixel words per
+        // channel and the position of their first value (lane = (channel sub, word slot)) are requested a task ahead, across bands
+        struct Bits { uint4 chunk; uint32_t next, first, at, lead, len; };
+        auto request = [&](uint32_t index, int n_first, int piece_of) {
+            const int yi0 = piece_of * p.yb * p.stride - p.pad, kx0 = p.flat ? piece_of * p.xb : 0;
+            const int run_end = p.flat ? min(p.W, kx0 + p.xb) : (int)plane_elems;   // no pixel of the plane from here on
+            Bits r;
+            r.chunk = make_uint4(0, 0, 0, 0);
+            r.next = r.first = r.at = r.lead = r.len = 0;
+            if (index >= 2u * p.slots) return r;
+            Place at = place_of(p, index >> 1, groups);
+            at.pixel += (index & 1u) * 32;
+            const int row = yi0 + (int)at.seg * p.in_step;                     // first input row of the segment
+            const int px = (p.flat ? kx0 : row * p.W) + (int)at.pixel;
+            const int c = c0 + (int)at.group * 8 + sub;
+            int lo = max(px, 0), hi = min(min(px + 32, run_end), px + p.seg_pixels - (int)at.pixel);
+            if (n_first + (int)at.img < p.B && c < p.Ca && lo < hi) {
+                r.at = ((uint32_t)(n_first + at.img) * p.Ca + c) * plane_elems + lo;   // flat index of the slot's first element
+                r.lead = lo - px;
+                r.len = hi - lo;
+                const uint32_t ch = r.at >> 7, w1 = (r.at >> 5) + 1;
+                r.first = __ldg(offsets + ch);
+                if (w1 < nwords) r.next = __ldg(mask + w1);
+                if (ch * 4 + 3 < nwords) {
+                    r.chunk = __ldg(reinterpret_cast<const uint4*>(mask) + ch);
+                } else {                             // the tensor's last chunk may be short
+                    r.chunk.x = __ldg(mask + ch * 4);
+                    if (ch * 4 + 1 < nwords) r.chunk.y = __ldg(mask + ch * 4 + 1);
+                    if (ch * 4 + 2 < nwords) r.chunk.z = __ldg(mask + ch * 4 + 2);
+                }
+            }
+            return r;
+        };
+        auto record = [&](const Bits& r) {
+            const uint32_t in = (r.at >> 5) & 3u, sh = r.at & 31u;
+            uint32_t m = r.chunk.x, pos = r.first;
+            if (in > 0) { pos += __popc(m); m = r.chunk.y; }
+            if (in > 1) { pos += __popc(m); m = r.chunk.z; }
+            if (in > 2) { pos += __popc(m); m = r.chunk.w; }
+            pos += __popc(m & ((1u << sh) - 1u));
+            uint32_t bits = __funnelshift_r(m, r.next, sh);
+            if (r.len < 32) bits &= (1u << r.len) - 1u;
+            if (pos + __popc(bits) > p.k) bits = 0;   // a table that does not match the mask must not read past the values
+            return make_uint2(bits << r.lead, pos);
+        };
+        Bits ahead = request(warp * 4 + slot, n0, piece);
         for (int i = 0; i < nb; ++i) {
             const int s = i % p.stages;
             const int y0 = p.flat ? 0 : piece * p.yb, k0 = p.flat ? piece * p.xb : 0;
+            const bool turn = piece + 1 == p.bands;                        // the next band opens another image
+            const int next_n = turn ? n0 + p.ni : n0, next_piece = turn ? 0 : piece + 1;
             const uint32_t xbuf = smem0 + s * stage_bytes, ybuf = xbuf + p.x_bytes;
-            // ---- X: a task is four slots, a slot 32 consecutive pixels of 8 channels.  First the mask bits of every slot and
-            // channel and the position of their first value: lane = (channel sub, slot)
-            const int yi0 = y0 * p.stride - p.pad;
-            const int run_end = p.flat ? min(p.W, k0 + p.xb) : (int)plane_elems;   // no pixel of the plane from here on
-            struct Bits { uint4 chunk; uint32_t next, first, at, lead, len; };
-            auto request = [&](uint32_t index) {
-                Bits r;
-                r.chunk = make_uint4(0, 0, 0, 0);
-                r.next = r.first = r.at = r.lead = r.len = 0;
-                if (index >= (uint32_t)p.slots) return r;
-                const Place at = place_of(p, index, groups);
-                const int row = yi0 + (int)at.seg * p.in_step;                     // first input row of the segment
-                const int px = (p.flat ? k0 : row * p.W) + (int)at.pixel;
-                const int c = c0 + (int)at.group * 8 + sub;
-                int lo = max(px, 0), hi = min(min(px + 32, run_end), px + p.seg_pixels - (int)at.pixel);
-                if (n0 + (int)at.img < p.B && c < p.Ca && lo < hi) {
-                    r.at = ((uint32_t)(n0 + at.img) * p.Ca + c) * plane_elems + lo;   // flat index of the slot's first element
-                    r.lead = lo - px;
-                    r.len = hi - lo;
-                    const uint32_t ch = r.at >> 7, w1 = (r.at >> 5) + 1;
-                    r.first = __ldg(offsets + ch);
-                    if (w1 < nwords) r.next = __ldg(mask + w1);
-                    if (ch * 4 + 3 < nwords) {
-                        r.chunk = __ldg(reinterpret_cast<const uint4*>(mask) + ch);
-                    } else {                             // the tensor's last chunk may be short
-                        r.chunk.x = __ldg(mask + ch * 4);
-                        if (ch * 4 + 1 < nwords) r.chunk.y = __ldg(mask + ch * 4 + 1);
-                        if (ch * 4 + 2 < nwords) r.chunk.z = __ldg(mask + ch * 4 + 2);
-                    }
-                }
+            // ---- dY: 8 channels x 8 pixels per lane, transposed in registers.  The eight lanes of a quarter-warp take eight
+            // channel groups (their pitch is 16 bytes modulo 128, so that the stores of a quarter-warp do not collide).  The
+            // loads of the warp's first task are issued before it waits for the stage and works on X.
+            struct DyPlace { int row, xc, jg; bool live; };
+            auto dy_place = [&](int t) {
+                DyPlace r;
+                const int jset = (int)quotient(t, p.step_magic);
+                const int core = (t - jset * dy_steps) * 4 + slot;
+                r.live = core < total_cores;
+                r.jg = jset * 8 + sub;
+                r.row = (int)quotient(core, p.cores_magic);
+                r.xc = core - r.row * p.cores;
                 return r;
             };
-            auto record = [&](const Bits& r) {
-                const uint32_t in = (r.at >> 5) & 3u, sh = r.at & 31u;
-                uint32_t m = r.chunk.x, pos = r.first;
-                if (in > 0) { pos += __popc(m); m = r.chunk.y; }
-                if (in > 1) { pos += __popc(m); m = r.chunk.z; }
-                if (in > 2) { pos += __popc(m); m = r.chunk.w; }
-                pos += __popc(m & ((1u << sh) - 1u));
-                uint32_t bits = __funnelshift_r(m, r.next, sh);
-                if (r.len < 32) bits &= (1u << r.len) - 1u;
-                if (pos + __popc(bits) > p.k) bits = 0;   // a table that does not match the mask must not read past the values
-                return make_uint2(bits << r.lead, pos);
+            auto load_dy = [&](int t, uint32_t (&w)[8][4]) {
+                const DyPlace at = dy_place(t);
+                const int img = (int)quotient(at.row, p.yb_magic), y = y0 + at.row - img * p.yb;
+                const int x = k0 + at.xc * 8, nv = min(8, p.Wo - x);       // pixels that exist
+                const bool in = at.live && n0 + img < p.B && y < p.Ho && nv > 0;
+                const int j = j0 + at.jg * 8;
+                const uint16_t* src = dy + ((size_t)(n0 + img) * p.Cz + j) * dy_plane + (size_t)y * p.Wo + x;
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    w[e][0] = w[e][1] = w[e][2] = w[e][3] = 0;
+                    if (in && j + e < p.Cz) {
+                        if constexpr (VEC == 8) {
+                            const uint4 v = ld_stream(reinterpret_cast<const uint4*>(src));
+                            w[e][0] = v.x; w[e][1] = v.y; w[e][2] = v.z; w[e][3] = v.w;
+                        } else if constexpr (VEC == 4) {
+                            const uint2 v = __ldg(reinterpret_cast<const uint2*>(src));
+                            w[e][0] = v.x; w[e][1] = v.y;
+                            if (nv > 4) {
+                                const uint2 u = __ldg(reinterpret_cast<const uint2*>(src) + 1);
+                                w[e][2] = u.x; w[e][3] = u.y;
+                            }
+                        } else if constexpr (VEC == 2) {
+#pragma unroll
+                            for (int h = 0; h < 4; ++h)
+                                if (2 * h < nv) w[e][h] = __ldg(reinterpret_cast<const uint32_t*>(src) + h);
+                        } else {
+                            // rows that start anywhere: the aligned words around the piece, shifted by half a word for odd starts
+                            const size_t at0 = (size_t)(src - dy);
+                            const uint32_t odd = (uint32_t)at0 & 1u;
+                            const uint32_t* words = reinterpret_cast<const uint32_t*>(dy) + (at0 >> 1);
+                            uint32_t raw[5];
+#pragma unroll
+                            for (int h = 0; h < 5; ++h) {
+                                raw[h] = 0;
+                                if (2 * h < nv + (int)odd) {     // the tensor's last element may have no right neighbour
+                                    if (((at0 >> 1) + h) * 2 + 1 < dy_total) raw[h] = __ldg(words + h);
+                                    else raw[h] = __ldg(reinterpret_cast<const uint16_t*>(words + h));
+                                }
+                            }
+#pragma unroll
+                            for (int h = 0; h < 4; ++h) {
+                                w[e][h] = odd ? __funnelshift_r(raw[h], raw[h + 1], 16) : raw[h];
+                                if (2 * h + 1 >= nv) w[e][h] &= 2 * h < nv ? 0xFFFFu : 0u;   // pixels of the next row
+                            }
+                        }
+                    }
+                    src += dy_plane;
+                }
             };
-            Bits ahead = request(warp * 4 + slot);
-            if (i >= p.stages) {
-                const bool ok = ptx::mbar_wait_warp(&ctl->empty[s], ((i / p.stages) - 1) & 1, wait_limit);
-                if (!ok) *abort_flag = 1;
-            }
-            if (__any_sync(kFullMask, *abort_flag != 0)) break;
-            for (int t = warp; t < x_tasks; t += kProdWarps) {
+            auto store_dy = [&](int t, const uint32_t (&w)[8][4]) {
+                const DyPlace at = dy_place(t);
+                if (!at.live) return;
+                const uint32_t dst = ybuf + at.row * dy_pitch + (at.jg * p.gpy + at.xc * 8) * 16;
+#pragma unroll
+                for (int px = 0; px < 8; ++px) {
+                    uint32_t o[4];
+#pragma unroll
+                    for (int h = 0; h < 4; ++h)
+                        o[h] = __byte_perm(w[2 * h][px >> 1], w[2 * h + 1][px >> 1], (px & 1) ? 0x7632 : 0x5410);
+                    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + px * 16), "r"(o[0]), "r"(o[1]), "r"(o[2]),
+                                 "r"(o[3]) : "memory");
+                }
+            };
+            // The retained values of a task are loaded into registers (a slot at a time: the lane gets the 8 channels of its two
+            // pixels), then stored; for the warp's first task of the band, and for its first dY task, the loads are on their
+            // way before it waits for the stage.
+            uint4 x4[4];
+            auto load_x = [&](int t) {
                 meta[lane] = record(ahead);
-                if (lane < 4) {
-                    const uint32_t index = t * 4 + lane;
+                if (lane < 2) {
+                    const uint32_t index = t * 2 + lane;
                     const Place at = place_of(p, index, groups);
                     home[lane] = make_uint2(xbuf + (at.img * p.x_rows + at.seg) * row_pitch + at.group * p.gp * 16,
                                             index < (uint32_t)p.slots ? at.pixel : (uint32_t)p.seg_pixels);
                 }
-                ahead = request((t + kProdWarps) * 4 + slot);
+                const bool more = t + kProdWarps < x_tasks;
+                if (more || i + 1 < nb)
+                    ahead = request((more ? t + kProdWarps : warp) * 4 + slot, more ? n0 : next_n, more ? piece : next_piece);
                 __syncwarp();
-                // a slot at a time: the lane builds the 16 bytes of its pixel's 8 channels
-#pragma unroll 2
-                for (int q = 0; q < 4; ++q) {
-                    uint32_t v[8];
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    uint32_t v[2][8];
 #pragma unroll
                     for (int h = 0; h < 4; ++h) {
-                        const uint4 m = reinterpret_cast<const uint4*>(meta)[q * 4 + h];
-                        v[2 * h] = ldg_u16_if(values + (m.y + __popc(m.x & lane_below)), m.x & lane_bit);
-                        v[2 * h + 1] = ldg_u16_if(values + (m.w + __popc(m.z & lane_below)), m.z & lane_bit);
+                        const uint4 m = reinterpret_cast<const uint4*>(meta)[(q * 2 + (lane >> 4)) * 4 + h];
+                        load_two(values, m.x, m.y, bit0, v[0][2 * h], v[1][2 * h]);
+                        load_two(values, m.z, m.w, bit0, v[0][2 * h + 1], v[1][2 * h + 1]);
                     }
-                    const uint2 at = home[q];            // where the slot's first pixel is: segment's address, pixel of the segment
-                    const uint32_t rel = at.y + lane;
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+                        x4[2 * q + e] = make_uint4(v[e][0] | (v[e][1] << 16), v[e][2] | (v[e][3] << 16), v[e][4] | (v[e][5] << 16),
+                                                   v[e][6] | (v[e][7] << 16));
+                }
+            };
+            auto store_x = [&]() {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const uint2 at = home[q >> 1];       // where the slot's first pixel is: segment's address, pixel of the segment
+                    const uint32_t rel = at.y + 2 * lane + (q & 1);
                     bool keep = rel < (uint32_t)p.seg_pixels;
                     uint32_t x = rel, to = at.x;
                     if (!p.flat) {
@@ -254,76 +358,34 @@ conv_wg_fused_kernel(const uint16_t* __restrict__ dy, const uint16_t* __restrict
                         }
                     }
                     if (keep)
-                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(to + x * 16), "r"(v[0] | (v[1] << 16)),
-                                     "r"(v[2] | (v[3] << 16)), "r"(v[4] | (v[5] << 16)), "r"(v[6] | (v[7] << 16)) : "memory");
+                        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(to + x * 16), "r"(x4[q].x), "r"(x4[q].y),
+                                     "r"(x4[q].z), "r"(x4[q].w) : "memory");
                 }
                 __syncwarp();                            // the records may be overwritten
+            };
+            uint32_t w[8][4];
+            if (warp < x_tasks) load_x(warp);
+            if (dy_first < dy_tasks) load_dy(dy_first, w);
+            if (i >= p.stages) {
+                const bool ok = ptx::mbar_wait_warp(&ctl->empty[s], ((i / p.stages) - 1) & 1, wait_limit);
+                if (!ok) *abort_flag = 1;
             }
-
-            // ---- dY: 8 channels x 8 pixels per lane, transposed in registers.  The eight lanes of a quarter-warp take eight
-            // channel groups (their pitch is 16 bytes modulo 128, so that the stores of a quarter-warp do not collide)
-            for (int t = (warp + kProdWarps - x_tasks % kProdWarps) % kProdWarps; t < dy_tasks; t += kProdWarps) {   // goes on where the X tasks ended
-                const int jset = (int)quotient(t, p.step_magic);
-                const int core = (t - jset * dy_steps) * 4 + slot, jg = jset * 8 + sub;
-                if (core >= total_cores) continue;
-                const int row = (int)quotient(core, p.cores_magic), xc = core - row * p.cores;
-                const int img = (int)quotient(row, p.yb_magic), y = y0 + row - img * p.yb;
-                const int x = k0 + xc * 8, nv = min(8, p.Wo - x);          // pixels that exist
-                const bool in = n0 + img < p.B && y < p.Ho && nv > 0;
-                const int j = j0 + jg * 8;
-                const uint16_t* src = dy + ((size_t)(n0 + img) * p.Cz + j) * dy_plane + (size_t)y * p.Wo + x;
-                uint32_t w[8][4];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    w[e][0] = w[e][1] = w[e][2] = w[e][3] = 0;
-                    if (in && j + e < p.Cz) {
-                        if constexpr (VEC == 8) {
-                            const uint4 v = ld_stream(reinterpret_cast<const uint4*>(src));
-                            w[e][0] = v.x; w[e][1] = v.y; w[e][2] = v.z; w[e][3] = v.w;
-                        } else if constexpr (VEC == 2) {
-#pragma unroll
-                            for (int h = 0; h < 4; ++h)
-                                if (2 * h < nv) w[e][h] = __ldg(reinterpret_cast<const uint32_t*>(src) + h);
-                        } else {
-#pragma unroll
-                            for (int h = 0; h < 8; ++h)
-                                if (h < nv) w[e][h >> 1] |= (uint32_t)__ldg(src + h) << ((h & 1) * 16);
-                        }
-                    }
-                    src += dy_plane;
-                }
-                const uint32_t dst = ybuf + row * dy_pitch + (jg * p.gpy + xc * 8) * 16;
-#pragma unroll
-                for (int px = 0; px < 8; ++px) {
-                    uint32_t o[4];
-#pragma unroll
-                    for (int h = 0; h < 4; ++h)
-                        o[h] = __byte_perm(w[2 * h][px >> 1], w[2 * h + 1][px >> 1], (px & 1) ? 0x7632 : 0x5410);
-                    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + px * 16), "r"(o[0]), "r"(o[1]), "r"(o[2]),
-                                 "r"(o[3]) : "memory");
-                }
+            if (__any_sync(kFullMask, *abort_flag != 0)) break;
+            if (warp < x_tasks) store_x();
+            for (int t = warp + kProdWarps; t < x_tasks; t += kProdWarps) {
+                load_x(t);
+                store_x();
+            }
+            for (int t = dy_first; t < dy_tasks; t += kProdWarps) {
+                if (t != dy_first) load_dy(t, w);
+                store_dy(t, w);
             }
 
             ptx::fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&ctl->full[s]);
-            if (i + 1 < nb) {
-                // the next band's dY is brought into L2 meanwhile (a lane's eight rows, one 16-byte piece of each 128-byte line)
-                const bool turn = piece + 1 == p.bands;
-                const int n1 = turn ? n0 + p.ni : n0, piece1 = turn ? 0 : piece + 1;
-                const int rows1 = p.flat ? 1 : min(p.yb, p.Ho - piece1 * p.yb);
-                const size_t first = p.flat ? (size_t)piece1 * p.xb : (size_t)piece1 * p.yb * p.Wo;
-                const int lines = (rows1 * (p.flat ? min(p.xb, p.Wo - piece1 * p.xb) : p.Wo) * 2 + 127) / 128;
-                const int per_img = min(p.mt, p.Cz - j0) * lines;
-                for (int q = threadIdx.x; q < per_img * min(p.ni, p.B - n1); q += 32 * kProdWarps) {
-                    const int img = q / per_img, rest = q - img * per_img, j = rest / lines, l = rest - j * lines;
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"(dy + ((size_t)(n1 + img) * p.Cz + j0 + j) * dy_plane + first + l * 64));
-                }
-            }
-            if (++piece == p.bands) {
-                piece = 0;
-                n0 += p.ni;
-            }
+            n0 = next_n;
+            piece = next_piece;
         }
         ptx::launch_dependents();
         // ---------------- epilogue: the accumulator leaves in the order it has in tensor memory ----------------
@@ -364,14 +426,26 @@ conv_wg_fused_kernel(const uint16_t* __restrict__ dy, const uint16_t* __restrict
             }
             ptx::tc_fence_after();
             const uint32_t stage = (smem0 + s * stage_bytes) >> 4;
+            // The horizontal taps of a K step share its dY operand, which is read from shared memory once: the MMAs would
+            // otherwise take all of its bandwidth (128 x 96 x 16: 7 KB per 48 cycles).
+            using ptx::CollectA;
+            const auto steps = [&](auto taps) {
+                constexpr int S = decltype(taps)::value;
 #pragma unroll 2
-            for (int q = 0; q < pairs; ++q) {
-                const uint64_t ad = desc_of(p.pairs[q].x + stage, high_a);
-                const uint32_t b_low = p.pairs[q].y + stage, acc = (i > 0 || q > 0) ? 1u : 0u;
-                ptx::umma_bf16_elected(tmem_base, ad, desc_of(b_low, high_b), idesc, acc, leader);
-                if (p.S > 1) ptx::umma_bf16_elected(tmem_base + n_inst, ad, desc_of(b_low + shift1, high_b), idesc, acc, leader);
-                if (p.S > 2) ptx::umma_bf16_elected(tmem_base + 2 * n_inst, ad, desc_of(b_low + shift2, high_b), idesc, acc, leader);
-            }
+                for (int q = 0; q < pairs; ++q) {
+                    const uint64_t ad = desc_of(p.pairs[q].x + stage, high_a);
+                    const uint32_t b_low = p.pairs[q].y + stage, acc = (i > 0 || q > 0) ? 1u : 0u;
+                    ptx::umma_bf16_elected<S == 1 ? CollectA::kDiscard : CollectA::kFill>(tmem_base, ad, desc_of(b_low, high_b), idesc, acc, leader);
+                    if constexpr (S > 1)
+                        ptx::umma_bf16_elected<S == 2 ? CollectA::kLastUse : CollectA::kUse>(tmem_base + n_inst, ad, desc_of(b_low + shift1, high_b),
+                                                                                             idesc, acc, leader);
+                    if constexpr (S > 2)
+                        ptx::umma_bf16_elected<CollectA::kLastUse>(tmem_base + 2 * n_inst, ad, desc_of(b_low + shift2, high_b), idesc, acc, leader);
+                }
+            };
+            if (p.S == 1) steps(std::integral_constant<int, 1>{});
+            else if (p.S == 2) steps(std::integral_constant<int, 2>{});
+            else steps(std::integral_constant<int, 3>{});
             if (leader) ptx::umma_commit(&ctl->empty[s]);
             __syncwarp();
         }
@@ -501,14 +575,14 @@ bool make_fused_conv_plan(FusedConvParams& p, int B, int Ca, int H, int W, int C
         p.bands_total = (B + ni - 1) / ni * p.bands;
         p.segs = p.in_step > 1 ? p.x_rows : 1;
         p.seg_pixels = p.flat ? p.xb : (p.in_step > 1 ? W : p.x_rows * W);
-        p.seg_slots = (p.seg_pixels + 31) / 32;
+        p.seg_slots = (p.seg_pixels + 63) / 64;
         p.slots = p.seg_slots * p.segs * p.ni * (p.cb / 8);
         int splits = (int)(sm_count() / tiles);
         if (splits < 1) splits = 1;
         if (splits > p.bands_total) splits = p.bands_total;
         p.bands_per_split = (p.bands_total + splits - 1) / splits;
         p.splits = (p.bands_total + p.bands_per_split - 1) / p.bands_per_split;
-        const int tasks = (p.slots + 3) / 4 + (p.ni * p.yb * p.cores + 3) / 4 * (p.mt / 64);
+        const int tasks = (p.slots + 1) / 2 + (p.ni * p.yb * p.cores + 3) / 4 * (p.mt / 64);
         return p.bands_per_split * (0.5f + (float)((tasks + kProdWarps - 1) / kProdWarps));
     };
     int best_pieces = 0, best_ni = 0;
@@ -533,9 +607,9 @@ bool make_fused_conv_plan(FusedConvParams& p, int B, int Ca, int H, int W, int C
     p.yb_magic = magic_of((uint32_t)p.yb);
     p.step_magic = magic_of((uint32_t)((cores_total + 3) / 4));
     // what the division by multiplication and the table of K steps can take
-    const int64_t most = p.slots + 4 * kProdWarps + 4;
+    const int64_t most = p.slots + 2 * kProdWarps + 2;
     if (cores_total > 2 * kMaxPairs || most * p.seg_slots >= (1 << 20) || most * p.segs >= (1 << 20) || most * p.ni >= (1 << 20) ||
-        (int64_t)cores_total * p.cores >= (1 << 20) || (!p.flat && (int64_t)(p.seg_pixels + 32) * W >= (1 << 20)))
+        (int64_t)cores_total * p.cores >= (1 << 20) || (!p.flat && (int64_t)(p.seg_pixels + 64) * W >= (1 << 20)))
         return false;
     p.ncols = R * S * p.cb;
     p.chunks = (p.ncols + 31) / 32;
@@ -596,10 +670,10 @@ dropit_status conv_fused_run(const void* dy, const void* values, const void* mas
     if (!cached_fused_conv_plan(p, B, Ca, H, W, Cz, R, S, stride, pad, k)) return DROPIT_ERR_UNSUPPORTED;
     const int tiles = p.tiles_c * p.tiles_j;
     if (workspace_bytes < (size_t)p.splits * tiles * p.chunks * 32 * kBM * 4) return DROPIT_ERR_WORKSPACE;
-    const int vec = p.Wo % 8 == 0 ? 8 : (p.Wo % 2 == 0 ? 2 : 1);
-    auto kern = vec == 8 ? conv_wg_fused_kernel<8> : (vec == 2 ? conv_wg_fused_kernel<2> : conv_wg_fused_kernel<1>);
-    static PerDeviceOnce attr[3];
-    PerDeviceOnce& once = attr[vec == 8 ? 0 : (vec == 2 ? 1 : 2)];
+    const int vec = p.Wo % 8 == 0 ? 3 : (p.Wo % 4 == 0 ? 2 : (p.Wo % 2 == 0 ? 1 : 0));
+    auto kern = vec == 3 ? conv_wg_fused_kernel<8> : (vec == 2 ? conv_wg_fused_kernel<4> : (vec == 1 ? conv_wg_fused_kernel<2> : conv_wg_fused_kernel<1>));
+    static PerDeviceOnce attr[4];
+    PerDeviceOnce& once = attr[vec];
     if (once.needed()) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBudget) != cudaSuccess)
             return DROPIT_ERR_CUDA;

@@ -154,17 +154,26 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint6
         : "memory");
 }
 // The same for a whole warp that runs the issuing loop together, `leader` being true in one thread: with the loop uniform over
-// the warp, the descriptors stay in uniform registers, where the instruction wants them.
+// the warp, the descriptors stay in uniform registers, where the instruction wants them.  A says what happens to the A
+// operand in the collector buffer: consecutive MMAs with the same A read it from shared memory once (fill, use .., lastuse).
+enum class CollectA { kDiscard, kFill, kUse, kLastUse };
+#define DROPIT_UMMA_ELECTED(USAGE)                                                                                       \
+    asm volatile(                                                                                                        \
+        "{\n\t.reg .pred p, e;\n\t"                                                                                     \
+        "setp.ne.b32 p, %4, 0;\n\t"                                                                                     \
+        "setp.ne.b32 e, %5, 0;\n\t"                                                                                     \
+        "@e tcgen05.mma.cta_group::1.kind::f16" USAGE " [%0], %1, %2, %3, p;\n\t}"                                      \
+        ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(leader)                                  \
+        : "memory")
+template <CollectA A>
 __device__ __forceinline__ void umma_bf16_elected(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                                   uint32_t accumulate, uint32_t leader) {
-    asm volatile(
-        "{\n\t.reg .pred p, e;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "setp.ne.b32 e, %5, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(leader)
-        : "memory");
+    if constexpr (A == CollectA::kFill) DROPIT_UMMA_ELECTED(".collector::a::fill");
+    else if constexpr (A == CollectA::kUse) DROPIT_UMMA_ELECTED(".collector::a::use");
+    else if constexpr (A == CollectA::kLastUse) DROPIT_UMMA_ELECTED(".collector::a::lastuse");
+    else DROPIT_UMMA_ELECTED("");
 }
+#undef DROPIT_UMMA_ELECTED
 __device__ __forceinline__ uint32_t elect_one() {
     uint32_t r;
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
