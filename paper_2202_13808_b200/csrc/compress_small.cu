@@ -15,11 +15,13 @@
 //      shared memory and leave coalesced.
 // Nothing is sampled and no scratch in global memory is used: any distribution of values takes the same path (equal keys
 // make the counting atomics collide, zeros are counted in registers because ReLU outputs are half zeros).
-// Bound by latency: barriers and the trips between CTAs, about 2 us a digit round.  Measured per call (graph replay,
-// gamma 0.9): bf16 8 Ki / 48 Ki / 196 Ki / 454 Ki elements 8.0 / 8.9 / 10.3 / 12.8 us, where the grid-wide kernel's full
-// histogram takes 60 us at any of these sizes; fp32 196 Ki / 454 Ki 16.9 / 20.7 us, where the three histogram launches and
-// the compaction take 27 us at 600 Ki.  At 2^19 bf16 elements (13.6 us) the sampled grid-wide kernel (15.8 us) is about to
-// overtake: two super-blocks per warp measured 17.4 us at 800 Ki against its 16.1, so there the line lies.
+// Bound by latency: barriers, the trips between CTAs (about 1 us a digit round) and the shared-memory counting.  Measured per
+// call (graph replay, gamma 0.9): bf16 8 Ki / 48 Ki / 196 Ki / 454 Ki elements 6.2 / 6.8 / 8.5 / 11.8 us, where the grid-wide
+// kernel's full histogram takes 60 us at any of these sizes; fp32 48 Ki / 196 Ki / 454 Ki 10.8 / 14.0 / 18.8 us, where the three
+// histogram launches and the compaction take 27 us at 600 Ki.  (Counting through a branch per element, only by the warps
+// that own a super-block, and a third barrier per round: 8.0 / 8.9 / 10.3 / 12.8 and 14.2 / 16.9 / 20.7 us.)  At 2^19 bf16
+// elements (12.5 us) the sampled grid-wide kernel (15.8 us) is about to overtake: two super-blocks per warp measured 17.4 us at
+// 800 Ki against its 16.1, so there the line lies.
 #include "common.cuh"
 #include "sm100_ptx.cuh"
 
@@ -39,9 +41,9 @@ constexpr size_t kGatherBytes = (size_t)2 * kMaxCtas * kRowBins * 4;
 
 struct SmallShared {
     uint32_t row[kRowBins];        // this CTA's counts of the current digit
-    uint32_t warp_tot[kWarps];
-    uint32_t gt[kMaxCtas], eq[kMaxCtas];   // per CTA of the cluster: keys above / at the digits fixed so far
-    uint32_t digit, cum;
+    uint2 warp_tot[kWarps];
+    uint32_t digit, cum;           // the digit found, keys above it
+    uint32_t before_gt, before_eq; // in the CTAs in front of this one: keys above / at the digit
 };
 
 template <typename Tr> struct SmallCfg {
@@ -68,11 +70,17 @@ __device__ __forceinline__ uint32_t warp_inclusive_scan(uint32_t v, int lane) {
     return v;
 }
 
+// [addr] += v if `on`; a predicated instruction, not a branch (a branch around every count tripled the counting passes).
+__device__ __forceinline__ void red_shared_if(uint32_t addr, uint32_t v, bool on) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p red.shared.add.u32 [%0], %1;\n\t}" ::"r"(addr), "r"(v), "r"(on ? 1u : 0u) : "memory");
+}
+
 // One digit round: sh.row[0 .. nb) holds this CTA's counts.  Finds the digit in which the descending running count
-// over the cluster reaches k_rem, subtracts from k_rem the keys above it and brings the per-CTA counts up to date.
+// over the cluster reaches k_rem, subtracts from k_rem the keys above it and brings run_gt / run_eq (keys above / at the
+// digits fixed so far, in the CTAs in front of this one) up to date.
 // `rows`: this round's gather buffer, [CTA][kRowBins] (two alternate: a CTA that is ahead by one round writes the other one).
 __device__ __forceinline__ uint32_t digit_round(SmallShared& sh, const uint32_t* rows, int nb, uint32_t rank, uint32_t ctas,
-                                                uint32_t& k_rem, bool first) {
+                                                uint32_t& k_rem, uint32_t& run_gt, uint32_t& run_eq, bool first) {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     __syncthreads();   // the row is complete
     if (first) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // every CTA of the cluster is running
@@ -82,37 +90,48 @@ __device__ __forceinline__ uint32_t digit_round(SmallShared& sh, const uint32_t*
         ptx::st_cluster_u32(ptx::map_shared_to_cta(mine + b * 4, dest), sh.row[b]);
     }
     ptx::cluster_sync_all();
-    // thread t < nb looks at bin nb - 1 - t: a prefix over the threads is a count from the top
+    // thread t < nb looks at bin nb - 1 - t: a prefix over the threads is a count from the top, over the cluster (h) and over
+    // the CTAs in front of this one (f)
     const int bin = nb - 1 - t;
-    uint32_t h = 0;
-    if (t < nb)
-        for (uint32_t r = 0; r < ctas; ++r) h += rows[r * kRowBins + bin];
-    const uint32_t inc = warp_inclusive_scan(h, lane);
-    if (lane == 31) sh.warp_tot[warp] = inc;
+    uint32_t h = 0, f = 0, h_inc = 0, f_inc = 0;
+    if (t < nb) {
+        for (uint32_t r = 0; r < ctas; ++r) {
+            const uint32_t v = rows[r * kRowBins + bin];
+            h += v;
+            if (r < rank) f += v;
+        }
+        h_inc = h;
+        f_inc = f;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t yh = __shfl_up_sync(kFullMask, h_inc, o), yf = __shfl_up_sync(kFullMask, f_inc, o);
+            if (lane >= o) { h_inc += yh; f_inc += yf; }
+        }
+        if (lane == 31) sh.warp_tot[warp] = make_uint2(h_inc, f_inc);
+    }
     __syncthreads();
     if (t < nb) {
-        uint32_t cum = inc - h;
-        for (int w = 0; w < warp; ++w) cum += sh.warp_tot[w];
+        uint32_t cum = h_inc - h, before = f_inc - f;
+#pragma unroll
+        for (int w = 0; w < kRowBins / 32 - 1; ++w) {
+            if (w < warp) {
+                const uint2 v = sh.warp_tot[w];
+                cum += v.x;
+                before += v.y;
+            }
+        }
         if (cum < k_rem && k_rem <= cum + h) {
             sh.digit = (uint32_t)bin;
             sh.cum = cum;
+            sh.before_gt = before;
+            sh.before_eq = f;
         }
     }
     __syncthreads();
-    const uint32_t digit = sh.digit;
     k_rem -= sh.cum;
-    if ((uint32_t)warp < ctas) {
-        uint32_t g = 0;
-        for (int b = (int)digit + 1 + lane; b < nb; b += 32) g += rows[warp * kRowBins + b];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(kFullMask, g, o);
-        if (lane == 0) {
-            sh.gt[warp] = (first ? 0u : sh.gt[warp]) + g;
-            sh.eq[warp] = rows[warp * kRowBins + digit];
-        }
-    }
-    __syncthreads();   // sh.row, sh.digit and sh.warp_tot may be written again
-    return digit;
+    run_gt += sh.before_gt;
+    run_eq = sh.before_eq;
+    return sh.digit;       // (the next round's first barrier comes before anything here is written again)
 }
 
 template <typename Tr, bool INDEX32>
@@ -165,32 +184,32 @@ small_compress_kernel(const uint4* __restrict__ x, uint32_t n, uint32_t k, uint3
     __syncthreads();
 
     // ---- counts of the upper 15 key bits ----
-    // visit(key) for every element of the warp's super-block that exists (zero padding is no data); any order
+    // visit(key, exists) for every element of the CTA's super-blocks (zero padding does not exist), in any order: all threads
+    // share the 16-byte vectors, also when only some warps own a super-block
+    const uint32_t cta_vecs = min(sb_per_cta, (n + kSb - 1) / kSb - min((n + kSb - 1) / kSb, rank * sb_per_cta)) * Cfg::kVecs;
+    const uint32_t cta_first = rank * sb_per_cta * kSb, data0 = ptx::smem_u32(ssm);
     auto for_each_key = [&](auto visit) {
-        if (active) {
-            const bool whole = ((uint64_t)sb + 1) * kSb <= n;
+        for (uint32_t v = t; v < cta_vecs; v += kThreads) {
+            uint32_t w[4];
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                         : "r"(data0 + v * 16) : "memory");
+            const uint32_t e0 = cta_first + v * G;
 #pragma unroll
-            for (int j = 0; j < OV; ++j) {
-                uint32_t w[4];
-                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
-                             : "r"(data + (j * 32 + lane) * 16) : "memory");
-                const uint32_t e0 = sb * kSb + (j * 32 + lane) * G;
-#pragma unroll
-                for (int e = 0; e < G; ++e) {
-                    uint32_t key;
-                    if constexpr (kF32) key = w[e] & 0x7FFFFFFFu;
-                    else key = ((e & 1) ? (w[e >> 1] >> 16) : w[e >> 1]) & 0x7FFFu;
-                    if (whole || e0 + e < n) visit(key);
-                }
+            for (int e = 0; e < G; ++e) {
+                uint32_t key;
+                if constexpr (kF32) key = w[e] & 0x7FFFFFFFu;
+                else key = ((e & 1) ? (w[e >> 1] >> 16) : w[e >> 1]) & 0x7FFFu;
+                visit(key, e0 + e < n);
             }
         }
     };
     {
         uint32_t zeros = 0;
-        for_each_key([&](uint32_t key) {
+        const uint32_t hist_addr = ptx::smem_u32(hist);
+        for_each_key([&](uint32_t key, bool exists) {
             const uint32_t top = kF32 ? key >> 16 : key;
-            if (top == 0) ++zeros;
-            else atomicAdd(&hist[top >> 1], 1u << ((top & 1u) * 16));
+            zeros += top == 0 && exists ? 1u : 0u;
+            red_shared_if(hist_addr + (top >> 1) * 4, 1u << ((top & 1u) * 16), top != 0 && exists);
         });
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) zeros += __shfl_xor_sync(kFullMask, zeros, o);
@@ -213,31 +232,29 @@ small_compress_kernel(const uint4* __restrict__ x, uint32_t n, uint32_t k, uint3
         sum += __shfl_xor_sync(kFullMask, sum, 2);
         if ((t & 3) == 0) sh.row[t >> 2] = sum;
     }
-    const uint32_t d1 = digit_round(sh, gather, 256, rank, ctas, k_rem, true);
+    uint32_t run_gt = 0, run_eq = 0;   // keys above / at T in front of this CTA
+    const uint32_t d1 = digit_round(sh, gather, 256, rank, ctas, k_rem, run_gt, run_eq, true);
     // ---- digit 2: the 128 counters behind that sum ----
     if (t < 128) {
         const uint32_t w = hist[d1 * 64 + (t >> 1)];
         sh.row[t] = (t & 1) ? w >> 16 : w & 0xFFFFu;
     }
-    uint32_t T = d1 * 128 + digit_round(sh, gather + kMaxCtas * kRowBins, 128, rank, ctas, k_rem, false);
+    uint32_t T = d1 * 128 + digit_round(sh, gather + kMaxCtas * kRowBins, 128, rank, ctas, k_rem, run_gt, run_eq, false);
     if constexpr (kF32) {
         // ---- digits 3 and 4: the lower 16 bits, over the keys whose upper bits match ----
+        const uint32_t row_addr = ptx::smem_u32(sh.row);
 #pragma unroll 1
         for (int shift = 8; shift >= 0; shift -= 8) {
             if (t < kRowBins) sh.row[t] = 0;
             __syncthreads();
-            for_each_key([&](uint32_t key) {
-                if ((key >> (shift + 8)) == T) atomicAdd(&sh.row[(key >> shift) & 0xFFu], 1u);
+            for_each_key([&](uint32_t key, bool exists) {
+                red_shared_if(row_addr + ((key >> shift) & 0xFFu) * 4, 1u, exists && (key >> (shift + 8)) == T);
             });
-            T = (T << 8) | digit_round(sh, gather + (shift == 8 ? 0 : kMaxCtas * kRowBins), 256, rank, ctas, k_rem, false);
+            T = (T << 8) | digit_round(sh, gather + (shift == 8 ? 0 : kMaxCtas * kRowBins), 256, rank, ctas, k_rem, run_gt, run_eq,
+                                         false);
         }
     }
     const uint32_t q = k_rem;          // ties at T that are retained, lowest flat indices first
-    uint32_t run_gt = 0, run_eq = 0;   // keys above / at T in front of this CTA
-    for (uint32_t r = 0; r < rank; ++r) {
-        run_gt += sh.gt[r];
-        run_eq += sh.eq[r];
-    }
     ptx::launch_dependents();
 
     // ---- ordered compaction ----
@@ -270,11 +287,11 @@ small_compress_kernel(const uint4* __restrict__ x, uint32_t n, uint32_t k, uint3
     const uint32_t cnt = __popc(g32) | (__popc(e32) << 16);      // a CTA has fewer than 2^16 elements: packed sums do not overflow
     const uint32_t inc = warp_inclusive_scan(cnt, lane);
     const uint32_t excl = inc - cnt, tot = __shfl_sync(kFullMask, inc, 31);
-    if (lane == 0) sh.warp_tot[warp] = tot;
+    if (lane == 0) sh.warp_tot[warp].x = tot;
     __syncthreads();
     if (!active) return;
     {
-        const uint32_t other = sh.warp_tot[lane];
+        const uint32_t other = sh.warp_tot[lane].x;
         const uint32_t before = warp_inclusive_scan(other, lane) - other;
         const uint32_t mine = __shfl_sync(kFullMask, before, warp);
         run_gt += mine & 0xFFFFu;
@@ -381,7 +398,7 @@ bool launch_small(const void* x, int64_t n, int64_t k, void* values, void* meta,
     const int limit = max_cluster<Tr, INDEX32>();
     const int64_t sbs = (n + kSb - 1) / kSb;
     if (limit == 0 || sbs > (int64_t)limit * kWarps) return false;
-    // 8 super-blocks per CTA until the cluster is full: 2 to 16 measure the same at 48 Ki elements, 32 costs 1.6 us there
+    // 8 super-blocks per CTA until the cluster is full: at 48 Ki elements 4 / 8 / 16 measure 7.0 / 6.8 / 7.5 us
     int ctas = 1;
     while (ctas < limit && sbs > (int64_t)ctas * kSbPerCta) ctas *= 2;
     const int64_t per = (sbs + ctas - 1) / ctas;
