@@ -41,12 +41,76 @@ constexpr int kEpiSubs = 2;                            // epilogue warps per TME
 constexpr int kEpiWarps = 4 * kEpiSubs;
 constexpr int kTcThreads = 64 + 32 * kEpiWarps;        // TMA warp, MMA warp, epilogue warps (idle until the accumulator is final)
 
+// Even split of tiles * blocks token blocks over `pairs` CTA pairs.  The first `full` * `len` blocks of every tile go to `full` pairs
+// of their own, which start at the same tokens in every tile, so that the rows of dY and of the scratch that the tiles share
+// are read at the same time; what is left of the tiles, one after the other, is cut into equal pieces for the remaining pairs.
+// A piece touches two tiles at most (the plan sees to that).  full = 0: everything is cut into equal pieces.
+struct StreamSplit {
+    int pairs, full, len;
+    int own;                                    // tiles * full: the first pair without a tile of its own
+    int left;                                   // blocks of a tile behind the full pairs' ones
+    uint32_t rest, all;                         // pieces of the rests, blocks of all rests: piece q starts at q * all / rest
+};
+constexpr int kStreamMaxBlocks = 1 << 18;       // of a tile: the products below stay under 2^32
+static StreamSplit make_stream_split(int pairs, int full, int len, int tiles, int blocks) {
+    StreamSplit s{pairs, full, len, tiles * full, blocks - full * len, 0, 0};
+    if (pairs > s.own && s.left > 0) {
+        s.rest = (uint32_t)(pairs - s.own);
+        s.all = (uint32_t)tiles * (uint32_t)s.left;
+    }
+    return s;
+}
+struct StreamPiece {
+    int tile, begin, first, next_begin, n;      // `first` blocks of `tile` from `begin` on, then n - first of the next one from next_begin on
+};
+__host__ __device__ __forceinline__ StreamPiece stream_piece(const StreamSplit& s, int p) {
+    StreamPiece r;
+    if (p < s.own) {
+        r.tile = p / s.full;
+        r.begin = (p - r.tile * s.full) * s.len;
+        r.first = r.n = s.len;
+        r.next_begin = 0;
+        return r;
+    }
+    const uint32_t q = (uint32_t)(p - s.own);
+    const int v = (int)(q * s.all / s.rest);
+    r.n = (int)((q + 1) * s.all / s.rest) - v;
+    r.tile = v / s.left;
+    const int off = v - r.tile * s.left;
+    r.next_begin = s.full * s.len;
+    r.begin = r.next_begin + off;
+    r.first = r.n < s.left - off ? r.n : s.left - off;
+    return r;
+}
+// The pairs that add to a tile: `full` of its own, then those whose piece touches its rest (first .. first + count - 1, counted
+// from the first pair without a tile of its own).
+__host__ __device__ __forceinline__ void stream_rest_pairs(const StreamSplit& s, int tile, int& first, int& count) {
+    first = count = 0;
+    if (s.left <= 0) return;
+    auto owner = [&](uint32_t v) {              // the piece of block v of the rests: the last one that starts at or before it
+        return (int)(((v + 1) * s.rest - 1) / s.all);
+    };
+    first = owner((uint32_t)(tile * s.left));
+    count = owner((uint32_t)((tile + 1) * s.left - 1)) - first + 1;
+}
+// Whether every piece has a block and touches two tiles at most.
+static bool stream_split_ok(const StreamSplit& s) {
+    if (s.left < 0 || (s.full > 0 && s.len < 1)) return false;
+    if (s.left == 0) return s.pairs == s.own;
+    if (s.pairs <= s.own || s.all < s.rest) return false;
+    for (int p = s.own; p < s.pairs; ++p) {
+        const StreamPiece c = stream_piece(s, p);
+        if (c.n - c.first > s.left) return false;
+    }
+    return true;
+}
+
 struct WgPlan {
     bool tensor_core;
     bool fused;               // weight_grad_tmem.cu: the cache is expanded into tensor memory inside the GEMM (no dense scratch)
     bool cluster;             // the splits of a tile form a thread-block cluster and add up through shared memory
     bool pair;                // CTA pairs compute 256 x 256 tiles (wg_pair_kernel); the splits add up through global memory
-    int stream_pairs;         // > 0: that many pairs share out all tiles' token blocks evenly (see StreamSplit), a second kernel adds up
+    StreamSplit stream;       // pairs > 0: they share out all tiles' token blocks evenly, a second kernel adds up
     int stream_slots;         // most pairs that share a tile
     int tiles_m, tiles_n, splits, kb_total, kb_per_split;
     size_t counters_off, counters_bytes;
@@ -67,21 +131,10 @@ static bool wg_path_is(const char* name) {
     return e && std::strcmp(e, name) == 0;
 }
 
-// Even split: pair p of `pairs` takes the token blocks [p * units / pairs, (p + 1) * units / pairs) of the sequence
-// "all blocks of tile 0, all blocks of tile 1, ..." (units = tiles * kb_total).  With at least as many pairs as tiles it touches
-// two tiles at most.
-__host__ __device__ __forceinline__ int stream_begin(int p, int units, int pairs) { return (int)((int64_t)p * units / pairs); }
-// The first pair that touches the tile whose blocks start at `unit`.
-__host__ __device__ __forceinline__ int stream_first_pair(int unit, int units, int pairs) {
-    int p = (int)((int64_t)unit * pairs / units);
-    while (p > 0 && stream_begin(p, units, pairs) > unit) --p;
-    while (stream_begin(p + 1, units, pairs) <= unit) ++p;
-    return p;
-}
-
 // Splits used to be as many as the SMs hold, whatever adding them up costs.  Measured per call, decompression included, before
-// and after choosing by cost: 591 x 768 -> 768 16.9 -> 12.5 us (no split), 1000 x 1024 -> 1024 21.8 -> 14.2, 8000 x 768 -> 768
-// 34.2 -> 26.3, 20000 x 256 -> 768 37.2 -> 27.2 and 25000 x 200 -> 800 40.9 -> 33.1 (even split).
+// and after choosing by cost: no split: 591 x 768 -> 768 16.9 -> 12.4 us, 1000 x 1024 -> 1024 21.8 -> 14.2; even split:
+// 5000 x 192 -> 768 36 -> 18, 8000 x 768 -> 768 34 -> 20, 20000 x 256 -> 768 37 -> 23, 30000 x 384 -> 384 42 -> 29,
+// 20000 x 800 -> 2400 109 -> 82, 32768 x 768 -> 2304 104 -> 94 (54 of the 72 pairs that find room used to work).
 // Microseconds, fitted on B200 (768 .. 3072 wide outputs, 591 .. 32768 tokens): a 144-token block of a pair's main loop,
 // and what adding up costs: tickets by the number of splits, or partial tiles written and read again by a second kernel.
 constexpr float kBlockUs = 0.66f;
@@ -91,7 +144,7 @@ static float ticket_us(int splits) {
 }
 // Pairs of CTAs that the device holds at once (not every SM finds a neighbour), defined behind the kernel.
 static int resident_pairs();
-static float stream_us(int pairs, int tiles) { return 6.f + 0.07f * (float)(pairs + tiles); }
+static float stream_us(int pairs, int tiles) { return 4.5f + 0.05f * (float)(pairs + tiles); }
 
 static WgPlan make_wg_plan(int64_t M, int64_t Ca, int64_t Cz, dropit_dtype dtype, dropit_format format, bool fused) {
     WgPlan p{};
@@ -135,21 +188,25 @@ static WgPlan make_wg_plan(int64_t M, int64_t Ca, int64_t Cz, dropit_dtype dtype
                 if (s == 1 || us < best) { best = us; splits = s; }
             }
             const int all_pairs = resident_pairs() < units ? resident_pairs() : units;
-            // Under the even split the pairs are at different tokens at any time, so that a row of dY or of the scratch that
-            // several tiles share is read from HBM for each of them unless L2 holds both operands (32768 x 768 -> 2304, 201 MB:
-            // 122 us against 92 with aligned ranges).
+            // Pairs at different tokens read what the tiles share from HBM once each, unless L2 holds both operands
+            // (32768 x 768 -> 2304, 201 MB: 122 us with full = 0, 92 with whole ranges).
             const bool in_l2 = (M * Ca + M * Cz) * 2 <= kStreamMaxBytes;
-            for (int s = 2; s <= most + 1 && pair_tiles <= all_pairs && in_l2; ++s) {
-                const int pairs = s * pair_tiles < all_pairs ? s * pair_tiles : all_pairs;
-                const float us = kBlockUs * ((units + pairs - 1) / pairs) + stream_us(pairs, pair_tiles);
-                if (us < best) { best = us; p.stream_pairs = pairs; }
+            for (int pairs = all_pairs; pairs > pair_tiles && pairs > all_pairs - 8 && p.kb_total < kStreamMaxBlocks; --pairs) {
+                const int len = (units + pairs - 1) / pairs;
+                // a pair that crosses from one tile into the next stores two accumulators
+                const float us = kBlockUs * len + stream_us(pairs, pair_tiles) + (pairs % pair_tiles ? 2.f : 0.f);
+                if (us >= best - (p.stream.pairs ? 0.5f : 0.f)) continue;      // fewer pairs only for a clear gain
+                const StreamSplit aligned = make_stream_split(pairs, pairs / pair_tiles, len, pair_tiles, p.kb_total);
+                const StreamSplit loose = make_stream_split(pairs, 0, 0, pair_tiles, p.kb_total);
+                if (stream_split_ok(aligned)) { best = us; p.stream = aligned; }
+                else if (in_l2 && stream_split_ok(loose)) { best = us; p.stream = loose; }
             }
-            if (p.stream_pairs) {
+            if (p.stream.pairs) {
                 splits = 1;
                 for (int t = 0; t < pair_tiles; ++t) {
-                    const int first = stream_first_pair(t * p.kb_total, units, p.stream_pairs);
-                    const int last = stream_first_pair((t + 1) * p.kb_total - 1, units, p.stream_pairs);
-                    if (last - first + 1 > p.stream_slots) p.stream_slots = last - first + 1;
+                    int first, count;
+                    stream_rest_pairs(p.stream, t, first, count);
+                    if (p.stream.full + count > p.stream_slots) p.stream_slots = p.stream.full + count;
                 }
             }
         }
@@ -166,11 +223,31 @@ static WgPlan make_wg_plan(int64_t M, int64_t Ca, int64_t Cz, dropit_dtype dtype
     p.dense_off = p.counters_off + p.counters_bytes;
     p.dense_bytes = align_up((size_t)M * Ca * es, 256);
     p.partial_off = p.dense_off + p.dense_bytes;
-    const int planes = p.stream_pairs ? p.stream_slots : (p.splits > 1 && !p.cluster ? p.splits : 0);
+    const int planes = p.stream.pairs ? p.stream_slots : (p.splits > 1 && !p.cluster ? p.splits : 0);
     p.partial_bytes = (size_t)planes * p.tiles_m * p.tiles_n * kBM * kBN * 4;   // whole tiles
     p.total_bytes = p.partial_off + p.partial_bytes;
     if (p.total_bytes == 0) p.total_bytes = 256;
     return p;
+}
+
+// The plans of the last shapes that this thread asked for: weighing the splits costs some microseconds, and a layer is planned
+// twice per call (workspace query and launch).
+static const WgPlan& cached_wg_plan(int64_t M, int64_t Ca, int64_t Cz, dropit_dtype dtype, dropit_format format, bool fused) {
+    struct Entry {
+        int64_t key[5];
+        WgPlan plan;
+    };
+    static thread_local Entry entries[8] = {};
+    static thread_local int next = 0;
+    const int64_t key[5] = {M, Ca, Cz, (int64_t)dtype | (int64_t)format << 4 | (int64_t)fused << 8 | (int64_t)wg_path_is("single") << 9,
+                            (int64_t)current_device() + 1};
+    for (const Entry& e : entries)
+        if (std::memcmp(e.key, key, sizeof(key)) == 0) return e.plan;
+    Entry& e = entries[next];
+    next = (next + 1) % 8;
+    e.plan = make_wg_plan(M, Ca, Cz, dtype, format, fused);
+    std::memcpy(e.key, key, sizeof(key));
+    return e.plan;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -656,10 +733,10 @@ constexpr size_t kPairSmemBytes = 1024 + (size_t)kPairStages * (kPairAStageBytes
 static_assert(kPairStages * (kPairAStageBytes + kPairBStageBytes) >= (int)(kEpiWarps * kEpiWarpFloats * sizeof(float)),
               "the epilogue stages its chunks in the pipeline buffers");
 
-// What a pair works on: `first` token blocks of one tile from kb_begin on and, under the even split, the blocks up to nkb from
-// the beginning of the next tile.
+// What a pair works on: `first` token blocks of one tile from kb_begin on and, under the even split, the blocks up to nkb of the
+// next tile from next_kb_begin on.
 struct PairSegments {
-    int nkb, first, kb_begin;
+    int nkb, first, kb_begin, next_kb_begin;
     int j0, cb;                      // first row of dY's columns / first of the tile's channels that this CTA loads
     int next_j0, next_cb;
 };
@@ -692,7 +769,7 @@ __device__ __forceinline__ void pair_producer(PairSmem* ctl, uint8_t* sA, uint8_
             const uint32_t bar = full0 + 8u * (uint32_t)s;
             if (!member) ptx::mbar_arrive_expect_tx(&ctl->full[s], 2u * kPairStageTx);
             const bool next = STREAM && i >= seg.first;
-            const int k0 = (next ? i - seg.first : seg.kb_begin + i) * kPairBK;
+            const int k0 = (next ? seg.next_kb_begin + i - seg.first : seg.kb_begin + i) * kPairBK;
             const int j0 = next ? seg.next_j0 : seg.j0, cb = next ? seg.next_cb : seg.cb;
             uint8_t* a = sA + s * kPairAStageBytes;
             uint8_t* b = sB + s * kPairBStageBytes;
@@ -721,7 +798,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CUtensorMap map_x, int Ca, int Cz,
                int tiles_n, int splits, int kb_per_split, int kb_total, float* __restrict__ dw, int accumulate,
                float* __restrict__ partial, uint32_t* counters, int32_t* dev_status, int grouped_maps,
-               uint32_t wait_limit, uint32_t epoch, int stream_pairs) {
+               uint32_t wait_limit, uint32_t epoch, const StreamSplit stream) {
     extern __shared__ uint8_t smem_raw[];
     // same offsets in both CTAs: the MMA addresses the operands of both with one descriptor
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -737,13 +814,14 @@ wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
     const int split = blockIdx.y;
     int pair = blockIdx.x >> 1;                    // pair of tiles; the pair's CTAs are neighbours along x
     PairSegments seg;
+    const int pair_tiles = ((Cz + 2 * kBM - 1) / (2 * kBM)) * tiles_n;
     if constexpr (STREAM) {
-        const int units = (int)(((Cz + 2 * kBM - 1) / (2 * kBM)) * tiles_n * kb_total);
-        const int u0 = stream_begin(pair, units, stream_pairs);
-        seg.nkb = stream_begin(pair + 1, units, stream_pairs) - u0;
-        pair = u0 / kb_total;
-        seg.kb_begin = u0 - pair * kb_total;
-        seg.first = min(seg.nkb, kb_total - seg.kb_begin);
+        const StreamPiece piece = stream_piece(stream, pair);
+        pair = piece.tile;
+        seg.nkb = piece.n;
+        seg.first = piece.first;
+        seg.kb_begin = piece.begin;
+        seg.next_kb_begin = piece.next_begin;
     } else {
         seg.kb_begin = split * kb_per_split;
         seg.first = seg.nkb = min(kb_total, seg.kb_begin + kb_per_split) - seg.kb_begin;
@@ -846,8 +924,8 @@ wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
         if constexpr (STREAM) {
             // Every segment's accumulator leaves for the pair's plane of the tile as it is.  The first of two does so under the
             // main loop of the second, by the four warps that do not produce.
-            const int units = (int)(((Cz + 2 * kBM - 1) / (2 * kBM)) * tiles_n * kb_total);
-            const size_t stride = (size_t)2 * ((Cz + 2 * kBM - 1) / (2 * kBM)) * tiles_n * kPlaneTileFloats;
+            const int me = (int)(blockIdx.x >> 1);
+            const size_t stride = (size_t)2 * pair_tiles * kPlaneTileFloats;
             for (int sg = 0; sg < segments; ++sg) {
                 const bool shared_out = sg == segments - 1;         // all eight warps
                 if (!shared_out && warp < 6) continue;
@@ -855,7 +933,12 @@ wg_pair_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant
                 ok = __all_sync(kFullMask, ok) && !*abort_flag;
                 if (!ok) { *abort_flag = 1; break; }
                 ptx::tc_fence_after();
-                const int slot = (int)(blockIdx.x >> 1) - stream_first_pair((pair + sg) * kb_total, units, stream_pairs);
+                int slot = me - pair * stream.full;
+                if (me >= stream.own) {
+                    int first, count;
+                    stream_rest_pairs(stream, pair + sg, first, count);
+                    slot = stream.full + me - stream.own - first;
+                }
                 float* plane = partial + (size_t)slot * stride + (size_t)(tile + 2 * sg) * kPlaneTileFloats;
                 const int g = warp & 3;
                 for (int ch = shared_out ? (warp - 2) >> 2 : 0; ch < kBN / 32; ch += shared_out ? kEpiSubs : 1) {
@@ -939,50 +1022,59 @@ static int resident_pairs() {
     return v;
 }
 
-// dw (=|+=) the planes of every tile, in pair order, after wg_pair_kernel under the even split.  A warp takes 32 rows x 32
-// columns: its lanes read their row's columns of each plane (512 contiguous bytes per load), turn the sum through shared
-// memory and write 128-byte row segments.
-__global__ void __launch_bounds__(128)
-wg_stream_reduce_kernel(const float* __restrict__ partial, int Ca, int Cz, int tiles_n, int kb_total, int stream_pairs,
+// dw (=|+=) the planes of every tile after wg_pair_kernel under the even split.  A block takes 32 rows x 32 columns; its four
+// warps share out the planes (warp w adds planes w, w + 4, ...), a lane reading its row's columns of a plane (512 contiguous
+// bytes per load), and the four sums are added in warp order: a fixed order for a given split.  Then every warp writes eight
+// 128-byte row segments.  (One warp per 32 x 32 columns took 19 us for the 24 planes of 20000 x 256 -> 768.)
+constexpr int kReduceWarps = 4;
+__global__ void __launch_bounds__(32 * kReduceWarps)
+wg_stream_reduce_kernel(const float* __restrict__ partial, int Ca, int Cz, int tiles_n, const StreamSplit stream,
                         float* __restrict__ dw, int accumulate) {
-    __shared__ __align__(16) float stage_all[4 * kEpiWarpFloats];
-    const int g = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    float* stage = stage_all + g * kEpiWarpFloats;
-    const int tile = blockIdx.x / (kBN / 32), ch = blockIdx.x % (kBN / 32);
-    const int pair_tiles = ((Cz + 2 * kBM - 1) / (2 * kBM)) * tiles_n, units = pair_tiles * kb_total;
+    __shared__ __align__(16) float stage_all[kReduceWarps * kEpiWarpFloats];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float* stage = stage_all + w * kEpiWarpFloats;
+    const int g = blockIdx.x & 3, ch = (blockIdx.x >> 2) % (kBN / 32), tile = (blockIdx.x >> 2) / (kBN / 32);
+    const int pair_tiles = ((Cz + 2 * kBM - 1) / (2 * kBM)) * tiles_n;
     const int pair = tile >> 1, member = tile & 1;
-    const int j0 = ((pair / tiles_n) * 2 + member) * kBM, c0 = (pair % tiles_n) * kBN;
+    const int j0 = ((pair / tiles_n) * 2 + member) * kBM + 32 * g, c0 = (pair % tiles_n) * kBN + ch * 32;
     ptx::grid_dependency_wait();
-    if (j0 + 32 * g >= Cz || c0 + ch * 32 >= Ca) return;       // uniform over the warp
-    const int first = stream_first_pair(pair * kb_total, units, stream_pairs);
-    const int count = stream_first_pair((pair + 1) * kb_total - 1, units, stream_pairs) - first + 1;
+    if (j0 >= Cz || c0 >= Ca) return;                          // uniform over the block
+    int first, count;
+    stream_rest_pairs(stream, pair, first, count);
+    count += stream.full;
     const size_t stride = (size_t)2 * pair_tiles * kPlaneTileFloats;
     const float* src = partial + (size_t)tile * kPlaneTileFloats + plane_offset(ch, g, 0, lane);
-    float4 acc[8], next[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) next[e] = __ldcg(reinterpret_cast<const float4*>(src + e * 128));
+    float4 acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s = 0; s < count; ++s) {
-        float4 cur[8];
+    for (int s = w; s < count; s += 2 * kReduceWarps) {        // two planes in flight
+        const bool two = s + kReduceWarps < count;
+        float4 a[8], b[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) cur[e] = next[e];
-        if (s + 1 < count) {
-#pragma unroll
-            for (int e = 0; e < 8; ++e) next[e] = __ldcg(reinterpret_cast<const float4*>(src + (size_t)(s + 1) * stride + e * 128));
+        for (int e = 0; e < 8; ++e) {
+            a[e] = __ldcg(reinterpret_cast<const float4*>(src + (size_t)s * stride + e * 128));
+            b[e] = two ? __ldcg(reinterpret_cast<const float4*>(src + (size_t)(s + kReduceWarps) * stride + e * 128))
+                       : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) { acc[e].x += cur[e].x; acc[e].y += cur[e].y; acc[e].z += cur[e].z; acc[e].w += cur[e].w; }
+        for (int e = 0; e < 8; ++e) {
+            acc[e].x += a[e].x; acc[e].y += a[e].y; acc[e].z += a[e].z; acc[e].w += a[e].w;
+            acc[e].x += b[e].x; acc[e].y += b[e].y; acc[e].z += b[e].z; acc[e].w += b[e].w;
+        }
     }
 #pragma unroll
     for (int e = 0; e < 8; ++e) *reinterpret_cast<float4*>(stage + lane * kEpiRowFloats + 4 * e) = acc[e];
-    __syncwarp();
-    const int rr0 = lane >> 3, q = lane & 7, col = c0 + ch * 32 + 4 * q;
+    __syncthreads();
+    const int q = lane & 7, col = c0 + 4 * q, warps = min(count, kReduceWarps);
 #pragma unroll
-    for (int it = 0; it < 8; ++it) {
-        const int row = j0 + 32 * g + it * 4 + rr0;
+    for (int it = 0; it < 2; ++it) {
+        const int r = w * 8 + it * 4 + (lane >> 3), row = j0 + r;
         if (col < Ca && row < Cz) {                             // Ca is a multiple of 8
-            float4 v = *reinterpret_cast<const float4*>(stage + (it * 4 + rr0) * kEpiRowFloats + 4 * q);
+            float4 v = *reinterpret_cast<const float4*>(stage_all + r * kEpiRowFloats + 4 * q);
+            for (int k = 1; k < warps; ++k) {
+                const float4 o = *reinterpret_cast<const float4*>(stage_all + k * kEpiWarpFloats + r * kEpiRowFloats + 4 * q);
+                v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
+            }
             float* dst = dw + (size_t)row * Ca + col;
             if (accumulate) {
                 const float4 o = *reinterpret_cast<const float4*>(dst);
@@ -1170,7 +1262,7 @@ extern "C" dropit_status dropit_weight_grad_workspace(int64_t M, int64_t Ca, int
     if (M < 0 || Ca <= 0 || Cz <= 0 || M * Ca >= ((int64_t)1 << 31)) return DROPIT_ERR_INVALID_ARG;
     if ((dtype != DROPIT_BF16 && dtype != DROPIT_F32) || (format != DROPIT_FMT_BITMASK && format != DROPIT_FMT_INDEX32))
         return DROPIT_ERR_INVALID_ARG;
-    if (workspace_bytes) *workspace_bytes = make_wg_plan(M, Ca, Cz, dtype, format, false).total_bytes;
+    if (workspace_bytes) *workspace_bytes = cached_wg_plan(M, Ca, Cz, dtype, format, false).total_bytes;
     return DROPIT_OK;
 }
 
@@ -1194,7 +1286,7 @@ static dropit_status weight_grad_impl(const void* dy, const void* values, const 
     if (!dy || !values || !meta || !is_aligned16(dy) || !is_aligned16(values) || !is_aligned16(meta))
         return DROPIT_ERR_INVALID_ARG;
     if (format == DROPIT_FMT_BITMASK && (!offsets || !is_aligned16(offsets))) return DROPIT_ERR_INVALID_ARG;
-    const WgPlan plan = make_wg_plan(M, Ca, Cz, dtype, format, force_fused || prefer_fused());
+    const WgPlan plan = cached_wg_plan(M, Ca, Cz, dtype, format, force_fused || prefer_fused());
     if (plan.fused)   // one launch, no scratch
         return launch_wg_tmem(dy, values, meta, offsets, M, Ca, Cz, k, plan.splits, plan.kb_per_split, plan.kb_total, dw,
                               accumulate, dev_status, stream);
@@ -1256,7 +1348,7 @@ static dropit_status weight_grad_impl(const void* dy, const void* values, const 
             return DROPIT_ERR_CUDA;
         smem_attr.mark();
     }
-    dim3 grid(plan.stream_pairs ? 2 * plan.stream_pairs : plan.tiles_m * plan.tiles_n, plan.splits);
+    dim3 grid(plan.stream.pairs ? 2 * plan.stream.pairs : plan.tiles_m * plan.tiles_n, plan.splits);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(kTcThreads);
@@ -1277,9 +1369,9 @@ static dropit_status weight_grad_impl(const void* dy, const void* values, const 
     attr[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
     ++cfg.numAttrs;
     const cudaError_t err =
-        plan.pair ? cudaLaunchKernelEx(&cfg, plan.stream_pairs ? wg_pair_kernel<true> : wg_pair_kernel<false>, map_dy, map_x, (int)Ca, (int)Cz, plan.tiles_n, plan.splits,
+        plan.pair ? cudaLaunchKernelEx(&cfg, plan.stream.pairs ? wg_pair_kernel<true> : wg_pair_kernel<false>, map_dy, map_x, (int)Ca, (int)Cz, plan.tiles_n, plan.splits,
                                        plan.kb_per_split, plan.kb_total, dw, accumulate, partial, counters, dev_status,
-                                       grouped ? 1 : 0, spin_limit(kWaitLimit), epoch, plan.stream_pairs)
+                                       grouped ? 1 : 0, spin_limit(kWaitLimit), epoch, plan.stream)
                   : cudaLaunchKernelEx(&cfg, wg_tc_kernel, map_dy, map_x, (int)Ca, (int)Cz, plan.tiles_n, plan.splits,
                                        plan.kb_per_split, plan.kb_total, dw, accumulate, partial, counters, dev_status,
                                        plan.cluster ? 1 : 0, grouped ? 1 : 0, spin_limit(kWaitLimit), epoch);
@@ -1287,16 +1379,16 @@ static dropit_status weight_grad_impl(const void* dy, const void* values, const 
         (void)cudaGetLastError();
         return DROPIT_ERR_CUDA;
     }
-    if (plan.stream_pairs == 0) return check_launch();
+    if (plan.stream.pairs == 0) return check_launch();
     s = check_launch();
     if (s != DROPIT_OK) return s;
-    cfg.gridDim = dim3((unsigned)(plan.tiles_m * plan.tiles_n * (kBN / 32)));
-    cfg.blockDim = dim3(128);
+    cfg.gridDim = dim3((unsigned)(plan.tiles_m * plan.tiles_n * (kBN / 32) * 4));
+    cfg.blockDim = dim3(32 * kReduceWarps);
     cfg.dynamicSmemBytes = 0;
     attr[0] = attr[cfg.numAttrs - 1];            // programmatic launch only
     cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, wg_stream_reduce_kernel, (const float*)partial, (int)Ca, (int)Cz, plan.tiles_n, plan.kb_total,
-                           plan.stream_pairs, dw, accumulate) != cudaSuccess) {
+    if (cudaLaunchKernelEx(&cfg, wg_stream_reduce_kernel, (const float*)partial, (int)Ca, (int)Cz, plan.tiles_n,
+                           plan.stream, dw, accumulate) != cudaSuccess) {
         (void)cudaGetLastError();
         return DROPIT_ERR_CUDA;
     }

@@ -15,6 +15,10 @@ CASES = [
     di.small_linear(9000, 256, 768, "bf16", 0.9),      # three tiles for all pairs: even split, many pairs per tile
     di.small_linear(10007, 200, 520, "bf16", 0.95),    # ... ragged tiles and a ragged last block
     di.small_linear(7000, 520, 776, "bf16", 0.95),     # twelve tiles: pairs cross tile boundaries at uneven places
+    di.small_linear(12000, 800, 2304, "bf16", 0.97),   # 36 tiles, whole ranges only
+    di.small_linear(9300, 776, 2056, "bf16", 0.97),    # 36 ragged tiles
+    di.small_linear(11000, 768, 2304, "bf16", 0.97),   # 27 tiles: two ranges per tile from the same tokens, the rests shared out
+    di.small_linear(7001, 1032, 2000, "bf16", 0.97),   # 40 tiles: one range per tile and the rests
     di.small_linear(700, 768, 768, "bf16", 0.9),       # a few blocks: no split
     di.small_linear(4000, 1536, 384, "bf16", 0.95),    # three ranges per tile with tickets
 ]
