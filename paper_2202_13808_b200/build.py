@@ -47,14 +47,14 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 def _build_native(force: bool):
     """Compile the torch binding against the installed torch's headers and link it to libdropit.so beside it."""
-    header = os.path.join(ROOT, "include", "dropit.h")
-    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) > max(os.path.getmtime(NATIVE_SRC), os.path.getmtime(header)):
+    deps = [NATIVE_SRC, os.path.join(CSRC, "layer_ops.h"), os.path.join(ROOT, "include", "dropit.h")]
+    if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) > max(os.path.getmtime(d) for d in deps):
         return
     import torch
 
     tdir = os.path.dirname(torch.__file__)
     cuda = os.path.join(os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc"))), "include")
-    includes = [os.path.join(ROOT, "include"), os.path.join(tdir, "include"),
+    includes = [os.path.join(ROOT, "include"), CSRC, os.path.join(tdir, "include"),
                 os.path.join(tdir, "include", "torch", "csrc", "api", "include"), cuda, sysconfig.get_path("include")]
     tmp = NATIVE + ".tmp.%d" % os.getpid()
     cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-DTORCH_API_INCLUDE_EXTENSION_H",

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "dropit.h"
+#include "layer_ops.h"
 
 namespace {
 
@@ -186,14 +187,37 @@ struct GeluLinear : public torch::autograd::Function<GeluLinear> {
         const auto saved = ctx->get_saved_variables();
         const Tensor &x2 = saved[0], &weight = saved[1], &values = saved[2];
         const auto cache = ctx->saved_data["cache"].toIntVector();
-        const Tensor dz2 = grads[0].reshape({-1, grads[0].size(-1)});
+        const Tensor dz2 = grads[0].reshape({-1, grads[0].size(-1)}).contiguous();
+        const bool bias = ctx->saved_data["bias"].toBool() && ctx->needs_input_grad(2);
         Tensor dx, dw, db;
-        if (ctx->needs_input_grad(0))                                    // Eq. 3: exact, needs theta only; the activation's cache is x
-            dx = at::gelu_backward(at::matmul(dz2, weight), x2).reshape(ctx->saved_data["shape"].toIntVector());
-        if (ctx->needs_input_grad(1))                                    // Eq. 6
-            dw = weight_grad(dz2.contiguous().to(values.scalar_type()), values, saved[3], saved[4], cache[0], cache[1], cache[2],
-                             (int)cache[3], c10::nullopt, false, c10::nullopt, false).to(weight.scalar_type());
-        if (ctx->saved_data["bias"].toBool() && ctx->needs_input_grad(2)) db = dz2.sum(0);
+        if (ctx->needs_input_grad(0)) {                                  // Eq. 3: exact, needs theta only; the activation's cache is x
+            const Tensor dy = at::matmul(dz2, weight);
+            if (dy.scalar_type() == at::kBFloat16 && x2.scalar_type() == at::kBFloat16 && dy.is_contiguous() &&
+                reinterpret_cast<uintptr_t>(x2.data_ptr()) % 16 == 0) {
+                c10::cuda::CUDAGuard guard(dy.device());
+                dx = at::empty_like(x2);
+                check(dropit::gelu_backward_bf16(ptr(dy), ptr(x2), ptr(dx), x2.numel(), current_stream(dy)), "gelu_backward");
+            } else {
+                dx = at::gelu_backward(dy, x2);
+            }
+            dx = dx.reshape(ctx->saved_data["shape"].toIntVector());
+        }
+        const bool own = weight.scalar_type() == at::kBFloat16 && dz2.scalar_type() == at::kBFloat16 && dz2.size(1) % 8 == 0 &&
+                         dz2.numel() != 0 && reinterpret_cast<uintptr_t>(dz2.data_ptr()) % 16 == 0;
+        if (ctx->needs_input_grad(1)) {                                  // Eq. 6
+            const Tensor full = weight_grad(dz2.to(values.scalar_type()), values, saved[3], saved[4], cache[0], cache[1], cache[2],
+                                            (int)cache[3], c10::nullopt, false, c10::nullopt, false);
+            if (own) {                                                   // rounded to the parameter's type together with the bias gradient
+                c10::cuda::CUDAGuard guard(dz2.device());
+                dw = at::detail::empty_cuda(full.sizes(), at::kBFloat16, full.device(), c10::nullopt);
+                if (bias) db = empty1(dz2.size(1), at::kBFloat16, dz2);
+                check(dropit::finish_linear_backward((const float*)ptr(full), ptr(dw), full.numel(), ptr(dz2), dz2.size(0), dz2.size(1),
+                                                     bias ? ptr(db) : nullptr, current_stream(dz2)), "finish_linear_backward");
+            } else {
+                dw = full.to(weight.scalar_type());
+            }
+        }
+        if (bias && !db.defined()) db = dz2.sum(0);
         return {dx, dw, db, Tensor(), Tensor(), Tensor()};
     }
 };
