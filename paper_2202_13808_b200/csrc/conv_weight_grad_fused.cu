@@ -6,9 +6,10 @@
 //   * inflate the band's piece of R(a-hat) into shared memory: a lane owns two pixels and builds the 16 bytes of their eight
 //     channels from eight mask words (the same for a half-warp), reading the retained values with predicated loads that are
 //     contiguous over the warp, so that 16-byte stores write zeros and values alike,
-//   * transpose the band of dY into shared memory (8 channels x 8 pixels per lane, in registers),
-// while one thread feeds the previous band to tcgen05.mma.  Both operands lie pixel-major: 8 channels (16 bytes) of
-// consecutive pixels of one image row follow one another,
+//   * copy the band of dY into shared memory as it is (cp.async; 8 pixels of a channel are 16 bytes, 8 channels a core matrix),
+// while one thread feeds the previous band to tcgen05.mma.  dY is the K-major operand: core matrix (8-pixel group of the band) *
+// (channels / 8) + channel / 8, without swizzle.  X lies pixel-major: 8 channels (16 bytes) of consecutive pixels of one image
+// row follow one another,
 //   address = row * row_pitch + (channel / 8) * group_pitch + pixel * 16 + (channel % 8) * 2,
 // which is the canonical MN-major layout without swizzle.  In it
 //   * the horizontal tap offset v is a start address 16 * v bytes further on (no shifted copies: with the 128-byte swizzle
@@ -20,14 +21,15 @@
 // Stride 2 keeps the even and the odd padded columns in separate planes.  The reduction is split over the CTAs; every split
 // stores its accumulator as it comes out of tensor memory and a second kernel adds the splits in order.
 //
-// Bound by the producers (some 150 warp instructions per 64 pixels x 8 channels of X) beside MMAs that take most of the shared
-// memory's bandwidth; both lanes' pixels of a pair share one mask lookup, the mask words are requested a task ahead and
-// the loads of a warp's first tasks are under way before it waits for the stage, so that one trip to memory per band is
+// Bound by the producers (some 240 warp instructions per 64 pixels x 8 channels of X, mask lookup included), which wait for the values'
+// trip through L2 at four warps a scheduler; both lanes' pixels of a pair share one mask lookup, the mask words are requested a task ahead and
+// the loads of a warp's first task are under way before it waits for the stage, so that one trip to memory per band is
 // exposed.  The taps of a K step share the dY operand in the collector.  16 producer warps: 20 (80 registers) are up to 8 %
 // slower.  Measured per call at batch 64, gamma 0.8 (graph replay), dense copies of conv_weight_grad_tc.cu (decompression,
-// shifted or gathered copies, GEMM on 64-pixel rows) -> first version of this kernel -> now: 3 x 3 64 -> 64 on 56 x 56
-// 59 -> 50 -> 50 us, 128 -> 128 on 28 x 28 131 -> 46 -> 39, 256 -> 256 on 14 x 14 125 -> 51 -> 45, 512 -> 512 on 7 x 7
-// 334 -> 93 -> 86, stride 2 128 -> 128 on 56 x 56 213 -> 70 -> 59; 1 x 1 of stride 2 256 -> 512 on 56 x 56 292 -> 170 -> 129.
+// shifted or gathered copies, GEMM on 64-pixel rows) -> dY transposed through registers (some 350 instructions per 32 pixels x
+// 64 channels, as much as X) -> now: 3 x 3 64 -> 64 on 56 x 56 59 -> 50 -> 37 us, 128 -> 128 on 28 x 28 131 -> 39 -> 36,
+// 256 -> 256 on 14 x 14 125 -> 45 -> 43, 512 -> 512 on 7 x 7 334 -> 86 -> 81, stride 2 128 -> 128 on 56 x 56 213 -> 59 -> 55;
+// 1 x 1 of stride 2 256 -> 512 on 56 x 56 292 -> 129 -> 117.
 #include <cstring>
 #include <type_traits>
 
@@ -51,7 +53,7 @@ struct FusedConvParams {
     int yb, ni;                                      // output rows per band; images per band (> 1 only for whole images)
     int xb;                                          // flat: pixels per band
     int cores;                                       // 8-pixel groups per output row
-    int gp, gpy;                                     // pixels per channel group and row: X (one plane), dY
+    int gp;                                          // pixels per channel group and row of X (one plane)
     int planes;                                      // column parities kept (1 or 2)
     int row_step, x_rows;                            // X rows per output row; X rows of one image in a band
     int in_step;                                     // input rows per X row
@@ -62,6 +64,8 @@ struct FusedConvParams {
     uint32_t w_magic;                                // pixel / W
     uint32_t cores_magic, yb_magic, step_magic;      // core / cores, row / yb, dY task / dY steps
     int x_bytes, dy_bytes, stages;                   // per pipeline stage
+    int vec;                                         // pixels per copy of dY that the row length allows: 8, 4, 2, 1
+    int dy_warp0, dy_idle, dy_extra;                 // see next_dy: first warp without a task of X in the last round, their number, their share
     int bands, bands_total, bands_per_split, splits; // bands per image (or per group of images); over the batch; per CTA
     int tiles_c, tiles_j;
     int ncols, chunks;                               // accumulator columns R * S * cb; 32-column chunks
@@ -82,14 +86,21 @@ struct FusedConvCtl {
 __host__ __device__ __forceinline__ uint32_t magic_of(uint32_t d) { return (1u << 20) / d + 1u; }
 __host__ __device__ __forceinline__ uint32_t quotient(uint32_t x, uint32_t magic) { return (x * magic) >> 20; }
 
-// Shared-memory matrix descriptor without swizzle, MN-major.  Low word: start address and the distance between the two 8-row
-// groups of a K = 16 step; high word: the distance between groups of eight columns, and the descriptor version.
+// Shared-memory matrix descriptor without swizzle.  Low word: start address and the distance between the two core matrices of a
+// K = 16 step; high word: the distance between groups of eight rows (dY) or columns (X), and the descriptor version.
 __host__ __device__ __forceinline__ uint32_t desc_low(uint32_t addr, uint32_t k_stride) { return (addr >> 4) | ((k_stride >> 4) << 16); }
 __device__ __forceinline__ uint64_t desc_of(uint32_t low, uint32_t high) { return (uint64_t)low | ((uint64_t)high << 32); }
 __device__ __forceinline__ uint32_t desc_high(uint32_t mn_stride) { return (mn_stride >> 4) | (1u << 14); }
 
 __device__ __forceinline__ void sts_zero16(uint32_t addr) {
     asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(addr), "r"(0u) : "memory");
+}
+
+// Asynchronous copy of `bytes` (0 or BYTES) to shared memory, zeros for the rest.
+template <int BYTES>
+__device__ __forceinline__ void cp_async_zfill(uint32_t dst, const uint16_t* src, uint32_t bytes) {
+    if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
 
 // *p if `bit` is not zero, else 0; a predicated load, not a branch.
@@ -123,13 +134,18 @@ __device__ __forceinline__ Place place_of(const FusedConvParams& p, uint32_t ind
     return r;
 }
 
-// VEC: pixels per load of dY that the row length allows (8: rows are whole aligned 16-byte groups; 4; 2; 1: rows that start anywhere)
+// Channels of a task of dY: half as many where its loads would otherwise take the registers that the prefetched values need.
+__host__ __device__ constexpr int dy_task_channels(int vec) { return vec <= 2 ? 32 : 64; }
+
+// VEC: pixels per copy of dY that the row length allows (8: rows are whole aligned 16-byte groups; 4; 2; 1: rows that start anywhere,
+// through registers)
 template <int VEC>
 __global__ void __launch_bounds__(kThreads, 1)
 conv_wg_fused_kernel(const uint16_t* __restrict__ dy, const uint16_t* __restrict__ values, const uint32_t* __restrict__ mask,
                      const uint32_t* __restrict__ offsets, const __grid_constant__ FusedConvParams p, float* __restrict__ partial,
                      int32_t* dev_status, uint32_t wait_limit) {
     extern __shared__ __align__(128) uint8_t csm[];
+    constexpr int kChannels = dy_task_channels(VEC);
     const int warp = __shfl_sync(kFullMask, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp: uniform
     const int stage_bytes = p.x_bytes + p.dy_bytes;
     const uint32_t smem0 = ptx::smem_u32(csm);
@@ -152,7 +168,7 @@ conv_wg_fused_kernel(const uint16_t* __restrict__ dy, const uint16_t* __restrict
         ptx::tmem_alloc(&ctl->tmem_base, p.tmem_cols);
         ptx::tmem_relinquish();
     }
-    const uint32_t row_pitch = (uint32_t)(p.cb / 8) * p.gp * 16, dy_pitch = (uint32_t)(p.mt / 8) * p.gpy * 16;
+    const uint32_t row_pitch = (uint32_t)(p.cb / 8) * p.gp * 16, core_pitch = (uint32_t)p.mt * 16;
     // padding columns, and the rows of dY behind a band's last one, are read but never written: zero
     for (int i = threadIdx.x; i < p.stages * stage_bytes / 16; i += kThreads) sts_zero16(smem0 + i * 16);
     const int total_cores = p.ni * p.yb * p.cores, pairs = (total_cores + 1) / 2;
@@ -169,10 +185,16 @@ conv_wg_fused_kernel(const uint16_t* __restrict__ dy, const uint16_t* __restrict
         const uint32_t nwords = (uint32_t)(((int64_t)p.B * p.Ca * p.H * p.W + 31) / 32);
         const uint32_t plane_elems = (uint32_t)p.H * p.W, plane_pitch = (uint32_t)p.x_bytes / p.planes;
         const int groups = p.cb / 8, x_tasks = (p.slots + 1) / 2;
-        const int dy_steps = (total_cores + 3) / 4, dy_tasks = dy_steps * (p.mt / 64);
+        const int dy_steps = (total_cores + 3) / 4, dy_tasks = dy_steps * (p.mt / kChannels);
         const size_t dy_plane = (size_t)p.Ho * p.Wo;
         [[maybe_unused]] const size_t dy_total = dy_plane * p.Cz * p.B;
-        const int dy_first = (warp + kProdWarps - x_tasks % kProdWarps) % kProdWarps;   // goes on where the X tasks end
+        const int dy_rank = (warp + kProdWarps - p.dy_warp0) % kProdWarps;
+        // the warps without a task of X in the last round take the first dy_extra tasks of dY, all warps share the others
+        const int dy_first = dy_rank < p.dy_idle && p.dy_extra > 0 ? dy_rank : p.dy_extra + dy_rank;
+        auto next_dy = [&](int t) {
+            if (t >= p.dy_extra) return t + kProdWarps;
+            return t + p.dy_idle < p.dy_extra ? t + p.dy_idle : p.dy_extra + dy_rank;
+        };
         const int slot = lane >> 3, sub = lane & 7;
         uint2* meta = ctl->meta[warp];
         uint2* home = ctl->home[warp];
@@ -230,86 +252,91 @@ conv_wg_fused_kernel(const uint16_t* __restrict__ dy, const uint16_t* __restrict
             const bool turn = piece + 1 == p.bands;                        // the next band opens another image
             const int next_n = turn ? n0 + p.ni : n0, next_piece = turn ? 0 : piece + 1;
             const uint32_t xbuf = smem0 + s * stage_bytes, ybuf = xbuf + p.x_bytes;
-            // ---- dY: 8 channels x 8 pixels per lane, transposed in registers.  The eight lanes of a quarter-warp take eight
-            // channel groups (their pitch is 16 bytes modulo 128, so that the stores of a quarter-warp do not collide).  The
-            // loads of the warp's first task are issued before it waits for the stage and works on X.
-            struct DyPlace { int row, xc, jg; bool live; };
+            // ---- dY: a task is four 8-pixel groups of 64 or 32 channels; a lane copies one group of the channels sub, sub + 8, ...
+            struct DyPlace { int core, row, xc, jset; bool live; };
             auto dy_place = [&](int t) {
                 DyPlace r;
-                const int jset = (int)quotient(t, p.step_magic);
-                const int core = (t - jset * dy_steps) * 4 + slot;
-                r.live = core < total_cores;
-                r.jg = jset * 8 + sub;
-                r.row = (int)quotient(core, p.cores_magic);
-                r.xc = core - r.row * p.cores;
+                r.jset = (int)quotient(t, p.step_magic);
+                r.core = (t - r.jset * dy_steps) * 4 + slot;
+                r.live = r.core < total_cores;
+                r.row = (int)quotient(r.core, p.cores_magic);
+                r.xc = r.core - r.row * p.cores;
                 return r;
             };
-            auto load_dy = [&](int t, uint32_t (&w)[8][4]) {
-                const DyPlace at = dy_place(t);
-                const int img = (int)quotient(at.row, p.yb_magic), y = y0 + at.row - img * p.yb;
-                const int x = k0 + at.xc * 8, nv = min(8, p.Wo - x);       // pixels that exist
-                const bool in = at.live && n0 + img < p.B && y < p.Ho && nv > 0;
-                const int j = j0 + at.jg * 8;
-                const uint16_t* src = dy + ((size_t)(n0 + img) * p.Cz + j) * dy_plane + (size_t)y * p.Wo + x;
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    w[e][0] = w[e][1] = w[e][2] = w[e][3] = 0;
-                    if (in && j + e < p.Cz) {
-                        if constexpr (VEC == 8) {
-                            const uint4 v = ld_stream(reinterpret_cast<const uint4*>(src));
-                            w[e][0] = v.x; w[e][1] = v.y; w[e][2] = v.z; w[e][3] = v.w;
-                        } else if constexpr (VEC == 4) {
-                            const uint2 v = __ldg(reinterpret_cast<const uint2*>(src));
-                            w[e][0] = v.x; w[e][1] = v.y;
-                            if (nv > 4) {
-                                const uint2 u = __ldg(reinterpret_cast<const uint2*>(src) + 1);
-                                w[e][2] = u.x; w[e][3] = u.y;
-                            }
-                        } else if constexpr (VEC == 2) {
-#pragma unroll
-                            for (int h = 0; h < 4; ++h)
-                                if (2 * h < nv) w[e][h] = __ldg(reinterpret_cast<const uint32_t*>(src) + h);
-                        } else {
-                            // rows that start anywhere: the aligned words around the piece, shifted by half a word for odd starts
-                            const size_t at0 = (size_t)(src - dy);
-                            const uint32_t odd = (uint32_t)at0 & 1u;
-                            const uint32_t* words = reinterpret_cast<const uint32_t*>(dy) + (at0 >> 1);
-                            uint32_t raw[5];
-#pragma unroll
-                            for (int h = 0; h < 5; ++h) {
-                                raw[h] = 0;
-                                if (2 * h < nv + (int)odd) {     // the tensor's last element may have no right neighbour
-                                    if (((at0 >> 1) + h) * 2 + 1 < dy_total) raw[h] = __ldg(words + h);
-                                    else raw[h] = __ldg(reinterpret_cast<const uint16_t*>(words + h));
-                                }
-                            }
-#pragma unroll
-                            for (int h = 0; h < 4; ++h) {
-                                w[e][h] = odd ? __funnelshift_r(raw[h], raw[h + 1], 16) : raw[h];
-                                if (2 * h + 1 >= nv) w[e][h] &= 2 * h < nv ? 0xFFFFu : 0u;   // pixels of the next row
-                            }
-                        }
-                    }
-                    src += dy_plane;
-                }
+            // the first channel's source and the pixels that exist there (not positive: none); where it goes
+            auto dy_source = [&](const DyPlace& at, int& nv) {
+                const int img = (int)quotient(at.row, p.yb_magic), y = y0 + at.row - img * p.yb, x = k0 + at.xc * 8;
+                nv = n0 + img < p.B && y < p.Ho ? min(8, p.Wo - x) : 0;
+                return dy + ((size_t)(n0 + img) * p.Cz + j0 + at.jset * kChannels + sub) * dy_plane + (size_t)y * p.Wo + x;
             };
-            auto store_dy = [&](int t, const uint32_t (&w)[8][4]) {
+            auto dy_target = [&](const DyPlace& at) { return ybuf + at.core * core_pitch + (at.jset * kChannels + sub) * 16; };
+            [[maybe_unused]] auto copy_dy = [&](int t) {
                 const DyPlace at = dy_place(t);
                 if (!at.live) return;
-                const uint32_t dst = ybuf + at.row * dy_pitch + (at.jg * p.gpy + at.xc * 8) * 16;
+                int nv;
+                const uint16_t* src = dy_source(at, nv);
+                size_t step = 8 * dy_plane;
+                if (nv <= 0) { src = dy; step = 0; }                       // zeros, from a valid address
+                uint32_t dst = dy_target(at);
+                const int left = p.Cz - (j0 + at.jset * kChannels + sub);
 #pragma unroll
-                for (int px = 0; px < 8; ++px) {
-                    uint32_t o[4];
+                for (int g = 0; g < kChannels / 8; ++g) {
+                    if (g * 8 < left) {
 #pragma unroll
-                    for (int h = 0; h < 4; ++h)
-                        o[h] = __byte_perm(w[2 * h][px >> 1], w[2 * h + 1][px >> 1], (px & 1) ? 0x7632 : 0x5410);
-                    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + px * 16), "r"(o[0]), "r"(o[1]), "r"(o[2]),
-                                 "r"(o[3]) : "memory");
+                        for (int h = 0; h < 8; h += VEC) cp_async_zfill<VEC * 2>(dst + h * 2, src + (h < nv ? h : 0), h < nv ? VEC * 2 : 0);
+                    }
+                    dst += 128;
+                    src += step;
                 }
             };
+            // Rows that are not 8-byte aligned (copied 4 bytes at a time, asynchronously, 256 -> 256 on 14 x 14 took 57 us instead of 43) go through registers: the aligned words around the piece, shifted by half a word for odd
+            // starts.  The loads of the warp's first task are issued before it waits for the stage and works on X.
+            [[maybe_unused]] auto load_dy = [&](int t, uint32_t (&w)[kChannels / 8][4]) {
+                const DyPlace at = dy_place(t);
+                int nv;
+                const uint16_t* src = dy_source(at, nv);
+                if (!at.live) nv = 0;
+                const int left = p.Cz - (j0 + at.jset * kChannels + sub);
+#pragma unroll
+                for (int g = 0; g < kChannels / 8; ++g) {
+                    w[g][0] = w[g][1] = w[g][2] = w[g][3] = 0;
+                    if constexpr (VEC == 2) {
+#pragma unroll
+                        for (int h = 0; h < 4; ++h)
+                            if (2 * h < nv && g * 8 < left) w[g][h] = __ldg(reinterpret_cast<const uint32_t*>(src) + h);
+                    } else if (nv > 0 && g * 8 < left) {
+                        const size_t at0 = (size_t)(src - dy);
+                        const uint32_t odd = (uint32_t)at0 & 1u;
+                        const uint32_t* words = reinterpret_cast<const uint32_t*>(dy) + (at0 >> 1);
+                        uint32_t raw[5];
+#pragma unroll
+                        for (int h = 0; h < 5; ++h) {
+                            raw[h] = 0;
+                            if (2 * h < nv + (int)odd) {     // the tensor's last element may have no right neighbour
+                                if (((at0 >> 1) + h) * 2 + 1 < dy_total) raw[h] = __ldg(words + h);
+                                else raw[h] = __ldg(reinterpret_cast<const uint16_t*>(words + h));
+                            }
+                        }
+#pragma unroll
+                        for (int h = 0; h < 4; ++h) {
+                            w[g][h] = odd ? __funnelshift_r(raw[h], raw[h + 1], 16) : raw[h];
+                            if (2 * h + 1 >= nv) w[g][h] &= 2 * h < nv ? 0xFFFFu : 0u;   // pixels of the next row
+                        }
+                    }
+                    src += 8 * dy_plane;
+                }
+            };
+            [[maybe_unused]] auto store_dy = [&](int t, const uint32_t (&w)[kChannels / 8][4]) {
+                const DyPlace at = dy_place(t);
+                if (!at.live) return;
+                const uint32_t dst = dy_target(at);
+#pragma unroll
+                for (int g = 0; g < kChannels / 8; ++g)
+                    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + g * 128), "r"(w[g][0]), "r"(w[g][1]), "r"(w[g][2]),
+                                 "r"(w[g][3]) : "memory");
+            };
             // The retained values of a task are loaded into registers (a slot at a time: the lane gets the 8 channels of its two
-            // pixels), then stored; for the warp's first task of the band, and for its first dY task, the loads are on their
-            // way before it waits for the stage.
+            // pixels), then stored; for the warp's first task of the band the loads are on their way before it waits for the stage.
             uint4 x4[4];
             auto load_x = [&](int t) {
                 meta[lane] = record(ahead);
@@ -363,24 +390,30 @@ conv_wg_fused_kernel(const uint16_t* __restrict__ dy, const uint16_t* __restrict
                 }
                 __syncwarp();                            // the records may be overwritten
             };
-            uint32_t w[8][4];
+            [[maybe_unused]] uint32_t w[kChannels / 8][4];
             if (warp < x_tasks) load_x(warp);
-            if (dy_first < dy_tasks) load_dy(dy_first, w);
+            if constexpr (VEC <= 2)
+                if (dy_first < dy_tasks) load_dy(dy_first, w);
             if (i >= p.stages) {
                 const bool ok = ptx::mbar_wait_warp(&ctl->empty[s], ((i / p.stages) - 1) & 1, wait_limit);
                 if (!ok) *abort_flag = 1;
             }
             if (__any_sync(kFullMask, *abort_flag != 0)) break;
+            if constexpr (VEC > 2)
+                for (int t = dy_first; t < dy_tasks; t = next_dy(t)) copy_dy(t);
             if (warp < x_tasks) store_x();
             for (int t = warp + kProdWarps; t < x_tasks; t += kProdWarps) {
                 load_x(t);
                 store_x();
             }
-            for (int t = dy_first; t < dy_tasks; t += kProdWarps) {
-                if (t != dy_first) load_dy(t, w);
-                store_dy(t, w);
+            if constexpr (VEC > 2) {
+                asm volatile("cp.async.wait_all;" ::: "memory");
+            } else {
+                for (int t = dy_first; t < dy_tasks; t = next_dy(t)) {
+                    if (t != dy_first) load_dy(t, w);
+                    store_dy(t, w);
+                }
             }
-
             ptx::fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive(&ctl->full[s]);
@@ -413,8 +446,8 @@ conv_wg_fused_kernel(const uint16_t* __restrict__ dy, const uint16_t* __restrict
         // ---------------- MMA issuer (the whole warp runs the loop, one thread issues) ----------------
         const uint32_t leader = ptx::elect_one();
         const uint32_t n_inst = (uint32_t)(p.R * p.cb);
-        const uint32_t idesc = ptx::make_idesc_bf16(kBM, (int)n_inst, true, true);
-        const uint32_t high_a = desc_high(p.gpy * 16), high_b = desc_high(p.gp * 16);
+        const uint32_t idesc = ptx::make_idesc_bf16(kBM, (int)n_inst, false, true);
+        const uint32_t high_a = desc_high(128), high_b = desc_high(p.gp * 16);
         const uint32_t plane_pitch = (uint32_t)p.x_bytes / p.planes;
         // where a horizontal tap's columns start, in descriptor units
         const uint32_t shift1 = (p.stride == 2 ? plane_pitch : 16u) >> 4, shift2 = (p.stride == 2 ? 16u : 32u) >> 4;
@@ -515,13 +548,13 @@ conv_fused_reduce_kernel(const float4* __restrict__ partial, const FusedConvPara
 }
 
 size_t stage_bytes_of(FusedConvParams& p) {
-    const size_t row_pitch = (size_t)(p.cb / 8) * p.gp * 16, dy_pitch = (size_t)(p.mt / 8) * p.gpy * 16;
+    const size_t row_pitch = (size_t)(p.cb / 8) * p.gp * 16;
     // With an odd number of 8-pixel groups the last K = 16 step reads one more K row than the band has: zeros in dY,
-    // anything finite in X.  With 64 rows of dY per band the instruction's rows 64..127 are the next image row (their
-    // results are not used).
+    // anything finite in X.  With 64 channels of dY per band the instruction's rows 64..127 are the next 8-pixel group
+    // (their results are not used).
     const int odd = (p.ni * p.yb * p.cores) & 1;
     const size_t x = (size_t)(p.ni * p.x_rows + odd * p.row_step) * row_pitch * p.planes;
-    const size_t y = (size_t)(p.ni * p.yb + odd + (p.mt == 64 ? 1 : 0)) * dy_pitch;
+    const size_t y = (size_t)(p.ni * p.yb * p.cores + odd + (p.mt == 64 ? 1 : 0)) * p.mt * 16;
     p.x_bytes = (int)align_up(x, 128 * p.planes);
     p.dy_bytes = (int)align_up(y, 128);
     return (size_t)p.x_bytes + p.dy_bytes;
@@ -546,11 +579,14 @@ bool make_fused_conv_plan(FusedConvParams& p, int B, int Ca, int H, int W, int C
     p.tiles_c = (Ca + p.cb - 1) / p.cb;
     p.tiles_j = (Cz + kBM - 1) / kBM;
     p.stages = 2;
+    p.vec = p.Wo % 8 == 0 ? 8 : (p.Wo % 4 == 0 ? 4 : (p.Wo % 2 == 0 ? 2 : 1));
+    // What a task of dY costs, in tasks of X; fitted: with half of it or twice as much the bands chosen are up to a quarter slower
+    // where rows are odd, and 5 to 10 % where they are even.
+    const float dy_cost = p.vec >= 4 ? 0.2f : (p.vec == 2 ? 0.3f : 0.6f);
     const int64_t tiles = (int64_t)p.tiles_c * p.tiles_j;
     if (tiles > 65535) return false;
     if (!p.flat) {
         p.cores = (p.Wo + 7) / 8;
-        p.gpy = p.cores * 8 + 1;
         // columns an 8-pixel group of any tap can reach, at the plane's resolution
         const int reach = p.cores * 8 + (S - 1) / stride + 1, padded = ((W + 7) / 8 * 8 + pad + stride - 1) / stride + 1;
         p.gp = reach > padded ? reach : padded;
@@ -563,7 +599,7 @@ bool make_fused_conv_plan(FusedConvParams& p, int B, int Ca, int H, int W, int C
         if (p.flat) {
             p.xb = (int)align_up((size_t)(p.W + pieces - 1) / pieces, pieces > 1 ? 32 : 16);
             p.cores = p.xb / 8;
-            p.gp = p.gpy = p.xb + 1;
+            p.gp = p.xb + 1;
             p.yb = 1;
             p.bands = (p.W + p.xb - 1) / p.xb;
         } else {
@@ -582,8 +618,12 @@ bool make_fused_conv_plan(FusedConvParams& p, int B, int Ca, int H, int W, int C
         if (splits > p.bands_total) splits = p.bands_total;
         p.bands_per_split = (p.bands_total + splits - 1) / splits;
         p.splits = (p.bands_total + p.bands_per_split - 1) / p.bands_per_split;
-        const int tasks = (p.slots + 1) / 2 + (p.ni * p.yb * p.cores + 3) / 4 * (p.mt / 64);
-        return p.bands_per_split * (0.5f + (float)((tasks + kProdWarps - 1) / kProdWarps));
+        const int x_tasks = (p.slots + 1) / 2, dy_tasks = (p.ni * p.yb * p.cores + 3) / 4 * (p.mt / dy_task_channels(p.vec));
+        p.dy_warp0 = x_tasks % kProdWarps;
+        p.dy_idle = p.dy_warp0 ? kProdWarps - p.dy_warp0 : 0;
+        p.dy_extra = p.dy_idle * (int)(1.f / dy_cost);
+        const int shared = dy_tasks > p.dy_extra ? dy_tasks - p.dy_extra : 0;
+        return p.bands_per_split * (0.5f + (float)((x_tasks + kProdWarps - 1) / kProdWarps) + (float)((shared + kProdWarps - 1) / kProdWarps) * dy_cost);
     };
     int best_pieces = 0, best_ni = 0;
     float best = 0.f;
@@ -617,14 +657,14 @@ bool make_fused_conv_plan(FusedConvParams& p, int B, int Ca, int H, int W, int C
     while ((int)p.tmem_cols < p.chunks * 32) p.tmem_cols *= 2;
     if (p.tmem_cols > 512) return false;
     {
-        const uint32_t row_pitch = (uint32_t)(p.cb / 8) * p.gp * 16, dy_pitch = (uint32_t)(p.mt / 8) * p.gpy * 16;
+        const uint32_t row_pitch = (uint32_t)(p.cb / 8) * p.gp * 16, core_pitch = (uint32_t)p.mt * 16;
         for (int i = 0; i < (cores_total + 1) / 2; ++i) {
             uint32_t a[2], b[2];
             for (int h = 0; h < 2; ++h) {
                 const int core = 2 * i + h, row = core / p.cores, xc = core % p.cores;
                 // the group behind the last row counts as a row of the last image
                 const int img = row / p.yb < p.ni ? row / p.yb : p.ni - 1, y = row - img * p.yb;
-                a[h] = p.x_bytes + row * dy_pitch + xc * 128;
+                a[h] = p.x_bytes + core * core_pitch;
                 b[h] = (img * p.x_rows + y * p.row_step) * row_pitch + xc * 128;
             }
             p.pairs[i] = make_uint2(desc_low(a[0], a[1] - a[0]), desc_low(b[0], b[1] - b[0]));
@@ -670,7 +710,7 @@ dropit_status conv_fused_run(const void* dy, const void* values, const void* mas
     if (!cached_fused_conv_plan(p, B, Ca, H, W, Cz, R, S, stride, pad, k)) return DROPIT_ERR_UNSUPPORTED;
     const int tiles = p.tiles_c * p.tiles_j;
     if (workspace_bytes < (size_t)p.splits * tiles * p.chunks * 32 * kBM * 4) return DROPIT_ERR_WORKSPACE;
-    const int vec = p.Wo % 8 == 0 ? 3 : (p.Wo % 4 == 0 ? 2 : (p.Wo % 2 == 0 ? 1 : 0));
+    const int vec = p.vec == 8 ? 3 : p.vec / 2;
     auto kern = vec == 3 ? conv_wg_fused_kernel<8> : (vec == 2 ? conv_wg_fused_kernel<4> : (vec == 1 ? conv_wg_fused_kernel<2> : conv_wg_fused_kernel<1>));
     static PerDeviceOnce attr[4];
     PerDeviceOnce& once = attr[vec];
