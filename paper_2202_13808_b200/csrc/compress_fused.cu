@@ -4,7 +4,7 @@
 // Every WARP owns one contiguous run of 1024-element super-blocks (two 512-element blocks) and keeps it for the
 // whole kernel, so
 // the ordered compaction needs no block-wide synchronisation and warps drift freely.
-//   sample  every CTA histograms the same 16 Ki-element jittered sample in shared memory and brackets
+//   sample  every CTA histograms the same 8 Ki-element jittered sample in shared memory and brackets
 //           the threshold key T between two keys [lo, hi] (6-sigma margin on the sample rank).
 //   phase 1 one read of the tensor: keys above hi are counted in a register, keys inside the band
 //           go to a small per-warp histogram, the rest is ignored (two packed bf16 per 32-bit word
@@ -18,11 +18,14 @@
 //           gt_before + min(eq_before, q).  The quota ends inside one warp's run; in all others one threshold decides.
 //           A lane owns 32 consecutive elements of a super-block; retained values are staged per warp and leave in
 //           aligned 16-byte pieces.
-// Bound by issue in both streaming phases (some 250 warp instructions per super-block each) on top of 11 us of fixed steps
-// (sample 5.5, barrier 2, phase 2 2.5).  What the one threshold, the flags gathered by a prmt with msb replication, the
+// Bound by issue in both streaming phases (some 250 warp instructions per super-block each) on top of 10 us of fixed steps
+// (sample 4.5, barrier 2, phase 2 2.5).  What the one threshold, the flags gathered by a prmt with msb replication, the
 // walk of dense words from registers and the rarer flushes gave, per call over rotating inputs (graph replay, gamma 0.9):
 // 12608 x 768 20.7 -> 19.3 us, 12608 x 3072 42.3 -> 39.1; 32768 x 768 at 0.5 48.3 -> 40.9; 32768 x 3072 at 0.8 96 -> 89,
-// at 0.5 134 -> 112 us (3.7 TB/s of the two reads and the outputs).
+// at 0.5 134 -> 112 us.  The sample's additions to shared memory take turns at the bank: half as many of them (8 Ki elements
+// instead of 16 Ki; the band, 1.4 times as wide, has 96 bins instead of 64) and none for zeros, which behind a ReLU are half of
+// them: 19.4 -> 18.3, 38.9 -> 38.3, 41.4 -> 39.2, 91 -> 88, 113 -> 109 us (3.8 TB/s of the two reads and the outputs); behind a
+// ReLU 64 x 256 x 56 x 56 57.5 -> 51.8, 64 x 64 x 56 x 56 26.9 -> 22.2 us.
 // When the band is wider than the per-warp histogram (small tensors, which are not sampled; key
 // distributions that are flat around T; a sample that missed) a general path is taken instead:
 // full CTA histogram in shared memory, global histogram by atomics, then one extra counting read.
@@ -42,10 +45,10 @@ constexpr int kBlkVecs = 32 * kVpl;                            // vectors per wa
 constexpr int kBlkElems = kBlkVecs * 8;                        // 512 bf16
 constexpr int kP1Blocks = 4 / kVpl;                            // blocks loaded per phase-1 iteration (4 loads per lane)
 constexpr int kKeySpace = 1 << 15;
-constexpr int kWarpBins = 64;                                  // per-warp band histogram
+constexpr int kWarpBins = 96;                                  // per-warp band histogram
 constexpr int kRowWords = kWarpBins + 2;                       // per-CTA row: bins, #key>hi, pad
 constexpr int kMaxGrid = 512;                                  // < 4096: departures are counted in 12 bits of the barrier word
-constexpr int kSampleVecs = 2048;                              // 16384 sampled elements
+constexpr int kSampleVecs = 1024;                              // 8192 sampled elements
 constexpr int64_t kSampleMinElems = kSmallMaxElems;            // below this the band is the full key range (the call normally goes to compress_small.cu)
 constexpr int kBarrierSpinLimit = 1 << 22;
 constexpr uint32_t kHiBits = 0x80008000u;
@@ -62,7 +65,8 @@ constexpr size_t kRingBytes = (size_t)kFusedWarps * kRingSlots * kSbBytes;   // 
 constexpr int kStageKeep = 264;
 constexpr int kStageVals = kSbElems + kStageKeep + 8;
 constexpr size_t kStageBytes = (size_t)kFusedWarps * kStageVals * 2;   // 81 KB
-static_assert(kStageBytes >= (size_t)kKeySpace * 2, "the sample's 16-bit histogram lives in the staging area");
+constexpr size_t kSampleBytes = (size_t)kKeySpace * 2;         // 16-bit key histogram of the sample
+static_assert(kStageBytes >= kSampleBytes, "the sample's 16-bit histogram lives in the staging area");
 
 struct FusedState {
     unsigned long long barrier;  // grid barrier: call epoch << 32 | arrivals (needs no clearing between calls)
@@ -230,7 +234,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* s
 }
 
 // ---------------------------------------------------------------------------------------------
-// Sample step: bracket the threshold key.  Every CTA runs it on the same 16 Ki elements (the first
+// Sample step: bracket the threshold key.  Every CTA runs it on the same 8 Ki elements (the first
 // CTA to ask brings them in from HBM, the others read them from L2) and therefore arrives at the
 // same band without any exchange.  `bins`: kKeySpace counters in shared memory; band[0..1] = lo, hi.
 // Ends with a block-wide barrier.
@@ -260,17 +264,23 @@ __device__ __forceinline__ void sample_band(const uint4* __restrict__ x, int64_t
         band[1] = kKeySpace - 1;
     }
     if (sampled) {
-        // two 16-bit counters per word (a counter holds at most the sample size, 16384)
+        // two 16-bit counters per word (a counter holds at most the sample size, 8192)
         uint4* z = reinterpret_cast<uint4*>(bins);
         for (int i = threadIdx.x; i < kKeySpace / 8; i += kFusedThreads) z[i] = make_uint4(0, 0, 0, 0);
         __syncthreads();
+        uint32_t zeros = 0;     // behind a ReLU they are half of the sample, and additions to one word take turns
 #pragma unroll
         for (int r = 0; r < kSampleVecs / kFusedThreads; ++r) {
             uint32_t key[8];
             keys_of(map(sv[r]), key);
 #pragma unroll
-            for (int e = 0; e < 8; ++e) atomicAdd(&bins[key[e] >> 1], 1u << ((key[e] & 1u) * 16));
+            for (int e = 0; e < 8; ++e) {
+                if (key[e] != 0) atomicAdd(&bins[key[e] >> 1], 1u << ((key[e] & 1u) * 16));
+                else ++zeros;
+            }
         }
+        zeros = __reduce_add_sync(kFullMask, zeros);
+        if ((threadIdx.x & 31) == 0 && zeros) atomicAdd(&bins[0], zeros);
         __syncthreads();
         // ranks (counted from the largest key) that bracket the threshold with a 6-sigma margin
         const float S = (float)(kSampleVecs * 8);
@@ -328,7 +338,6 @@ __device__ __forceinline__ void sample_band(const uint4* __restrict__ x, int64_t
 struct FusedShared {
     uint32_t warp[32];
     unsigned long long red64[32];
-    uint32_t whist[kFusedWarps][kWarpBins];   // per-warp band histograms (fast path)
     uint32_t w_hi[kFusedWarps];               // per-warp #{key > hi}
     uint32_t tot[kRowWords];                  // band histogram over all CTAs (+ #key>hi)
     uint32_t pre[kRowWords];                  // ... over the CTAs before this one
@@ -497,13 +506,14 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                       uint16_t* __restrict__ values, uint32_t* __restrict__ mask, int32_t* __restrict__ indices,
                       uint32_t* __restrict__ offsets, int32_t* dev_status, int spin_max, const unsigned char* prep) {
     // shared memory: [input ring, 128 KB | general path: full key histogram]
-    //                [phase 3: per-warp value staging, 81 KB | sample step: 16-bit key histogram]
+    //                [phase 3: per-warp value staging, 81 KB | sample step: 16-bit key histogram | phases 1-2: band histograms]
     //                [control block of phases 1-2]
     extern __shared__ __align__(16) unsigned char fsm[];
     uint32_t* bins = reinterpret_cast<uint32_t*>(fsm);
     uint32_t* sample_bins = reinterpret_cast<uint32_t*>(fsm + kRingBytes);
     uint16_t* s_vals_all = reinterpret_cast<uint16_t*>(fsm + kRingBytes);   // phase 3: per-warp staging
     FusedShared& sh = *reinterpret_cast<FusedShared*>(fsm + kRingBytes + kStageBytes);
+    uint32_t (*whist)[kWarpBins] = reinterpret_cast<uint32_t (*)[kWarpBins]>(fsm + kRingBytes);   // per-warp band histograms (fast path)
 
     FusedState* st = reinterpret_cast<FusedState*>(ws);
     unsigned long long* agg = reinterpret_cast<unsigned long long*>(ws + agg_off);
@@ -549,7 +559,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
         }
         const uint32_t* wh = prep_warp_hist(prep, ph->grid) + (size_t)blockIdx.x * kFusedWarps * kPrepWarpWords;
         for (int i = threadIdx.x; i < kFusedWarps * kWarpBins; i += blockDim.x)
-            (&sh.whist[0][0])[i] = wh[(i / kWarpBins) * kPrepWarpWords + (i % kWarpBins)];
+            (&whist[0][0])[i] = wh[(i / kWarpBins) * kPrepWarpWords + (i % kWarpBins)];
         if (threadIdx.x < kFusedWarps) sh.w_hi[threadIdx.x] = wh[threadIdx.x * kPrepWarpWords + kWarpBins];
         rows = const_cast<uint32_t*>(prep_rows(prep));
         __syncthreads();
@@ -575,7 +585,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
         if (!(prepared && attempt == 0)) {
             // ---------------- phase 1: band histogram ----------------
             if (narrow) {
-                for (int i = threadIdx.x; i < kFusedWarps * kWarpBins; i += blockDim.x) (&sh.whist[0][0])[i] = 0;
+                for (int i = threadIdx.x; i < kFusedWarps * kWarpBins; i += blockDim.x) (&whist[0][0])[i] = 0;
             } else {
                 if (prefetched) {   // the histogram takes the ring's memory: let the requested blocks land first
                     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -584,7 +594,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                 for (uint32_t i = threadIdx.x; i <= width; i += blockDim.x) bins[i] = 0;
             }
             __syncthreads();
-            uint32_t* hist = narrow ? sh.whist[warp] : bins;
+            uint32_t* hist = narrow ? whist[warp] : bins;
             const uint32_t c_hi = ge_const(hi + 1), c_lo = ge_const(lo);
             uint32_t cnt_hi = 0, cnt_lo = 0;   // keys above the band / keys equal to lo
             auto count_vec = [&](const uint4& v, int nvalid) {
@@ -730,7 +740,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                 if (threadIdx.x < kRowWords) {
                     uint32_t v = 0;
                     if (threadIdx.x < kWarpBins) {
-                        for (int w = 0; w < kFusedWarps; ++w) v += sh.whist[w][threadIdx.x];
+                        for (int w = 0; w < kFusedWarps; ++w) v += whist[w][threadIdx.x];
                     } else if (threadIdx.x == kWarpBins) {
                         v = cta_hi;
                     }
@@ -768,24 +778,24 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
             }
             __syncthreads();
             {
-                // thread (g, c) adds column c of rows g, g + kGroups, ...: consecutive threads read consecutive
+                // thread (g, c) adds column c of rows g, g + groups, ...: consecutive threads read consecutive
                 // words of a row, and a thread's loads are independent of one another
-                constexpr int kGroups = kFusedThreads / kRowWords;
-                constexpr int kInFlight = 10;
+                constexpr uint32_t groups = kFusedThreads / kRowWords;
+                constexpr int kInFlight = 15;
                 const uint32_t g = threadIdx.x / kRowWords, c = threadIdx.x - g * kRowWords;
-                if (g < (uint32_t)kGroups && (c <= width || c == (uint32_t)kWarpBins)) {
+                if (g < groups && (c <= width || c == (uint32_t)kWarpBins)) {
                     uint32_t t_sum = 0, p_sum = 0;
-                    for (uint32_t r0 = g; r0 < gridDim.x; r0 += kInFlight * kGroups) {
+                    for (uint32_t r0 = g; r0 < gridDim.x; r0 += kInFlight * groups) {
                         uint32_t val[kInFlight];
 #pragma unroll
                         for (int u = 0; u < kInFlight; ++u) {
-                            const uint32_t r = r0 + u * kGroups;
+                            const uint32_t r = r0 + u * groups;
                             val[u] = (r < gridDim.x) ? __ldcg(&rows[(size_t)r * kRowWords + c]) : 0u;
                         }
 #pragma unroll
                         for (int u = 0; u < kInFlight; ++u) {
                             t_sum += val[u];
-                            if (r0 + u * kGroups < blockIdx.x) p_sum += val[u];
+                            if (r0 + u * groups < blockIdx.x) p_sum += val[u];
                         }
                     }
                     if (t_sum) atomicAdd(&sh.tot[c], t_sum);
@@ -794,11 +804,12 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
             }
             __syncthreads();
             if (warp == 0) {
-                // bins in descending key order, two per lane: the bin that takes the running count past k is T
+                // bins in descending key order: the bin that takes the running count past k is T
                 const unsigned long long above = sh.tot[kWarpBins];   // keys above the band
-                uint32_t h[2], inc[2];
+                constexpr int kPerLane = kWarpBins / 32;
+                uint32_t h[kPerLane], inc[kPerLane];
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
+                for (int j = 0; j < kPerLane; ++j) {
                     const uint32_t pos = j * 32 + lane;
                     h[j] = (pos <= width) ? sh.tot[width - pos] : 0u;
                     inc[j] = h[j];
@@ -808,9 +819,10 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                         if (lane >= o) inc[j] += y;
                     }
                 }
-                inc[1] += __shfl_sync(kFullMask, inc[0], 31);
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
+                for (int j = 1; j < kPerLane; ++j) inc[j] += __shfl_sync(kFullMask, inc[j - 1], 31);
+#pragma unroll
+                for (int j = 0; j < kPerLane; ++j) {
                     const uint32_t pos = j * 32 + lane;
                     const unsigned long long cum = above + (inc[j] - h[j]);
                     if (pos <= width && cum < k && k <= cum + h[j]) {
@@ -830,7 +842,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                 // this warp's (#key > T, #key == T) and the same over the CTAs before this one
                 uint32_t g = 0, pg = 0;
                 for (uint32_t d = dT + 1 + lane; d <= width; d += 32) {
-                    g += sh.whist[warp][d];
+                    g += whist[warp][d];
                     pg += sh.pre[d];
                 }
                 for (int o = 16; o > 0; o >>= 1) {
@@ -839,7 +851,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                 }
                 if (lane == 0) {
                     sh.wpre_gt[warp] = g + sh.w_hi[warp];
-                    sh.wpre_eq[warp] = sh.whist[warp][dT];
+                    sh.wpre_eq[warp] = whist[warp][dT];
                 }
                 __syncthreads();
                 // exclusive scan over the CTA's warps (lane = warp index), done by every warp for itself
@@ -1299,8 +1311,9 @@ produce_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, int64_t n, un
                const uint16_t* __restrict__ table, unsigned char* prep) {
     extern __shared__ __align__(16) unsigned char fsm[];
     uint32_t* sample_bins = reinterpret_cast<uint32_t*>(fsm + kRingBytes);
-    FusedShared& sh = *reinterpret_cast<FusedShared*>(fsm + kRingBytes + kStageBytes);
-    const uint32_t lut_addr = ptx_smem(fsm + kRingBytes + kStageBytes + ((sizeof(FusedShared) + 15) / 16) * 16);
+    FusedShared& sh = *reinterpret_cast<FusedShared*>(fsm + kRingBytes + kSampleBytes);
+    uint32_t (*whist)[kWarpBins] = reinterpret_cast<uint32_t (*)[kWarpBins]>(fsm + kRingBytes);
+    const uint32_t lut_addr = ptx_smem(fsm + kRingBytes + kSampleBytes + ((sizeof(FusedShared) + 15) / 16) * 16);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t ring_warp = ptx_smem(fsm) + warp * (kRingSlots * kSbBytes);
     const uint32_t ring_copy = ring_warp + lane * 16;
@@ -1314,7 +1327,7 @@ produce_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, int64_t n, un
     const int64_t sb0 = blk0 / 2, sb1 = (blk1 + 1) / 2;
     const int64_t sb_full_end = (nvec_full / kSbVecs < sb1) ? nvec_full / kSbVecs : sb1;
     if constexpr (ACT == kActTable) {
-        uint16_t* lut = reinterpret_cast<uint16_t*>(fsm + kRingBytes + kStageBytes + ((sizeof(FusedShared) + 15) / 16) * 16);
+        uint16_t* lut = reinterpret_cast<uint16_t*>(fsm + kRingBytes + kSampleBytes + ((sizeof(FusedShared) + 15) / 16) * 16);
         for (uint32_t i = threadIdx.x; i < 2 * kLutSpan; i += blockDim.x)
             lut[i] = table[(i >= kLutSpan ? 0x8000u : 0u) | (kLutKeyLo + (i >= kLutSpan ? i - kLutSpan : i))];
         __syncthreads();
@@ -1329,9 +1342,9 @@ produce_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, int64_t n, un
     const uint32_t lo = sh.band[0], hi = sh.band[1];
     const uint32_t width = hi - lo;
     const bool stats = n >= kSampleMinElems && width < (uint32_t)kWarpBins;   // uniform over the grid
-    for (int i = threadIdx.x; i < kFusedWarps * kWarpBins; i += blockDim.x) (&sh.whist[0][0])[i] = 0;
+    for (int i = threadIdx.x; i < kFusedWarps * kWarpBins; i += blockDim.x) (&whist[0][0])[i] = 0;
     __syncthreads();
-    uint32_t* hist = sh.whist[warp];
+    uint32_t* hist = whist[warp];
     const uint32_t c_hi = ge_const(hi + 1), c_lo = ge_const(lo);
     uint32_t cnt_hi = 0, cnt_lo = 0;
     // ---- whole super-blocks through the ring ----
@@ -1432,12 +1445,12 @@ produce_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, int64_t n, un
     uint32_t* wh = const_cast<uint32_t*>(prep_warp_hist(prep, gridDim.x)) + (size_t)blockIdx.x * kFusedWarps * kPrepWarpWords;
     for (int i = threadIdx.x; i < kFusedWarps * kPrepWarpWords; i += blockDim.x) {
         const int w = i / kPrepWarpWords, c = i % kPrepWarpWords;
-        wh[i] = c < kWarpBins ? sh.whist[w][c] : (c == kWarpBins ? sh.w_hi[w] : 0u);
+        wh[i] = c < kWarpBins ? whist[w][c] : (c == kWarpBins ? sh.w_hi[w] : 0u);
     }
     if (threadIdx.x < kRowWords) {
         uint32_t v = 0;
         if (threadIdx.x < kWarpBins) {
-            for (int w = 0; w < kFusedWarps; ++w) v += sh.whist[w][threadIdx.x];
+            for (int w = 0; w < kFusedWarps; ++w) v += whist[w][threadIdx.x];
         } else if (threadIdx.x == kWarpBins) {
             for (int w = 0; w < kFusedWarps; ++w) v += sh.w_hi[w];
         }
@@ -1449,7 +1462,7 @@ template <int ACT>
 static dropit_status launch_produce(const void* x, void* y, int64_t n, int64_t k, const uint16_t* table, unsigned char* prep,
                                     cudaStream_t stream) {
     const FusedPlan plan = make_fused_plan(n);
-    const size_t smem = kRingBytes + kStageBytes + ((sizeof(FusedShared) + 15) / 16) * 16 + kLutBytes;
+    const size_t smem = kRingBytes + kSampleBytes + ((sizeof(FusedShared) + 15) / 16) * 16 + kLutBytes;
     static PerDeviceOnce attr;
     if (attr.needed()) {
         if (cudaFuncSetAttribute(produce_kernel<ACT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
