@@ -21,13 +21,13 @@
 // Stride 2 keeps the even and the odd padded columns in separate planes.  The reduction is split over the CTAs; every split
 // stores its accumulator as it comes out of tensor memory and a second kernel adds the splits in order.
 //
-// Bound by the producers (some 240 warp instructions per 64 pixels x 8 channels of X, mask lookup included), which wait for the values'
-// trip through L2 at four warps a scheduler; both lanes' pixels of a pair share one mask lookup, the mask words are requested a task ahead and
+// Bound by the producers (some 400 warp instructions per 64 pixels x 8 channels of X, everything included; 13.7 M for 64 -> 64 on
+// 56 x 56), which wait for the values' trip through L2 and for shared memory at four warps a scheduler (issue slots 40 % busy); both lanes' pixels of a pair share one mask lookup, the mask words are requested a task ahead and
 // the loads of a warp's first task are under way before it waits for the stage, so that one trip to memory per band is
 // exposed.  The taps of a K step share the dY operand in the collector.  16 producer warps: 20 (80 registers) are up to 8 %
 // slower.  Measured per call at batch 64, gamma 0.8 (graph replay), dense copies of conv_weight_grad_tc.cu (decompression,
-// shifted or gathered copies, GEMM on 64-pixel rows) -> dY transposed through registers (some 350 instructions per 32 pixels x
-// 64 channels, as much as X) -> now: 3 x 3 64 -> 64 on 56 x 56 59 -> 50 -> 37 us, 128 -> 128 on 28 x 28 131 -> 39 -> 36,
+// shifted or gathered copies, GEMM on 64-pixel rows) -> dY transposed through registers (15.6 M instructions, and
+// its loads not in flight during the work on X) -> now: 3 x 3 64 -> 64 on 56 x 56 59 -> 50 -> 37 us, 128 -> 128 on 28 x 28 131 -> 39 -> 36,
 // 256 -> 256 on 14 x 14 125 -> 45 -> 43, 512 -> 512 on 7 x 7 334 -> 86 -> 81, stride 2 128 -> 128 on 56 x 56 213 -> 59 -> 55;
 // 1 x 1 of stride 2 256 -> 512 on 56 x 56 292 -> 129 -> 117.
 #include <cstring>
