@@ -78,7 +78,7 @@ __device__ __forceinline__ void red_shared_if(uint32_t addr, uint32_t v, bool on
 // One digit round: sh.row[0 .. nb) holds this CTA's counts.  Finds the digit in which the descending running count
 // over the cluster reaches k_rem, subtracts from k_rem the keys above it and brings run_gt / run_eq (keys above / at the
 // digits fixed so far, in the CTAs in front of this one) up to date.
-// `rows`: this round's gather buffer, [CTA][kRowBins] (two alternate: a CTA that is ahead by one round writes the other one).
+// `rows`: gather buffer of the current digit round, [CTA][kRowBins] (two alternate: a CTA that is ahead by one round writes the other one).
 __device__ __forceinline__ uint32_t digit_round(SmallShared& sh, const uint32_t* rows, int nb, uint32_t rank, uint32_t ctas,
                                                 uint32_t& k_rem, uint32_t& run_gt, uint32_t& run_eq, bool first) {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
