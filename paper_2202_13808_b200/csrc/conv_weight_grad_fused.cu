@@ -495,11 +495,71 @@ conv_wg_fused_kernel(const uint16_t* __restrict__ dy, const uint16_t* __restrict
     if (*abort_flag && threadIdx.x == 0 && dev_status) atomicExch(dev_status, (int)DROPIT_ERR_TIMEOUT);
 }
 
-// dw[j,c,u,v] (=|+=) sum over splits, in split order within a warp's share and then over the warps.  A block takes 32 rows of
-// one 4-column group; its eight warps share out the splits.
+// Number of retained elements in front of flat index e; `kept`: whether e is one of them.
+__device__ __forceinline__ uint32_t retained_before(const uint32_t* __restrict__ mask, const uint32_t* __restrict__ offsets, uint32_t e,
+                                                    bool& kept) {
+    const uint32_t w = e >> 5, bit = 1u << (e & 31u);
+    uint32_t pos = __ldg(offsets + (e >> 7));
+    for (uint32_t i = w & ~3u; i < w; ++i) pos += __popc(__ldg(mask + i));
+    const uint32_t word = __ldg(mask + w);
+    kept = (word & bit) != 0;
+    return pos + __popc(word & (bit - 1u));
+}
+
 constexpr int kRedWarps = 8;
-__global__ void __launch_bounds__(32 * kRedWarps)
-conv_fused_reduce_kernel(const float4* __restrict__ partial, const FusedConvParams p, float* __restrict__ dw, int accumulate) {
+
+// dW[j0 + lane, c, u, v] term by term, for a channel that holds an infinity or a NaN (false: it holds none, nothing is computed).  The
+// K steps cover whole 8-pixel groups; behind a row's last output and behind the band's last group dY is zero there, but X may be a
+// pixel that the tap (u, v) does not see, and zero times infinity is NaN.  Called by the whole block; `part`: a float per thread.
+// Positions are shared out among the warps in runs of 32, whose pixels the lanes look up; then a lane is an output channel.
+__device__ __noinline__ bool sum_term_by_term(const FusedConvParams& p, const uint16_t* __restrict__ dy, const uint16_t* __restrict__ values,
+                                              const uint32_t* __restrict__ mask, const uint32_t* __restrict__ offsets, int j0, int c, int u,
+                                              int v, float* part, float& sum) {
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const uint32_t plane = (uint32_t)p.H * p.W, total = (uint32_t)p.B * p.Ca * plane, dy_plane = (uint32_t)p.Ho * p.Wo;
+    bool kept, found = false;
+    for (int n = g; n < p.B; n += kRedWarps) {
+        const uint32_t e = ((uint32_t)n * p.Ca + c) * plane;
+        const uint32_t first = retained_before(mask, offsets, e, kept);
+        const uint32_t last = e + plane < total ? min(retained_before(mask, offsets, e + plane, kept), p.k) : p.k;
+        for (uint32_t i = first + lane; i < last; i += 32) found |= (__ldg(values + i) & 0x7F80u) == 0x7F80u;
+    }
+    if (!__syncthreads_or(found)) return false;
+    float acc = 0.f;
+    const uint32_t positions = (uint32_t)p.B * dy_plane;
+    for (uint32_t q0 = g * 32; q0 < positions; q0 += 32 * kRedWarps) {
+        const uint32_t q = q0 + lane, n = q / dy_plane, at = q - n * dy_plane;
+        const int iy = (int)(at / p.Wo) * p.stride + u - p.pad, ix = (int)(at % p.Wo) * p.stride + v - p.pad;
+        const unsigned long long from = (unsigned long long)n * p.Cz * dy_plane + at;
+        float x = 0.f;
+        kept = false;
+        if (q < positions && iy >= 0 && iy < p.H && ix >= 0 && ix < p.W) {
+            const uint32_t pos = retained_before(mask, offsets, ((n * p.Ca + c) * p.H + iy) * p.W + ix, kept);
+            kept = kept && pos < p.k;
+            if (kept) x = __uint_as_float((uint32_t)__ldg(values + pos) << 16);
+        }
+        for (uint32_t todo = __ballot_sync(kFullMask, kept); todo; todo &= todo - 1) {
+            const int b = __ffs(todo) - 1;
+            const float xb = __shfl_sync(kFullMask, x, b);
+            const unsigned long long fb = __shfl_sync(kFullMask, from, b);
+            if (j0 + lane < p.Cz) acc = fmaf(__uint_as_float((uint32_t)__ldg(dy + fb + (unsigned long long)(j0 + lane) * dy_plane) << 16), xb, acc);
+        }
+    }
+    part[threadIdx.x] = acc;
+    __syncthreads();
+    sum = 0.f;
+    for (int w = 0; w < kRedWarps; ++w) sum += part[w * 32 + lane];
+    __syncthreads();
+    return true;
+}
+
+// dw[j,c,u,v] (=|+=) sum over splits, in split order within a warp's share and then over the warps.  A block takes 32 rows of
+// one 4-column group; its eight warps share out the splits.  Sums that are not finite are looked at again (sum_term_by_term): the look
+// costs up to 0.5 us (14 x 14), one infinity in the input of 64 -> 64 on 56 x 56 at batch 64 brings the call from 40 us to 2 ms.
+__global__ void __launch_bounds__(32 * kRedWarps, 5)
+conv_fused_reduce_kernel(const float4* __restrict__ partial, const __grid_constant__ FusedConvParams p, const uint16_t* __restrict__ dy,
+                         const uint16_t* __restrict__ values, const uint32_t* __restrict__ mask, const uint32_t* __restrict__ offsets,
+                         float* __restrict__ dw, int accumulate) {
     __shared__ float4 sums[kRedWarps][32];
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
     const int quarters = (min(kBM, p.Cz) + 31) / 32;
@@ -528,15 +588,35 @@ conv_fused_reduce_kernel(const float4* __restrict__ partial, const FusedConvPara
     }
     sums[g][lane] = acc;
     __syncthreads();
-    if (g == 0 && j < p.Cz) {
+    int v = 0, u = 0, c = 0;
+    auto tap = [&]() {                                  // cb is a multiple of 16: the four columns belong to one tap
+        const int n_inst = p.R * p.cb;
+        v = col / n_inst;
+        u = (col % n_inst) / p.cb;
+        c = c0 + col % p.cb;
+    };
+    bool odd = false;
+    if (g == 0) {                                       // one warp: with the divisions in all of them 256 -> 256 on 14 x 14 (4608 blocks) took 2.4 us more
 #pragma unroll
         for (int w = 1; w < kRedWarps; ++w) {
-            const float4 v = sums[w][lane];
-            acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+            const float4 o = sums[w][lane];
+            acc.x += o.x; acc.y += o.y; acc.z += o.z; acc.w += o.w;
         }
-        const int n_inst = p.R * p.cb;
-        const int v = col / n_inst, u = (col % n_inst) / p.cb, c = c0 + col % p.cb;   // cb is a multiple of 16: one tap
-        const float a[4] = {acc.x, acc.y, acc.z, acc.w};
+        tap();
+        odd = !isfinite(acc.x * 0.f + acc.y * 0.f + acc.z * 0.f + acc.w * 0.f) && j < p.Cz;   // one of the four is not finite
+    }
+    odd = __syncthreads_or(odd);
+    float a[4] = {acc.x, acc.y, acc.z, acc.w};
+    if (odd) {
+        tap();
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            float sum;
+            if (c + e < p.Ca && sum_term_by_term(p, dy, values, mask, offsets, j - lane, c + e, u, v, &sums[0][0].x, sum) && !isfinite(a[e]))
+                a[e] = sum;
+        }
+    }
+    if (g == 0 && j < p.Cz) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             if (c + e < p.Ca) {
@@ -550,7 +630,7 @@ conv_fused_reduce_kernel(const float4* __restrict__ partial, const FusedConvPara
 size_t stage_bytes_of(FusedConvParams& p) {
     const size_t row_pitch = (size_t)(p.cb / 8) * p.gp * 16;
     // With an odd number of 8-pixel groups the last K = 16 step reads one more K row than the band has: zeros in dY,
-    // anything finite in X.  With 64 channels of dY per band the instruction's rows 64..127 are the next 8-pixel group
+    // pixels or zeros in X (sum_term_by_term mends what infinities make of that).  With 64 channels of dY per band the instruction's rows 64..127 are the next 8-pixel group
     // (their results are not used).
     const int odd = (p.ni * p.yb * p.cores) & 1;
     const size_t x = (size_t)(p.ni * p.x_rows + odd * p.row_step) * row_pitch * p.planes;
@@ -742,7 +822,9 @@ dropit_status conv_fused_run(const void* dy, const void* values, const void* mas
     cfg.gridDim = dim3((unsigned)(tiles * p.chunks * 8 * quarters));
     cfg.blockDim = dim3(32 * kRedWarps);
     cfg.dynamicSmemBytes = 0;
-    if (cudaLaunchKernelEx(&cfg, conv_fused_reduce_kernel, reinterpret_cast<const float4*>(partial), p, dw, accumulate) != cudaSuccess) {
+    if (cudaLaunchKernelEx(&cfg, conv_fused_reduce_kernel, reinterpret_cast<const float4*>(partial), p, reinterpret_cast<const uint16_t*>(dy),
+                           reinterpret_cast<const uint16_t*>(values), reinterpret_cast<const uint32_t*>(mask), offsets, dw,
+                           accumulate) != cudaSuccess) {
         (void)cudaGetLastError();
         return DROPIT_ERR_CUDA;
     }
