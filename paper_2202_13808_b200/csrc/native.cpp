@@ -17,12 +17,17 @@ namespace {
 
 using at::Tensor;
 
-struct StatusError {
-    int code;
-    const char* where;
-};
+py::object* g_error_class = nullptr;
+
+// A status that is not OK becomes the package's DropITError.  It travels as a python_error, which is a std::exception: the autograd
+// engine hands those from the thread of a backward pass to the caller, anything else that leaves a node ends the process.
 void check(dropit_status s, const char* where) {
-    if (s != DROPIT_OK) throw StatusError{(int)s, where};
+    if (s == DROPIT_OK) return;
+    py::gil_scoped_acquire gil;
+    PyErr_SetObject(g_error_class ? g_error_class->ptr() : PyExc_RuntimeError, py::make_tuple((int)s, where).ptr());
+    python_error error;
+    error.persist();
+    throw error;
 }
 
 dropit_dtype dtype_code(const Tensor& t, const char* name) {
@@ -226,16 +231,14 @@ Tensor gelu_linear(const Tensor& x, const Tensor& weight, const c10::optional<Te
     return GeluLinear::apply(x, weight, bias, gamma, fmt, table);
 }
 
-py::object* g_error_class = nullptr;
-
 }  // namespace
 
 PYBIND11_MODULE(_native, m) {
     py::register_exception_translator([](std::exception_ptr p) {
         try {
             if (p) std::rethrow_exception(p);
-        } catch (const StatusError& e) {
-            PyErr_SetObject(g_error_class ? g_error_class->ptr() : PyExc_RuntimeError, py::make_tuple(e.code, e.where).ptr());
+        } catch (python_error& e) {
+            e.restore();
         }
     });
     m.def("set_error_class", [](py::object cls) { g_error_class = new py::object(cls); });
