@@ -194,10 +194,12 @@ struct GeluLinear : public torch::autograd::Function<GeluLinear> {
         const auto cache = ctx->saved_data["cache"].toIntVector();
         const Tensor dz2 = grads[0].reshape({-1, grads[0].size(-1)}).contiguous();
         const bool bias = ctx->saved_data["bias"].toBool() && ctx->needs_input_grad(2);
+        // With create_graph the gradients are to be differentiated again: what can be is then formed by operations that autograd knows.
+        const bool graph = at::GradMode::is_enabled();
         Tensor dx, dw, db;
         if (ctx->needs_input_grad(0)) {                                  // Eq. 3: exact, needs theta only; the activation's cache is x
             const Tensor dy = at::matmul(dz2, weight);
-            if (dy.scalar_type() == at::kBFloat16 && x2.scalar_type() == at::kBFloat16 && dy.is_contiguous() &&
+            if (!graph && dy.scalar_type() == at::kBFloat16 && x2.scalar_type() == at::kBFloat16 && dy.is_contiguous() &&
                 reinterpret_cast<uintptr_t>(x2.data_ptr()) % 16 == 0) {
                 c10::cuda::CUDAGuard guard(dy.device());
                 dx = at::empty_like(x2);
@@ -207,7 +209,7 @@ struct GeluLinear : public torch::autograd::Function<GeluLinear> {
             }
             dx = dx.reshape(ctx->saved_data["shape"].toIntVector());
         }
-        const bool own = weight.scalar_type() == at::kBFloat16 && dz2.scalar_type() == at::kBFloat16 && dz2.size(1) % 8 == 0 &&
+        const bool own = !graph && weight.scalar_type() == at::kBFloat16 && dz2.scalar_type() == at::kBFloat16 && dz2.size(1) % 8 == 0 &&
                          dz2.numel() != 0 && reinterpret_cast<uintptr_t>(dz2.data_ptr()) % 16 == 0;
         if (ctx->needs_input_grad(1)) {                                  // Eq. 6
             const Tensor full = weight_grad(dz2.to(values.scalar_type()), values, saved[3], saved[4], cache[0], cache[1], cache[2],

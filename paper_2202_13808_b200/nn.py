@@ -141,7 +141,8 @@ class DropITGeluLinearFn:
     """z = GELU(x) W^T + b for bf16 tensors, with the GELU written by the library's producer kernel so that the
     selection statistics of GELU(x), the tensor the Linear caches, are taken while it is written (Sec. 3.5: the
     activation keeps its own cache x; only the Linear's cache is replaced by D(GELU(x))).  The autograd node is native
-    (csrc/native.cpp): forward and backward make a dozen calls, whose host side in Python took twice their GPU time."""
+    (csrc/native.cpp): forward and backward make a dozen calls, whose host side in Python took twice their GPU time.
+    dx and db can be differentiated again, with respect to dz and W (x is a constant there, and dW is one)."""
 
     @staticmethod
     def apply(x, weight, bias, gamma: float, fmt: str):

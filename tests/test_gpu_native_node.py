@@ -28,3 +28,25 @@ def test_an_error_in_the_backward_pass_reaches_the_caller(cuda_device, Cz):
     lin(x).backward(dz)                      # nothing is left behind
     dropit.check_device_status(cuda_device)
     assert bool(torch.isfinite(lin.weight.grad).all())
+
+
+def test_a_gradient_penalty_reaches_the_weight(cuda_device):
+    """dx = (dz W) GELU'(x) can be differentiated again: the gradients of |dx|^2 with respect to W and dz."""
+    lin, x, dz = _layer(37, 64, 24, cuda_device)
+    dz.requires_grad_(True)
+    dx, = torch.autograd.grad(lin(x), x, dz, create_graph=True)
+    dW, ddz = torch.autograd.grad((dx.double() ** 2).sum(), (lin.weight, dz))
+    W, z, xd = lin.weight.detach().double(), dz.detach().double(), x.detach().double()
+    g = 0.5 * torch.erfc(-xd / 2 ** 0.5) + xd * torch.exp(-0.5 * xd * xd) / (2 * torch.pi) ** 0.5
+    inner, size = 2 * (z @ W) * g * g, 2 * (z.abs() @ W.abs()) * g * g      # d|dx|^2 / d(dz W), and what it is summed from
+    # bf16 roundings on the way, half a unit (2^-8) each: dz W, dx, its gradient, that times GELU'(x), and the result
+    for got, want, bound in ((dW, z.t() @ inner, z.abs().t() @ size), (ddz, inner @ W.t(), size @ W.t().abs())):
+        assert bool(((got.double() - want).abs() <= 6 * 2.0 ** -8 * bound).all())
+
+
+def test_a_bias_gradient_can_be_differentiated(cuda_device):
+    lin, x, dz = _layer(37, 64, 24, cuda_device)
+    dz.requires_grad_(True)
+    _, db = torch.autograd.grad(lin(x), (lin.weight, lin.bias), dz, create_graph=True)
+    back, = torch.autograd.grad(db.float().sum(), dz)
+    assert torch.equal(back, torch.ones_like(dz))
