@@ -267,7 +267,7 @@ decompress_index32_kernel(const typename Tr::elem_t* __restrict__ values, const 
     }
 }
 
-// ... without a seek table
+// ... without a seek table that can be used
 template <typename Tr>
 __global__ void __launch_bounds__(256)
 scatter_index32_kernel(const typename Tr::elem_t* __restrict__ values, const int32_t* __restrict__ idx, int64_t k,
@@ -309,7 +309,7 @@ static dropit_status run_decompress(const void* values, const void* meta, const 
         }
         return check_launch();
     }
-    if (offsets != nullptr) {
+    if (offsets != nullptr && is_aligned16(offsets)) {      // coordinate caches are accepted without a table too, or with an unaligned one
         const int64_t steps = (n + 1023) / 1024;
         int64_t blocks = (steps + kIdxWarps - 1) / kIdxWarps;
         const int64_t resident = (int64_t)sm_count() * (Tr::kElemBytes == 2 ? 8 : 6);

@@ -48,6 +48,7 @@ Tensor empty1(int64_t n, at::ScalarType type, const Tensor& like) {
     return at::detail::empty_cuda({n}, type, like.device(), c10::nullopt);
 }
 void* ptr(const Tensor& t) { return t.defined() && t.numel() ? t.data_ptr() : nullptr; }
+void* table_ptr(const c10::optional<Tensor>& t) { return t.has_value() ? ptr(*t) : nullptr; }
 void* current_stream(const Tensor& t) { return c10::cuda::getCurrentCUDAStream(t.device().index()).stream(); }
 
 // One status word per device, which every kernel's bounded waits report to.
@@ -128,8 +129,9 @@ std::string mismatch(const Tensor& dy, const Tensor& values) {
     return std::string("dy dtype ") + toString(dy.scalar_type()) + " != cache dtype " + toString(values.scalar_type());
 }
 
-Tensor weight_grad(const Tensor& dy, const Tensor& values, const Tensor& meta, const Tensor& offsets, int64_t n, int64_t Ca, int64_t k,
-                   int fmt, const c10::optional<Tensor>& out, bool accumulate, const c10::optional<Tensor>& workspace, bool no_scratch) {
+// `offsets` may be absent: a coordinate cache can do without its seek table.
+Tensor weight_grad(const Tensor& dy, const Tensor& values, const Tensor& meta, const c10::optional<Tensor>& offsets, int64_t n, int64_t Ca,
+                   int64_t k, int fmt, const c10::optional<Tensor>& out, bool accumulate, const c10::optional<Tensor>& workspace, bool no_scratch) {
     const dropit_dtype dt = require_cuda(dy, "dy");
     if (dy.scalar_type() != values.scalar_type()) throw py::type_error(mismatch(dy, values));
     const int64_t M = Ca ? n / Ca : 0, Cz = dy.dim() ? dy.size(-1) : 0;
@@ -142,14 +144,14 @@ Tensor weight_grad(const Tensor& dy, const Tensor& values, const Tensor& meta, c
     check(dropit_weight_grad_workspace(M, Ca, Cz, dt, (dropit_format)fmt, &bytes), "dropit_weight_grad_workspace");
     const Tensor ws = scratch(workspace, bytes, dy);
     auto fn = no_scratch ? dropit_weight_grad_fused : dropit_weight_grad;
-    check(fn(ptr(dy), ptr(values), ptr(meta), (const uint32_t*)ptr(offsets), M, Ca, Cz, k, dt, (dropit_format)fmt, (float*)ptr(dw),
+    check(fn(ptr(dy), ptr(values), ptr(meta), (const uint32_t*)table_ptr(offsets), M, Ca, Cz, k, dt, (dropit_format)fmt, (float*)ptr(dw),
              accumulate ? 1 : 0, ptr(ws), (size_t)ws.numel(), status_ptr(dy), current_stream(dy)),
           no_scratch ? "dropit_weight_grad_fused" : "dropit_weight_grad");
     return dw;
 }
 
-Tensor conv_weight_grad(const Tensor& dy, const Tensor& values, const Tensor& meta, const Tensor& offsets, int B, int Ca, int H, int W,
-                        int R, int S, int stride, int pad, int dilation, int64_t k, int fmt, const c10::optional<Tensor>& out,
+Tensor conv_weight_grad(const Tensor& dy, const Tensor& values, const Tensor& meta, const c10::optional<Tensor>& offsets, int B, int Ca, int H,
+                        int W, int R, int S, int stride, int pad, int dilation, int64_t k, int fmt, const c10::optional<Tensor>& out,
                         bool accumulate, const c10::optional<Tensor>& workspace) {
     const dropit_dtype dt = require_cuda(dy, "dy");
     if (dy.scalar_type() != values.scalar_type()) throw py::type_error(mismatch(dy, values));
@@ -161,7 +163,7 @@ Tensor conv_weight_grad(const Tensor& dy, const Tensor& values, const Tensor& me
     check(dropit_conv_weight_grad_workspace(B, Ca, H, W, Cz, R, S, stride, pad, dt, (dropit_format)fmt, &bytes),
           "dropit_conv_weight_grad_workspace");
     const Tensor ws = scratch(workspace, bytes, dy);
-    check(dropit_conv_weight_grad(ptr(dy), ptr(values), ptr(meta), (const uint32_t*)ptr(offsets), B, Ca, H, W, Cz, R, S, stride, pad,
+    check(dropit_conv_weight_grad(ptr(dy), ptr(values), ptr(meta), (const uint32_t*)table_ptr(offsets), B, Ca, H, W, Cz, R, S, stride, pad,
                                   dilation, k, dt, (dropit_format)fmt, (float*)ptr(dw), accumulate ? 1 : 0, ptr(ws),
                                   (size_t)ws.numel(), status_ptr(dy), current_stream(dy)), "dropit_conv_weight_grad");
     return dw;
