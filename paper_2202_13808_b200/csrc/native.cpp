@@ -246,11 +246,12 @@ PYBIND11_MODULE(_native, m) {
         }
     });
     m.def("set_error_class", [](py::object cls) { g_error_class = new py::object(cls); });
-    m.def("status_word", &status_word);
-    m.def("compress", &compress);
-    m.def("produce", &produce);
-    m.def("compress_prepared", &compress_prepared);
-    m.def("weight_grad", &weight_grad);
-    m.def("conv_weight_grad", &conv_weight_grad);
-    m.def("gelu_linear", &gelu_linear);
+    // Without the interpreter's lock, as a call through ctypes is: a launch can wait for room in the stream's queue.
+    m.def("status_word", torch::wrap_pybind_function_no_gil(status_word));
+    m.def("compress", torch::wrap_pybind_function_no_gil(compress));
+    m.def("produce", torch::wrap_pybind_function_no_gil(produce));
+    m.def("compress_prepared", torch::wrap_pybind_function_no_gil(compress_prepared));
+    m.def("weight_grad", torch::wrap_pybind_function_no_gil(weight_grad));
+    m.def("conv_weight_grad", torch::wrap_pybind_function_no_gil(conv_weight_grad));
+    m.def("gelu_linear", torch::wrap_pybind_function_no_gil(gelu_linear));
 }
