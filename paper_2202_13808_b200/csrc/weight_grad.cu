@@ -1093,8 +1093,8 @@ __device__ __forceinline__ float to_float(float f) { return f; }
 
 // dY tile (kFmaK tokens x TILE outputs) and R(a-hat) tile (x TILE channels) in shared memory, the next ones on their way in
 // registers.  A thread holds MICRO x MICRO sums, packed in pairs for the two-wide FMA; the threads form groups that each
-// cover the tile and share out the tokens of a stage, and the groups' sums are added in group order.  64-wide tiles: 8 x 8
-// sums, 4 groups of 64 threads.  32-wide tiles, for outputs too small to fill the chip with 64-wide ones: 4 x 4 sums, 4 groups.
+// cover the tile and share out the tokens of a stage, and the groups' sums are added in group order.  ffma_kernel() says which
+// of the four forms takes a call; CTAS: how many of them an SM is to hold.
 // Bound by the FMA rate (256 x 768 x 768: 2.2 us at the two-wide rate) and the latency of its eight stages.
 constexpr int kFmaK = 32;
 __device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
@@ -1108,12 +1108,13 @@ __device__ __forceinline__ void unpack2(unsigned long long v, float& lo, float& 
 __device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
-template <typename T, int TILE>
-__global__ void __launch_bounds__(256)
+template <typename T, int TILE, int MICRO, int CTAS>
+__global__ void __launch_bounds__(256, CTAS)
 wg_ffma_kernel(const T* __restrict__ dy, const T* __restrict__ xd, int M, int Ca, int Cz, float* __restrict__ dw,
                int accumulate) {
-    constexpr int kMicro = TILE / 8;                           // 8 or 4
-    constexpr int kGroups = 4, kSide = 8;                      // 4 groups of 8 x 8 threads
+    constexpr int kMicro = MICRO;
+    constexpr int kSide = TILE / MICRO, kGroups = 256 / (kSide * kSide);      // groups of kSide x kSide threads
+    constexpr int kStep = kSide * 4;                           // a thread's sums: 4-wide pieces this many columns (rows) apart
     constexpr int kCols4 = TILE / 4;
     constexpr int kUnits = kFmaK * kCols4 / 256;               // 4-element pieces per thread and operand
     constexpr int kPitch = TILE + 4;
@@ -1122,7 +1123,7 @@ wg_ffma_kernel(const T* __restrict__ dy, const T* __restrict__ xd, int M, int Ca
     auto& sB = smem[1];
     const int j0 = blockIdx.y * TILE, c0 = blockIdx.x * TILE;
     const int group = threadIdx.x / (kSide * kSide), tg = threadIdx.x % (kSide * kSide);
-    const int tx = tg % kSide, ty = tg / kSide;                // a thread's sums: 4-wide pieces 32 columns (rows) apart
+    const int tx = tg % kSide, ty = tg / kSide;
     const bool vec_a = (Cz & 3) == 0, vec_b = (Ca & 3) == 0;   // rows start on a 4-element boundary
     float4 ra[kUnits], rb[kUnits];
     auto load4 = [&](const T* p, int n, int col, int cols, bool vec) {
@@ -1176,12 +1177,13 @@ wg_ffma_kernel(const T* __restrict__ dy, const T* __restrict__ xd, int M, int Ca
 #pragma unroll
         for (int kk = 0; kk < kFmaK / kGroups; ++kk) {
             const int row = group * (kFmaK / kGroups) + kk;
+            if (kGroups == 1 && row >= M - k0) break;          // the stages of few tokens are mostly padding
             float a[kMicro];
             unsigned long long b[kMicro / 2];
 #pragma unroll
             for (int h = 0; h < kMicro / 4; ++h) {
-                const float4 a4 = *reinterpret_cast<const float4*>(&sA[buf][row][h * 32 + ty * 4]);
-                const float4 b4 = *reinterpret_cast<const float4*>(&sB[buf][row][h * 32 + tx * 4]);
+                const float4 a4 = *reinterpret_cast<const float4*>(&sA[buf][row][h * kStep + ty * 4]);
+                const float4 b4 = *reinterpret_cast<const float4*>(&sB[buf][row][h * kStep + tx * 4]);
                 a[4 * h] = a4.x; a[4 * h + 1] = a4.y; a[4 * h + 2] = a4.z; a[4 * h + 3] = a4.w;
                 b[2 * h] = pack2(b4.x, b4.y);
                 b[2 * h + 1] = pack2(b4.z, b4.w);
@@ -1205,7 +1207,7 @@ wg_ffma_kernel(const T* __restrict__ dy, const T* __restrict__ xd, int M, int Ca
     float4* share = reinterpret_cast<float4*>(&smem[0][0][0][0]);
     constexpr int kPieces = kMicro * kMicro / 4;
     static_assert(sizeof(smem) >= (size_t)kSide * kSide * kPieces * sizeof(float4), "room for one group's sums");
-    for (int g = 1; g < kGroups; ++g) {
+    for (int g = 1; g < kGroups && g * (kFmaK / kGroups) < M; ++g) {      // (groups without a token have nothing to add)
         if (group == g)
 #pragma unroll
             for (int q = 0; q < kPieces; ++q) {
@@ -1225,11 +1227,11 @@ wg_ffma_kernel(const T* __restrict__ dy, const T* __restrict__ xd, int M, int Ca
     if (group != 0) return;
 #pragma unroll
     for (int i = 0; i < kMicro; ++i) {
-        const int j = j0 + (i / 4) * 32 + ty * 4 + i % 4;
+        const int j = j0 + (i / 4) * kStep + ty * 4 + i % 4;
         if (j >= Cz) continue;
 #pragma unroll
         for (int h = 0; h < kMicro / 4; ++h) {
-            const int c = c0 + h * 32 + tx * 4;
+            const int c = c0 + h * kStep + tx * 4;
             float* d = dw + (size_t)j * Ca + c;
             if (vec_b && c + 4 <= Ca) {
                 float4 v = make_float4(out[i][4 * h], out[i][4 * h + 1], out[i][4 * h + 2], out[i][4 * h + 3]);
@@ -1245,6 +1247,29 @@ wg_ffma_kernel(const T* __restrict__ dy, const T* __restrict__ xd, int M, int Ca
             }
         }
     }
+}
+
+// The forms, by the number of 64 x 64 tiles.  Measured with the decompression, us per call:
+//  * kNarrow, 32 x 32 tiles, 4 groups with 4 x 4 sums: outputs that 64 x 64 tiles would leave more than half of the chip without.
+//  * kAlone, 4 groups with 8 x 8 sums, all registers: up to one tile per SM (256 x 768 x 768 13.4; with the registers cut 15.6).
+//  * kShared, the same with two CTAs per SM: more tiles (8 x 1024 -> 4096 23.2 with one, 12.4 with two; 1000 x 768 -> 3072 132, 129).
+//  * kFew, one group with 4 x 4 sums, four CTAs per SM, nothing to add up at the end: few tokens (8 x 1024 -> 4096 8.3; 64 tokens 22.4
+//    against 24.3, 96 tokens equal; 768 -> 768, one tile per SM, 32 tokens 5.9 against 6.3, 64 tokens 7.9 against 7.3), and, where rows are
+//    read by the element, many tiles (1000 x 2050 -> 1002 159 against 168; two CTAs per SM do the rest in a last wave).
+enum class FfmaKernel { kNarrow, kAlone, kShared, kFew };
+static FfmaKernel ffma_kernel(int64_t M, int64_t Ca, int64_t Cz) {
+    const int64_t tiles = ((Ca + 63) / 64) * ((Cz + 63) / 64), sms = sm_count();
+    if (2 * tiles <= sms) return FfmaKernel::kNarrow;
+    if (tiles <= sms) return M <= 48 ? FfmaKernel::kFew : FfmaKernel::kAlone;
+    const bool by_element = (Ca & 3) != 0 || (Cz & 3) != 0;
+    return M <= (by_element ? 112 : 80) || (by_element && tiles > 2 * sms) ? FfmaKernel::kFew : FfmaKernel::kShared;
+}
+template <typename T>
+static cudaError_t launch_ffma(const cudaLaunchConfig_t& cfg, FfmaKernel form, const void* dy, const void* dense, int M, int Ca, int Cz, float* dw,
+                               int accumulate) {
+    auto kernel = form == FfmaKernel::kNarrow ? wg_ffma_kernel<T, 32, 4, 5> : form == FfmaKernel::kAlone ? wg_ffma_kernel<T, 64, 8, 1>
+                  : form == FfmaKernel::kShared ? wg_ffma_kernel<T, 64, 8, 2> : wg_ffma_kernel<T, 64, 4, 1>;
+    return cudaLaunchKernelEx(&cfg, kernel, reinterpret_cast<const T*>(dy), reinterpret_cast<const T*>(dense), M, Ca, Cz, dw, accumulate);
 }
 
 __global__ void zero_or_keep_kernel(float* dw, int64_t count, int accumulate) {
@@ -1298,9 +1323,8 @@ static dropit_status weight_grad_impl(const void* dy, const void* values, const 
     if (s != DROPIT_OK) return s;
 
     if (!plan.tensor_core) {
-        // 32-wide tiles where 64-wide ones would leave more than half of the chip idle
-        const bool narrow = 2 * (int64_t)plan.tiles_n * plan.tiles_m <= sm_count();
-        const int tile = narrow ? 32 : 64;
+        const FfmaKernel form = ffma_kernel(M, Ca, Cz);
+        const int tile = form == FfmaKernel::kNarrow ? 32 : 64;
         cudaLaunchAttribute pdl[1];
         pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         pdl[0].val.programmaticStreamSerializationAllowed = 1;
@@ -1310,15 +1334,8 @@ static dropit_status weight_grad_impl(const void* dy, const void* values, const 
         cfg.stream = stream;
         cfg.attrs = pdl;
         cfg.numAttrs = 1;
-        cudaError_t err;
-        if (dtype == DROPIT_BF16)
-            err = cudaLaunchKernelEx(&cfg, narrow ? wg_ffma_kernel<uint16_t, 32> : wg_ffma_kernel<uint16_t, 64>,
-                                     reinterpret_cast<const uint16_t*>(dy), reinterpret_cast<const uint16_t*>(dense), (int)M, (int)Ca,
-                                     (int)Cz, dw, accumulate);
-        else
-            err = cudaLaunchKernelEx(&cfg, narrow ? wg_ffma_kernel<float, 32> : wg_ffma_kernel<float, 64>,
-                                     reinterpret_cast<const float*>(dy), reinterpret_cast<const float*>(dense), (int)M, (int)Ca,
-                                     (int)Cz, dw, accumulate);
+        const cudaError_t err = dtype == DROPIT_BF16 ? launch_ffma<uint16_t>(cfg, form, dy, dense, (int)M, (int)Ca, (int)Cz, dw, accumulate)
+                                                     : launch_ffma<float>(cfg, form, dy, dense, (int)M, (int)Ca, (int)Cz, dw, accumulate);
         if (err != cudaSuccess) {
             (void)cudaGetLastError();
             return DROPIT_ERR_CUDA;
