@@ -13,8 +13,11 @@
 //   4. element i is retained iff key_i > T, or key_i == T and fewer than q equal keys precede it.  A lane owns 32
 //      consecutive elements, i.e. one mask word; the retained values are moved to the front of the super-block in
 //      shared memory and leave coalesced.
-// Nothing is sampled and no scratch in global memory is used: any distribution of values takes the same path (equal keys
-// make the counting atomics collide, zeros are counted in registers because ReLU outputs are half zeros).
+// Nothing is sampled and no scratch in global memory is used: any distribution of values takes the same path.  Equal keys
+// make the counting atomics collide; zeros are counted in registers because ReLU outputs are half zeros.  Other values that fill more
+// than half of an fp32 tensor of 300 Ki elements and more are slower here than with the histogram launches (2^19 elements, half of them equal
+// 31.6 against 27.2 us, all 39.7 against 26.1; none 21.2 against 26.0).  Counting the commonest key of a sample in registers, not zero,
+// brought these to 26 us and cost all other calls 0.6 to 1 us.
 // Bound by latency: barriers, the trips between CTAs (about 1 us a digit round) and the shared-memory counting.  Measured per
 // call (graph replay, gamma 0.9): bf16 8 Ki / 48 Ki / 196 Ki / 454 Ki elements 6.2 / 6.8 / 8.5 / 11.8 us, where the grid-wide
 // kernel's full histogram takes 60 us at any of these sizes; fp32 48 Ki / 196 Ki / 454 Ki 10.8 / 14.0 / 18.8 us, where the three

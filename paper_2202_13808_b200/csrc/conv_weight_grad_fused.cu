@@ -665,6 +665,12 @@ bool make_fused_conv_plan(FusedConvParams& p, int B, int Ca, int H, int W, int C
     const float dy_cost = p.vec >= 4 ? 0.2f : (p.vec == 2 ? 0.3f : 0.6f);
     const int64_t tiles = (int64_t)p.tiles_c * p.tiles_j;
     if (tiles > 65535) return false;
+    // 1 x 1 filters of stride 2: every block of 128 outputs inflates X again, for a single tap and in slots of 64 pixels that a short
+    // row fills by less than half (0.84 us per million elements of all slots).  From some size on the dense copies, made once, are ahead, if
+    // there are channels enough for their GEMM: batch 64, 1024 -> 2048 on 14 x 14 (470 M elements) 401 against 358 us, 512 -> 2048 on
+    // 28 x 28 411 / 346; batch 128 760 / 614 and 841 / 625.  Not so below (batch 64, 512 -> 1024 on 28 x 28, 235 M: 197 / 209), with fewer channels
+    // (batch 128, 256 -> 1024 on 28 x 28 197 / 262) or on longer rows (batch 64, 512 -> 1280 on 40 x 40 350 / 527).
+    if (R == 1 && S == 1 && stride == 2 && W <= 32 && Ca >= 512 && (int64_t)p.tiles_j * B * Ca * p.Ho * 64 >= 240000000) return false;
     if (!p.flat) {
         p.cores = (p.Wo + 7) / 8;
         // columns an 8-pixel group of any tap can reach, at the plane's resolution

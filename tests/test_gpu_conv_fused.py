@@ -53,3 +53,22 @@ def test_fused_conv_waits_give_up_and_recover(cuda_device, monkeypatch):
     again = dropit.dropit_conv_weight_grad(dy, cache, (3, 3), 1, 1)
     dropit.check_device_status(cuda_device)
     assert torch.equal(again, good)
+
+
+# strided 1 x 1 filters with many outputs: the most work that is inflated per block of outputs, and the first that takes dense copies
+@pytest.mark.parametrize("batch", [56, 64])
+def test_strided_pointwise_either_side_of_the_line(cuda_device, batch):
+    B, Ca, side, Cz = batch, 512, 27, 1024 + 8
+    inflated = -(-Cz // 128) * B * Ca * ((side + 1) // 2) * 64
+    assert (inflated >= 240_000_000) == (batch == 64)
+    x = torch.randn(B, Ca, side, side, generator=torch.Generator().manual_seed(batch)).to(torch.bfloat16).to(cuda_device)
+    cache = dropit.dropit_compress(x, 0.9)
+    dy = torch.randn(B, Cz, 14, 14, device=cuda_device).to(torch.bfloat16)
+    before = dropit.dropit_launch_count()
+    dw = dropit.dropit_conv_weight_grad(dy, cache, (1, 1), 2, 0)
+    launches = dropit.dropit_launch_count() - before
+    dropit.check_device_status(cuda_device)
+    assert (launches == 2) == (batch == 56)               # product and reduction, without decompression and gathered copies
+    a = dropit.dropit_decompress(cache)[:, :, ::2, ::2].double()
+    ref = torch.einsum("njyx,ncyx->jc", dy.double(), a)
+    assert float((dw[:, :, 0, 0].double() - ref).abs().max()) <= 2e-4 * float(ref.abs().max())
