@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import glob
+import importlib.util
 import os
 import subprocess
 import sys
@@ -48,7 +49,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 def _build_native(force: bool):
     """Compile the torch binding against the installed torch's headers and link it to libdropit.so beside it."""
-    deps = [NATIVE_SRC, os.path.join(CSRC, "layer_ops.h"), os.path.join(ROOT, "include", "dropit.h")]
+    deps = [NATIVE_SRC, os.path.join(CSRC, "layer_ops.h"), os.path.join(ROOT, "include", "dropit.h"),
+            os.path.join(os.path.dirname(importlib.util.find_spec("torch").origin), "version.py")]     # another torch, another ABI
     if not force and os.path.exists(NATIVE) and os.path.getmtime(NATIVE) > max(os.path.getmtime(d) for d in deps):
         return
     import torch
