@@ -50,3 +50,32 @@ def test_a_bias_gradient_can_be_differentiated(cuda_device):
     _, db = torch.autograd.grad(lin(x), (lin.weight, lin.bias), dz, create_graph=True)
     back, = torch.autograd.grad(db.float().sum(), dz)
     assert torch.equal(back, torch.ones_like(dz))
+
+
+# Widths that the kernel for the bias gradient and the rounding of dW does not take, a gradient that is expanded, not stored, one that
+# has gaps between its rows, and a weight that is not trained.
+@pytest.mark.parametrize("Cz", [8, 10, 100, 200])
+@pytest.mark.parametrize("form", ["stored", "expanded", "sliced", "frozen"])
+def test_gradients_of_other_forms(cuda_device, Cz, form):
+    M, Ca = 61, 72
+    lin, x, dz = _layer(M, Ca, Cz, cuda_device)
+    if form == "expanded":
+        dz = dz[0, 0].expand(M, Cz)
+    elif form == "sliced":
+        dz = torch.cat([dz, dz], 1)[:, Cz // 2:Cz // 2 + Cz]
+    lin.weight.requires_grad_(form != "frozen")
+    lin(x).backward(dz)
+    dropit.check_device_status(cuda_device)
+    z, xd, W = dz.double(), x.detach().double(), lin.weight.detach().double()
+    u, eps = 2.0 ** -8, M * 2.0 ** -24
+    g = 0.5 * torch.erfc(-xd / 2 ** 0.5) + xd * torch.exp(-0.5 * xd * xd) / (2 * torch.pi) ** 0.5
+    # bf16 roundings of dz W and of dx; one rounding of an fp32 sum of M terms for the others
+    assert bool(((x.grad.double() - (z @ W) * g).abs() <= 2.1 * u * (z.abs() @ W.abs()) * g.abs() + 1e-5 * (z.abs() @ W.abs())).all())
+    assert bool(((lin.bias.grad.double() - z.sum(0)).abs() <= u * z.sum(0).abs() + 2 * eps * z.abs().sum(0)).all())
+    if form == "frozen":
+        assert lin.weight.grad is None
+        return
+    y, prep = dropit.dropit_produce(x.detach(), 0.5, "gelu")
+    kept = dropit.dropit_decompress(dropit.dropit_compress_prepared(y, 0.5, prep)).double()
+    want, size = z.t() @ kept, z.abs().t() @ kept.abs()
+    assert bool(((lin.weight.grad.double() - want).abs() <= u * want.abs() + 2 * eps * size).all())

@@ -17,10 +17,10 @@ CASES = [
     di.small_linear(7000, 520, 776, "bf16", 0.95),     # twelve tiles: pairs cross tile boundaries at uneven places
     di.small_linear(12000, 800, 2304, "bf16", 0.97),   # 36 tiles, whole ranges only
     di.small_linear(9300, 776, 2056, "bf16", 0.97),    # 36 ragged tiles
-    di.small_linear(11000, 768, 2304, "bf16", 0.97),   # 27 tiles: two ranges per tile from the same tokens, the rests shared out
+    di.small_linear(11000, 768, 2304, "bf16", 0.97),   # 27 tiles: two ranges per tile with tickets
     di.small_linear(7001, 1032, 2000, "bf16", 0.97),   # 40 tiles: one range per tile and the rests
     di.small_linear(700, 768, 768, "bf16", 0.9),       # a few blocks: no split
-    di.small_linear(4000, 1536, 384, "bf16", 0.95),    # three ranges per tile with tickets
+    di.small_linear(4000, 1536, 384, "bf16", 0.95),    # 12 tiles: six pairs each, none of which crosses into the next
 ]
 
 
@@ -37,6 +37,32 @@ def test_split_weight_grad_matches_oracle(cuda_device, case):
     assert torch.equal(dropit.dropit_weight_grad(dyd, cache), dw)                                     # fixed order
     assert torch.equal(dropit.dropit_weight_grad(dyd, cache, out=dw.clone(), accumulate=True), dw + dw)
     dropit.check_device_status(cuda_device)
+
+
+# The way that the plan takes, as it shows outside: the even split adds up in a launch of its own, and the workspace holds a plane of
+# whole tiles per range.
+WAYS = [
+    (di.small_linear(700, 768, 768, "bf16", 0.9), 2, 0),       # no split
+    (di.small_linear(2000, 768, 2304, "bf16", 0.97), 2, 2),    # two ranges with tickets
+    (di.small_linear(3001, 1024, 1536, "bf16", 0.97), 2, 3),   # three
+    (di.small_linear(4000, 1536, 384, "bf16", 0.95), 3, 6),    # even split, whole ranges of equal length
+    (di.small_linear(9000, 256, 768, "bf16", 0.9), 3, 24),     # ... of many pairs
+    (di.small_linear(7001, 1032, 2000, "bf16", 0.97), 3, 3),   # ... one range per tile, the rests shared out by pairs that cross tiles
+    (di.small_linear(13001, 768, 2304, "bf16", 0.98), 3, 4),   # ... two ranges per tile and the rests
+]
+
+
+@pytest.mark.parametrize("case, launches, planes", WAYS, ids=lambda v: getattr(v, "name", None))
+def test_every_way_to_split_is_taken_and_matches_oracle(cuda_device, case, launches, planes):
+    size = dropit.dropit_weight_grad_workspace(case.M, case.Ca, case.Cz, dropit.BF16, dropit.FMT_BITMASK, cuda_device)
+    tiles = 2 * -(-case.Cz // 256) * -(-case.Ca // 256)
+    assert (size - case.M * case.Ca * 2) // (tiles * 128 * 256 * 4) == planes
+    cache = dropit.dropit_compress(di.make_x(case).to(cuda_device), case.gamma)
+    dy = di.make_dy(case).to(cuda_device)
+    before = dropit.dropit_launch_count()
+    dropit.dropit_weight_grad(dy, cache)
+    assert dropit.dropit_launch_count() - before == launches
+    test_split_weight_grad_matches_oracle(cuda_device, case)
 
 
 def test_even_split_waits_give_up_and_recover(cuda_device, monkeypatch):
