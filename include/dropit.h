@@ -209,7 +209,7 @@ dropit_status dropit_dequantize_values(const uint8_t* codes, const uint32_t* sca
  * host that has no allocator to call at all.  For them the scratch that
  * dropit_compress takes from its `workspace` argument lives in a fixed array
  * inside the library's device image: dropit_compress_static_scratch_bytes()
- * bytes (about 400 KB) that every GPU which loads the library holds until the
+ * bytes (about 470 KB) that every GPU which loads the library holds until the
  * process exits.
  *  - Same inputs, outputs, selection rule and cache layout as dropit_compress
  *    with dtype = DROPIT_BF16; the caller still provides x, values, meta, offsets.
@@ -292,10 +292,12 @@ dropit_status dropit_conv_weight_grad_workspace(int B, int Ca, int H, int W, int
  *   dy [device, B x Cz x Ho x Wo, dtype] with Ho = (H + 2 pad - R)/stride + 1,
  *   Wo likewise; values/meta/offsets [device] = cache of a [B x Ca x H x W];
  *   dw [device, Cz x Ca x R x S, float], overwritten or accumulated into.
- * bf16 bitmask caches with filters of up to 3 x 3 and stride 1 or 2 are multiplied on the tensor cores
- * straight from the cache; other bf16 shapes with S <= 7 (and Wo <= W when stride is 1) on the tensor
- * cores from dense copies (one implicit GEMM per filter tap over (n, y, x)); fp32 accumulation and a
- * fixed summation order either way.  The rest and fp32 inputs use an fp32 FMA kernel.  A bounded device wait that expires is reported
+ * bf16 bitmask caches with filters of up to 3 x 3, stride 1 or 2 and pad <= 2 are multiplied on the tensor
+ * cores straight from the cache where a band of image rows fits shared memory, except 1 x 1 filters of
+ * stride 1 on planes of whole 16-byte groups and large 1 x 1 layers of stride 2 on rows of up to 32 pixels;
+ * these and other bf16 shapes with S <= 7 (and Wo <= W when stride is 1) on the tensor cores from dense
+ * copies (one implicit GEMM per filter tap over (n, y, x)); fp32 accumulation and a fixed summation order
+ * either way.  The rest and fp32 inputs use an fp32 FMA kernel.  A bounded device wait that expires is reported
  * through dev_status as DROPIT_ERR_TIMEOUT.
  */
 dropit_status dropit_conv_weight_grad(const void* dy, const void* values, const void* meta, const uint32_t* offsets,

@@ -962,7 +962,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
     // ---------------- phase 3: ordered compaction, one warp per run of super-blocks ----------------
     // A lane owns 32 consecutive elements = one mask word, so a super-block costs one warp scan and the
     // mask needs no exchange.  Retained values are staged per warp at (final position - head) and leave
-    // for global memory in aligned 16-byte pieces after every super-block; the < 8 that remain are
+    // for global memory in aligned 16-byte pieces once more than kStageKeep are waiting; the < 8 that remain are
     // carried to the front of the buffer.
     ptx::launch_dependents();   // a programmatically launched kernel behind this one may be brought up
     unsigned long long departed_before = 0;   // see the end of the kernel

@@ -159,7 +159,7 @@ small_compress_kernel(const uint4* __restrict__ x, uint32_t n, uint32_t k, uint3
     const uint32_t data = ptx::smem_u32(ssm) + warp * Cfg::kSlotBytes;
     const uint32_t nvec_full = n / G;
 
-    ptx::grid_dependency_wait();
+    ptx::grid_dependency_wait();      // (for a programmatic launch; launch_small makes an ordinary one, where it returns at once)
     if (active) {
 #pragma unroll
         for (int j = 0; j < OV; ++j) {

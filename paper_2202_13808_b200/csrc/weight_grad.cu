@@ -230,7 +230,7 @@ static WgPlan make_wg_plan(int64_t M, int64_t Ca, int64_t Cz, dropit_dtype dtype
     return p;
 }
 
-// The plans of the last shapes that this thread asked for: weighing the splits costs some microseconds, and a layer is planned
+// The plans of the last shapes that this thread asked for: weighing the splits costs up to a microsecond, and a layer is planned
 // twice per call (workspace query and launch).
 static const WgPlan& cached_wg_plan(int64_t M, int64_t Ca, int64_t Cz, dropit_dtype dtype, dropit_format format, bool fused) {
     struct Entry {
