@@ -713,6 +713,7 @@ bool make_fused_conv_plan(FusedConvParams& p, int B, int Ca, int H, int W, int C
     };
     int best_pieces = 0, best_ni = 0;
     float best = 0.f;
+    // (no more than 64 pieces are tried: a plane of more than 128 rows that fits shared memory only row by row is refused)
     const int most_pieces = p.flat ? (p.W + 31) / 32 : p.Ho;
     for (int pieces = 1; pieces <= most_pieces && pieces <= 64; ++pieces) {
         if (!p.flat && pieces > 1 && (p.Ho + pieces - 1) / pieces == (p.Ho + pieces - 2) / (pieces - 1)) continue;

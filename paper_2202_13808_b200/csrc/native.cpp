@@ -30,10 +30,11 @@ void check(dropit_status s, const char* where) {
     throw error;
 }
 
+std::string type_name(const Tensor& t) { return "torch." + c10::getDtypeNames(t.scalar_type()).first; }
 dropit_dtype dtype_code(const Tensor& t, const char* name) {
     if (t.scalar_type() == at::kBFloat16) return DROPIT_BF16;
     if (t.scalar_type() == at::kFloat) return DROPIT_F32;
-    throw py::type_error(std::string(name) + ": dtype " + toString(t.scalar_type()) + " is not supported (bf16 or fp32)");
+    throw py::type_error(std::string(name) + ": dtype " + type_name(t) + " is not supported (bf16 or fp32)");
 }
 dropit_dtype require_cuda(const Tensor& t, const char* name) {
     if (!t.is_cuda()) throw py::value_error(std::string(name) + " must be a CUDA tensor (there is no CPU path)");
@@ -126,7 +127,7 @@ CacheTuple compress_prepared(const Tensor& y, double gamma, const Tensor& prep, 
 }
 
 std::string mismatch(const Tensor& dy, const Tensor& values) {
-    return std::string("dy dtype ") + toString(dy.scalar_type()) + " != cache dtype " + toString(values.scalar_type());
+    return "dy dtype " + type_name(dy) + " != cache dtype " + type_name(values);
 }
 
 // `offsets` may be absent: a coordinate cache can do without its seek table.
@@ -134,7 +135,7 @@ Tensor weight_grad(const Tensor& dy, const Tensor& values, const Tensor& meta, c
                    int64_t k, int fmt, const c10::optional<Tensor>& out, bool accumulate, const c10::optional<Tensor>& workspace, bool no_scratch) {
     const dropit_dtype dt = require_cuda(dy, "dy");
     if (dy.scalar_type() != values.scalar_type()) throw py::type_error(mismatch(dy, values));
-    const int64_t M = Ca ? n / Ca : 0, Cz = dy.dim() ? dy.size(-1) : 0;
+    const int64_t M = Ca ? n / Ca : 0, Cz = dy.size(-1);
     if (dy.numel() != M * Cz)
         throw py::value_error("dy has " + std::to_string(dy.numel()) + " elements, expected " + std::to_string(M) + " x " + std::to_string(Cz));
     if (!out.has_value() && accumulate) throw py::value_error("accumulate=True needs out");

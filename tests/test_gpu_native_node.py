@@ -79,3 +79,14 @@ def test_gradients_of_other_forms(cuda_device, Cz, form):
     kept = dropit.dropit_decompress(dropit.dropit_compress_prepared(y, 0.5, prep)).double()
     want, size = z.t() @ kept, z.abs().t() @ kept.abs()
     assert bool(((lin.weight.grad.double() - want).abs() <= u * want.abs() + 2 * eps * size).all())
+
+
+def test_refusals_read_as_torch_writes_types(cuda_device):
+    x = torch.randn(8, 16, device=cuda_device)
+    with pytest.raises(TypeError, match=r"x: dtype torch\.float16 is not supported"):
+        dropit.dropit_compress(x.half(), 0.5)
+    cache = dropit.dropit_compress(x.bfloat16(), 0.5)
+    with pytest.raises(TypeError, match=r"dy dtype torch\.float32 != cache dtype torch\.bfloat16"):
+        dropit.dropit_weight_grad(x, cache)
+    with pytest.raises(IndexError):
+        dropit.dropit_weight_grad(x[0, 0].bfloat16(), cache)
