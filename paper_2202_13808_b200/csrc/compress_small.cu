@@ -9,7 +9,9 @@
 //   3. the threshold is found digit by digit: 8 bits, then 7 (fp32: then 8 and 8 more over the keys that still match).
 //      A round is: each CTA writes its row of 128 or 256 counts into every CTA of the cluster, one cluster barrier, and
 //      every CTA finds the same digit from the same rows.  The rows of the CTAs in front of it also give a CTA its
-//      exclusive prefix of keys above and at the threshold, so the ordered compaction needs no further exchange;
+//      exclusive prefix of keys above and at the threshold, so the ordered compaction needs no further exchange.
+//      fp32, up to 4096 keys that match in their upper 15 bits: their lower halves are sent round once instead, and every CTA
+//      finds both lower digits from that list (4.9 -> 3.8 us of the kernel at 196 Ki normal values, where some 300 match);
 //   4. element i is retained iff key_i > T, or key_i == T and fewer than q equal keys precede it.  A lane owns 32
 //      consecutive elements, i.e. one mask word; the retained values are moved to the front of the super-block in
 //      shared memory and leave coalesced.
@@ -20,7 +22,8 @@
 // brought these to 26 us and cost all other calls 0.6 to 1 us.
 // Bound by latency: barriers, the trips between CTAs (about 1 us a digit round) and the shared-memory counting.  Measured per
 // call (graph replay, gamma 0.9): bf16 8 Ki / 48 Ki / 196 Ki / 454 Ki elements 6.2 / 6.8 / 8.5 / 11.8 us, where the grid-wide
-// kernel's full histogram takes 60 us at any of these sizes; fp32 48 Ki / 196 Ki / 454 Ki 10.8 / 14.0 / 18.8 us, where the three
+// kernel's full histogram takes 60 us at any of these sizes; fp32 48 Ki / 196 Ki / 454 Ki 10.8 / 14.0 / 18.8 us (196 Ki / 512 Ki now 13.0 / 19.2, 14.4 / 20.5 on the same day without the list
+// and the programmatic launch, which takes 0.7 us off every call behind a kernel that leaves SMs free), where the three
 // histogram launches and the compaction take 27 us at 600 Ki.  (Counting through a branch per element, only by the warps
 // that own a super-block, and a third barrier per round: 8.0 / 8.9 / 10.3 / 12.8 and 14.2 / 16.9 / 20.7 us.)  At 2^19 bf16
 // elements (12.5 us) the sampled grid-wide kernel (15.8 us) is about to overtake: two super-blocks per warp measured 17.4 us at
@@ -41,12 +44,15 @@ constexpr uint32_t kTopBins = 1u << 15;
 constexpr int kRowBins = 256;                            // counts of one CTA in one digit round
 constexpr size_t kHistBytes = (size_t)kTopBins * 2;
 constexpr size_t kGatherBytes = (size_t)2 * kMaxCtas * kRowBins * 4;
+constexpr uint32_t kListCap = kMaxCtas * kRowBins;          // a gather buffer, a word per key
 
 struct SmallShared {
     uint32_t row[kRowBins];        // this CTA's counts of the current digit
     uint2 warp_tot[kWarps];
     uint32_t digit, cum;           // the digit found, keys above it
     uint32_t before_gt, before_eq; // in the CTAs in front of this one: keys above / at the digit
+    uint32_t at;                   // keys at the digit, over the cluster
+    uint32_t listed, list_before;  // keys this CTA has put on the list; on the list in front of its own: keys above | at T << 16
 };
 
 template <typename Tr> struct SmallCfg {
@@ -128,6 +134,7 @@ __device__ __forceinline__ uint32_t digit_round(SmallShared& sh, const uint32_t*
             sh.cum = cum;
             sh.before_gt = before;
             sh.before_eq = f;
+            sh.at = h;
         }
     }
     __syncthreads();
@@ -135,6 +142,33 @@ __device__ __forceinline__ uint32_t digit_round(SmallShared& sh, const uint32_t*
     run_gt += sh.before_gt;
     run_eq = sh.before_eq;
     return sh.digit;       // (the next round's first barrier comes before anything here is written again)
+}
+
+// One digit of the keys on a list of `m` entries, found by every warp for itself from the counts of its 256 values in sh.row: the
+// largest one with k_rem entries at or above it; k_rem loses those above it.
+__device__ __forceinline__ uint32_t list_digit(const SmallShared& sh, int lane, uint32_t& k_rem) {
+    constexpr int kPer = kRowBins / 32;          // values per lane
+    static_assert(kPer == 8, "");
+    const uint4 a = reinterpret_cast<const uint4*>(sh.row)[lane * 2], b = reinterpret_cast<const uint4*>(sh.row)[lane * 2 + 1];
+    uint32_t ge = a.x + a.y + a.z + a.w + b.x + b.y + b.z + b.w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_down_sync(kFullMask, ge, o);
+        if (lane + o < 32) ge += y;
+    }
+    const int owner = 31 - __clz(__ballot_sync(kFullMask, ge >= k_rem));      // (lane 0 holds all entries that still match: at least k_rem)
+    const uint32_t behind = __shfl_sync(kFullMask, ge, (owner + 1) & 31);
+    k_rem -= owner < 31 ? behind : 0u;
+    const uint32_t c = sh.row[owner * kPer + (lane & 7)];
+    ge = c;
+#pragma unroll
+    for (int o = 1; o < kPer; o <<= 1) {
+        const uint32_t y = __shfl_down_sync(kFullMask, ge, o, kPer);
+        if ((lane & 7) + o < kPer) ge += y;
+    }
+    const int bin = 31 - __clz(__ballot_sync(kFullMask, ge >= k_rem) & 0xFFu);
+    k_rem -= __shfl_sync(kFullMask, ge - c, bin);
+    return (uint32_t)(owner * kPer + bin);
 }
 
 template <typename Tr, bool INDEX32>
@@ -159,7 +193,7 @@ small_compress_kernel(const uint4* __restrict__ x, uint32_t n, uint32_t k, uint3
     const uint32_t data = ptx::smem_u32(ssm) + warp * Cfg::kSlotBytes;
     const uint32_t nvec_full = n / G;
 
-    ptx::grid_dependency_wait();      // (for a programmatic launch; launch_small makes an ordinary one, where it returns at once)
+    ptx::grid_dependency_wait();      // launched programmatically: the input may come from the kernel before this one
     if (active) {
 #pragma unroll
         for (int j = 0; j < OV; ++j) {
@@ -182,6 +216,7 @@ small_compress_kernel(const uint4* __restrict__ x, uint32_t n, uint32_t k, uint3
         }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
+    if (t == 0) sh.listed = sh.list_before = 0;
     for (uint32_t i = t; i < kHistBytes / 16; i += kThreads) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0, 0, 0, 0);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
@@ -246,15 +281,48 @@ small_compress_kernel(const uint4* __restrict__ x, uint32_t n, uint32_t k, uint3
     if constexpr (kF32) {
         // ---- digits 3 and 4: the lower 16 bits, over the keys whose upper bits match ----
         const uint32_t row_addr = ptx::smem_u32(sh.row);
-#pragma unroll 1
-        for (int shift = 8; shift >= 0; shift -= 8) {
+        const uint32_t m = sh.at;
+        if (m <= kListCap) {
+            // Few keys match (some 300 of 196 Ki normal ones): their lower halves go on a list that every CTA holds, this CTA's
+            // behind those of the CTAs in front of it, and every CTA finds both digits on its own.  One trip through the cluster
+            // and one pass over the elements instead of two.
+            const uint32_t front = run_eq, list_addr = ptx::smem_u32(gather);        // (the first round's rows are read)
+            for_each_key([&](uint32_t key, bool exists) {
+                if (exists && (key >> 16) == T) {
+                    const uint32_t to = list_addr + (front + atomicAdd(&sh.listed, 1u)) * 4;
+                    for (uint32_t r = 0; r < ctas; ++r) ptx::st_cluster_u32(ptx::map_shared_to_cta(to, r), key & 0xFFFFu);
+                }
+            });
+            if (t < kRowBins) sh.row[t] = 0;
+            ptx::cluster_sync_all();
+            for (uint32_t i = t; i < m; i += kThreads) red_shared_if(row_addr + (gather[i] >> 8) * 4, 1u, true);
+            __syncthreads();
+            const uint32_t d3 = list_digit(sh, lane, k_rem);
+            __syncthreads();
             if (t < kRowBins) sh.row[t] = 0;
             __syncthreads();
-            for_each_key([&](uint32_t key, bool exists) {
-                red_shared_if(row_addr + ((key >> shift) & 0xFFu) * 4, 1u, exists && (key >> (shift + 8)) == T);
-            });
-            T = (T << 8) | digit_round(sh, gather + (shift == 8 ? 0 : kMaxCtas * kRowBins), 256, rank, ctas, k_rem, run_gt, run_eq,
-                                         false);
+            for (uint32_t i = t; i < m; i += kThreads) red_shared_if(row_addr + (gather[i] & 0xFFu) * 4, 1u, (gather[i] >> 8) == d3);
+            __syncthreads();
+            const uint32_t low = d3 << 8 | list_digit(sh, lane, k_rem);
+            uint32_t before = 0;
+            for (uint32_t i = t; i < front; i += kThreads) before += (gather[i] > low ? 1u : 0u) | (gather[i] == low ? 1u << 16 : 0u);
+            before = __reduce_add_sync(kFullMask, before);
+            if (lane == 0 && before) atomicAdd(&sh.list_before, before);
+            __syncthreads();
+            run_gt += sh.list_before & 0xFFFFu;
+            run_eq = sh.list_before >> 16;
+            T = T << 16 | low;
+        } else {
+#pragma unroll 1
+            for (int shift = 8; shift >= 0; shift -= 8) {
+                if (t < kRowBins) sh.row[t] = 0;
+                __syncthreads();
+                for_each_key([&](uint32_t key, bool exists) {
+                    red_shared_if(row_addr + ((key >> shift) & 0xFFu) * 4, 1u, exists && (key >> (shift + 8)) == T);
+                });
+                T = (T << 8) | digit_round(sh, gather + (shift == 8 ? 0 : kMaxCtas * kRowBins), 256, rank, ctas, k_rem, run_gt,
+                                           run_eq, false);
+            }
         }
     }
     const uint32_t q = k_rem;          // ties at T that are retained, lowest flat indices first
@@ -405,17 +473,20 @@ bool launch_small(const void* x, int64_t n, int64_t k, void* values, void* meta,
     int ctas = 1;
     while (ctas < limit && sbs > (int64_t)ctas * kSbPerCta) ctas *= 2;
     const int64_t per = (sbs + ctas - 1) / ctas;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (unsigned)ctas;
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    // programmatic: the cluster may be set up while the kernel before it drains; it waits before it reads anything
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)ctas);
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = Cfg::kSmemBytes;
     cfg.stream = stream;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     if (cudaLaunchKernelEx(&cfg, small_compress_kernel<Tr, INDEX32>, reinterpret_cast<const uint4*>(x), (uint32_t)n, (uint32_t)k,
                            (uint32_t)per, reinterpret_cast<typename Tr::elem_t*>(values),
                            INDEX32 ? (uint32_t*)nullptr : reinterpret_cast<uint32_t*>(meta),

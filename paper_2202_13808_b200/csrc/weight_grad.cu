@@ -1167,6 +1167,7 @@ wg_ffma_kernel(const T* __restrict__ dy, const T* __restrict__ xd, int M, int Ca
 #pragma unroll
         for (int l = 0; l < kMicro / 2; ++l) acc[i][l] = 0ull;
     ptx::grid_dependency_wait();                               // the dense scratch comes from the kernel before this one
+    ptx::launch_dependents();
     load_stage(0);
     store_stage(0);
     __syncthreads();

@@ -31,3 +31,22 @@ def test_small_tensors_match_the_oracle(cuda_device, n, dtype, fmt):
         cache = dropit.dropit_compress(x.to(cuda_device), gamma, fmt)
         dropit.check_device_status(cuda_device)
         assert_cache_matches_oracle(cache, bits, dt, keep, k, fmt)
+
+
+# fp32 keys that share their upper 15 bits: up to 4096 of them are ranked from a list, more by counting their lower digits in turn
+@pytest.mark.parametrize("matching", [1, 37, 4095, 4096, 4097, 9000])
+@pytest.mark.parametrize("front", [0, 20000])
+def test_keys_that_match_in_their_upper_bits(cuda_device, matching, front):
+    gen = torch.Generator().manual_seed(matching + front)
+    low = torch.randint(0, 1 << 16, (matching,), generator=gen)
+    low[::5] = low[0]                                          # ties, at the threshold too for some of the counts below
+    same = (low + (0x3F80 << 16)).to(torch.int32)              # 1.0 .. 1.0078
+    others = torch.where(torch.rand(front, generator=gen) < 0.5, 0.25, -3.0).view(torch.int32)
+    bits = torch.cat([others, same])[torch.randperm(matching + front, generator=gen)]
+    x = bits.view(torch.float32)
+    above = int((others.view(torch.float32).abs() > 1).sum())
+    for kept in {above + 1, above + (matching + 1) // 2, above + matching}:
+        gamma = 1.0 - kept / x.numel()
+        xb, dt, keep, k = oracle_cache(x, gamma)
+        cache = dropit.dropit_compress(x.to(cuda_device), gamma)
+        assert_cache_matches_oracle(cache, xb, dt, keep, k, "bitmask")
