@@ -26,6 +26,10 @@
 // instead of 16 Ki; the band, 1.4 times as wide, has 96 bins instead of 64) and none for zeros, which behind a ReLU are half of
 // them: 19.4 -> 18.3, 38.9 -> 38.3, 41.4 -> 39.2, 91 -> 88, 113 -> 109 us (3.8 TB/s of the two reads and the outputs); behind a
 // ReLU 64 x 256 x 56 x 56 57.5 -> 51.8, 64 x 64 x 56 x 56 26.9 -> 22.2 us.
+// The steps between the two passes are one-time code and trips to L2: sums over a warp's lanes by one reduction instead of shuffles,
+// the band's ends looked up by a warp instead of one thread, the counters of a sample thread added in pairs, and the barrier's
+// look at whether its word is this call's made ahead of time: 600 Ki / 3.2 M / 9.7 M elements 15.1 / 16.4 / 19.1 -> 13.7 / 15.1 / 17.1 us
+// (replayed; 38.7 M 38.9 -> 36.9).  Finding T by halving, in every warp, instead of one warp's scan: 0.7 us slower.
 // When the band is wider than the per-warp histogram (small tensors, which are not sampled; key
 // distributions that are flat around T; a sample that missed) a general path is taken instead:
 // full CTA histogram in shared memory, global histogram by atomics, then one extra counting read.
@@ -209,8 +213,8 @@ __device__ __forceinline__ uint32_t element_order(uint32_t x) {
     return x ^ t ^ (t << 1);
 }
 
-// Exclusive prefix over the block's threads of `v`; also returns the block total.
-__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* s_warp, uint32_t* total) {
+// Exclusive prefix over the block's threads of `v`.
+__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* s_warp) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t inc = v;
 #pragma unroll
@@ -221,16 +225,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* s
     __syncthreads();   // protect s_warp from a previous use
     if (lane == 31) s_warp[warp] = inc;
     __syncthreads();
-    uint32_t wt = (lane < (int)(blockDim.x >> 5)) ? s_warp[lane] : 0u;
-    uint32_t winc = wt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        uint32_t y = __shfl_up_sync(kFullMask, winc, o);
-        if (lane >= o) winc += y;
-    }
-    const uint32_t wprefix = __shfl_sync(kFullMask, winc - wt, warp);
-    *total = __shfl_sync(kFullMask, winc, 31);
-    return wprefix + inc - v;
+    return __reduce_add_sync(kFullMask, lane < warp ? s_warp[lane] : 0u) + inc - v;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -297,36 +292,32 @@ __device__ __forceinline__ void sample_band(const uint4* __restrict__ x, int64_t
         // the thread's 16 words hold its 32 counters; the four 16-byte reads go in an order rotated by (t/2) mod 4,
         // so that the threads of a quarter-warp (64 bytes apart) touch different banks
         const uint4* mine = reinterpret_cast<const uint4*>(bins + (kKeySpace / 2 - (t + 1) * (PER / 2)));
-        uint32_t sum = 0;
+        uint32_t pair = 0;
 #pragma unroll
         for (int j = 0; j < PER / 8; ++j) {
             const uint4 v = mine[j ^ ((t >> 1) & 3)];
-            sum += (v.x & 0xFFFFu) + (v.x >> 16) + (v.y & 0xFFFFu) + (v.y >> 16) + (v.z & 0xFFFFu) + (v.z >> 16) +
-                   (v.w & 0xFFFFu) + (v.w >> 16);
+            pair += v.x + v.y + v.z + v.w;         // (a half never exceeds the sample's size)
         }
+        const uint32_t sum = (pair & 0xFFFFu) + (pair >> 16);
         after_loads();   // what the caller wants in flight while the thresholds are worked out (issued earlier, it delays the sample)
-        uint32_t total;
-        const uint32_t excl = block_exclusive_scan(sum, s_warp, &total);
-        // key at descending rank r: cum_before < r <= cum_before + h
-        if ((excl < R_hi && R_hi <= excl + sum) || (excl < R_lo && R_lo <= excl + sum)) {
-            // one or two threads of the CTA get here: they read their counters again, in key order
-            uint32_t cw[PER / 2];
+        const uint32_t excl = block_exclusive_scan(sum, s_warp);
+        // key at descending rank r: cum_before < r <= cum_before + h.  Of at most two threads' counters: their warp takes one each
+        const bool has_hi = excl < R_hi && R_hi <= excl + sum, has_lo = excl < R_lo && R_lo <= excl + sum;
+        uint32_t todo = __ballot_sync(kFullMask, has_hi || has_lo);
+        while (todo) {
+            const int owner = __ffs(todo) - 1;
+            todo &= todo - 1u;
+            const uint32_t key = kKeySpace - 1 - (((t & ~31) + owner) * PER + (t & 31));
+            const uint32_t h = (bins[key >> 1] >> ((key & 1u) * 16)) & 0xFFFFu;
+            uint32_t cum = h;
 #pragma unroll
-            for (int j = 0; j < PER / 8; ++j) {
-                const uint4 v = mine[j];
-                cw[4 * j] = v.x; cw[4 * j + 1] = v.y; cw[4 * j + 2] = v.z; cw[4 * j + 3] = v.w;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFullMask, cum, o);
+                if ((t & 31) >= o) cum += y;
             }
-            uint32_t cum = excl;
-#pragma unroll
-            for (int r = 0; r < PER; ++r) {
-                // key = kKeySpace-1 - (t*PER + r) lives in word 15 - r/2 of the thread, upper half when r is even
-                const uint32_t key = kKeySpace - 1 - (t * PER + r);
-                const uint32_t cwr = cw[PER / 2 - 1 - r / 2];
-                const uint32_t hh = (r & 1) ? (cwr & 0xFFFFu) : (cwr >> 16);
-                if (cum < R_hi && R_hi <= cum + hh) band[1] = key;
-                if (cum < R_lo && R_lo <= cum + hh) band[0] = key;
-                cum += hh;
-            }
+            cum += __shfl_sync(kFullMask, excl, owner);
+            if (cum - h < R_hi && R_hi <= cum) band[1] = key;
+            if (cum - h < R_lo && R_lo <= cum) band[0] = key;
         }
     }
     __syncthreads();
@@ -359,19 +350,19 @@ __device__ __forceinline__ void barrier_open(unsigned long long* word, uint32_t 
         asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(word), "l"((unsigned long long)epoch << 32) : "memory");
     }
 }
+// `early` (thread 0): the word as it was some time ago; if it carried the epoch then, no trip to L2 is made to look again.
 __device__ __forceinline__ bool grid_barrier(unsigned long long* word, uint32_t epoch, uint32_t target, int* s_ok,
-                                             int spin_max) {
+                                             int spin_max, unsigned long long early) {
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         bool ok = true;
         int spins = 0;
-        unsigned long long v;
-        for (;;) {   // the word belongs to this call
-            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
-            if ((uint32_t)(v >> 32) == epoch) break;
+        unsigned long long v = early;
+        while ((uint32_t)(v >> 32) != epoch) {   // the word belongs to this call
             if (++spins > spin_max) { ok = false; break; }
             __nanosleep(32);
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
         }
         if (ok) {
             atomicAdd(word, 1ull);
@@ -383,7 +374,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long* word, uint32_t 
                 __nanosleep(32);
             }
         }
-        __threadfence();
         *s_ok = ok ? 1 : 0;
     }
     __syncthreads();
@@ -568,6 +558,8 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                     [&] { if (sb0 < sb1) issue_sb(sb1 - 1, 0); }, [](const uint4& v) { return v; });
     }
     bool prefetched = !prepared;
+    // requested here, looked at by the first barrier
+    const unsigned long long early_word = threadIdx.x == 0 ? ld_relaxed_u64(&st->barrier) : 0ull;
     uint32_t lo = sh.band[0], hi = sh.band[1];
     uint32_t T = 0, q = 0;
     uint32_t run_gt = 0, run_eq = 0;   // this warp's exclusive prefix (absolute)
@@ -724,34 +716,34 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                 }
             }
             prefetched = false;
-            for (int o = 16; o > 0; o >>= 1) {
-                cnt_lo += __shfl_xor_sync(kFullMask, cnt_lo, o);
-                cnt_hi += __shfl_xor_sync(kFullMask, cnt_hi, o);
-            }
+            cnt_lo = __reduce_add_sync(kFullMask, cnt_lo);
+            cnt_hi = __reduce_add_sync(kFullMask, cnt_hi);
             if (lane == 0) {
                 if (cnt_lo) atomicAdd(&hist[0], cnt_lo);
                 sh.w_hi[warp] = cnt_hi;
             }
             __syncthreads();
-            uint32_t cta_hi = 0;
-            for (int w = 0; w < kFusedWarps; ++w) cta_hi += sh.w_hi[w];
+            static_assert(kFusedWarps == 32 && kWarpBins % 32 == 0, "one lane per warp, one warp for the row's last words");
             if (narrow) {
                 // publish this CTA's row: band bins and #key>hi
-                if (threadIdx.x < kRowWords) {
+                if (threadIdx.x < kWarpBins) {
                     uint32_t v = 0;
-                    if (threadIdx.x < kWarpBins) {
-                        for (int w = 0; w < kFusedWarps; ++w) v += whist[w][threadIdx.x];
-                    } else if (threadIdx.x == kWarpBins) {
-                        v = cta_hi;
-                    }
+#pragma unroll
+                    for (int w = 0; w < kFusedWarps; ++w) v += whist[w][threadIdx.x];
                     rows[(size_t)blockIdx.x * kRowWords + threadIdx.x] = v;
+                } else if (warp == kWarpBins / 32) {
+                    const uint32_t v = __reduce_add_sync(kFullMask, sh.w_hi[lane]);
+                    if (lane < kRowWords - kWarpBins) rows[(size_t)blockIdx.x * kRowWords + kWarpBins + lane] = lane ? 0u : v;
                 }
             } else {
+                uint32_t cta_hi = 0;
+                if (threadIdx.x == 0)
+                    for (int w = 0; w < kFusedWarps; ++w) cta_hi += sh.w_hi[w];
                 // the global histogram is scratch that nobody cleared: every CTA clears a slice, and one more
                 // grid barrier separates the clearing from the accumulation
                 for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i <= width; i += gridDim.x * blockDim.x) ghist[i] = 0;
                 barrier_target += gridDim.x;
-                if (!grid_barrier(&st->barrier, epoch, barrier_target, &sh.ok, spin_max)) {
+                if (!grid_barrier(&st->barrier, epoch, barrier_target, &sh.ok, spin_max, early_word)) {
                     if (threadIdx.x == 0 && dev_status) atomicExch(dev_status, (int)DROPIT_ERR_TIMEOUT);
                     return;
                 }
@@ -762,7 +754,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
                 if (threadIdx.x == 0 && cta_hi) atomicAdd(&st->n_hi[attempt], (unsigned long long)cta_hi);
             }
             barrier_target += gridDim.x;
-            if (!grid_barrier(&st->barrier, epoch, barrier_target, &sh.ok, spin_max)) {
+            if (!grid_barrier(&st->barrier, epoch, barrier_target, &sh.ok, spin_max, early_word)) {
                 if (threadIdx.x == 0 && dev_status) atomicExch(dev_status, (int)DROPIT_ERR_TIMEOUT);
                 return;
             }
@@ -841,30 +833,24 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
             {
                 // this warp's (#key > T, #key == T) and the same over the CTAs before this one
                 uint32_t g = 0, pg = 0;
-                for (uint32_t d = dT + 1 + lane; d <= width; d += 32) {
-                    g += whist[warp][d];
-                    pg += sh.pre[d];
+#pragma unroll
+                for (int j = 0; j < kWarpBins / 32; ++j) {
+                    const uint32_t d = j * 32 + lane;
+                    if (d > dT && d <= width) {
+                        g += whist[warp][d];
+                        pg += sh.pre[d];
+                    }
                 }
-                for (int o = 16; o > 0; o >>= 1) {
-                    g += __shfl_xor_sync(kFullMask, g, o);
-                    pg += __shfl_xor_sync(kFullMask, pg, o);
-                }
+                g = __reduce_add_sync(kFullMask, g);
+                pg = __reduce_add_sync(kFullMask, pg);
                 if (lane == 0) {
                     sh.wpre_gt[warp] = g + sh.w_hi[warp];
                     sh.wpre_eq[warp] = whist[warp][dT];
                 }
                 __syncthreads();
-                // exclusive scan over the CTA's warps (lane = warp index), done by every warp for itself
-                const uint32_t og = (lane < kFusedWarps) ? sh.wpre_gt[lane] : 0u;
-                const uint32_t oe = (lane < kFusedWarps) ? sh.wpre_eq[lane] : 0u;
-                uint32_t gi = og, ei = oe;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t yg = __shfl_up_sync(kFullMask, gi, o), ye = __shfl_up_sync(kFullMask, ei, o);
-                    if (lane >= o) { gi += yg; ei += ye; }
-                }
-                run_gt = pg + sh.pre[kWarpBins] + __shfl_sync(kFullMask, gi - og, warp);
-                run_eq = sh.pre[dT] + __shfl_sync(kFullMask, ei - oe, warp);
+                // the warps in front of this one (lane = warp index), summed by every warp for itself
+                run_gt = pg + sh.pre[kWarpBins] + __reduce_add_sync(kFullMask, lane < warp ? sh.wpre_gt[lane] : 0u);
+                run_eq = sh.pre[dT] + __reduce_add_sync(kFullMask, lane < warp ? sh.wpre_eq[lane] : 0u);
             }
             break;
         }
@@ -877,8 +863,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
             const uint32_t pos = threadIdx.x * per + r;
             if (pos < nb) sum += __ldcg(&ghist[width - pos]);
         }
-        uint32_t total;
-        const uint32_t excl = block_exclusive_scan(sum, sh.warp, &total);
+        const uint32_t excl = block_exclusive_scan(sum, sh.warp);
         {
             unsigned long long cum = n_hi + excl;
             if (cum < k && k <= cum + sum) {
@@ -942,7 +927,7 @@ fused_compress_kernel(const uint4* __restrict__ x, int64_t n, unsigned long long
             }
             if (threadIdx.x == 0) st_relaxed_u64(&agg[blockIdx.x], ((unsigned long long)ce << 32) | cg);
             barrier_target += gridDim.x;
-            if (!grid_barrier(&st->barrier, epoch, barrier_target, &sh.ok, spin_max)) {
+            if (!grid_barrier(&st->barrier, epoch, barrier_target, &sh.ok, spin_max, early_word)) {
                 if (threadIdx.x == 0 && dev_status) atomicExch(dev_status, (int)DROPIT_ERR_TIMEOUT);
                 return;
             }
@@ -1420,10 +1405,8 @@ produce_kernel(const uint4* __restrict__ x, uint4* __restrict__ y, int64_t n, un
             }
         }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        cnt_lo += __shfl_xor_sync(kFullMask, cnt_lo, o);
-        cnt_hi += __shfl_xor_sync(kFullMask, cnt_hi, o);
-    }
+    cnt_lo = __reduce_add_sync(kFullMask, cnt_lo);
+    cnt_hi = __reduce_add_sync(kFullMask, cnt_hi);
     if (lane == 0) {
         if (cnt_lo) atomicAdd(&hist[0], cnt_lo);
         sh.w_hi[warp] = cnt_hi;
