@@ -553,76 +553,102 @@ __device__ __noinline__ bool sum_term_by_term(const FusedConvParams& p, const ui
     return true;
 }
 
-// dw[j,c,u,v] (=|+=) sum over splits, in split order within a warp's share and then over the warps.  A block takes 32 rows of
-// one 4-column group; its eight warps share out the splits.  Sums that are not finite are looked at again (sum_term_by_term): the look
-// costs up to 0.5 us (14 x 14), one infinity in the input of 64 -> 64 on 56 x 56 at batch 64 brings the call from 40 us to 2 ms.
-__global__ void __launch_bounds__(32 * kRedWarps, 5)
+// dw[j,c,u,v] (=|+=) sum over splits, in split order within a warp's share and then over the warps.  A block takes 32 rows, four
+// channels and TAPS of the filter's taps (CHANNELS, 1 x 1 filters: TAPS times four channels); its eight warps share out the splits.
+// Sums that are not finite are looked at again (sum_term_by_term), tap by tap.
+// All taps of a channel in one block write whole stretches of dW (144 bytes of a row of 3 x 3 filters, where one tap wrote 4 bytes in
+// every 36), keep nine loads per thread in flight and are a ninth of the blocks.  Per call at batch 64, gamma 0.8: 3 x 3 256 -> 256 on
+// 14 x 14 46.6 -> 38.4 us, 512 -> 512 on 7 x 7 98.7 -> 71.2, stride 2 256 -> 256 on 28 x 28 67.7 -> 59.5.
+template <int TAPS, bool CHANNELS = false>
+__global__ void __launch_bounds__(32 * kRedWarps, TAPS == 1 ? 5 : (TAPS < 9 ? 4 : 2))
 conv_fused_reduce_kernel(const float4* __restrict__ partial, const __grid_constant__ FusedConvParams p, const uint16_t* __restrict__ dy,
                          const uint16_t* __restrict__ values, const uint32_t* __restrict__ mask, const uint32_t* __restrict__ offsets,
                          float* __restrict__ dw, int accumulate) {
-    __shared__ float4 sums[kRedWarps][32];
+    constexpr int kRowFloats = 4 * TAPS, kPitch = kRowFloats + 1;
+    __shared__ float4 sums[kRedWarps][TAPS][32];
+    __shared__ float out[32 * kPitch];                  // [row][channel][tap]
+    __shared__ float part[32 * kRedWarps];
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
-    const int quarters = (min(kBM, p.Cz) + 31) / 32;
+    const int quarters = (min(kBM, p.Cz) + 31) / 32, groups = p.cb / (CHANNELS ? 4 * TAPS : 4), sets = CHANNELS ? 1 : p.R * p.S / TAPS;
     int b = blockIdx.x;
     const int quarter = b % quarters; b /= quarters;
-    const int e4 = b % (p.chunks * 8), tile = b / (p.chunks * 8);
-    const int tiles = p.tiles_c * p.tiles_j;
-    const int c0 = (tile % p.tiles_c) * p.cb, j = (tile / p.tiles_c) * kBM + 32 * quarter + lane;
-    const int col = e4 * 4;
+    const int group = b % groups; b /= groups;
+    const int tap0 = (b % sets) * TAPS, tile = b / sets;
+    const int c = (tile % p.tiles_c) * p.cb + group * (CHANNELS ? 4 * TAPS : 4), j0 = (tile / p.tiles_c) * kBM + 32 * quarter;
     ptx::grid_dependency_wait();                        // the partial tiles come from the kernel before this one
-    if (col >= p.ncols || j - lane >= p.Cz) return;
-    const size_t plane = (size_t)tiles * p.chunks * 8 * kBM;
-    const float4* src = partial + ((size_t)tile * p.chunks * 8 + e4) * kBM + 32 * quarter + lane;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (c >= p.Ca || j0 >= p.Cz) return;
+    const size_t plane = (size_t)p.tiles_c * p.tiles_j * p.chunks * 8 * kBM;
+    const float4* src = partial + ((size_t)tile * p.chunks * 8 + group * (CHANNELS ? TAPS : 1)) * kBM + 32 * quarter + lane;
+    uint32_t at[TAPS];                                  // columns are in the order [v][u][channel]
+#pragma unroll
+    for (int t = 0; t < TAPS; ++t) {
+        const int u = (tap0 + t) / p.S, v = tap0 + t - u * p.S;
+        at[t] = (uint32_t)(CHANNELS ? t : (v * p.R + u) * groups) * kBM;
+    }
+    constexpr int kTapFloats = CHANNELS ? 4 : 1, kChFloats = CHANNELS ? 1 : TAPS;      // how far apart in a row of `out`
+    float4 acc[TAPS];
+#pragma unroll
+    for (int t = 0; t < TAPS; ++t) acc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
     int s = g;
-    for (; s + 3 * kRedWarps < p.splits; s += 4 * kRedWarps) {
-        float4 v[4];
+    if constexpr (TAPS < 9) {
+        for (; s + 3 * kRedWarps < p.splits; s += 4 * kRedWarps) {
+            float4 x[4][TAPS];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = __ldcg(src + (size_t)(s + u * kRedWarps) * plane);
+            for (int w = 0; w < 4; ++w)
 #pragma unroll
-        for (int u = 0; u < 4; ++u) { acc.x += v[u].x; acc.y += v[u].y; acc.z += v[u].z; acc.w += v[u].w; }
+                for (int t = 0; t < TAPS; ++t) x[w][t] = __ldcg(src + (size_t)(s + w * kRedWarps) * plane + at[t]);
+#pragma unroll
+            for (int w = 0; w < 4; ++w)
+#pragma unroll
+                for (int t = 0; t < TAPS; ++t) { acc[t].x += x[w][t].x; acc[t].y += x[w][t].y; acc[t].z += x[w][t].z; acc[t].w += x[w][t].w; }
+        }
     }
     for (; s < p.splits; s += kRedWarps) {
-        const float4 v = __ldcg(src + (size_t)s * plane);
-        acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+        float4 x[TAPS];
+#pragma unroll
+        for (int t = 0; t < TAPS; ++t) x[t] = __ldcg(src + (size_t)s * plane + at[t]);
+#pragma unroll
+        for (int t = 0; t < TAPS; ++t) { acc[t].x += x[t].x; acc[t].y += x[t].y; acc[t].z += x[t].z; acc[t].w += x[t].w; }
     }
-    sums[g][lane] = acc;
+#pragma unroll
+    for (int t = 0; t < TAPS; ++t) sums[g][t][lane] = acc[t];
     __syncthreads();
-    int v = 0, u = 0, c = 0;
-    auto tap = [&]() {                                  // cb is a multiple of 16: the four columns belong to one tap
-        const int n_inst = p.R * p.cb;
-        v = col / n_inst;
-        u = (col % n_inst) / p.cb;
-        c = c0 + col % p.cb;
-    };
     bool odd = false;
-    if (g == 0) {                                       // one warp: with the divisions in all of them 256 -> 256 on 14 x 14 (4608 blocks) took 2.4 us more
+    for (int i = threadIdx.x; i < 32 * TAPS; i += 32 * kRedWarps) {
+        const int t = i >> 5, row = i & 31;
+        float4 a = sums[0][t][row];
 #pragma unroll
         for (int w = 1; w < kRedWarps; ++w) {
-            const float4 o = sums[w][lane];
-            acc.x += o.x; acc.y += o.y; acc.z += o.z; acc.w += o.w;
+            const float4 o = sums[w][t][row];
+            a.x += o.x; a.y += o.y; a.z += o.z; a.w += o.w;
         }
-        tap();
-        odd = !isfinite(acc.x * 0.f + acc.y * 0.f + acc.z * 0.f + acc.w * 0.f) && j < p.Cz;   // one of the four is not finite
+        float* o = out + row * kPitch + t * kTapFloats;
+        o[0] = a.x; o[kChFloats] = a.y; o[2 * kChFloats] = a.z; o[3 * kChFloats] = a.w;
+        odd |= !isfinite(a.x * 0.f + a.y * 0.f + a.z * 0.f + a.w * 0.f) && j0 + row < p.Cz;   // one of the four is not finite
     }
-    odd = __syncthreads_or(odd);
-    float a[4] = {acc.x, acc.y, acc.z, acc.w};
-    if (odd) {
-        tap();
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            float sum;
-            if (c + e < p.Ca && sum_term_by_term(p, dy, values, mask, offsets, j - lane, c + e, u, v, &sums[0][0].x, sum) && !isfinite(a[e]))
-                a[e] = sum;
-        }
-    }
-    if (g == 0 && j < p.Cz) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if (c + e < p.Ca) {
-                float* d = dw + (((size_t)j * p.Ca + c + e) * p.R + u) * p.S + v;
-                *d = accumulate ? *d + a[e] : a[e];
+    if (__syncthreads_or(odd)) {
+        for (int t = 0; t < TAPS; ++t) {
+            float* o = out + lane * kPitch + t * kTapFloats;
+            odd = !isfinite(o[0] * 0.f + o[kChFloats] * 0.f + o[2 * kChFloats] * 0.f + o[3 * kChFloats] * 0.f) && j0 + lane < p.Cz;
+            if (!__syncthreads_or(odd)) continue;
+            const int u = CHANNELS ? 0 : (tap0 + t) / p.S, v = CHANNELS ? 0 : tap0 + t - u * p.S;
+            for (int e = 0; e < 4; ++e) {
+                float sum;
+                const int ch = c + (CHANNELS ? 4 * t : 0) + e;
+                if (ch < p.Ca && sum_term_by_term(p, dy, values, mask, offsets, j0, ch, u, v, part, sum) && g == 0 &&
+                    !isfinite(o[e * kChFloats]))
+                    o[e * kChFloats] = sum;
             }
+            __syncthreads();
+        }
+    }
+    const int taps = p.R * p.S;
+    for (int i = threadIdx.x; i < 32 * kRowFloats; i += 32 * kRedWarps) {
+        const int row = i / kRowFloats, e = i - row * kRowFloats, ch = e / kChFloats;
+        if (j0 + row < p.Cz && c + ch < p.Ca) {
+            float* d = dw + ((size_t)(j0 + row) * p.Ca + c + ch) * taps + tap0 + (e - ch * kChFloats);
+            const float v = out[row * kPitch + e];
+            *d = accumulate ? *d + v : v;
         }
     }
 }
@@ -825,11 +851,18 @@ dropit_status conv_fused_run(const void* dy, const void* values, const void* mas
     }
     dropit_status st = check_launch();
     if (st != DROPIT_OK) return st;
-    const int quarters = ((Cz < kBM ? Cz : kBM) + 31) / 32;
-    cfg.gridDim = dim3((unsigned)(tiles * p.chunks * 8 * quarters));
+    const int quarters = ((Cz < kBM ? Cz : kBM) + 31) / 32, sets = R * S, blocks = tiles * quarters * (p.cb / 4);
+    // as many taps (channels) per block as leave two blocks per SM: 64 -> 64 on 56 x 56 (32 blocks with nine taps, 96 with three) 43.4 /
+    // 41.3 us against 41.4 with one, 16 images of it 21.9 / 19.4 / 19.5; stride 2 128 -> 128 on 56 x 56 (144 / 432) 57.4 / 56.6 / 58.4
+    const int least = 2 * sm_count();
+    const int per = sets == 1 ? (blocks / 4 >= least ? 4 : 1)
+                              : (sets == 9 && blocks >= least ? 9 : (sets % 3 == 0 && blocks * (sets / 3) >= least ? 3 : 1));
+    auto reduce = per == 9 ? conv_fused_reduce_kernel<9> : (per == 4 ? conv_fused_reduce_kernel<4, true>
+                                                                     : (per == 3 ? conv_fused_reduce_kernel<3> : conv_fused_reduce_kernel<1>));
+    cfg.gridDim = dim3((unsigned)(per == 4 ? blocks / 4 : blocks * (sets / per)));
     cfg.blockDim = dim3(32 * kRedWarps);
     cfg.dynamicSmemBytes = 0;
-    if (cudaLaunchKernelEx(&cfg, conv_fused_reduce_kernel, reinterpret_cast<const float4*>(partial), p, reinterpret_cast<const uint16_t*>(dy),
+    if (cudaLaunchKernelEx(&cfg, reduce, reinterpret_cast<const float4*>(partial), p, reinterpret_cast<const uint16_t*>(dy),
                            reinterpret_cast<const uint16_t*>(values), reinterpret_cast<const uint32_t*>(mask), offsets, dw,
                            accumulate) != cudaSuccess) {
         (void)cudaGetLastError();

@@ -48,3 +48,17 @@ def test_nonfinite_values_stay_where_they_are_seen(cuda_device, case):
         assert (got[np.isinf(ref)] == ref[np.isinf(ref)]).all() and (np.isnan(got) == np.isnan(ref)).all(), (y, x)
         # exact bf16 products, fp32 sums: the bound that the other bf16 gradients are held to
         assert max_rel_err(got[finite], ref[finite]) <= 2e-4
+
+
+# the reduction's forms: all nine taps of four channels per block, three taps, 16 channels of a 1 x 1 filter; ragged in both channel counts
+@pytest.mark.parametrize("case", [
+    di.small_conv(2, 299, 6, 6, 250, 3, 3, 1, 1, "bf16", 0.5),
+    di.small_conv(2, 61, 6, 9, 250, 3, 3, 1, 1, "bf16", 0.5),
+    di.small_conv(2, 300, 5, 5, 500, 1, 1, 1, 0, "bf16", 0.5),
+], ids=lambda c: c.name)
+def test_every_form_of_the_reduction(cuda_device, case):
+    cache = dropit.dropit_compress(di.make_x(case).to(cuda_device), case.gamma, "bitmask")
+    args = (di.make_dy(case).to(cuda_device), cache, (case.R, case.S), case.stride, case.pad)
+    dw = dropit.dropit_conv_weight_grad(*args)
+    assert torch.equal(dropit.dropit_conv_weight_grad(*args, out=dw.clone(), accumulate=True), dw + dw)
+    test_nonfinite_values_stay_where_they_are_seen(cuda_device, case)
