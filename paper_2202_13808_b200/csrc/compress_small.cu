@@ -10,8 +10,8 @@
 //      A round is: each CTA writes its row of 128 or 256 counts into every CTA of the cluster, one cluster barrier, and
 //      every CTA finds the same digit from the same rows.  The rows of the CTAs in front of it also give a CTA its
 //      exclusive prefix of keys above and at the threshold, so the ordered compaction needs no further exchange.
-//      fp32, up to 4096 keys that match in their upper 15 bits: their lower halves are sent round once instead, and every CTA
-//      finds both lower digits from that list (4.9 -> 3.8 us of the kernel at 196 Ki normal values, where some 300 match);
+//      fp32, up to 1024 keys that match in their upper 15 bits: their lower halves are sent round once instead, and every CTA
+//      finds both lower digits from that list;
 //   4. element i is retained iff key_i > T, or key_i == T and fewer than q equal keys precede it.  A lane owns 32
 //      consecutive elements, i.e. one mask word; the retained values are moved to the front of the super-block in
 //      shared memory and leave coalesced.
@@ -22,7 +22,7 @@
 // brought these to 26 us and cost all other calls 0.6 to 1 us.
 // Bound by latency: barriers, the trips between CTAs (about 1 us a digit round) and the shared-memory counting.  Measured per
 // call (graph replay, gamma 0.9): bf16 8 Ki / 48 Ki / 196 Ki / 454 Ki elements 6.2 / 6.8 / 8.5 / 11.8 us, where the grid-wide
-// kernel's full histogram takes 60 us at any of these sizes; fp32 48 Ki / 196 Ki / 454 Ki 10.8 / 14.0 / 18.8 us (196 Ki / 512 Ki now 13.0 / 19.2, 14.4 / 20.5 on the same day without the list
+// kernel's full histogram takes 60 us at any of these sizes; fp32 48 Ki / 196 Ki / 454 Ki 10.8 / 14.0 / 18.8 us (48 Ki / 196 Ki / 512 Ki now 10.0 / 12.0 / 17.4, 10.9 / 14.3 / 21.1 on the same day without the list
 // and the programmatic launch, which takes 0.7 us off every call behind a kernel that leaves SMs free), where the three
 // histogram launches and the compaction take 27 us at 600 Ki.  (Counting through a branch per element, only by the warps
 // that own a super-block, and a third barrier per round: 8.0 / 8.9 / 10.3 / 12.8 and 14.2 / 16.9 / 20.7 us.)  At 2^19 bf16
@@ -44,7 +44,11 @@ constexpr uint32_t kTopBins = 1u << 15;
 constexpr int kRowBins = 256;                            // counts of one CTA in one digit round
 constexpr size_t kHistBytes = (size_t)kTopBins * 2;
 constexpr size_t kGatherBytes = (size_t)2 * kMaxCtas * kRowBins * 4;
-constexpr uint32_t kListCap = kMaxCtas * kRowBins;          // a gather buffer, a word per key
+// Most keys that are ranked from a list, a word each.  Keys that lie side by side are found by a few warps, one key after the other: 1000 /
+// 2000 / 4090 of them take 13.6 / 15.7 / 20.3 us at 196 Ki elements, where the two digit rounds take 14.4 / 14.5 / 15.5, and 11.0 / 12.3 / 15.1 at
+// 48 Ki (11.3 / 11.3 / 12.3).  Scattered ones are ahead up to 3000.
+constexpr uint32_t kListCap = 1024;
+static_assert(kListCap <= kMaxCtas * kRowBins, "a gather buffer holds the list");
 
 struct SmallShared {
     uint32_t row[kRowBins];        // this CTA's counts of the current digit
@@ -285,14 +289,20 @@ small_compress_kernel(const uint4* __restrict__ x, uint32_t n, uint32_t k, uint3
         if (m <= kListCap) {
             // Few keys match (some 300 of 196 Ki normal ones): their lower halves go on a list that every CTA holds, this CTA's
             // behind those of the CTAs in front of it, and every CTA finds both digits on its own.  One trip through the cluster
-            // and one pass over the elements instead of two.
-            const uint32_t front = run_eq, list_addr = ptx::smem_u32(gather);        // (the first round's rows are read)
+            // and one pass over the elements instead of two.  They are collected first and sent by all threads: sent by the thread
+            // that finds a key, to one CTA after the other, 300 of 196 Ki took 13.0 us instead of 12.3, 1000 of 512 Ki 20.1 instead of 18.3.
+            const uint32_t front = run_eq;
+            // (this CTA has read the second round's rows, the cluster the first round's; a CTA on its own finds its keys where the list is)
+            uint32_t* found = gather + (ctas > 1 ? kMaxCtas * kRowBins : 0);
             for_each_key([&](uint32_t key, bool exists) {
-                if (exists && (key >> 16) == T) {
-                    const uint32_t to = list_addr + (front + atomicAdd(&sh.listed, 1u)) * 4;
-                    for (uint32_t r = 0; r < ctas; ++r) ptx::st_cluster_u32(ptx::map_shared_to_cta(to, r), key & 0xFFFFu);
-                }
+                if (exists && (key >> 16) == T) found[atomicAdd(&sh.listed, 1u)] = key & 0xFFFFu;
             });
+            if (ctas > 1) {
+                __syncthreads();
+                const uint32_t own = sh.listed;
+                const uint32_t to = ptx::map_shared_to_cta(ptx::smem_u32(gather + front), (uint32_t)warp & (ctas - 1u));    // (a power of two)
+                for (uint32_t i = (uint32_t)warp / ctas * 32 + lane; i < own; i += kThreads / ctas) ptx::st_cluster_u32(to + i * 4, found[i]);
+            }
             if (t < kRowBins) sh.row[t] = 0;
             ptx::cluster_sync_all();
             for (uint32_t i = t; i < m; i += kThreads) red_shared_if(row_addr + (gather[i] >> 8) * 4, 1u, true);
