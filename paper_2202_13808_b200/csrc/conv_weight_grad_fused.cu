@@ -63,6 +63,7 @@ struct FusedConvParams {
     uint32_t seg_magic, segs_magic, ni_magic;        // slot / seg_slots = (slot * seg_magic) >> 20 and so on
     uint32_t w_magic;                                // pixel / W
     uint32_t cores_magic, yb_magic, step_magic;      // core / cores, row / yb, dY task / dY steps
+    uint32_t s_magic;                                // tap / S
     int x_bytes, dy_bytes, stages;                   // per pipeline stage
     int vec;                                         // pixels per copy of dY that the row length allows: 8, 4, 2, 1
     int dy_warp0, dy_idle, dy_extra;                 // see next_dy: first warp without a task of X in the last round, their number, their share
@@ -569,21 +570,24 @@ conv_fused_reduce_kernel(const float4* __restrict__ partial, const __grid_consta
     __shared__ float out[32 * kPitch];                  // [row][channel][tap]
     __shared__ float part[32 * kRedWarps];
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
-    const int quarters = (min(kBM, p.Cz) + 31) / 32, groups = p.cb / (CHANNELS ? 4 * TAPS : 4), sets = CHANNELS ? 1 : p.R * p.S / TAPS;
-    int b = blockIdx.x;
-    const int quarter = b % quarters; b /= quarters;
-    const int group = b % groups; b /= groups;
-    const int tap0 = (b % sets) * TAPS, tile = b / sets;
-    const int c = (tile % p.tiles_c) * p.cb + group * (CHANNELS ? 4 * TAPS : 4), j0 = (tile / p.tiles_c) * kBM + 32 * quarter;
+    // Blocks: (32 rows of a tile, groups of channels and sets of taps, tile).  The columns of the partial tiles are in the order [v][u][channel]:
+    // with one tap per block, or none but channels, blockIdx.y counts them as they lie.  What else the block's number says is worked out behind
+    // the loads: with the divisions in front of them calls of 8 images took 14.7 instead of 13.6 us (64 -> 64 on 56 x 56), 13.1 / 11.8 (40 -> 72
+    // on 23 x 23), 32.7 / 28.7 (512 -> 512 on 7 x 7).
+    const int groups = p.cb / (CHANNELS ? 4 * TAPS : 4), quarter = blockIdx.x, tile = blockIdx.z;
+    const int tap_set = TAPS == 3 ? (int)blockIdx.y / groups : 0;      // (nine taps are all there are)
+    const uint32_t first = CHANNELS ? blockIdx.y * TAPS : blockIdx.y - (uint32_t)(tap_set * groups);
     ptx::grid_dependency_wait();                        // the partial tiles come from the kernel before this one
-    if (c >= p.Ca || j0 >= p.Cz) return;
     const size_t plane = (size_t)p.tiles_c * p.tiles_j * p.chunks * 8 * kBM;
-    const float4* src = partial + ((size_t)tile * p.chunks * 8 + group * (CHANNELS ? TAPS : 1)) * kBM + 32 * quarter + lane;
-    uint32_t at[TAPS];                                  // columns are in the order [v][u][channel]
+    const float4* src = partial + ((size_t)tile * p.chunks * 8 + first) * kBM + 32 * quarter + lane;
+    uint32_t at[TAPS];
 #pragma unroll
     for (int t = 0; t < TAPS; ++t) {
-        const int u = (tap0 + t) / p.S, v = tap0 + t - u * p.S;
-        at[t] = (uint32_t)(CHANNELS ? t : (v * p.R + u) * groups) * kBM;
+        if constexpr (TAPS == 9) at[t] = (uint32_t)(t % 3 * 3 + t / 3) * groups * kBM;
+        else if constexpr (TAPS == 3) {
+            const uint32_t tap = tap_set * TAPS + t, u = quotient(tap, p.s_magic), v = tap - u * p.S;
+            at[t] = (v * p.R + u) * groups * kBM;
+        } else at[t] = (uint32_t)t * kBM;
     }
     constexpr int kTapFloats = CHANNELS ? 4 : 1, kChFloats = CHANNELS ? 1 : TAPS;      // how far apart in a row of `out`
     float4 acc[TAPS];
@@ -612,6 +616,17 @@ conv_fused_reduce_kernel(const float4* __restrict__ partial, const __grid_consta
     }
 #pragma unroll
     for (int t = 0; t < TAPS; ++t) sums[g][t][lane] = acc[t];
+    int group = first, tap0 = tap_set * TAPS;
+    if constexpr (TAPS == 1) {
+        const int column = group / groups, v = column / p.R;
+        group -= column * groups;
+        tap0 = (column - v * p.R) * p.S + v;
+    } else if constexpr (CHANNELS) {
+        group = blockIdx.y;
+    }
+    const int tile_j = tile / p.tiles_c, j0 = tile_j * kBM + 32 * quarter;
+    const int c = (tile - tile_j * p.tiles_c) * p.cb + group * (CHANNELS ? 4 * TAPS : 4);
+    if (c >= p.Ca || j0 >= p.Cz) return;                // (what such a block has read is not used)
     __syncthreads();
     bool odd = false;
     for (int i = threadIdx.x; i < 32 * TAPS; i += 32 * kRedWarps) {
@@ -756,6 +771,7 @@ bool make_fused_conv_plan(FusedConvParams& p, int B, int Ca, int H, int W, int C
     p.segs_magic = magic_of((uint32_t)p.segs);
     p.ni_magic = magic_of((uint32_t)p.ni);
     p.w_magic = magic_of((uint32_t)W);
+    p.s_magic = magic_of((uint32_t)S);
     p.cores_magic = magic_of((uint32_t)p.cores);
     p.yb_magic = magic_of((uint32_t)p.yb);
     p.step_magic = magic_of((uint32_t)((cores_total + 3) / 4));
@@ -859,7 +875,7 @@ dropit_status conv_fused_run(const void* dy, const void* values, const void* mas
                               : (sets == 9 && blocks >= least ? 9 : (sets % 3 == 0 && blocks * (sets / 3) >= least ? 3 : 1));
     auto reduce = per == 9 ? conv_fused_reduce_kernel<9> : (per == 4 ? conv_fused_reduce_kernel<4, true>
                                                                      : (per == 3 ? conv_fused_reduce_kernel<3> : conv_fused_reduce_kernel<1>));
-    cfg.gridDim = dim3((unsigned)(per == 4 ? blocks / 4 : blocks * (sets / per)));
+    cfg.gridDim = dim3((unsigned)quarters, (unsigned)(per == 4 ? p.cb / 16 : p.cb / 4 * (sets / per)), (unsigned)tiles);
     cfg.blockDim = dim3(32 * kRedWarps);
     cfg.dynamicSmemBytes = 0;
     if (cudaLaunchKernelEx(&cfg, reduce, reinterpret_cast<const float4*>(partial), p, reinterpret_cast<const uint16_t*>(dy),
