@@ -72,6 +72,8 @@ struct FusedConvParams {
     int ncols, chunks;                               // accumulator columns R * S * cb; 32-column chunks
     uint32_t tmem_cols;
     uint32_t k;
+    const uint16_t *dy, *values;                     // for mend_nonfinite
+    const uint32_t *mask, *offsets;
     uint2 pairs[kMaxPairs];                          // low descriptor words of a band's K = 16 steps, relative to the stage: dY, X
 };
 
@@ -499,76 +501,163 @@ conv_wg_fused_kernel(const uint16_t* __restrict__ dy, const uint16_t* __restrict
 // Number of retained elements in front of flat index e; `kept`: whether e is one of them.
 __device__ __forceinline__ uint32_t retained_before(const uint32_t* __restrict__ mask, const uint32_t* __restrict__ offsets, uint32_t e,
                                                     bool& kept) {
-    const uint32_t w = e >> 5, bit = 1u << (e & 31u);
-    uint32_t pos = __ldg(offsets + (e >> 7));
-    for (uint32_t i = w & ~3u; i < w; ++i) pos += __popc(__ldg(mask + i));
-    const uint32_t word = __ldg(mask + w);
+    const uint32_t w = e >> 5, bit = 1u << (e & 31u), word = __ldg(mask + w);
+    uint32_t pos = __ldg(offsets + (e >> 7)) + __popc(word & (bit - 1u));
+#pragma unroll
+    for (uint32_t i = 1; i < 4; ++i)
+        if ((w & 3u) >= i) pos += __popc(__ldg(mask + (w - i)));
     kept = (word & bit) != 0;
-    return pos + __popc(word & (bit - 1u));
+    return pos;
 }
 
 constexpr int kRedWarps = 8;
 
-// dW[j0 + lane, c, u, v] term by term, for a channel that holds an infinity or a NaN (false: it holds none, nothing is computed).  The
-// K steps cover whole 8-pixel groups; behind a row's last output and behind the band's last group dY is zero there, but X may be a
-// pixel that the tap (u, v) does not see, and zero times infinity is NaN.  Called by the whole block; `part`: a float per thread.
-// Positions are shared out among the warps in runs of 32, whose pixels the lanes look up; then a lane is an output channel.
-__device__ __noinline__ bool sum_term_by_term(const FusedConvParams& p, const uint16_t* __restrict__ dy, const uint16_t* __restrict__ values,
-                                              const uint32_t* __restrict__ mask, const uint32_t* __restrict__ offsets, int j0, int c, int u,
-                                              int v, float* part, float& sum) {
+// Where the sums of a block of the reduction go, and its output: 32 rows of dW from j0 on, TAPS taps from tap0 on of four channels from c on
+// (CHANNELS, 1 x 1 filters: 4 * TAPS channels).
+template <int FORM_TAPS, bool CHANNELS>
+struct RedBlock {
+    static constexpr int kTaps = CHANNELS ? 1 : FORM_TAPS, kChannels = CHANNELS ? 4 * FORM_TAPS : 4;
+    static constexpr int kRowFloats = kTaps * kChannels, kPitch = kRowFloats + 1;      // a row of the sums, [channel][tap]
+    int c, j0, tap0;
+    __device__ __forceinline__ void store(const FusedConvParams& p, const float* sums, float* __restrict__ dw, int accumulate) const {
+        const int taps = p.R * p.S;
+        for (int i = threadIdx.x; i < 32 * kRowFloats; i += 32 * kRedWarps) {
+            const int row = i / kRowFloats, e = i - row * kRowFloats, ch = e / kTaps;
+            if (j0 + row < p.Cz && c + ch < p.Ca) {
+                float* d = dw + ((size_t)(j0 + row) * p.Ca + c + ch) * taps + tap0 + (e - ch * kTaps);
+                const float v = sums[row * kPitch + e];
+                *d = accumulate ? *d + v : v;
+            }
+        }
+    }
+};
+
+// The channels c .. c + chs - 1 (chs < 32) that hold an infinity or a NaN, a bit each.  Called by the whole block; a warp takes an image's
+// channels, whose values follow one another in the cache, in one go (lane i: the values in front of channel c + i).
+__device__ __forceinline__ uint32_t nonfinite_channels(const FusedConvParams& p, int c, int chs, uint32_t* found) {
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
-    const uint32_t plane = (uint32_t)p.H * p.W, total = (uint32_t)p.B * p.Ca * plane, dy_plane = (uint32_t)p.Ho * p.Wo;
-    bool kept, found = false;
+    const uint32_t plane = (uint32_t)p.H * p.W, total = (uint32_t)p.B * p.Ca * plane;
+    if (threadIdx.x == 0) *found = 0;
+    __syncthreads();
     for (int n = g; n < p.B; n += kRedWarps) {
-        const uint32_t e = ((uint32_t)n * p.Ca + c) * plane;
-        const uint32_t first = retained_before(mask, offsets, e, kept);
-        const uint32_t last = e + plane < total ? min(retained_before(mask, offsets, e + plane, kept), p.k) : p.k;
-        for (uint32_t i = first + lane; i < last; i += 32) found |= (__ldg(values + i) & 0x7F80u) == 0x7F80u;
-    }
-    if (!__syncthreads_or(found)) return false;
-    float acc = 0.f;
-    const uint32_t positions = (uint32_t)p.B * dy_plane;
-    for (uint32_t q0 = g * 32; q0 < positions; q0 += 32 * kRedWarps) {
-        const uint32_t q = q0 + lane, n = q / dy_plane, at = q - n * dy_plane;
-        const int iy = (int)(at / p.Wo) * p.stride + u - p.pad, ix = (int)(at % p.Wo) * p.stride + v - p.pad;
-        const unsigned long long from = (unsigned long long)n * p.Cz * dy_plane + at;
-        float x = 0.f;
-        kept = false;
-        if (q < positions && iy >= 0 && iy < p.H && ix >= 0 && ix < p.W) {
-            const uint32_t pos = retained_before(mask, offsets, ((n * p.Ca + c) * p.H + iy) * p.W + ix, kept);
-            kept = kept && pos < p.k;
-            if (kept) x = __uint_as_float((uint32_t)__ldg(values + pos) << 16);
-        }
-        for (uint32_t todo = __ballot_sync(kFullMask, kept); todo; todo &= todo - 1) {
-            const int b = __ffs(todo) - 1;
-            const float xb = __shfl_sync(kFullMask, x, b);
-            const unsigned long long fb = __shfl_sync(kFullMask, from, b);
-            if (j0 + lane < p.Cz) acc = fmaf(__uint_as_float((uint32_t)__ldg(dy + fb + (unsigned long long)(j0 + lane) * dy_plane) << 16), xb, acc);
+        const uint32_t e = ((uint32_t)n * p.Ca + c + min(lane, chs)) * plane;
+        bool kept;
+        const uint32_t at = e < total ? min(retained_before(p.mask, p.offsets, e, kept), p.k) : p.k;
+        const uint32_t first = __shfl_sync(kFullMask, at, 0), last = __shfl_sync(kFullMask, at, chs);
+        bool odd = false;
+        for (uint32_t i = first + lane; i < last; i += 32) odd |= (__ldg(p.values + i) & 0x7F80u) == 0x7F80u;
+        if (!__any_sync(kFullMask, odd)) continue;
+        for (int ch = 0; ch < chs; ++ch) {
+            const uint32_t from = __shfl_sync(kFullMask, at, ch), to = __shfl_sync(kFullMask, at, ch + 1);
+            odd = false;
+            for (uint32_t i = from + lane; i < to; i += 32) odd |= (__ldg(p.values + i) & 0x7F80u) == 0x7F80u;
+            if (odd) atomicOr(found, 1u << ch);
         }
     }
-    part[threadIdx.x] = acc;
     __syncthreads();
-    sum = 0.f;
-    for (int w = 0; w < kRedWarps; ++w) sum += part[w * 32 + lane];
+    return *found;
+}
+
+// The sums in `out` ([row][channel][tap]) that are not finite, of the channels that hold an infinity or a NaN: added up again term by term.
+// The K steps cover whole 8-pixel groups; behind a row's last output and behind the band's last group dY is zero there, but X may be a
+// pixel that the tap does not see, and zero times infinity is NaN.
+// A thread looks up what its pixel of dY meets at each tap, a round of 256 pixels ahead; then a warp goes over the 256 pixels with four rows of
+// dY, whose loads are contiguous.  A channel is searched once for all of its taps.  64 images, gamma 0.8, nothing odd / one infinity in
+// X / one NaN in dY: 256 -> 256 on 14 x 14 34 / 297 / 40 us (with the taps one after the other, each searching, and a lane per row of dY,
+// whose loads are 32 sectors: 1369 / 359; the same in nine times as many blocks, one per tap: 222 / 98); 512 -> 512 on 7 x 7 54 / 114 / 60
+// (481 / 300; 138 / 144); 64 -> 64 on 56 x 56, one tap per block either way, 36 / 2390 / 94 (2330 / 151).
+// What bounds it: two barriers and the trips to L2 in every round, on the few SMs that have such a channel.
+// Called by the whole block, whose sums it stores: it is not part of the kernel's own code, whose registers it would take, and nothing of that is
+// kept across the call.
+template <int TAPS>
+struct MendShared {
+    uint32_t x[kRedWarps][TAPS][32];       // bf16 in the upper half; bit 0: retained
+    size_t from[kRedWarps * 32];           // the pixel in the first row of dY
+    uint32_t found;
+};
+template <typename Block>
+__device__ __noinline__ void mend_nonfinite(const FusedConvParams& p, const Block blk, float* out, MendShared<Block::kTaps>& sh,
+                                            float* __restrict__ dw, int accumulate) {
+    constexpr int TAPS = Block::kTaps, kRows = 32 / kRedWarps;
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, c = blk.c;
+    const uint32_t dy_plane = (uint32_t)p.Ho * p.Wo, pixels = (uint32_t)p.B * dy_plane;
+    const int j = min(blk.j0 + g * kRows, p.Cz - 1), more = p.Cz - 1 - j;       // (behind the last row: not used)
+    for (uint32_t todo = nonfinite_channels(p, c, min(Block::kChannels, p.Ca - c), &sh.found); todo; todo &= todo - 1u) {
+        const int ch = __ffs(todo) - 1;
+        float acc[kRows][TAPS];
+#pragma unroll
+        for (int r = 0; r < kRows; ++r)
+#pragma unroll
+            for (int t = 0; t < TAPS; ++t) acc[r][t] = 0.f;
+        uint32_t met[TAPS];                                 // looked up one round ahead
+        size_t at_dy;
+        auto look_up = [&](uint32_t q0) {
+            const uint32_t q = min(q0 + threadIdx.x, pixels - 1u), n = q / dy_plane, at = q - n * dy_plane;
+            const int y = (int)(at / p.Wo) * p.stride - p.pad, x = (int)(at % p.Wo) * p.stride - p.pad;
+            int u = blk.tap0 / p.S, v = blk.tap0 - u * p.S;
+            at_dy = (size_t)n * p.Cz * dy_plane + at;
+#pragma unroll
+            for (int t = 0; t < TAPS; ++t) {
+                const int iy = y + u, ix = x + v;
+                const bool in = q0 + threadIdx.x < pixels && iy >= 0 && iy < p.H && ix >= 0 && ix < p.W;
+                bool kept;
+                const uint32_t pos = retained_before(p.mask, p.offsets, in ? ((n * p.Ca + c + ch) * p.H + iy) * p.W + ix : 0u, kept);
+                const uint32_t value = __ldg(p.values + min(pos, p.k - 1u));
+                met[t] = in && kept && pos < p.k ? value << 16 | 1u : 0u;
+                if (++v == p.S) { v = 0; ++u; }
+            }
+        };
+        look_up(0);
+        for (uint32_t q0 = 0; q0 < pixels; q0 += 32 * kRedWarps) {
+            __syncthreads();                                // the pixels before these are done with
+            sh.from[threadIdx.x] = at_dy;
+#pragma unroll
+            for (int t = 0; t < TAPS; ++t) sh.x[g][t][lane] = met[t];
+            __syncthreads();
+            if (q0 + 32 * kRedWarps < pixels) look_up(q0 + 32 * kRedWarps);
+#pragma unroll(TAPS == 1 ? 2 : 4)
+            for (int w = 0; w < kRedWarps; ++w) {
+                const uint16_t* src = p.dy + sh.from[w * 32 + lane] + (size_t)j * dy_plane;
+                float d[kRows];
+#pragma unroll
+                for (int r = 0; r < kRows; ++r) d[r] = __uint_as_float((uint32_t)__ldg(src + (size_t)min(r, more) * dy_plane) << 16);
+#pragma unroll
+                for (int t = 0; t < TAPS; ++t) {
+                    const uint32_t xv = sh.x[w][t][lane];
+                    if (xv & 1u) {
+#pragma unroll
+                        for (int r = 0; r < kRows; ++r) acc[r][t] = fmaf(d[r], __uint_as_float(xv & 0xFFFF0000u), acc[r][t]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < kRows; ++r)
+#pragma unroll
+            for (int t = 0; t < TAPS; ++t) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) acc[r][t] += __shfl_xor_sync(kFullMask, acc[r][t], o);
+                float* sum = out + (g * kRows + r) * Block::kPitch + ch * TAPS + t;
+                if (lane == 0 && !isfinite(*sum)) *sum = acc[r][t];
+            }
+    }
     __syncthreads();
-    return true;
+    blk.store(p, out, dw, accumulate);
 }
 
 // dw[j,c,u,v] (=|+=) sum over splits, in split order within a warp's share and then over the warps.  A block takes 32 rows, four
 // channels and TAPS of the filter's taps (CHANNELS, 1 x 1 filters: TAPS times four channels); its eight warps share out the splits.
-// Sums that are not finite are looked at again (sum_term_by_term), tap by tap.
+// Sums that are not finite are looked at again (mend_nonfinite).
 // All taps of a channel in one block write whole stretches of dW (144 bytes of a row of 3 x 3 filters, where one tap wrote 4 bytes in
 // every 36), keep nine loads per thread in flight and are a ninth of the blocks.  Per call at batch 64, gamma 0.8: 3 x 3 256 -> 256 on
 // 14 x 14 46.6 -> 38.4 us, 512 -> 512 on 7 x 7 98.7 -> 71.2, stride 2 256 -> 256 on 28 x 28 67.7 -> 59.5.
 template <int TAPS, bool CHANNELS = false>
 __global__ void __launch_bounds__(32 * kRedWarps, TAPS == 1 ? 5 : (TAPS < 9 ? 4 : 2))
-conv_fused_reduce_kernel(const float4* __restrict__ partial, const __grid_constant__ FusedConvParams p, const uint16_t* __restrict__ dy,
-                         const uint16_t* __restrict__ values, const uint32_t* __restrict__ mask, const uint32_t* __restrict__ offsets,
-                         float* __restrict__ dw, int accumulate) {
-    constexpr int kRowFloats = 4 * TAPS, kPitch = kRowFloats + 1;
+conv_fused_reduce_kernel(const float4* __restrict__ partial, const __grid_constant__ FusedConvParams p, float* __restrict__ dw, int accumulate) {
+    using Block = RedBlock<TAPS, CHANNELS>;
+    constexpr int kPitch = Block::kPitch;
     __shared__ float4 sums[kRedWarps][TAPS][32];
     __shared__ float out[32 * kPitch];                  // [row][channel][tap]
-    __shared__ float part[32 * kRedWarps];
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
     // Blocks: (32 rows of a tile, groups of channels and sets of taps, tile).  The columns of the partial tiles are in the order [v][u][channel]:
     // with one tap per block, or none but channels, blockIdx.y counts them as they lie.  What else the block's number says is worked out behind
@@ -641,37 +730,20 @@ conv_fused_reduce_kernel(const float4* __restrict__ partial, const __grid_consta
         o[0] = a.x; o[kChFloats] = a.y; o[2 * kChFloats] = a.z; o[3 * kChFloats] = a.w;
         odd |= !isfinite(a.x * 0.f + a.y * 0.f + a.z * 0.f + a.w * 0.f) && j0 + row < p.Cz;   // one of the four is not finite
     }
+    const Block blk = {c, j0, tap0};
     if (__syncthreads_or(odd)) {
-        for (int t = 0; t < TAPS; ++t) {
-            float* o = out + lane * kPitch + t * kTapFloats;
-            odd = !isfinite(o[0] * 0.f + o[kChFloats] * 0.f + o[2 * kChFloats] * 0.f + o[3 * kChFloats] * 0.f) && j0 + lane < p.Cz;
-            if (!__syncthreads_or(odd)) continue;
-            const int u = CHANNELS ? 0 : (tap0 + t) / p.S, v = CHANNELS ? 0 : tap0 + t - u * p.S;
-            for (int e = 0; e < 4; ++e) {
-                float sum;
-                const int ch = c + (CHANNELS ? 4 * t : 0) + e;
-                if (ch < p.Ca && sum_term_by_term(p, dy, values, mask, offsets, j0, ch, u, v, part, sum) && g == 0 &&
-                    !isfinite(o[e * kChFloats]))
-                    o[e * kChFloats] = sum;
-            }
-            __syncthreads();
-        }
+        using Mend = MendShared<Block::kTaps>;
+        static_assert(sizeof(Mend) <= sizeof(sums), "");
+        mend_nonfinite(p, blk, out, reinterpret_cast<Mend&>(sums), dw, accumulate);      // (the sums have been read)
+        return;
     }
-    const int taps = p.R * p.S;
-    for (int i = threadIdx.x; i < 32 * kRowFloats; i += 32 * kRedWarps) {
-        const int row = i / kRowFloats, e = i - row * kRowFloats, ch = e / kChFloats;
-        if (j0 + row < p.Cz && c + ch < p.Ca) {
-            float* d = dw + ((size_t)(j0 + row) * p.Ca + c + ch) * taps + tap0 + (e - ch * kChFloats);
-            const float v = out[row * kPitch + e];
-            *d = accumulate ? *d + v : v;
-        }
-    }
+    blk.store(p, out, dw, accumulate);
 }
 
 size_t stage_bytes_of(FusedConvParams& p) {
     const size_t row_pitch = (size_t)(p.cb / 8) * p.gp * 16;
     // With an odd number of 8-pixel groups the last K = 16 step reads one more K row than the band has: zeros in dY,
-    // pixels or zeros in X (sum_term_by_term mends what infinities make of that).  With 64 channels of dY per band the instruction's rows 64..127 are the next 8-pixel group
+    // pixels or zeros in X (mend_nonfinite mends what infinities make of that).  With 64 channels of dY per band the instruction's rows 64..127 are the next 8-pixel group
     // (their results are not used).
     const int odd = (p.ni * p.yb * p.cores) & 1;
     const size_t x = (size_t)(p.ni * p.x_rows + odd * p.row_step) * row_pitch * p.planes;
@@ -878,9 +950,11 @@ dropit_status conv_fused_run(const void* dy, const void* values, const void* mas
     cfg.gridDim = dim3((unsigned)quarters, (unsigned)(per == 4 ? p.cb / 16 : p.cb / 4 * (sets / per)), (unsigned)tiles);
     cfg.blockDim = dim3(32 * kRedWarps);
     cfg.dynamicSmemBytes = 0;
-    if (cudaLaunchKernelEx(&cfg, reduce, reinterpret_cast<const float4*>(partial), p, reinterpret_cast<const uint16_t*>(dy),
-                           reinterpret_cast<const uint16_t*>(values), reinterpret_cast<const uint32_t*>(mask), offsets, dw,
-                           accumulate) != cudaSuccess) {
+    p.dy = reinterpret_cast<const uint16_t*>(dy);
+    p.values = reinterpret_cast<const uint16_t*>(values);
+    p.mask = reinterpret_cast<const uint32_t*>(mask);
+    p.offsets = offsets;
+    if (cudaLaunchKernelEx(&cfg, reduce, reinterpret_cast<const float4*>(partial), p, dw, accumulate) != cudaSuccess) {
         (void)cudaGetLastError();
         return DROPIT_ERR_CUDA;
     }

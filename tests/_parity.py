@@ -56,3 +56,16 @@ def max_rel_err(got: np.ndarray, ref: np.ndarray) -> float:
     if denom == 0:
         return float(np.abs(got).max())
     return float(np.abs(got.astype(np.float64) - ref).max() / denom)
+
+
+def conv_weight_grad_f64(dy, a, kernel_size, stride, pad):
+    """dW of the dense tensors dy and a in fp64, tap by tap over the pixels that the tap sees (zeros in the padding)."""
+    R, S = kernel_size
+    ho, wo = dy.shape[2:]
+    a = torch.nn.functional.pad(a.double(), (pad, pad, pad, pad))
+    dw = torch.empty(dy.shape[1], a.shape[1], R, S, dtype=torch.float64, device=dy.device)
+    for u in range(R):
+        for v in range(S):
+            seen = a[:, :, u:u + (ho - 1) * stride + 1:stride, v:v + (wo - 1) * stride + 1:stride]
+            dw[:, :, u, v] = torch.einsum("njyx,ncyx->jc", dy.double(), seen)
+    return dw
