@@ -683,15 +683,17 @@ conv_fused_reduce_kernel(const float4* __restrict__ partial, const __grid_consta
 #pragma unroll
     for (int t = 0; t < TAPS; ++t) acc[t] = make_float4(0.f, 0.f, 0.f, 0.f);
     int s = g;
-    if constexpr (TAPS < 9) {
-        for (; s + 3 * kRedWarps < p.splits; s += 4 * kRedWarps) {
-            float4 x[4][TAPS];
+    // Splits whose loads are in flight: as many as fit the registers; the 16 channels' form hardly ever has more than two for a warp
+    constexpr int kDeep = TAPS == 1 ? 4 : (TAPS == 3 ? 2 : 1);
+    if constexpr (kDeep > 1) {
+        for (; s + (kDeep - 1) * kRedWarps < p.splits; s += kDeep * kRedWarps) {
+            float4 x[kDeep][TAPS];
 #pragma unroll
-            for (int w = 0; w < 4; ++w)
+            for (int w = 0; w < kDeep; ++w)
 #pragma unroll
                 for (int t = 0; t < TAPS; ++t) x[w][t] = __ldcg(src + (size_t)(s + w * kRedWarps) * plane + at[t]);
 #pragma unroll
-            for (int w = 0; w < 4; ++w)
+            for (int w = 0; w < kDeep; ++w)
 #pragma unroll
                 for (int t = 0; t < TAPS; ++t) { acc[t].x += x[w][t].x; acc[t].y += x[w][t].y; acc[t].z += x[w][t].z; acc[t].w += x[w][t].w; }
         }
