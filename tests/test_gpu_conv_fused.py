@@ -5,7 +5,7 @@ import torch
 import dropit_inputs as di
 import oracle
 import paper_2202_13808_b200 as dropit
-from _parity import max_rel_err, oracle_cache
+from _parity import conv_weight_grad_f64, max_rel_err, oracle_cache
 
 pytestmark = pytest.mark.gpu
 
@@ -72,3 +72,33 @@ def test_strided_pointwise_either_side_of_the_line(cuda_device, batch):
     a = dropit.dropit_decompress(cache)[:, :, ::2, ::2].double()
     ref = torch.einsum("njyx,ncyx->jc", dy.double(), a)
     assert float((dw[:, :, 0, 0].double() - ref).abs().max()) <= 2e-4 * float(ref.abs().max())
+
+
+# The forms of the reduction with more splits than a warp takes at once: three taps (all filters that have them in threes), nine taps, 16
+# channels of a 1 x 1 filter, one tap.  (case, columns of a tile's sums in chunks of 32, tiles, splits at least)
+SPLITS = [
+    (di.small_conv(64, 120, 28, 28, 120, 3, 3, 1, 1, "bf16", 0.8), 14, 3, 33),
+    (di.small_conv(64, 300, 9, 9, 100, 1, 3, 1, 1, "bf16", 0.8), 15, 2, 33),
+    (di.small_conv(64, 300, 9, 9, 100, 3, 1, 1, 1, "bf16", 0.8), 8, 4, 25),
+    (di.small_conv(64, 300, 9, 9, 100, 2, 3, 1, 1, "bf16", 0.8), 15, 4, 25),
+    (di.small_conv(64, 300, 9, 9, 100, 3, 2, 2, 1, "bf16", 0.8), 15, 4, 25),
+    (di.small_conv(24, 250, 14, 14, 250, 3, 3, 1, 1, "bf16", 0.8), 14, 12, 9),
+    (di.small_conv(64, 250, 15, 15, 600, 1, 1, 1, 0, "bf16", 0.8), 8, 5, 17),
+    (di.small_conv(64, 60, 28, 28, 60, 3, 3, 1, 1, "bf16", 0.8), 9, 2, 33),
+]
+
+
+@pytest.mark.parametrize("case,chunks,tiles,splits", SPLITS, ids=lambda v: getattr(v, "name", str(v)))
+def test_many_splits_are_added_up(cuda_device, case, chunks, tiles, splits):
+    size = dropit.dropit_conv_weight_grad_workspace(case.B, case.Ca, case.H, case.W, case.Cz, case.R, case.S, case.stride, case.pad, dropit.BF16,
+                                                    dropit.FMT_BITMASK, cuda_device)
+    assert size % (chunks * 32 * 128 * 4 * tiles) == 0 and size // (chunks * 32 * 128 * 4 * tiles) >= splits
+    cache = dropit.dropit_compress(di.make_x(case).to(cuda_device), case.gamma, "bitmask")
+    dy = di.make_dy(case).to(cuda_device)
+    ref = conv_weight_grad_f64(dy, dropit.dropit_decompress(cache), (case.R, case.S), case.stride, case.pad)
+    args = (dy, cache, (case.R, case.S), case.stride, case.pad)
+    dw = dropit.dropit_conv_weight_grad(*args)
+    assert float((dw.double() - ref).abs().max()) <= 2e-4 * float(ref.abs().max())
+    twice = dropit.dropit_conv_weight_grad(*args, out=dw.clone(), accumulate=True)
+    dropit.check_device_status(cuda_device)
+    assert torch.equal(twice, dw + dw)
