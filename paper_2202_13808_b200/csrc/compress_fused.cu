@@ -19,7 +19,7 @@
 //           A lane owns 32 consecutive elements of a super-block; retained values are staged per warp and leave in
 //           aligned 16-byte pieces.
 // Bound by issue in both streaming phases (some 250 warp instructions per super-block each) on top of 10 us of fixed steps
-// (sample 4.5, barrier 2, phase 2 2.5).  What the one threshold, the flags gathered by a prmt with msb replication, the
+// (sample 3.8, a CTA's sums 0.5 to 0.9, barrier 1.5 to 2, column sums 1.2 to 1.8, T 2.6, prefixes 0.45).  What the one threshold, the flags gathered by a prmt with msb replication, the
 // walk of dense words from registers and the rarer flushes gave, per call over rotating inputs (graph replay, gamma 0.9):
 // 12608 x 768 20.7 -> 19.3 us, 12608 x 3072 42.3 -> 39.1; 32768 x 768 at 0.5 48.3 -> 40.9; 32768 x 3072 at 0.8 96 -> 89,
 // at 0.5 134 -> 112 us.  The sample's additions to shared memory take turns at the bank: half as many of them (8 Ki elements

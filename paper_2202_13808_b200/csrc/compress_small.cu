@@ -21,12 +21,12 @@
 // 31.6 against 27.2 us, all 39.7 against 26.1; none 21.2 against 26.0).  Counting the commonest key of a sample in registers, not zero,
 // brought these to 26 us and cost all other calls 0.6 to 1 us.
 // Bound by latency: barriers, the trips between CTAs (about 1 us a digit round) and the shared-memory counting.  Measured per
-// call (graph replay, gamma 0.9): bf16 8 Ki / 48 Ki / 196 Ki / 454 Ki elements 6.2 / 6.8 / 8.5 / 11.8 us, where the grid-wide
-// kernel's full histogram takes 60 us at any of these sizes; fp32 48 Ki / 196 Ki / 454 Ki 10.8 / 14.0 / 18.8 us (48 Ki / 196 Ki / 512 Ki now 10.0 / 12.0 / 17.4, 10.9 / 14.3 / 21.1 on the same day without the list
-// and the programmatic launch, which takes 0.7 us off every call behind a kernel that leaves SMs free), where the three
+// call (graph replay, gamma 0.9): bf16 8 Ki / 48 Ki / 196 Ki / 512 Ki elements 5.8 / 6.3 / 8.0 / 11.9 us, where the grid-wide
+// kernel's full histogram takes 60 us at any of these sizes; fp32 9.3 / 9.9 / 12.0 / 17.5 us (9.8 / 10.9 / 13.9 / 20.3 without the list and
+// the programmatic launch, which takes 0.7 us off every call behind a kernel that leaves SMs free), where the three
 // histogram launches and the compaction take 27 us at 600 Ki.  (Counting through a branch per element, only by the warps
 // that own a super-block, and a third barrier per round: 8.0 / 8.9 / 10.3 / 12.8 and 14.2 / 16.9 / 20.7 us.)  At 2^19 bf16
-// elements (12.5 us) the sampled grid-wide kernel (15.8 us) is about to overtake: two super-blocks per warp measured 17.4 us at
+// elements (11.9 us) the sampled grid-wide kernel (13.2 us) is about to overtake: two super-blocks per warp measured 17.4 us at
 // 800 Ki against its 16.1, so there the line lies.
 #include "common.cuh"
 #include "sm100_ptx.cuh"

@@ -21,8 +21,9 @@ dropit_status conv_tc_run(const void* dy, const void* values, const void* meta, 
 // Straight from a bitmask cache (bf16, filters of up to 3 x 3), defined in conv_weight_grad_fused.cu.  Asked for all shapes but
 // one (and refusing those that it has no band for, see make_fused_conv_plan): a 1 x 1 filter of stride 1 on planes of whole 16-byte groups is a
 // plain GEMM on the decompressed tensor without any further copy, and the dense path's TMA tiles then mostly beat the producer
-// warps.  Batch 64, dense / fused: 56 x 56 64 -> 256 38 / 62, 256 -> 256 79 / 117, 256 -> 64 54.7 / 52.4; 28 x 28 512 -> 512 64 / 119; the fused
-// kernel is ahead on small planes and batches (8 x 8 256 -> 256 17 / 13, batch 8 28 x 28 256 -> 256 18.6 / 15.5), which this line leaves out.
+// warps.  Batch 64, dense / fused: 56 x 56 64 -> 256 38 / 61, 256 -> 256 79 / 116, 256 -> 64 54.4 / 55.1; 28 x 28 512 -> 512 65 / 119; the fused
+// kernel is ahead on small planes and batches (8 x 8 256 -> 256 16.5 / 11.7, 2048 -> 512 66 / 46, batch 8 28 x 28 256 -> 256 18.3 / 14.7), which this
+// line leaves out.
 size_t conv_fused_workspace_bytes(int B, int Ca, int H, int W, int Cz, int R, int S, int stride, int pad);
 dropit_status conv_fused_run(const void* dy, const void* values, const void* mask, const uint32_t* offsets, int B, int Ca, int H,
                              int W, int Cz, int R, int S, int stride, int pad, int64_t k, float* dw, int accumulate,

@@ -21,15 +21,18 @@
 // Stride 2 keeps the even and the odd padded columns in separate planes.  The reduction is split over the CTAs; every split
 // stores its accumulator as it comes out of tensor memory and a second kernel adds the splits in order.
 //
-// Bound by the producers (some 400 warp instructions per 64 pixels x 8 channels of X, everything included; 13.7 M for 64 -> 64 on
-// 56 x 56), which wait for the values' trip through L2 and for shared memory at four warps a scheduler (issue slots 40 % busy); both lanes' pixels of a pair share one mask lookup, the mask words are requested a task ahead and
-// the loads of a warp's first task are under way before it waits for the stage, so that one trip to memory per band is
-// exposed.  The taps of a K step share the dY operand in the collector.  16 producer warps: 20 (80 registers) are up to 8 %
-// slower.  Measured per call at batch 64, gamma 0.8 (graph replay), dense copies of conv_weight_grad_tc.cu (decompression,
-// shifted or gathered copies, GEMM on 64-pixel rows) -> dY transposed through registers (15.6 M instructions, and
-// its loads not in flight during the work on X) -> now: 3 x 3 64 -> 64 on 56 x 56 59 -> 50 -> 37 us, 128 -> 128 on 28 x 28 131 -> 39 -> 36,
-// 256 -> 256 on 14 x 14 125 -> 45 -> 43, 512 -> 512 on 7 x 7 334 -> 86 -> 81, stride 2 128 -> 128 on 56 x 56 213 -> 59 -> 55;
-// 1 x 1 of stride 2 256 -> 512 on 56 x 56 292 -> 129 -> 117.
+// Bound by filling the stages: some 400 warp instructions per 64 pixels x 8 channels of X, everything included (13.7 M for 64 -> 64 on
+// 56 x 56), at four warps a scheduler, which wait for the values' trip through L2 and for shared memory (issue slots 40 % busy); both lanes'
+// pixels of a pair share one mask lookup, the mask words are requested a task ahead and the loads of a warp's first task are under way before it
+// waits for the stage, so that one trip to memory per band is exposed.  The taps of a K step share the dY operand in the collector.  16
+// producer warps: 20 (80 registers) are up to 8 % slower.  64 images, gamma 0.8, graph replay, a whole call / filling by itself / the product by
+// itself / launches, epilogue and reduction (by handing over stages that were not filled, and by leaving all MMAs but one out): 3 x 3
+// 64 -> 64 on 56 x 56 36.1 / 21.4 / 13.1 / 10.7 us (525 MMAs of 128 x 96 x 16 at 49 cycles, the full rate; half of their rows are unused),
+// 256 -> 256 on 14 x 14 34.0 / 15.5 / 9.2 / 15.2, 512 -> 512 on 7 x 7 53.9 / 25.4 / 9.0 / 24.8, 128 -> 128 on 28 x 28 33.3 / 17.1 / 9.0 / 13.0, stride 2
+// 128 -> 128 on 56 x 56 53.2 / 37.8 / 7.7 / 14.9.  Where it came from, over rotating inputs: dense copies of conv_weight_grad_tc.cu (decompression,
+// shifted or gathered copies, GEMM on 64-pixel rows) -> dY transposed through registers -> dY copied as it lies, before the reduction had
+// forms: 64 -> 64 on 56 x 56 59 -> 50 -> 37 us, 28 x 28 131 -> 39 -> 36, 14 x 14 125 -> 45 -> 43, 7 x 7 334 -> 86 -> 81, stride 2 on 56 x 56
+// 213 -> 59 -> 55; 1 x 1 of stride 2 256 -> 512 on 56 x 56 292 -> 129 -> 117.
 #include <cstring>
 #include <type_traits>
 
@@ -649,8 +652,9 @@ __device__ __noinline__ void mend_nonfinite(const FusedConvParams& p, const Bloc
 // channels and TAPS of the filter's taps (CHANNELS, 1 x 1 filters: TAPS times four channels); its eight warps share out the splits.
 // Sums that are not finite are looked at again (mend_nonfinite).
 // All taps of a channel in one block write whole stretches of dW (144 bytes of a row of 3 x 3 filters, where one tap wrote 4 bytes in
-// every 36), keep nine loads per thread in flight and are a ninth of the blocks.  Per call at batch 64, gamma 0.8: 3 x 3 256 -> 256 on
-// 14 x 14 46.6 -> 38.4 us, 512 -> 512 on 7 x 7 98.7 -> 71.2, stride 2 256 -> 256 on 28 x 28 67.7 -> 59.5.
+// every 36), keep nine loads per thread in flight and are a ninth of the blocks.  256 -> 256 on 14 x 14, 64 images, against one tap per block:
+// 4.9 sectors a store request instead of 32, 130 k sectors written to L2 instead of 885 k, 2.5 M warp instructions instead of 10.9 M; per call
+// 43.3 -> 35.0 us, 512 -> 512 on 7 x 7 82.2 -> 57.6, stride 2 256 -> 256 on 28 x 28 64.3 -> 56.1 (with the divisions behind the loads 33.8, 53.5, 53.6).
 template <int TAPS, bool CHANNELS = false>
 __global__ void __launch_bounds__(32 * kRedWarps, TAPS == 1 ? 5 : (TAPS < 9 ? 4 : 2))
 conv_fused_reduce_kernel(const float4* __restrict__ partial, const __grid_constant__ FusedConvParams p, float* __restrict__ dw, int accumulate) {
@@ -942,8 +946,10 @@ dropit_status conv_fused_run(const void* dy, const void* values, const void* mas
     dropit_status st = check_launch();
     if (st != DROPIT_OK) return st;
     const int quarters = ((Cz < kBM ? Cz : kBM) + 31) / 32, sets = R * S, blocks = tiles * quarters * (p.cb / 4);
-    // as many taps (channels) per block as leave two blocks per SM: 64 -> 64 on 56 x 56 (32 blocks with nine taps, 96 with three) 43.4 /
-    // 41.3 us against 41.4 with one, 16 images of it 21.9 / 19.4 / 19.5; stride 2 128 -> 128 on 56 x 56 (144 / 432) 57.4 / 56.6 / 58.4
+    // As many taps (channels) per block as leave two blocks per SM.  One / three / nine taps (blocks with nine): 64 -> 64 on 56 x 56 (32)
+    // 35.9 / 36.6 / 38.2 us, 8 images of 40 -> 72 on 23 x 23 (36) 12.3 / 12.8 / 15.1, stride 2 128 -> 128 on 56 x 56 (144) 55.2 / 53.5 / 54.7, 8 images
+    // of 64 -> 320 on 13 x 13 (176) 14.6 / 11.9 / 12.5, 32 images of 200 -> 312 on 9 x 9 (720) 35.8 / 29.9 / 28.9, of 512 -> 512 on 7 x 7 (2112),
+    // 8 images, 48.3 / 32.9 / 29.1.
     const int least = 2 * sm_count();
     const int per = sets == 1 ? (blocks / 4 >= least ? 4 : 1)
                               : (sets == 9 && blocks >= least ? 9 : (sets % 3 == 0 && blocks * (sets / 3) >= least ? 3 : 1));
