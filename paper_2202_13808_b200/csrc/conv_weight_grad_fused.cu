@@ -663,14 +663,18 @@ conv_fused_reduce_kernel(const float4* __restrict__ partial, const __grid_consta
     __shared__ float4 sums[kRedWarps][TAPS][32];
     __shared__ float out[32 * kPitch];                  // [row][channel][tap]
     const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
-    // Blocks: (32 rows of a tile, groups of channels and sets of taps, tile).  The columns of the partial tiles are in the order [v][u][channel]:
+    // Blocks: (32 rows, groups of channels and sets of taps, block of channels).  The columns of the partial tiles are in the order [v][u][channel]:
     // with one tap per block, or none but channels, blockIdx.y counts them as they lie.  What else the block's number says is worked out behind
     // the loads: with the divisions in front of them calls of 8 images took 14.7 instead of 13.6 us (64 -> 64 on 56 x 56), 13.1 / 11.8 (40 -> 72
     // on 23 x 23), 32.7 / 28.7 (512 -> 512 on 7 x 7).
-    const int groups = p.cb / (CHANNELS ? 4 * TAPS : 4), quarter = blockIdx.x, tile = blockIdx.z;
+    const int groups = p.cb / Block::kChannels, j0 = 32 * blockIdx.x, quarter = blockIdx.x % (kBM / 32);
+    const int tile = (int)(blockIdx.x / (kBM / 32)) * p.tiles_c + blockIdx.z, c0 = blockIdx.z * p.cb;
     const int tap_set = TAPS == 3 ? (int)blockIdx.y / groups : 0;      // (nine taps are all there are)
-    const uint32_t first = CHANNELS ? blockIdx.y * TAPS : blockIdx.y - (uint32_t)(tap_set * groups);
+    int group = (int)blockIdx.y - tap_set * groups;
+    const uint32_t first = CHANNELS ? group * TAPS : group;
     ptx::grid_dependency_wait();                        // the partial tiles come from the kernel before this one
+    // Groups behind the last channel; one tap per block has to divide to tell, and does so later.
+    if (TAPS > 1 && c0 + group * Block::kChannels >= p.Ca) return;
     const size_t plane = (size_t)p.tiles_c * p.tiles_j * p.chunks * 8 * kBM;
     const float4* src = partial + ((size_t)tile * p.chunks * 8 + first) * kBM + 32 * quarter + lane;
     uint32_t at[TAPS];
@@ -711,17 +715,14 @@ conv_fused_reduce_kernel(const float4* __restrict__ partial, const __grid_consta
     }
 #pragma unroll
     for (int t = 0; t < TAPS; ++t) sums[g][t][lane] = acc[t];
-    int group = first, tap0 = tap_set * TAPS;
+    int tap0 = tap_set * TAPS;
     if constexpr (TAPS == 1) {
         const int column = group / groups, v = column / p.R;
         group -= column * groups;
         tap0 = (column - v * p.R) * p.S + v;
-    } else if constexpr (CHANNELS) {
-        group = blockIdx.y;
     }
-    const int tile_j = tile / p.tiles_c, j0 = tile_j * kBM + 32 * quarter;
-    const int c = (tile - tile_j * p.tiles_c) * p.cb + group * (CHANNELS ? 4 * TAPS : 4);
-    if (c >= p.Ca || j0 >= p.Cz) return;                // (what such a block has read is not used)
+    const int c = c0 + group * Block::kChannels;
+    if (TAPS == 1 && c >= p.Ca) return;
     __syncthreads();
     bool odd = false;
     for (int i = threadIdx.x; i < 32 * TAPS; i += 32 * kRedWarps) {
@@ -955,7 +956,7 @@ dropit_status conv_fused_run(const void* dy, const void* values, const void* mas
                               : (sets == 9 && blocks >= least ? 9 : (sets % 3 == 0 && blocks * (sets / 3) >= least ? 3 : 1));
     auto reduce = per == 9 ? conv_fused_reduce_kernel<9> : (per == 4 ? conv_fused_reduce_kernel<4, true>
                                                                      : (per == 3 ? conv_fused_reduce_kernel<3> : conv_fused_reduce_kernel<1>));
-    cfg.gridDim = dim3((unsigned)quarters, (unsigned)(per == 4 ? p.cb / 16 : p.cb / 4 * (sets / per)), (unsigned)tiles);
+    cfg.gridDim = dim3((unsigned)((Cz + 31) / 32), (unsigned)(per == 4 ? p.cb / 16 : p.cb / 4 * (sets / per)), (unsigned)p.tiles_c);
     cfg.blockDim = dim3(32 * kRedWarps);
     cfg.dynamicSmemBytes = 0;
     p.dy = reinterpret_cast<const uint16_t*>(dy);
