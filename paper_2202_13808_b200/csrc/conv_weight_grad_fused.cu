@@ -949,8 +949,8 @@ dropit_status conv_fused_run(const void* dy, const void* values, const void* mas
     const int quarters = ((Cz < kBM ? Cz : kBM) + 31) / 32, sets = R * S, blocks = tiles * quarters * (p.cb / 4);
     // As many taps (channels) per block as leave two blocks per SM.  One / three / nine taps (blocks with nine): 64 -> 64 on 56 x 56 (32)
     // 35.9 / 36.6 / 38.2 us, 8 images of 40 -> 72 on 23 x 23 (36) 12.3 / 12.8 / 15.1, stride 2 128 -> 128 on 56 x 56 (144) 55.2 / 53.5 / 54.7, 8 images
-    // of 64 -> 320 on 13 x 13 (176) 14.6 / 11.9 / 12.5, 32 images of 200 -> 312 on 9 x 9 (720) 35.8 / 29.9 / 28.9, of 512 -> 512 on 7 x 7 (2112),
-    // 8 images, 48.3 / 32.9 / 29.1.
+    // of 64 -> 320 on 13 x 13 (176) 14.6 / 11.9 / 12.5, 256 -> 256 on 14 x 14 (576) 40.2 / 34.2 / 33.9, 8 images of 512 -> 512 on 7 x 7 (2112)
+    // 48.3 / 32.9 / 29.1.
     const int least = 2 * sm_count();
     const int per = sets == 1 ? (blocks / 4 >= least ? 4 : 1)
                               : (sets == 9 && blocks >= least ? 9 : (sets % 3 == 0 && blocks * (sets / 3) >= least ? 3 : 1));
